@@ -350,6 +350,13 @@ moe_status moe_dispatch_layout_static(const int32_t* topk_idx, int32_t T, int32_
                                       int32_t* counts, int32_t* offsets, int32_t* perm, int32_t* inv_perm,
                                       void* cuda_stream);
 
+/* One whole step on device arrays: moe_route, moe_dispatch_layout, moe_grouped_ffn and moe_combine in order, with the
+ * arguments of each; returns the status of the first that fails (the step is then where that call left it). */
+moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias, const void* x, int32_t T,
+                     int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
+                     int32_t* inv_perm, const void* w_gate_up, const void* w_down, const void* ws_gate_up,
+                     const void* ws_down, void* out);
+
 /* One whole step with HOST activations: copies logits_host [T,E] fp32 and x_host [T,H] bf16
  * to the device (cudaMemcpyAsync into context-owned staging), runs a1..a9, copies out
  * [T,H] bf16 back to out_host and synchronises the stream before returning.  Pinned host

@@ -29,7 +29,7 @@ STATUS_NAMES = {0: "MOE_OK", 1: "MOE_ERR_INVALID_ARG", 2: "MOE_ERR_CAPACITY", 3:
 # every symbol include/moe_pd.h declares
 EXPORTS = ("moe_version", "moe_ctx_workspace_bytes", "moe_ctx_create", "moe_ctx_destroy", "moe_ctx_status",
            "moe_last_error", "moe_route", "moe_dispatch_layout", "moe_grouped_ffn", "moe_grouped_ffn_fp8", "moe_combine",
-           "moe_layer_host", "moe_layer_host_submit", "moe_layer_host_wait",
+           "moe_layer", "moe_layer_host", "moe_layer_host_submit", "moe_layer_host_wait",
            "moe_ctx_debug_ptrs", "moe_ctx_debug_ptrs_fp8", "moe_ctx_launch_count", "moe_ctx_set_profiling", "moe_ctx_read_profile",
            "moe_dispatch_layout_static", "moe_ctx_set_segments", "moe_ctx_abandon_step", "moe_turnstile_create", "moe_turnstile_destroy",
            "moe_turnstile_set_span", "moe_turnstile_begin_epoch", "moe_turnstile_publish", "moe_turnstile_task_done",
@@ -99,6 +99,8 @@ def load_library() -> ctypes.CDLL:
     lib.moe_grouped_ffn_fp8.argtypes = [vp] * 9 + [i32]
     lib.moe_combine.restype = i32
     lib.moe_combine.argtypes = [vp, vp, vp, i32, vp]
+    lib.moe_layer.restype = i32
+    lib.moe_layer.argtypes = [vp] * 4 + [i32] + [vp] * 11
     lib.moe_layer_host.restype = i32
     lib.moe_layer_host.argtypes = [vp, vp, vp, vp, i32, vp, vp, vp, vp, vp]
     lib.moe_layer_host_submit.restype = i32
@@ -158,13 +160,17 @@ def _ptr(t: Optional[torch.Tensor]):
     return ctypes.c_void_p(t.data_ptr())
 
 
-def _dev(t: Optional[torch.Tensor], dtype, name):
+def _arg(t: Optional[torch.Tensor], dtype, name: str):
+    """Device address of a contiguous CUDA tensor of the given type (None stays None)."""
     if t is None:
-        return
-    if not t.is_cuda:
-        raise ValueError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
+        return None
+    if t.dtype is not dtype or not t.is_cuda:
+        if not t.is_cuda:
+            raise ValueError(f"{name} must be a CUDA tensor")
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
+    if not t.is_contiguous():
+        raise ValueError("tensor must be contiguous")
+    return t.data_ptr()
 
 
 def make_config(hidden, n_experts, top_k, inter, shared_inter=0, max_tokens=1, phase=MOE_PHASE_PREFILL, sm_budget=0,
@@ -288,32 +294,30 @@ class MoeContext:
         return {n: (float(t.ms[i]), int(t.calls[i])) for i, n in enumerate(STAGE_NAMES)}
 
     def moe_route(self, logits, select_bias, topk_idx, topk_w, T=None):
-        _dev(logits, torch.float32, "logits"); _dev(select_bias, torch.float32, "select_bias")
-        _dev(topk_idx, torch.int32, "topk_idx"); _dev(topk_w, torch.float32, "topk_w")
         T = logits.shape[0] if T is None else T
-        self._check(self.lib.moe_route(self.handle, _ptr(logits), _ptr(select_bias), T, _ptr(topk_idx), _ptr(topk_w)))
+        self._check(self.lib.moe_route(self.handle, _arg(logits, torch.float32, "logits"),
+                                       _arg(select_bias, torch.float32, "select_bias"), T,
+                                       _arg(topk_idx, torch.int32, "topk_idx"), _arg(topk_w, torch.float32, "topk_w")))
 
     def moe_dispatch_layout(self, topk_idx, x, counts=None, offsets=None, perm=None, inv_perm=None, T=None):
-        _dev(topk_idx, torch.int32, "topk_idx"); _dev(x, torch.bfloat16, "x")
-        for n, t in (("counts", counts), ("offsets", offsets), ("perm", perm), ("inv_perm", inv_perm)):
-            _dev(t, torch.int32, n)
         T = topk_idx.shape[0] if T is None else T
-        self._check(self.lib.moe_dispatch_layout(self.handle, _ptr(topk_idx), T, _ptr(x), _ptr(counts), _ptr(offsets),
-                                                 _ptr(perm), _ptr(inv_perm)))
+        i32 = torch.int32
+        self._check(self.lib.moe_dispatch_layout(self.handle, _arg(topk_idx, i32, "topk_idx"), T,
+                                                 _arg(x, torch.bfloat16, "x"), _arg(counts, i32, "counts"),
+                                                 _arg(offsets, i32, "offsets"), _arg(perm, i32, "perm"),
+                                                 _arg(inv_perm, i32, "inv_perm")))
 
     def moe_dispatch_notify(self, topk_idx, counts=None, offsets=None, perm=None, inv_perm=None, T=None):
         """First half of a split dispatch (counts, scan, permutation); the context then holds a pending dispatch."""
-        _dev(topk_idx, torch.int32, "topk_idx")
-        for n, t in (("counts", counts), ("offsets", offsets), ("perm", perm), ("inv_perm", inv_perm)):
-            _dev(t, torch.int32, n)
         T = topk_idx.shape[0] if T is None else T
-        self._check(self.lib.moe_dispatch_notify(self.handle, _ptr(topk_idx), T, _ptr(counts), _ptr(offsets),
-                                                 _ptr(perm), _ptr(inv_perm)))
+        i32 = torch.int32
+        self._check(self.lib.moe_dispatch_notify(self.handle, _arg(topk_idx, i32, "topk_idx"), T,
+                                                 _arg(counts, i32, "counts"), _arg(offsets, i32, "offsets"),
+                                                 _arg(perm, i32, "perm"), _arg(inv_perm, i32, "inv_perm")))
 
     def moe_dispatch_move(self, x):
         """Second half: the routed data movement of the pending dispatch."""
-        _dev(x, torch.bfloat16, "x")
-        self._check(self.lib.moe_dispatch_move(self.handle, _ptr(x)))
+        self._check(self.lib.moe_dispatch_move(self.handle, _arg(x, torch.bfloat16, "x")))
 
     def moe_ctx_pending_dispatch(self) -> dict:
         p, t, d = ctypes.c_int32(0), ctypes.c_int32(0), ctypes.c_int32(0)
@@ -321,32 +325,28 @@ class MoeContext:
         return {"pending": bool(p.value), "tokens": int(t.value), "notified_done": bool(d.value)}
 
     def moe_grouped_ffn(self, w_gate_up, w_down, x, ws_gate_up=None, ws_down=None, T=None):
-        for n, t in (("w_gate_up", w_gate_up), ("w_down", w_down), ("x", x), ("ws_gate_up", ws_gate_up),
-                     ("ws_down", ws_down)):
-            _dev(t, torch.bfloat16, n)
         T = x.shape[0] if T is None else T
-        self._check(self.lib.moe_grouped_ffn(self.handle, _ptr(w_gate_up), _ptr(w_down), _ptr(x), _ptr(ws_gate_up),
-                                             _ptr(ws_down), T))
+        bf16 = torch.bfloat16
+        self._check(self.lib.moe_grouped_ffn(self.handle, _arg(w_gate_up, bf16, "w_gate_up"),
+                                             _arg(w_down, bf16, "w_down"), _arg(x, bf16, "x"),
+                                             _arg(ws_gate_up, bf16, "ws_gate_up"), _arg(ws_down, bf16, "ws_down"), T))
 
     def moe_grouped_ffn_fp8(self, wq_gate_up, sw_gate_up, wq_down, sw_down, wsq_gate_up=None, sws_gate_up=None,
                             wsq_down=None, sws_down=None, T=None):
         """wq_* are uint8 tensors of E4M3 codes, sw_* fp32 per-output-channel scales."""
-        for n, t in (("wq_gate_up", wq_gate_up), ("wq_down", wq_down), ("wsq_gate_up", wsq_gate_up),
-                     ("wsq_down", wsq_down)):
-            _dev(t, torch.uint8, n)
-        for n, t in (("sw_gate_up", sw_gate_up), ("sw_down", sw_down), ("sws_gate_up", sws_gate_up),
-                     ("sws_down", sws_down)):
-            _dev(t, torch.float32, n)
         if T is None:
             raise ValueError("T is required")
-        self._check(self.lib.moe_grouped_ffn_fp8(self.handle, _ptr(wq_gate_up), _ptr(sw_gate_up), _ptr(wq_down),
-                                                 _ptr(sw_down), _ptr(wsq_gate_up), _ptr(sws_gate_up), _ptr(wsq_down),
-                                                 _ptr(sws_down), T))
+        u8, f32 = torch.uint8, torch.float32
+        self._check(self.lib.moe_grouped_ffn_fp8(self.handle, _arg(wq_gate_up, u8, "wq_gate_up"),
+                                                 _arg(sw_gate_up, f32, "sw_gate_up"), _arg(wq_down, u8, "wq_down"),
+                                                 _arg(sw_down, f32, "sw_down"), _arg(wsq_gate_up, u8, "wsq_gate_up"),
+                                                 _arg(sws_gate_up, f32, "sws_gate_up"),
+                                                 _arg(wsq_down, u8, "wsq_down"), _arg(sws_down, f32, "sws_down"), T))
 
     def moe_combine(self, topk_w, inv_perm, out, T=None):
-        _dev(topk_w, torch.float32, "topk_w"); _dev(inv_perm, torch.int32, "inv_perm"); _dev(out, torch.bfloat16, "out")
         T = out.shape[0] if T is None else T
-        self._check(self.lib.moe_combine(self.handle, _ptr(topk_w), _ptr(inv_perm), T, _ptr(out)))
+        self._check(self.lib.moe_combine(self.handle, _arg(topk_w, torch.float32, "topk_w"),
+                                         _arg(inv_perm, torch.int32, "inv_perm"), T, _arg(out, torch.bfloat16, "out")))
 
     def moe_layer_host(self, logits_host, select_bias, x_host, w_gate_up, w_down, ws_gate_up, ws_down, out_host,
                        T=None):
@@ -403,22 +403,30 @@ class MoeContext:
         if out is None:
             out = torch.empty(T, self.cfg.hidden, dtype=torch.bfloat16, device=device)
             fresh.append(out)
-        cur = torch.cuda.current_stream(self.device)
-        if fresh and cur != self.stream:
-            self.stream.wait_stream(cur)
-            for t in fresh:
-                t.record_stream(self.stream)
+        if fresh:
+            cur = torch.cuda.current_stream(self.device)
+            if cur != self.stream:
+                self.stream.wait_stream(cur)
+                for t in fresh:
+                    t.record_stream(self.stream)
         return bufs, out
 
-    # -- convenience: one whole step on device tensors (calls the four entry points in order)
+    # -- convenience: one whole step on device tensors (the four entry points in order, in one call: a step's host time
+    # is what bounds the smallest ones)
     def layer(self, x, logits, select_bias, w_gate_up, w_down, ws_gate_up=None, ws_down=None, out=None, bufs=None):
         T, k, E = x.shape[0], self.cfg.top_k, self.cfg.n_experts
-        bufs, out = self._step_tensors(T, k, E, x.device, bufs, out)
-        self.moe_route(logits, select_bias, bufs["topk_idx"], bufs["topk_w"], T=T)
-        self.moe_dispatch_layout(bufs["topk_idx"], x, bufs["counts"], bufs["offsets"], bufs["perm"], bufs["inv_perm"],
-                                 T=T)
-        self.moe_grouped_ffn(w_gate_up, w_down, x, ws_gate_up, ws_down, T=T)
-        self.moe_combine(bufs["topk_w"], bufs["inv_perm"], out, T=T)
+        if bufs is None or out is None:
+            bufs, out = self._step_tensors(T, k, E, x.device, bufs, out)
+        i32, f32, bf16 = torch.int32, torch.float32, torch.bfloat16
+        st = self.lib.moe_layer(self.handle, _arg(logits, f32, "logits"), _arg(select_bias, f32, "select_bias"),
+                                _arg(x, bf16, "x"), T, _arg(bufs["topk_idx"], i32, "topk_idx"),
+                                _arg(bufs["topk_w"], f32, "topk_w"), _arg(bufs["counts"], i32, "counts"),
+                                _arg(bufs["offsets"], i32, "offsets"), _arg(bufs["perm"], i32, "perm"),
+                                _arg(bufs["inv_perm"], i32, "inv_perm"), _arg(w_gate_up, bf16, "w_gate_up"),
+                                _arg(w_down, bf16, "w_down"), _arg(ws_gate_up, bf16, "ws_gate_up"),
+                                _arg(ws_down, bf16, "ws_down"), _arg(out, bf16, "out"))
+        if st != MOE_OK:
+            self._check(st)
         return out, bufs
 
     def layer_fp8(self, x, logits, select_bias, w8: dict, out=None, bufs=None):
@@ -453,12 +461,12 @@ def moe_dispatch_layout_static(topk_idx, n_experts, counts, offsets, perm, inv_p
     lib = load_library()
     T = topk_idx.shape[0] if T is None else T
     top_k = topk_idx.shape[1] if top_k is None else top_k
-    for n, t in (("topk_idx", topk_idx), ("counts", counts), ("offsets", offsets), ("perm", perm), ("inv_perm", inv_perm)):
-        _dev(t, torch.int32, n)
+    i32 = torch.int32
+    args = [_arg(t, i32, n) for n, t in (("topk_idx", topk_idx), ("counts", counts), ("offsets", offsets),
+                                         ("perm", perm), ("inv_perm", inv_perm))]
     s = stream if stream is not None else torch.cuda.current_stream(topk_idx.device)
     with torch.cuda.device(topk_idx.device):
-        return int(lib.moe_dispatch_layout_static(_ptr(topk_idx), T, top_k, n_experts, _ptr(counts), _ptr(offsets),
-                                                  _ptr(perm), _ptr(inv_perm), ctypes.c_void_p(s.cuda_stream)))
+        return int(lib.moe_dispatch_layout_static(args[0], T, top_k, n_experts, *args[1:], ctypes.c_void_p(s.cuda_stream)))
 
 
 class Turnstile:

@@ -207,6 +207,8 @@ struct moe_ctx {
   std::mutex* yield_mu;
   int* stopped_host;  // pinned host word: CTAs that stopped in the last launch
   int64_t yields;     // launches that ended on a yield request
+  bool unmarked;      // launches have been enqueued since `done` was last recorded
+  moe::StreamPlan* plans[2][4];  // tensor maps of the small-M GEMM: [buffer set][2 * (dense problem by itself) + down pass]
   unsigned long long wait_limit_ns;  // time limit of every bounded device-side wait (0 = the kernels' default)
   bool debug_stall;                  // failure-detection hook: the GEMM producers issue no copies
   char err[256];
@@ -253,11 +255,19 @@ bool capturing(const moe_ctx* ctx) {
   return st != cudaStreamCaptureStatusNone;
 }
 
-// After the last enqueue of a call: count the launches and mark the stream position.  While the stream is
-// being captured into a CUDA graph nothing executes, so there is no position to mark (and an event recorded
-// during capture could not be queried later).
+// After the last enqueue of a call: count the launches.
 void mark(moe_ctx* ctx, int n) {
   ctx->launches += n;
+  ctx->unmarked = true;
+}
+
+// Marks the stream position that moe_ctx_destroy asks about: at the end of a step (an event record between two kernels
+// of a step would cost host time on every call), or when a step is given up.  While the stream is being captured into a
+// CUDA graph nothing executes, so there is no position to mark (and an event recorded during capture could not be
+// queried later).
+void mark_position(moe_ctx* ctx) {
+  if (!ctx->unmarked) return;
+  ctx->unmarked = false;
   if (!capturing(ctx)) cudaEventRecord(ctx->done, ctx->stream);
 }
 
@@ -284,6 +294,12 @@ struct StageTimer {
     if (span) cudaEventRecord(span->end, ctx->stream);
   }
 };
+
+void free_ctx(moe_ctx* ctx) {
+  for (auto& set : ctx->plans)
+    for (moe::StreamPlan* plan : set) moe::stream_plan_destroy(plan);
+  delete ctx;
+}
 
 int gemm_ctas(const moe_ctx* ctx) {
   return (ctx->cfg.sm_budget > 0 && ctx->cfg.sm_budget < ctx->n_sms) ? ctx->cfg.sm_budget : ctx->n_sms;
@@ -349,6 +365,7 @@ cudaError_t run_gemm(moe_ctx* ctx, moe::GemmProblem p, const moe::GemmDenseGroup
   p.offsets_settled = true;
   p.tile_counters = reinterpret_cast<int*>(ctx->ws + kTileCounterOffset) + 2 * (ctx->gemm_seq++ % kTileCounterPairs);
   p.max_group_rows = T;
+  p.plan = ctx->plans[ctx->cur][(p.offsets == nullptr ? 2 : 0) + (p.gated ? 0 : 1)];
   if (variant == MOE_GEMM_VALIDATION) {
     cudaError_t e = moe::launch_gemm_validation(p, ctx->stream, n);
     if (e == cudaSuccess && dense != nullptr) {
@@ -460,6 +477,17 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
   ctx->status = reinterpret_cast<int*>(ctx->ws);
   for (int s = 0; s < l.n_sets; ++s) carve_set(*cfg, ctx->ws + kStatusBlock + (size_t)s * l.set_bytes, &ctx->sets[s]);
   ctx->host_pipeline = false;
+  ctx->unmarked = false;
+  bool have_plans = true;
+  for (int i = 0; i < 8; ++i) {
+    moe::StreamPlan*& plan = ctx->plans[i / 4][i % 4];
+    plan = i / 4 < l.n_sets ? moe::stream_plan_create() : nullptr;
+    if (i / 4 < l.n_sets && plan == nullptr) have_plans = false;
+  }
+  if (!have_plans) {
+    free_ctx(ctx);
+    return fail(nullptr, MOE_ERR_CUDA, "host allocation failed");
+  }
   ctx->wait_limit_ns = 0;
   ctx->debug_stall = false;
   ctx->preemptible = false;
@@ -485,11 +513,11 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
     std::lock_guard<std::mutex> lock(g_registry_mutex);
     for (const moe_ctx* o : g_registry) {
       if (o->device == ctx->device && ctx->ws < o->ws + o->ws_bytes && o->ws < ctx->ws + ctx->ws_bytes) {
-        delete ctx;
+        free_ctx(ctx);
         return fail(nullptr, MOE_ERR_STATE, "workspace overlaps the workspace of a live context");
       }
       if (o->device == ctx->device && o->stream == ctx->stream && o->cfg.phase != ctx->cfg.phase) {
-        delete ctx;
+        free_ctx(ctx);
         return fail(nullptr, MOE_ERR_STATE, "stream is already bound to a live context of the other phase");
       }
     }
@@ -514,7 +542,7 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
         break;
       }
     moe_status st = cuda_fail(nullptr, e, "context set-up");
-    delete ctx;
+    free_ctx(ctx);
     return st;
   }
   ctx->n_sms = sms;
@@ -525,6 +553,7 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
 moe_status moe_ctx_destroy(moe_ctx* ctx) {
   if (!ctx) return MOE_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
+  mark_position(ctx);  // (a step that stopped half way)
   cudaError_t q = cudaEventQuery(ctx->done);
   if (q == cudaErrorNotReady) return fail(ctx, MOE_ERR_STATE, "work is still in flight on the context's stream");
   if (q != cudaSuccess) (void)cudaGetLastError();
@@ -559,13 +588,17 @@ moe_status moe_ctx_destroy(moe_ctx* ctx) {
     cudaEventDestroy(sp.beg);
     cudaEventDestroy(sp.end);
   }
-  delete ctx;
+  free_ctx(ctx);
   return MOE_OK;
 }
 
 moe_status moe_ctx_abandon_step(moe_ctx* ctx) {
   if (!ctx) return MOE_ERR_INVALID_ARG;
   if (ctx->state == ST_IDLE) return MOE_OK;
+  {
+    DeviceGuard guard(ctx->device);
+    mark_position(ctx);
+  }
   ctx->state = ST_IDLE;
   ctx->T = 0;
   ctx->pending_dispatch = false;  // a pending dispatch is retired with the step
@@ -961,7 +994,19 @@ moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_per
   ctx->split_step = false;
   if (ctx->n_sets == 2) ctx->cur ^= 1;  // D: the next step works in the other buffer set
   mark(ctx, n);
+  mark_position(ctx);
   return MOE_OK;
+}
+
+moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias, const void* x, int32_t T,
+                     int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
+                     int32_t* inv_perm, const void* w_gate_up, const void* w_down, const void* ws_gate_up,
+                     const void* ws_down, void* out) {
+  moe_status st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
+  if (st == MOE_OK) st = moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm);
+  if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T);
+  if (st == MOE_OK) st = moe_combine(ctx, topk_w, inv_perm, T, out);
+  return st;
 }
 
 moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* select_bias, const void* x_host,

@@ -35,6 +35,8 @@
 #include <cuda_bf16.h>
 
 #include <cstdlib>
+#include <cstring>
+#include <new>
 
 #include "kernels.h"
 #include "tc_common.cuh"
@@ -812,6 +814,19 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   }
 }
 
+// What an operand's tensor maps depend on.
+struct OperandKey {
+  const void* W = nullptr;
+  const void* A = nullptr;
+  int64_t rows = 0;
+  int32_t groups = 0, n_feat = 0, K = 0;
+  bool gated = false, fp8 = false;
+  bool same_weights(const OperandKey& o) const {
+    return W == o.W && groups == o.groups && n_feat == o.n_feat && K == o.K && gated == o.gated && fp8 == o.fp8;
+  }
+  bool same_rows(const OperandKey& o) const { return A == o.A && rows == o.rows && K == o.K && fp8 == o.fp8; }
+};
+
 template <typename Kernel>
 cudaError_t launch_variant(Kernel kern, const CUtensorMap& mw, const CUtensorMap& mw2, const StreamMaps& xm,
                            const StreamParams& prm, int grid, size_t smem, cudaStream_t stream, bool overlap) {
@@ -821,6 +836,23 @@ cudaError_t launch_variant(Kernel kern, const CUtensorMap& mw, const CUtensorMap
 }
 
 }  // namespace
+
+struct StreamPlan {
+  OperandKey key, key2;  // the routed problem's and the dense group's
+  CUtensorMap mw, mw2;
+  StreamMaps xm;
+};
+
+StreamPlan* stream_plan_create() {
+  StreamPlan* p = new (std::nothrow) StreamPlan();
+  if (p != nullptr) {
+    memset(&p->mw, 0, sizeof p->mw);
+    memset(&p->mw2, 0, sizeof p->mw2);
+    memset(&p->xm, 0, sizeof p->xm);
+  }
+  return p;
+}
+void stream_plan_destroy(StreamPlan* plan) { delete plan; }
 
 cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense, int max_ctas, int* status,
                                cudaStream_t stream, int* n_launches) {
@@ -844,38 +876,53 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   const int e_end = (p.offsets && p.e_end >= 0) ? p.e_end : groups;
   if (e_begin < 0 || e_end > groups || e_begin >= e_end) return cudaErrorInvalidValue;
 
-  CUtensorMap mw, mw2;
-  StreamMaps xm;
   // Weights: one box holds both 128-row weight boxes of a k-block.  Gated pass: [groups][2][n_feat][K] with a box
   // of 128 rows x 2 (gate rows and the matching up rows); down pass: [groups][n_feat][K] with a box of 256 rows.
-  auto encode_w = [&](CUtensorMap* m, const void* W, uint64_t K, uint64_t n_feat, uint64_t n_groups) {
-    if (p.gated) {
+  auto encode_w = [&](CUtensorMap* m, const OperandKey& k) {
+    const uint64_t K = (uint64_t)k.K, n_feat = (uint64_t)k.n_feat, n_groups = (uint64_t)k.groups;
+    if (k.gated) {
       const uint64_t dims[4] = {K, n_feat, 2, n_groups};
       const uint64_t str[3] = {K * esz, n_feat * K * esz, 2 * n_feat * K * esz};
       const uint32_t box[4] = {box_k, (uint32_t)kWBoxRows, 2u, 1u};
-      return encode_map(m, W, 4, dims, str, box, fp8);
+      return encode_map(m, k.W, 4, dims, str, box, fp8);
     }
     const uint64_t dims[3] = {K, n_feat, n_groups};
     const uint64_t str[2] = {K * esz, n_feat * K * esz};
     const uint32_t box[3] = {box_k, 2u * kWBoxRows, 1u};
-    return encode_map(m, W, 3, dims, str, box, fp8);
+    return encode_map(m, k.W, 3, dims, str, box, fp8);
   };
-  auto encode_x = [&](CUtensorMap* maps, const void* A, uint64_t K, uint64_t rows) {
-    for (int b = 0; b < kXMaps; ++b) {
-      const uint64_t dims[2] = {K, rows};
-      const uint64_t str[1] = {K * esz};
-      const uint32_t box[2] = {box_k, 16u * (uint32_t)(b + 1)};
-      if (!encode_map(&maps[b], A, 2, dims, str, box, fp8)) return false;
-    }
-    return true;
+  auto encode_x = [&](CUtensorMap* m, const OperandKey& k, int b) {  // the box of 16 (b + 1) rows
+    const uint64_t dims[2] = {(uint64_t)k.K, (uint64_t)k.rows};
+    const uint64_t str[1] = {(uint64_t)k.K * esz};
+    const uint32_t box[2] = {box_k, 16u * (uint32_t)(b + 1)};
+    return encode_map(m, k.A, 2, dims, str, box, fp8);
   };
-  if (!encode_w(&mw, p.W, (uint64_t)p.K, (uint64_t)p.n_feat, (uint64_t)groups)) return cudaErrorInvalidValue;
-  if (!encode_x(xm.x, p.A, (uint64_t)p.K, (uint64_t)p.rows_bound)) return cudaErrorInvalidValue;
-  mw2 = mw;
-  for (int b = 0; b < kXMaps; ++b) xm.x2[b] = xm.x[b];
+  // The routed rows' maps span the buffer's capacity, not this call's rows, so that a call with another T finds them as
+  // they are: a tile's last box may then read rows that an earlier, larger step left there; their columns of the
+  // accumulator are never stored.  The dense group has two box sizes at most (its equal chunks and the last one).
+  if (p.plan == nullptr) return cudaErrorInvalidValue;
+  StreamPlan& plan = *p.plan;
+  {
+    const OperandKey k{p.W, p.A, p.rows_cap, groups, p.n_feat, p.K, p.gated, fp8}, had = plan.key;
+    plan.key = OperandKey{};  // a failure half way leaves no valid key
+    if (!had.same_weights(k) && !encode_w(&plan.mw, k)) return cudaErrorInvalidValue;
+    if (!had.same_rows(k))
+      for (int b = 0; b < kXMaps; ++b)
+        if (!encode_x(&plan.xm.x[b], k, b)) return cudaErrorInvalidValue;
+    plan.key = k;
+  }
   if (dense != nullptr) {
-    if (!encode_w(&mw2, dense->W, (uint64_t)dense->K, (uint64_t)dense->n_feat, 1)) return cudaErrorInvalidValue;
-    if (!encode_x(xm.x2, dense->A, (uint64_t)dense->K, (uint64_t)dense->rows)) return cudaErrorInvalidValue;
+    const OperandKey k{dense->W, dense->A, dense->rows, 1, dense->n_feat, dense->K, p.gated, fp8}, had = plan.key2;
+    plan.key2 = OperandKey{};
+    if (!had.same_weights(k) && !encode_w(&plan.mw2, k)) return cudaErrorInvalidValue;
+    if (!had.same_rows(k)) {
+      const int chunks = (dense->rows + kMaxTileRows - 1) / kMaxTileRows;
+      const int chunk = ((dense->rows + chunks - 1) / chunks + 15) & ~15;
+      const int last = (dense->rows - (chunks - 1) * chunk + 15) & ~15;
+      if (!encode_x(&plan.xm.x2[chunk / 16 - 1], k, chunk / 16 - 1)) return cudaErrorInvalidValue;
+      if (last != chunk && !encode_x(&plan.xm.x2[last / 16 - 1], k, last / 16 - 1)) return cudaErrorInvalidValue;
+    }
+    plan.key2 = k;
   }
 
   StreamParams prm;
@@ -931,11 +978,11 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   const bool overlap = p.rows_bound <= kGemmOverlapMaxRows;
   cudaError_t err;
   if (fp8)
-    err = p.gated ? launch_variant(grouped_gemm_stream_kernel<true, true>, mw, mw2, xm, prm, grid, smem, stream, overlap)
-                  : launch_variant(grouped_gemm_stream_kernel<false, true>, mw, mw2, xm, prm, grid, smem, stream, overlap);
+    err = p.gated ? launch_variant(grouped_gemm_stream_kernel<true, true>, plan.mw, plan.mw2, plan.xm, prm, grid, smem, stream, overlap)
+                  : launch_variant(grouped_gemm_stream_kernel<false, true>, plan.mw, plan.mw2, plan.xm, prm, grid, smem, stream, overlap);
   else
-    err = p.gated ? launch_variant(grouped_gemm_stream_kernel<true, false>, mw, mw2, xm, prm, grid, smem, stream, overlap)
-                  : launch_variant(grouped_gemm_stream_kernel<false, false>, mw, mw2, xm, prm, grid, smem, stream, overlap);
+    err = p.gated ? launch_variant(grouped_gemm_stream_kernel<true, false>, plan.mw, plan.mw2, plan.xm, prm, grid, smem, stream, overlap)
+                  : launch_variant(grouped_gemm_stream_kernel<false, false>, plan.mw, plan.mw2, plan.xm, prm, grid, smem, stream, overlap);
   if (err == cudaSuccess && n_launches) *n_launches += 1;
   return err;
 }

@@ -82,6 +82,14 @@ cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32
                            void* out, int T, int k, int H, int* status, cudaStream_t stream, int* n_launches,
                            unsigned long long wait_limit_ns = 0);
 
+// Tensor maps of one small-M GEMM launch (host memory, opaque outside gemm_stream.cu).  A context keeps one plan per
+// buffer set and pass; a launch whose operands (addresses and shapes) are the plan's re-encodes nothing.  (Looking 34
+// maps up per launch in a locked table cost 3.4 us of host time; with that, an event record per call and four calls from
+// Python a 64-token step of the tiny layer took 36.4 us, all of it host time; 28.3 us now, bound by the GPU.)
+struct StreamPlan;
+StreamPlan* stream_plan_create();
+void stream_plan_destroy(StreamPlan* plan);
+
 // ---- a6-a8 grouped GEMM --------------------------------------------------------------------
 // One grouped GEMM pass:  out[r, :] = epilogue( A[r, :] . W[e]^T )  for r in expert e's segment.
 //   gated:     W[e] is [2*n_feat, K]; out[r,i] = silu(A.W[e,i]) * (A.W[e,n_feat+i]),  i < n_feat
@@ -135,6 +143,7 @@ struct GemmProblem {
   // Upper bound on the rows of any one group (a token reaches an expert at most once, so T), or 0 if unknown.  With
   // at most 16, every non-empty group is one tile of the same cost and the small-M kernel skips ordering them.
   int32_t max_group_rows = 0;
+  StreamPlan* plan = nullptr;  // small-M kernel: the launch's tensor maps
 };
 
 // A dense group (the shared expert) that rides in the same launch as a grouped problem: its tiles are added
