@@ -359,8 +359,10 @@ moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias
 
 /* One whole step with HOST activations: copies logits_host [T,E] fp32 and x_host [T,H] bf16
  * to the device (cudaMemcpyAsync into context-owned staging), runs a1..a9, copies out
- * [T,H] bf16 back to out_host and synchronises the stream before returning.  Pinned host
- * memory is recommended.  select_bias and all weights are DEVICE pointers as above. */
+ * [T,H] bf16 back to out_host and waits for all of it before returning.  With pinned host
+ * memory (recommended) the copies run on copy streams of the context and overlap the kernels:
+ * the output leaves in pieces of columns while the down pass computes the next, and a large
+ * prefill batch is cut into two chunks of tokens.  Results are those of the device calls, bit for bit.  select_bias and all weights are DEVICE pointers as above. */
 moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* select_bias, const void* x_host,
                           int32_t T, const void* w_gate_up, const void* w_down, const void* ws_gate_up,
                           const void* ws_down, void* out_host);

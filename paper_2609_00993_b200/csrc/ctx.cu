@@ -4,6 +4,7 @@
 
 #include <cstdarg>
 #include <cstdio>
+#include <algorithm>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -198,6 +199,7 @@ struct moe_ctx {
     bool in_flight;
   } slots[MOE_HOST_SLOTS];
   cudaStream_t h2d_stream, d2h_stream;
+  cudaEvent_t copied_in, computed;  // stream positions inside moe_layer_host (a wait takes the last record before it)
   bool host_pipeline;
   // preemption of prefill GEMM passes at tile granularity (off by default)
   bool preemptible;
@@ -324,6 +326,16 @@ int gemm_ctas(const moe_ctx* ctx) {
 constexpr int64_t kSmallMRowsGated = 1024, kSmallMRowsGatedShortKFrom = 448, kSmallMRowsDown = 320;
 constexpr int64_t kSmallMRowsFp8Gated = 256, kSmallMRowsFp8Down = 128;
 constexpr int kLongK = 4096, kShortDownK = 1536;
+
+// moe_layer_host: the down pass in one piece for every 1.5 MB of output, up to four; two chunks of tokens from 200 rows
+// per expert and 4 MB a chunk on.  Measured on the Qwen3-30B-shaped layer with pinned buffers (whole call; before: copy,
+// compute, copy):
+//   T = 1531   534 us -> 513 (rows behind the router's work), 486 with two or four pieces, 520 with eight
+//   T = 701    369 us -> 343 with two pieces, 352 with four;  hidden 2560, 512 experts, T = 5001: 2517 -> 2261 us with four
+//   two chunks against one: T = 2600 (162 rows per expert) 737 : 690 us, 3500 (219) 824 : 845, 5200 (325) 1066 : 1235,
+//   8192 (512) 1400 : 1957 before;  three or four chunks at 8192: 1466, 1590 us.
+constexpr size_t kHostPieceBytes = 1536 * 1024, kHostChunkBytes = 4 << 20;
+constexpr int kHostMaxPieces = 4, kHostChunkFromRows = 200;
 
 // AUTO: a DECODE context always streams; a PREFILL context chooses per launch from the problem's rows (T * top_k
 // rows over n_experts; T rows over one group for the shared expert by itself) and K: the choice is a function of T
@@ -567,6 +579,8 @@ moe_status moe_ctx_destroy(moe_ctx* ctx) {
       cudaEventDestroy(ctx->slots[s].comp);
       cudaEventDestroy(ctx->slots[s].done);
     }
+    cudaEventDestroy(ctx->copied_in);
+    cudaEventDestroy(ctx->computed);
     cudaStreamDestroy(ctx->h2d_stream);
     cudaStreamDestroy(ctx->d2h_stream);
   }
@@ -717,6 +731,130 @@ int ffn_boundaries(const moe_ctx* ctx) {
 
 }  // namespace
 
+namespace {
+
+// moe_grouped_ffn.  With piece_cols > 0 (an unsegmented step; a multiple of 256) the down pass runs in pieces of that many
+// output features, and after_piece(first, end) is called when each has been enqueued.
+template <class AfterPiece>
+moe_status grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, const void* x, const void* ws_gate_up,
+                       const void* ws_down, int32_t T, int piece_cols, AfterPiece after_piece) {
+  if (!ctx) return MOE_ERR_INVALID_ARG;
+  if (ctx->cfg.weight_format != MOE_WEIGHTS_BF16)
+    return fail(ctx, MOE_ERR_STATE, "the context was created for FP8 weights: call moe_grouped_ffn_fp8");
+  if (ctx->state != ST_LAID_OUT)
+    return fail(ctx, MOE_ERR_STATE, "moe_grouped_ffn needs a moe_dispatch_layout with x in the same step");
+  if (T != ctx->T) return fail(ctx, MOE_ERR_INVALID_ARG, "T = %d differs from the layout's T = %d", T, ctx->T);
+  if (!w_gate_up || !w_down) return fail(ctx, MOE_ERR_INVALID_ARG, "routed weights are NULL");
+  const bool shared = ctx->cfg.n_shared != 0;
+  if (shared && (!ws_gate_up || !ws_down || (!x && T > 0)))
+    return fail(ctx, MOE_ERR_INVALID_ARG, "the shared expert needs ws_gate_up, ws_down and x");
+  if (gathers_rows(ctx) && !x && T > 0) return fail(ctx, MOE_ERR_INVALID_ARG, "the row gather needs x");
+  if (misaligned(w_gate_up) || misaligned(w_down) || misaligned(x) || misaligned(ws_gate_up) || misaligned(ws_down))
+    return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
+  DeviceGuard guard(ctx->device);
+  BufferSet& b = ctx->sets[ctx->cur];
+  const moe_config& c = ctx->cfg;
+  const int64_t N = (int64_t)T * c.top_k, Ncap = (int64_t)c.max_tokens * c.top_k;
+  int n = 0;
+  cudaError_t e = cudaSuccess;
+  if (T > 0) {
+    // One launch per pass, or one per group of seg_experts experts with a boundary call after each.
+    const int span = (ctx->seg_experts > 0 && ctx->seg_experts < c.n_experts) ? ctx->seg_experts : c.n_experts;
+    const int routed_segs = (c.n_experts + span - 1) / span;
+    const int first = ctx->split_step ? 1 : 0;  // a split dispatch reported boundary 0 after its notification
+    const int n_bound = first + 2 * routed_segs + (shared ? 2 : 0);
+    int bound = first;
+    auto boundary = [&]() {
+      if (ctx->seg_experts > 0 && ctx->boundary_fn) {
+        if (!capturing(ctx)) cudaEventRecord(ctx->done, ctx->stream);
+        ctx->boundary_fn(ctx->boundary_user, bound, n_bound);
+      }
+      ++bound;
+    };
+    moe::GemmProblem g1{b.x_perm, w_gate_up, b.act, ctx->offsets, 0, Ncap, N, c.n_experts, c.inter, c.hidden, true};
+    moe::GemmProblem g2{b.act, w_down, b.y_perm, ctx->offsets, 0, Ncap, N, c.n_experts, c.hidden, c.inter, false};
+    if (gathers_rows(ctx)) {
+      g1.gather_src = x;
+      g1.perm = ctx->perm;
+      g1.top_k = c.top_k;
+    }
+    moe::GemmDenseGroup s1{x, ws_gate_up, b.act_shared, T, c.shared_inter, c.hidden};
+    moe::GemmDenseGroup s2{b.act_shared, ws_down, b.y_shared, T, c.hidden, c.shared_inter};
+    // Unsegmented: the shared expert's two passes ride in the routed launches (two launches in all).
+    // Segmented: they are segments of their own, after the routed ones.
+    const bool fuse_shared = shared && ctx->seg_experts == 0;
+    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+      moe::GemmProblem& g = pass == 0 ? g1 : g2;
+      for (int e0 = 0; e0 < c.n_experts && e == cudaSuccess; e0 += span) {
+        g.e_begin = e0;
+        g.e_end = e0 + span < c.n_experts ? e0 + span : c.n_experts;
+        const int step = pass == 1 && piece_cols > 0 ? piece_cols : g.n_feat;
+        for (int f0 = 0; f0 < g.n_feat && e == cudaSuccess; f0 += step) {
+          g.f_begin = f0;
+          g.f_end = f0 + step < g.n_feat ? f0 + step : g.n_feat;
+          {
+            StageTimer tm(ctx, pass == 0 ? 3 : 4);
+            e = run_gemm(ctx, g, fuse_shared ? (pass == 0 ? &s1 : &s2) : nullptr, T, &n);
+          }
+          if (pass == 1 && piece_cols > 0 && e == cudaSuccess) e = after_piece(g.f_begin, g.f_end);
+        }
+        if (e == cudaSuccess) boundary();
+      }
+    }
+    if (e == cudaSuccess && shared && !fuse_shared) {
+      moe::GemmProblem d1{s1.A, s1.W, s1.out, nullptr, T, T, T, 1, s1.n_feat, s1.K, true};
+      {
+        StageTimer tm(ctx, 5);
+        e = run_gemm(ctx, d1, nullptr, T, &n);
+      }
+      if (e == cudaSuccess) {
+        boundary();
+        moe::GemmProblem d2{s2.A, s2.W, s2.out, nullptr, T, T, T, 1, s2.n_feat, s2.K, false};
+        {
+          StageTimer tm(ctx, 6);
+          e = run_gemm(ctx, d2, nullptr, T, &n);
+        }
+        if (e == cudaSuccess) boundary();
+      }
+    }
+  }
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "moe_grouped_ffn");
+  ctx->state = ST_FFN_DONE;
+  mark(ctx, n);
+  return MOE_OK;
+}
+
+// The copy streams and events of the host path, created by its first call.
+moe_status ensure_host_streams(moe_ctx* ctx, const char* who) {
+  if (ctx->host_pipeline) return MOE_OK;
+  constexpr int kEvents = 3 * MOE_HOST_SLOTS + 2;
+  cudaEvent_t ev[kEvents] = {};
+  cudaStream_t st[2] = {};
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < kEvents && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&st[i], cudaStreamNonBlocking);
+  if (e != cudaSuccess) {
+    for (int i = 0; i < kEvents; ++i)
+      if (ev[i]) cudaEventDestroy(ev[i]);
+    for (int i = 0; i < 2; ++i)
+      if (st[i]) cudaStreamDestroy(st[i]);
+    return cuda_fail(ctx, e, who);
+  }
+  for (int s = 0; s < MOE_HOST_SLOTS; ++s) {
+    ctx->slots[s].h2d = ev[3 * s];
+    ctx->slots[s].comp = ev[3 * s + 1];
+    ctx->slots[s].done = ev[3 * s + 2];
+  }
+  ctx->copied_in = ev[kEvents - 2];
+  ctx->computed = ev[kEvents - 1];
+  ctx->h2d_stream = st[0];
+  ctx->d2h_stream = st[1];
+  ctx->host_pipeline = true;
+  return MOE_OK;
+}
+
+}  // namespace
+
 extern "C" {
 
 moe_status moe_dispatch_layout(moe_ctx* ctx, const int32_t* topk_idx, int32_t T, const void* x, int32_t* counts,
@@ -790,84 +928,7 @@ moe_status moe_ctx_pending_dispatch(moe_ctx* ctx, int32_t* pending, int32_t* tok
 
 moe_status moe_grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, const void* x,
                            const void* ws_gate_up, const void* ws_down, int32_t T) {
-  if (!ctx) return MOE_ERR_INVALID_ARG;
-  if (ctx->cfg.weight_format != MOE_WEIGHTS_BF16)
-    return fail(ctx, MOE_ERR_STATE, "the context was created for FP8 weights: call moe_grouped_ffn_fp8");
-  if (ctx->state != ST_LAID_OUT)
-    return fail(ctx, MOE_ERR_STATE, "moe_grouped_ffn needs a moe_dispatch_layout with x in the same step");
-  if (T != ctx->T) return fail(ctx, MOE_ERR_INVALID_ARG, "T = %d differs from the layout's T = %d", T, ctx->T);
-  if (!w_gate_up || !w_down) return fail(ctx, MOE_ERR_INVALID_ARG, "routed weights are NULL");
-  const bool shared = ctx->cfg.n_shared != 0;
-  if (shared && (!ws_gate_up || !ws_down || (!x && T > 0)))
-    return fail(ctx, MOE_ERR_INVALID_ARG, "the shared expert needs ws_gate_up, ws_down and x");
-  if (gathers_rows(ctx) && !x && T > 0) return fail(ctx, MOE_ERR_INVALID_ARG, "the row gather needs x");
-  if (misaligned(w_gate_up) || misaligned(w_down) || misaligned(x) || misaligned(ws_gate_up) || misaligned(ws_down))
-    return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
-  DeviceGuard guard(ctx->device);
-  BufferSet& b = ctx->sets[ctx->cur];
-  const moe_config& c = ctx->cfg;
-  const int64_t N = (int64_t)T * c.top_k, Ncap = (int64_t)c.max_tokens * c.top_k;
-  int n = 0;
-  cudaError_t e = cudaSuccess;
-  if (T > 0) {
-    // One launch per pass, or one per group of seg_experts experts with a boundary call after each.
-    const int span = (ctx->seg_experts > 0 && ctx->seg_experts < c.n_experts) ? ctx->seg_experts : c.n_experts;
-    const int routed_segs = (c.n_experts + span - 1) / span;
-    const int first = ctx->split_step ? 1 : 0;  // a split dispatch reported boundary 0 after its notification
-    const int n_bound = first + 2 * routed_segs + (shared ? 2 : 0);
-    int bound = first;
-    auto boundary = [&]() {
-      if (ctx->seg_experts > 0 && ctx->boundary_fn) {
-        if (!capturing(ctx)) cudaEventRecord(ctx->done, ctx->stream);
-        ctx->boundary_fn(ctx->boundary_user, bound, n_bound);
-      }
-      ++bound;
-    };
-    moe::GemmProblem g1{b.x_perm, w_gate_up, b.act, ctx->offsets, 0, Ncap, N, c.n_experts, c.inter, c.hidden, true};
-    moe::GemmProblem g2{b.act, w_down, b.y_perm, ctx->offsets, 0, Ncap, N, c.n_experts, c.hidden, c.inter, false};
-    if (gathers_rows(ctx)) {
-      g1.gather_src = x;
-      g1.perm = ctx->perm;
-      g1.top_k = c.top_k;
-    }
-    moe::GemmDenseGroup s1{x, ws_gate_up, b.act_shared, T, c.shared_inter, c.hidden};
-    moe::GemmDenseGroup s2{b.act_shared, ws_down, b.y_shared, T, c.hidden, c.shared_inter};
-    // Unsegmented: the shared expert's two passes ride in the routed launches (two launches in all).
-    // Segmented: they are segments of their own, after the routed ones.
-    const bool fuse_shared = shared && ctx->seg_experts == 0;
-    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
-      moe::GemmProblem& g = pass == 0 ? g1 : g2;
-      for (int e0 = 0; e0 < c.n_experts && e == cudaSuccess; e0 += span) {
-        g.e_begin = e0;
-        g.e_end = e0 + span < c.n_experts ? e0 + span : c.n_experts;
-        {
-          StageTimer tm(ctx, pass == 0 ? 3 : 4);
-          e = run_gemm(ctx, g, fuse_shared ? (pass == 0 ? &s1 : &s2) : nullptr, T, &n);
-        }
-        if (e == cudaSuccess) boundary();
-      }
-    }
-    if (e == cudaSuccess && shared && !fuse_shared) {
-      moe::GemmProblem d1{s1.A, s1.W, s1.out, nullptr, T, T, T, 1, s1.n_feat, s1.K, true};
-      {
-        StageTimer tm(ctx, 5);
-        e = run_gemm(ctx, d1, nullptr, T, &n);
-      }
-      if (e == cudaSuccess) {
-        boundary();
-        moe::GemmProblem d2{s2.A, s2.W, s2.out, nullptr, T, T, T, 1, s2.n_feat, s2.K, false};
-        {
-          StageTimer tm(ctx, 6);
-          e = run_gemm(ctx, d2, nullptr, T, &n);
-        }
-        if (e == cudaSuccess) boundary();
-      }
-    }
-  }
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "moe_grouped_ffn");
-  ctx->state = ST_FFN_DONE;
-  mark(ctx, n);
-  return MOE_OK;
+  return grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T, 0, [](int, int) { return cudaSuccess; });
 }
 
 moe_status moe_grouped_ffn_fp8(moe_ctx* ctx, const void* wq_gate_up, const float* sw_gate_up, const void* wq_down,
@@ -1014,31 +1075,100 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
                           const void* ws_down, void* out_host) {
   if (!ctx) return MOE_ERR_INVALID_ARG;
   if (ctx->state != ST_IDLE) return fail(ctx, MOE_ERR_STATE, "moe_layer_host called in the middle of a step");
+  if (ctx->cfg.weight_format != MOE_WEIGHTS_BF16)
+    return fail(ctx, MOE_ERR_STATE, "the host path serves contexts created for BF16 weights");
   if (T < 0) return fail(ctx, MOE_ERR_INVALID_ARG, "T < 0");
   if (T > ctx->cfg.max_tokens) return fail(ctx, MOE_ERR_CAPACITY, "T = %d exceeds max_tokens = %d", T, ctx->cfg.max_tokens);
   if (T > 0 && (!logits_host || !x_host || !out_host)) return fail(ctx, MOE_ERR_INVALID_ARG, "NULL host pointer");
   DeviceGuard guard(ctx->device);
+  moe_status st = ensure_host_streams(ctx, "moe_layer_host set-up");
+  if (st != MOE_OK) return st;
   BufferSet& b = ctx->sets[ctx->cur];
   const moe_config& c = ctx->cfg;
-  const size_t x_bytes = (size_t)T * c.hidden * 2;
-  cudaError_t e = cudaSuccess;
-  if (T > 0) {
-    e = cudaMemcpyAsync(b.logits, logits_host, (size_t)T * c.n_experts * 4, cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b.x_stage, x_host, x_bytes, cudaMemcpyHostToDevice, ctx->stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "host-to-device copy");
-  }
-  moe_status st = moe_route(ctx, b.logits, select_bias, T, b.topk_idx, b.topk_w);
-  if (st == MOE_OK) st = moe_dispatch_layout(ctx, b.topk_idx, T, b.x_stage, nullptr, nullptr, nullptr, nullptr);
-  if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, b.x_stage, ws_gate_up, ws_down, T);
-  if (st == MOE_OK) st = moe_combine(ctx, b.topk_w, nullptr, T, b.out_stage);
-  if (st != MOE_OK) {
+  const size_t row_bytes = (size_t)c.hidden * 2;
+  // Both copies overlap the kernels as far as the step allows.  In: the router starts on the logits while the rows are
+  // still on their way.  Out: the down pass runs in pieces of output features, and a piece is combined and copied while
+  // the next is computed -- a piece costs two launches more, so there is one for every kHostPieceBytes, up to four.
+  // A prefill batch of at least kHostChunkFromRows rows per expert is also cut into two chunks of tokens, so that the
+  // second comes in while the first is computed; with fewer rows the pass is bound by streaming the weights, which each
+  // chunk would do again.  Segments and preemption keep their one sequence of boundaries.
+  // So does pageable memory, whose copies the runtime makes while the call waits.
+  cudaPointerAttributes attr;
+  const bool pinned = T > 0 && cudaPointerGetAttributes(&attr, out_host) == cudaSuccess && attr.type == cudaMemoryTypeHost;
+  const bool whole = ctx->seg_experts > 0 || ctx->preemptible || c.gemm_variant == MOE_GEMM_VALIDATION || !pinned;
+  const bool halves = !whole && c.phase == MOE_PHASE_PREFILL &&
+                      (int64_t)T * c.top_k >= (int64_t)kHostChunkFromRows * c.n_experts && T * row_bytes >= 2 * kHostChunkBytes;
+  const int n_chunks = halves ? 2 : 1;
+  const int chunk = ((T + n_chunks - 1) / n_chunks + 15) / 16 * 16;  // keeps every chunk's arrays 16-byte aligned
+  cudaError_t e = cudaEventRecord(ctx->computed, ctx->stream);  // the staging buffers are the stream's until here
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->h2d_stream, ctx->computed, 0);
+  for (const moe_ctx::HostSlot& s : ctx->slots)  // (a slot of the pipelined path may still be copying out of them)
+    if (e == cudaSuccess && s.in_flight) e = cudaStreamWaitEvent(ctx->stream, s.done, 0);
+  for (int t0 = 0; (t0 < T || T == 0) && e == cudaSuccess && st == MOE_OK; t0 += chunk) {
+    const int n_tok = std::min(chunk, T - t0);
+    float* const logits = b.logits + (size_t)t0 * c.n_experts;
+    char* const x = b.x_stage + (size_t)t0 * row_bytes;
+    char* const out = b.out_stage + (size_t)t0 * row_bytes;
+    char* const out_to = static_cast<char*>(out_host) + (size_t)t0 * row_bytes;
+    int32_t* const idx = b.topk_idx + (size_t)t0 * c.top_k;
+    float* const w = b.topk_w + (size_t)t0 * c.top_k;
+    if (T > 0) {
+      e = cudaMemcpyAsync(logits, logits_host + (size_t)t0 * c.n_experts, (size_t)n_tok * c.n_experts * 4,
+                          cudaMemcpyHostToDevice, ctx->h2d_stream);
+      if (e == cudaSuccess) e = cudaEventRecord(ctx->copied_in, ctx->h2d_stream);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->copied_in, 0);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(x, static_cast<const char*>(x_host) + (size_t)t0 * row_bytes, (size_t)n_tok * row_bytes,
+                            cudaMemcpyHostToDevice, ctx->h2d_stream);
+      if (e == cudaSuccess) e = cudaEventRecord(ctx->copied_in, ctx->h2d_stream);
+      if (e != cudaSuccess) break;
+    }
+    st = moe_route(ctx, logits, select_bias, n_tok, idx, w);
+    if (st == MOE_OK) st = enqueue_layout(ctx, "moe_layer_host", idx, n_tok, nullptr, nullptr, nullptr, nullptr);
+    if (st != MOE_OK) break;
+    if ((e = cudaStreamWaitEvent(ctx->stream, ctx->copied_in, 0)) != cudaSuccess) break;
+    st = enqueue_row_movement(ctx, "moe_layer_host", x);
+    if (st != MOE_OK) break;
+    ctx->state = ST_LAID_OUT;
+    ctx->split_step = false;
+    int pieces = 1;
+    if (!whole && t0 + n_tok == T)
+      pieces = (int)std::min<size_t>(kHostMaxPieces, 1 + (size_t)n_tok * row_bytes / kHostPieceBytes);
+    const int piece_cols = (c.hidden / pieces + 255) / 256 * 256;
+    const char* const y_shared = c.n_shared ? ctx->sets[ctx->cur].y_shared : nullptr;
+    auto finish = [&](int c0, int c1) -> cudaError_t {  // combine the columns [c0, c1) and send them
+      int n = 0;
+      cudaError_t err;
+      {
+        StageTimer tm(ctx, 7);
+        err = moe::launch_combine(ctx->sets[ctx->cur].y_perm, y_shared, ctx->inv_perm, w, out, n_tok, c.top_k, c.hidden,
+                                  ctx->status, ctx->stream, &n, ctx->wait_limit_ns, c0, c1);
+      }
+      ctx->launches += n;
+      if (err == cudaSuccess) err = cudaEventRecord(ctx->computed, ctx->stream);
+      if (err == cudaSuccess) err = cudaStreamWaitEvent(ctx->d2h_stream, ctx->computed, 0);
+      if (err == cudaSuccess && n_tok > 0)
+        err = cudaMemcpy2DAsync(out_to + (size_t)c0 * 2, row_bytes, out + (size_t)c0 * 2, row_bytes, (size_t)(c1 - c0) * 2,
+                                n_tok, cudaMemcpyDeviceToHost, ctx->d2h_stream);
+      return err;
+    };
+    st = grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, n_tok, pieces > 1 ? piece_cols : 0, finish);
+    if (st != MOE_OK) break;
+    if (pieces == 1) e = finish(0, c.hidden);
     ctx->state = ST_IDLE;
-    return st;
+    if (ctx->n_sets == 2) ctx->cur ^= 1;
+    if (T == 0) break;
   }
-  if (T > 0) e = cudaMemcpyAsync(out_host, b.out_stage, x_bytes, cudaMemcpyDeviceToHost, ctx->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "device-to-host copy");
-  return MOE_OK;
+  mark(ctx, 0);
+  mark_position(ctx);
+  // nothing of the caller's memory is in use when this returns, whatever happened
+  for (cudaStream_t s : {ctx->h2d_stream, ctx->stream, ctx->d2h_stream}) {
+    const cudaError_t sync = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = sync;
+  }
+  if (st != MOE_OK || e != cudaSuccess) ctx->state = ST_IDLE;
+  if (st != MOE_OK) return st;
+  return e == cudaSuccess ? MOE_OK : cuda_fail(ctx, e, "moe_layer_host");
 }
 
 moe_status moe_layer_host_submit(moe_ctx* ctx, int32_t slot, const float* logits_host, const float* select_bias,
@@ -1055,28 +1185,8 @@ moe_status moe_layer_host_submit(moe_ctx* ctx, int32_t slot, const float* logits
   if (T > 0 && (!logits_host || !x_host || !out_host)) return fail(ctx, MOE_ERR_INVALID_ARG, "NULL host pointer");
   DeviceGuard guard(ctx->device);
   cudaError_t e = cudaSuccess;
-  if (!ctx->host_pipeline) {
-    constexpr int kEvents = 3 * MOE_HOST_SLOTS;
-    cudaEvent_t ev[kEvents] = {};
-    cudaStream_t st[2] = {};
-    for (int i = 0; i < kEvents && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&st[i], cudaStreamNonBlocking);
-    if (e != cudaSuccess) {
-      for (int i = 0; i < kEvents; ++i)
-        if (ev[i]) cudaEventDestroy(ev[i]);
-      for (int i = 0; i < 2; ++i)
-        if (st[i]) cudaStreamDestroy(st[i]);
-      return cuda_fail(ctx, e, "moe_layer_host_submit set-up");
-    }
-    for (int s = 0; s < MOE_HOST_SLOTS; ++s) {
-      ctx->slots[s].h2d = ev[3 * s];
-      ctx->slots[s].comp = ev[3 * s + 1];
-      ctx->slots[s].done = ev[3 * s + 2];
-    }
-    ctx->h2d_stream = st[0];
-    ctx->d2h_stream = st[1];
-    ctx->host_pipeline = true;
-  }
+  moe_status st = ensure_host_streams(ctx, "moe_layer_host_submit set-up");
+  if (st != MOE_OK) return st;
   moe_ctx::HostSlot& hs = ctx->slots[slot];
   BufferSet& b = ctx->sets[ctx->cur];
   const moe_config& c = ctx->cfg;
@@ -1088,7 +1198,7 @@ moe_status moe_layer_host_submit(moe_ctx* ctx, int32_t slot, const float* logits
   if (e == cudaSuccess) e = cudaEventRecord(hs.h2d, ctx->h2d_stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, hs.h2d, 0);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "host-to-device copy");
-  moe_status st = moe_route(ctx, hs.logits, select_bias, T, b.topk_idx, b.topk_w);
+  st = moe_route(ctx, hs.logits, select_bias, T, b.topk_idx, b.topk_w);
   if (st == MOE_OK) st = moe_dispatch_layout(ctx, b.topk_idx, T, hs.x, nullptr, nullptr, nullptr, nullptr);
   if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, hs.x, ws_gate_up, ws_down, T);
   if (st == MOE_OK) st = moe_combine(ctx, b.topk_w, nullptr, T, hs.out);

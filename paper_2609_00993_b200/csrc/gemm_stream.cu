@@ -81,6 +81,7 @@ struct StreamParams {
   int32_t E;               // experts covered by this launch
   int32_t e_base;          // index of the launch's first expert in the weight tensor
   int32_t n_feat;          // output features (I for the gated pass, H for the down pass)
+  int32_t ft0, n_ft, n_ft2;  // feature tiles of this launch: the first, and how many (n_ft2: of the dense group)
   int32_t K;
   __nv_bfloat16* out;      // [rows, n_feat]
   int32_t ring_slots;
@@ -150,7 +151,7 @@ __device__ __forceinline__ int size_class(int cnt) {
 
 // tile -> (expert, first row, valid rows, feature tile).  The dense group's tiles come first (chunk major),
 // then the experts' in the order `order` (largest first): prefix[i] = chunks of the experts at positions < i.
-__device__ __forceinline__ STile decode_tile(int tile, int dense_tiles, int n_ft2, int rows2, int n_ft, int E,
+__device__ __forceinline__ STile decode_tile(int tile, int dense_tiles, int n_ft2, int rows2, int n_ft, int ft0, int E,
                                              const int* prefix, const int* order, const int* beg, const int* cnts) {
   STile t;
   int tiles, chunk;
@@ -158,7 +159,7 @@ __device__ __forceinline__ STile decode_tile(int tile, int dense_tiles, int n_ft
     const int rt = tile / n_ft2;
     chunking(rows2, tiles, chunk);
     t.e = 0;
-    t.ft = tile - rt * n_ft2;
+    t.ft = ft0 + tile - rt * n_ft2;
     t.row0 = rt * chunk;
     t.rows = min(chunk, rows2 - t.row0);
     t.dense = true;
@@ -175,7 +176,7 @@ __device__ __forceinline__ STile decode_tile(int tile, int dense_tiles, int n_ft
   chunking(cnt, tiles, chunk);
   const int mt = rt - prefix[lo];
   t.e = e;
-  t.ft = tile - rt * n_ft;
+  t.ft = ft0 + tile - rt * n_ft;
   t.row0 = beg[e] + mt * chunk;
   t.rows = min(chunk, cnt - mt * chunk);
   t.dense = false;
@@ -216,9 +217,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   [[maybe_unused]] const int unit = (int)blockIdx.x;
   if (threadIdx.x == 0) PROF_STAMP(0);
   constexpr int kFeatPerTile = GATED ? 128 : 256;
-  const int n_ft = (p.n_feat + kFeatPerTile - 1) / kFeatPerTile;
+  const int n_ft = p.n_ft, n_ft2 = p.n_ft2;
   const int num_kb1 = (p.K + kbk - 1) / kbk, num_kb2 = (p.K2 + kbk - 1) / kbk;
-  const int n_ft2 = (p.n_feat2 + kFeatPerTile - 1) / kFeatPerTile;
   const int dense_tiles = p.rows2 > 0 ? ((p.rows2 + kMaxTileRows - 1) / kMaxTileRows) * n_ft2 : 0;
   const unsigned long long limit = p.wait_limit_ns;
 
@@ -401,7 +401,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         }
         if (tile < 0) break;
         bool stop_after = false;
-        const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.E, prefix, order, beg, cnts);
+        const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, order, beg, cnts);
         const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
         const int w_row0 = t.ft * kFeatPerTile;
         const CUtensorMap* mw = t.dense ? &map_w2 : &map_w;
@@ -508,7 +508,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         mbar_arrive(bar_tqempty + 8u * q);
         ++tcount;
         if (tile < 0) break;
-        const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.E, prefix, order, beg, cnts);
+        const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, order, beg, cnts);
         const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
         const bool big = n > 128u;
         uint32_t d_a, d_b;
@@ -616,7 +616,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       if (lane == 0) mbar_arrive(bar_tqempty + 8u * q);
       ++tcount;
       if (tile < 0) break;
-      const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.E, prefix, order, beg, cnts);
+      const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, order, beg, cnts);
       const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
       const bool big = n > 128u;
       uint32_t h = 0, d_a, d_b;
@@ -968,11 +968,19 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   const size_t smem = 1024 + (size_t)slots * kSlotBytes + tail;
 
   const int feat_per_tile = p.gated ? 128 : 256;
-  const int64_t n_ft = (p.n_feat + feat_per_tile - 1) / feat_per_tile;
+  const int f_end = p.f_end < 0 ? p.n_feat : p.f_end;
+  const bool part = p.f_begin != 0 || f_end != p.n_feat;
+  if (p.f_begin < 0 || p.f_begin % 256 != 0 || f_end > p.n_feat || p.f_begin >= f_end ||
+      (f_end % feat_per_tile != 0 && f_end != p.n_feat) || (part && dense != nullptr && dense->n_feat != p.n_feat))
+    return cudaErrorInvalidValue;
+  const int64_t n_ft = (f_end + feat_per_tile - 1) / feat_per_tile - p.f_begin / feat_per_tile;
+  prm.ft0 = p.f_begin / feat_per_tile;
+  prm.n_ft = (int)n_ft;
+  prm.n_ft2 = dense == nullptr ? 1 : part ? (int)n_ft : (dense->n_feat + feat_per_tile - 1) / feat_per_tile;
   const int64_t row_tiles = p.rows_bound / kMaxTileRows + (prm.E < p.rows_bound ? prm.E : p.rows_bound);
   int64_t tiles = row_tiles * n_ft;
   if (dense != nullptr)
-    tiles += (int64_t)((dense->rows + kMaxTileRows - 1) / kMaxTileRows) * ((dense->n_feat + feat_per_tile - 1) / feat_per_tile);
+    tiles += (int64_t)((dense->rows + kMaxTileRows - 1) / kMaxTileRows) * prm.n_ft2;
   int grid = (int)(tiles < (int64_t)max_ctas ? tiles : (int64_t)max_ctas);
   if (grid < 1) grid = 1;
   const bool overlap = p.rows_bound <= kGemmOverlapMaxRows;

@@ -53,6 +53,7 @@ struct TcParams {
   int32_t E;               // experts covered by this launch
   int32_t e_base;          // index of the launch's first expert in the weight tensor
   int32_t n_feat;          // output features (I for the gated pass, H for the down pass)
+  int32_t ft0, n_ft, n_ft2;  // feature tiles of this launch: the first, and how many (n_ft2: of the dense group)
   int32_t K;
   __nv_bfloat16* out;      // [rows, n_feat]
   int32_t row_tile;        // tokens per tile: 128
@@ -95,13 +96,13 @@ struct Tile {
 
 // tile -> (expert, first row, valid rows, feature tile).  The dense group's tiles come first (row tile major),
 // then the experts': prefix[e] = row tiles of experts < e.
-__device__ __forceinline__ Tile decode_tile(int tile, int dense_tiles, int n_ft2, int rows2, int n_ft, int E,
+__device__ __forceinline__ Tile decode_tile(int tile, int dense_tiles, int n_ft2, int rows2, int n_ft, int ft0, int E,
                                             const int* prefix, const int* seg, int row_tile) {
   Tile t;
   if (tile < dense_tiles) {
     const int rt = tile / n_ft2;
     t.e = 0;
-    t.ft = tile - rt * n_ft2;
+    t.ft = ft0 + tile - rt * n_ft2;
     t.row0 = rt * row_tile;
     t.rows = min(row_tile, rows2 - t.row0);
     t.dense = true;
@@ -115,7 +116,7 @@ __device__ __forceinline__ Tile decode_tile(int tile, int dense_tiles, int n_ft2
     if (prefix[mid] <= rt) lo = mid; else hi = mid;
   }
   t.e = lo;
-  t.ft = tile - rt * n_ft;
+  t.ft = ft0 + tile - rt * n_ft;
   const int mt = rt - prefix[lo];
   t.row0 = seg[lo] + mt * row_tile;
   t.rows = min(row_tile, seg[lo + 1] - t.row0);
@@ -160,9 +161,8 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
   const int unit = (int)blockIdx.x, n_units = (int)gridDim.x;
   const int tile_rows = p.row_tile;  // token rows per tile of the list
   constexpr int kFeatPerTile = GATED ? 128 : 256;
-  const int n_ft = (p.n_feat + kFeatPerTile - 1) / kFeatPerTile;
+  const int n_ft = p.n_ft, n_ft2 = p.n_ft2;
   const int num_kb1 = (p.K + kbk - 1) / kbk, num_kb2 = (p.K2 + kbk - 1) / kbk;
-  const int n_ft2 = (p.n_feat2 + kFeatPerTile - 1) / kFeatPerTile;
   const int dense_tiles = p.rows2 > 0 ? ((p.rows2 + p.row_tile - 1) / p.row_tile) * n_ft2 : 0;
   constexpr uint32_t acc_cols = 256u;  // TMEM columns per accumulator stage
   constexpr uint32_t tmem_cols = 2u * acc_cols;
@@ -220,7 +220,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
       RingCursor ring;
       bool ok = true;
       for (int tile = unit; tile < total_tiles && ok; tile += n_units) {
-        const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.E, prefix, seg, tile_rows);
+        const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, seg, tile_rows);
         const int w_row0 = t.ft * kFeatPerTile;
         const int w_row1 = GATED ? (t.dense ? p.n_feat2 : p.n_feat) + t.ft * kFeatPerTile : w_row0 + kWBoxRows;
         const CUtensorMap* mw = t.dense ? &map_w2 : &map_w;
@@ -257,7 +257,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
       const uint32_t lo_base = (uint32_t)umma_smem_desc(base_addr);  // stage 0, weight box 0
       const uint32_t lo_stage = (uint32_t)stage_bytes >> 4, lo_box = (uint32_t)kWBoxBytes >> 4;
       for (int tile = unit; tile < total_tiles && ok; tile += n_units, ++tile_iter) {
-        const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.E, prefix, seg, tile_rows);
+        const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, seg, tile_rows);
         const uint32_t as = tile_iter & 1u, aph = (tile_iter >> 1) & 1u;
         if (!mbar_wait(bar_tempty + 8u * as, aph ^ 1u, abort_flag, p.wait_limit_ns)) { ok = false; break; }
         tc_fence_after();
@@ -304,7 +304,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     int slot_next[8];
     auto fetch_slots = [&](int tile, int (&slot)[8]) {
       if (tile >= total_tiles) return;
-      const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.E, prefix, seg, tile_rows);
+      const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, seg, tile_rows);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int r = rbase + 16 * i;
@@ -314,7 +314,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     };
     fetch_slots(unit, slot_next);
     for (int tile = unit; tile < total_tiles && ok; tile += n_units) {
-      const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.E, prefix, seg, tile_rows);
+      const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, seg, tile_rows);
       const __nv_bfloat16* src = t.dense ? p.gather_src2 : p.gather_src;
       const int Kt = t.dense ? p.K2 : p.K;
       const __nv_bfloat16* row_ptr[8];  // nullptr: the row is left as it is; its result is never stored
@@ -344,7 +344,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     bool ok = true;
     const uint32_t lane_base = ((uint32_t)(warp * 32)) << 16;
     for (int tile = unit; tile < total_tiles && ok; tile += n_units, ++tile_iter) {
-      const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.E, prefix, seg, tile_rows);
+      const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, seg, tile_rows);
       const uint32_t as = tile_iter & 1u, aph = (tile_iter >> 1) & 1u;
       auto release_acc = [&]() {  // hand the accumulator stage back to the MMA issuer
         tc_fence_before();
@@ -653,11 +653,19 @@ cudaError_t launch_gemm_tc(const GemmProblem& p, const GemmDenseGroup* dense, in
   const size_t smem = 1024 + (size_t)stages * stage_bytes + tail;
 
   const int feat_per_tile = p.gated ? 128 : 256;
-  const int64_t n_ft = (p.n_feat + feat_per_tile - 1) / feat_per_tile;
+  const int f_end = p.f_end < 0 ? p.n_feat : p.f_end;
+  const bool part = p.f_begin != 0 || f_end != p.n_feat;
+  if (p.f_begin < 0 || p.f_begin % 256 != 0 || f_end > p.n_feat || p.f_begin >= f_end ||
+      (f_end % feat_per_tile != 0 && f_end != p.n_feat) || (part && dense != nullptr && dense->n_feat != p.n_feat))
+    return cudaErrorInvalidValue;
+  const int64_t n_ft = (f_end + feat_per_tile - 1) / feat_per_tile - p.f_begin / feat_per_tile;
+  prm.ft0 = p.f_begin / feat_per_tile;
+  prm.n_ft = (int)n_ft;
+  prm.n_ft2 = dense == nullptr ? 1 : part ? (int)n_ft : (dense->n_feat + feat_per_tile - 1) / feat_per_tile;
   const int64_t row_tiles = p.rows_bound / row_tile + (prm.E < p.rows_bound ? prm.E : p.rows_bound);
   int64_t tiles = row_tiles * n_ft;
   if (dense != nullptr)
-    tiles += (int64_t)((dense->rows + row_tile - 1) / row_tile) * ((dense->n_feat + feat_per_tile - 1) / feat_per_tile);
+    tiles += (int64_t)((dense->rows + row_tile - 1) / row_tile) * prm.n_ft2;
 
   int grid = (int)(tiles < (int64_t)max_ctas ? tiles : (int64_t)max_ctas);
   if (grid < 1) grid = 1;

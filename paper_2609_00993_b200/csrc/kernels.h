@@ -78,9 +78,10 @@ cudaError_t launch_layout(const int32_t* topk_idx, int64_t n_slots, int E, int32
 cudaError_t launch_permute(const void* x, const int32_t* inv_perm, void* x_perm, int T, int k, int H, int* status,
                            cudaStream_t stream, int* n_launches, const float* row_val = nullptr,
                            float* row_val_perm = nullptr, unsigned long long wait_limit_ns = 0);
+// Columns [c_begin, c_end) of the rows (c_end < 0: all; multiples of 8).
 cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32_t* inv_perm, const float* topk_w,
                            void* out, int T, int k, int H, int* status, cudaStream_t stream, int* n_launches,
-                           unsigned long long wait_limit_ns = 0);
+                           unsigned long long wait_limit_ns = 0, int c_begin = 0, int c_end = -1);
 
 // Tensor maps of one small-M GEMM launch (host memory, opaque outside gemm_stream.cu).  A context keeps one plan per
 // buffer set and pass; a launch whose operands (addresses and shapes) are the plan's re-encodes nothing.  (Looking 34
@@ -109,6 +110,8 @@ struct GemmProblem {
   bool gated;
   int32_t e_begin = 0;     // this launch covers experts [e_begin, e_end) only (a prefill segment);
   int32_t e_end = -1;      // e_end < 0 means E
+  int32_t f_begin = 0;     // ... and output features [f_begin, f_end) only (f_begin a multiple of 256; f_end < 0 means
+  int32_t f_end = -1;      // n_feat); a dense group in the same launch then has the same n_feat and range
   // Row gather (tensor-core large-M gated pass only): when gather_src is set, A is not read; row p of the
   // operand is gather_src[perm[p] / top_k, :] instead (gather_src is bf16 [T, K], perm is [rows_bound]).
   const void* gather_src = nullptr;

@@ -159,7 +159,7 @@ __device__ __forceinline__ void fma_bf16x8(float (&acc)[8], const uint4& v, floa
   }
 }
 
-// out[t, c0:c1] = sum_j w[t,j] * y_perm[inv_perm[t*k+j], c0:c1] (+ y_shared[t, c0:c1]); ascending j, then shared.
+// Columns [c_begin, c_end): out[t, c0:c1] = sum_j w[t,j] * y_perm[inv_perm[t*k+j], c0:c1] (+ y_shared[t, c0:c1]); ascending j, then shared.
 // dynamic shared memory, per stage: (k+1) row chunks of chunk_bytes | k weights | valid mask; then barriers.
 // Producer lane j gathers row j; lane 0 also fetches the shared row.  KT > 0 fixes k at compile time (the sum
 // over experts is then fully unrolled); KT = 0 takes k at run time.
@@ -167,8 +167,8 @@ template <int KT>
 __global__ void __launch_bounds__(kCombineThreads)
 combine_kernel(const __nv_bfloat16* __restrict__ y_perm, const __nv_bfloat16* __restrict__ y_shared,
                const int32_t* __restrict__ inv_perm, const float* __restrict__ topk_w, __nv_bfloat16* __restrict__ out,
-               int T, int k, int H, int col_blocks, int chunk_bytes, int stage_bytes, int n_stages, int* status,
-               unsigned long long wait_limit_ns) {
+               int T, int k, int H, int c_begin, int c_end, int col_blocks, int chunk_bytes, int stage_bytes, int n_stages,
+               int* status, unsigned long long wait_limit_ns) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
   const uint32_t bar_full = base + (uint32_t)(n_stages * stage_bytes);
@@ -194,8 +194,8 @@ combine_kernel(const __nv_bfloat16* __restrict__ y_perm, const __nv_bfloat16* __
     bool ok = true;
     long long n = 0;
     for (long long it = blockIdx.x; it < n_items; it += gridDim.x, ++n) {
-      const int t = (int)(it / col_blocks), c0 = (int)(it % col_blocks) * kCombineChunkCols;
-      const uint32_t bytes = (uint32_t)(min(kCombineChunkCols, H - c0) * 2);
+      const int t = (int)(it / col_blocks), c0 = c_begin + (int)(it % col_blocks) * kCombineChunkCols;
+      const uint32_t bytes = (uint32_t)(min(kCombineChunkCols, c_end - c0) * 2);
       const uint32_t s = (uint32_t)(n % n_stages), ph = (uint32_t)((n / n_stages) & 1);
       int row = -1;
       float wv = 0.f;
@@ -227,8 +227,8 @@ combine_kernel(const __nv_bfloat16* __restrict__ y_perm, const __nv_bfloat16* __
     long long n = 0;
     const int v = threadIdx.x;
     for (long long it = blockIdx.x; it < n_items; it += gridDim.x, ++n) {
-      const int t = (int)(it / col_blocks), c0 = (int)(it % col_blocks) * kCombineChunkCols;
-      const int cols = min(kCombineChunkCols, H - c0);
+      const int t = (int)(it / col_blocks), c0 = c_begin + (int)(it % col_blocks) * kCombineChunkCols;
+      const int cols = min(kCombineChunkCols, c_end - c0);
       const uint32_t s = (uint32_t)(n % n_stages), ph = (uint32_t)((n / n_stages) & 1);
       ok = __all_sync(0xffffffffu, mbar_wait(bar_full + 8u * s, ph, wait_limit_ns));
       if (!ok) break;
@@ -306,11 +306,13 @@ cudaError_t launch_permute(const void* x, const int32_t* inv_perm, void* x_perm,
 
 cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32_t* inv_perm, const float* topk_w,
                            void* out, int T, int k, int H, int* status, cudaStream_t stream, int* n_launches,
-                           unsigned long long wait_limit_ns) {
-  if (T <= 0) return cudaSuccess;
-  if (k > 32) return cudaErrorNotSupported;  // one gathering lane per row
-  const int col_blocks = (H + kCombineChunkCols - 1) / kCombineChunkCols;
-  const int chunk_bytes = (H < kCombineChunkCols ? H : kCombineChunkCols) * 2;
+                           unsigned long long wait_limit_ns, int c_begin, int c_end) {
+  if (c_end < 0) c_end = H;
+  if (T <= 0 || c_begin >= c_end) return cudaSuccess;
+  if (k > 32 || c_begin < 0 || c_end > H || c_begin % 8 != 0 || c_end % 8 != 0) return cudaErrorNotSupported;  // one gathering lane per row
+  const int cols = c_end - c_begin;
+  const int col_blocks = (cols + kCombineChunkCols - 1) / kCombineChunkCols;
+  const int chunk_bytes = (cols < kCombineChunkCols ? cols : kCombineChunkCols) * 2;
   const int stage_bytes = ((k + 1) * chunk_bytes + 4 * k + 4 + 127) / 128 * 128;
   int stages = (64 * 1024) / stage_bytes;  // about 64 KB of slots per CTA, three CTAs per SM
   if (stages > kCombineMaxStages) stages = kCombineMaxStages;
@@ -324,7 +326,7 @@ cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32
     const int grid = (int)(n_items < cap ? n_items : cap);
     return launch_pdl(true, kern, dim3(grid), dim3(kCombineThreads), smem, stream, static_cast<const __nv_bfloat16*>(y_perm),
                       static_cast<const __nv_bfloat16*>(y_shared), inv_perm, topk_w, static_cast<__nv_bfloat16*>(out), T, k,
-                      H, col_blocks, chunk_bytes, stage_bytes, stages, status,
+                      H, c_begin, c_end, col_blocks, chunk_bytes, stage_bytes, stages, status,
                       wait_limit_ns ? wait_limit_ns : kWaitLimitNs);
   };
   cudaError_t err = k == 8 ? launch(combine_kernel<8>) : k == 4 ? launch(combine_kernel<4>)
