@@ -338,7 +338,7 @@ moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_per
  * The call allocates nothing and frees nothing.  It works on the device that is current when it is called:
  * the pointers and the stream must belong to that device.  The first call on each device looks up the
  * array's device address (a host-side set-up step); make that first call before any stream capture begins.
- * A call with more experts than any earlier call on that device (single-launch path, T*top_k <= 16384) also
+ * A call with more experts than any earlier call on that device also
  * raises a kernel's shared-memory limit on the host, so it too should come before capture.
  * All calls on one device share the array: two calls whose kernels can overlap on the GPU (different
  * streams without an ordering between them) race on it -- order them.  Nothing in the array needs clearing

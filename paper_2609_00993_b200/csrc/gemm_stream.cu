@@ -290,7 +290,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       const unsigned lt_mask = (1u << lane) - 1u;
       for (int b = 0; b < p.E; b += 32) {
         const int e = b + lane;
-        const int key = e < p.E ? size_class(cnts[e]) : kSizeClasses + lane;  // lanes past the end group with nobody
+        const int key = e < p.E ? size_class(cnts[e]) : kSizeClasses;
         const unsigned peers = __match_any_sync(0xffffffffu, key);
         int pos = 0;
         if (e < p.E) pos = class_pos[key] + __popc(peers & lt_mask);

@@ -1,11 +1,16 @@
 // Stages a2-a4: per-expert counts, exclusive scan, stable token-to-expert permutation.
 //
 // The permutation must be bit-exact and run-to-run identical, so no slot is claimed with a global
-// atomic.  The flat slots are cut into warp-owned chunks; a warp walks its chunk 32 slots at a time
-// and ranks equal experts inside a step with __match_any_sync, which keeps ascending slot order.
-//   small N (decode, low latency): ONE CTA does count -> scan -> place in shared memory, one launch.
-//   large N (prefill):             count per chunk -> per-expert scan over chunks (one CTA per 32
-//                                  experts) -> scan over experts and place per chunk.
+// atomic.  The flat slots are cut into chunks, one per CTA, and a chunk into 32 runs, one per warp; a warp walks its run
+// 32 slots at a time and ranks equal experts inside a step with __match_any_sync, which keeps ascending slot order.
+// What a CTA needs beyond its own chunk -- how many slots of each expert lie in earlier chunks, and in all -- it finds out
+// by itself, so that no kernel only scans:
+//   up to kRecountMaxSlots slots   one launch: every CTA counts the other chunks too (a few slots per thread);
+//   more                           a launch that counts each chunk, then the same kernel reading those counts.
+// The arithmetic is nothing; what it costs is launches, dependent round trips and the slots one SM can walk.  Back to
+// back in a CUDA graph, against one CTA up to 16384 slots and count -> scan -> place in three launches above: 512 slots of
+// 256 experts 4.1 -> 3.2 us, 5600 10.3 -> 5.9, 12248 of 128 17.7 -> 6.8, 32768 of 512 10.7 -> 8.5, 65536 of 128 8.4 -> 7.9,
+// 262144 of 256 14.3 -> 12.2.  (Recounting up to 32768 slots instead of 16384: 0.3 us less at 20000, 0.5 more at 32000.)
 #include <mutex>
 
 #include "kernels.h"
@@ -13,69 +18,16 @@
 namespace moe {
 namespace {
 
-constexpr int kFusedWarps = 32;           // single-CTA path: 32 warps
-constexpr int kFusedMaxSlotsPerWarp = 512;  // -> up to 16384 slots in one CTA
-constexpr int kChunkWarpsPerBlock = 4;    // multi-CTA path: warps (= chunks) per CTA
+constexpr int kWarps = 32;                // warps (= runs) per CTA
+constexpr int kThreads = 32 * kWarps;
+constexpr int kMinChunk = 1024;           // slots per CTA at least: one step of 32 per warp
+constexpr int kMaxChunk = 4096;           // ... and at most
+constexpr int kChunkTarget = 64;          // CTAs wanted between those two
+constexpr int64_t kRecountMaxSlots = 16384;  // see above
+constexpr int kBatch = 8;                 // loads issued together (latency hiding)
 
 __device__ __forceinline__ void flag_status(int* status, int code) {
   if (status != nullptr) atomicCAS(status, kStOk, code);
-}
-
-constexpr int kBatch = 8;  // steps of 32 slots whose index loads are issued together (latency hiding)
-
-// Counts one chunk [f0, f1) into hist[0..E) (shared memory, zeroed by the caller).
-__device__ __forceinline__ void count_chunk(const int32_t* __restrict__ topk_idx, int64_t f0, int64_t f1, int E,
-                                            int* hist, int* status) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t base = f0; base < f1; base += 32 * kBatch) {
-    int ev[kBatch];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int64_t f = base + 32 * u + lane;
-      ev[u] = (f < f1) ? __ldg(topk_idx + f) : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      if (base + 32 * u + lane >= f1) continue;
-      const int e = ev[u];
-      if (e >= 0 && e < E) atomicAdd(&hist[e], 1);  // integer adds commute: the count is order-independent
-      else flag_status(status, kStBadIndex);
-    }
-  }
-}
-
-// Places one chunk.  run[e] holds the destination of the chunk's next slot of expert e.
-__device__ __forceinline__ void place_chunk(const int32_t* __restrict__ topk_idx, int64_t f0, int64_t f1, int E,
-                                            int* run, int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  for (int64_t base0 = f0; base0 < f1; base0 += 32 * kBatch) {
-    int ev[kBatch];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int64_t f = base0 + 32 * u + lane;
-      ev[u] = (f < f1) ? __ldg(topk_idx + f) : -1;
-    }
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int64_t base = base0 + 32 * u;
-      if (base >= f1) break;  // uniform across the warp
-      const int64_t f = base + lane;
-      const int e = ev[u];
-      const bool valid = (e >= 0 && e < E);
-      const int keyv = valid ? e : (E + lane);  // invalid lanes never group with anyone
-      const unsigned peers = __match_any_sync(0xffffffffu, keyv);
-      int p = -1;
-      if (valid) p = run[e] + __popc(peers & lt_mask);
-      __syncwarp();
-      if (valid && (peers & lt_mask) == 0u) run[e] += __popc(peers);  // the lowest lane of a group advances it
-      __syncwarp();
-      if (f < f1) {
-        inv_perm[f] = p;
-        if (valid) perm[p] = (int32_t)f;
-      }
-    }
-  }
 }
 
 // Block-wide exclusive scan of counts[0..E) -> offsets[0..E]; E <= 1024, blockDim.x a multiple of 32 and >= E...
@@ -122,144 +74,196 @@ __device__ void block_exclusive_scan(const int* counts_sh, int E, int32_t* __res
   __syncthreads();
 }
 
-// ---- single-CTA path: count, scan and place in one launch -------------------------------------
-// shared memory: hist[kFusedWarps][E] | offsets_sh[E+1] | counts_sh[E] | warp_sums[33]
-__global__ void __launch_bounds__(kFusedWarps * 32)
-layout_fused_kernel(const int32_t* __restrict__ topk_idx, int n_slots, int E, int slots_per_warp,
-                    int32_t* __restrict__ counts, int32_t* __restrict__ offsets, int32_t* __restrict__ perm,
-                    int32_t* __restrict__ inv_perm, int* status) {
-  pdl_wait();
-  pdl_launch_dependents();
-  extern __shared__ int sh[];
-  int* hist = sh;
-  int* offsets_sh = hist + kFusedWarps * E;
-  int* counts_sh = offsets_sh + (E + 1);
-  int* warp_sums = counts_sh + E;
-  const int warp = threadIdx.x >> 5;
-
-  for (int i = threadIdx.x; i < kFusedWarps * E; i += blockDim.x) hist[i] = 0;
-  __syncthreads();
-  const int64_t f0 = min((int64_t)warp * slots_per_warp, (int64_t)n_slots);
-  const int64_t f1 = min(f0 + slots_per_warp, (int64_t)n_slots);
-  count_chunk(topk_idx, f0, f1, E, hist + warp * E, status);
-  __syncthreads();
-  // per expert: exclusive prefix over the warps' chunks, total into counts
-  for (int e = threadIdx.x; e < E; e += blockDim.x) {
-    int sum = 0;
-    for (int wv = 0; wv < kFusedWarps; ++wv) {
-      const int c = hist[wv * E + e];
-      hist[wv * E + e] = sum;
-      sum += c;
-    }
-    counts_sh[e] = sum;
-    counts[e] = sum;
-  }
-  __syncthreads();
-  block_exclusive_scan(counts_sh, E, offsets, offsets_sh, warp_sums);
-  int* run = hist + warp * E;
-  for (int e = threadIdx.x & 31; e < E; e += 32) run[e] += offsets_sh[e];
-  __syncwarp();
-  place_chunk(topk_idx, f0, f1, E, run, perm, inv_perm);
-}
-
-// ---- multi-CTA path ------------------------------------------------------------------------------
-// (1) per-chunk histograms: chunk_counts[chunk][e]
-__global__ void __launch_bounds__(kChunkWarpsPerBlock * 32)
-layout_count_kernel(const int32_t* __restrict__ topk_idx, int64_t n_slots, int E, int n_chunks,
-                    int32_t* __restrict__ chunk_counts, int* status) {
-  pdl_wait();
-  pdl_launch_dependents();
-  extern __shared__ int sh[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunk = blockIdx.x * kChunkWarpsPerBlock + warp;
-  int* hist = sh + warp * E;
-  for (int e = lane; e < E; e += 32) hist[e] = 0;
-  __syncwarp();
-  if (chunk >= n_chunks) return;
-  const int64_t f0 = (int64_t)chunk * kLayoutChunk;
-  const int64_t f1 = min(f0 + kLayoutChunk, n_slots);
-  count_chunk(topk_idx, f0, f1, E, hist, status);
-  __syncwarp();
-  for (int e = lane; e < E; e += 32) chunk_counts[(size_t)chunk * E + e] = hist[e];
-}
-
-// (2) per expert an exclusive prefix over chunks (in place) and the total -> counts.  One CTA per 32 experts;
-//     warp w owns the w-th of 32 contiguous runs of chunks, lane l the CTA's l-th expert, so a warp's loads are
-//     one 128-byte line per chunk and go out in batches of kBatch before anything depends on them.  A run of
-//     at most kBatch chunks (up to 65536 slots) is read once and kept in registers for the second walk.
-__global__ void __launch_bounds__(1024)
-layout_scan_kernel(int32_t* __restrict__ chunk_counts, int n_chunks, int E, int32_t* __restrict__ counts) {
-  pdl_wait();
-  pdl_launch_dependents();
-  __shared__ int partial[32][33];
-  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
-  const int e = blockIdx.x * 32 + lane;
-  const bool active = e < E;
-  const int per = (n_chunks + 31) / 32;
-  const int c0 = min(part * per, n_chunks), c1 = min(c0 + per, n_chunks);
-  int first[kBatch];  // the run's first batch
-#pragma unroll
-  for (int u = 0; u < kBatch; ++u) first[u] = (active && c0 + u < c1) ? chunk_counts[(size_t)(c0 + u) * E + e] : 0;
-  int sum = 0;
-#pragma unroll
-  for (int u = 0; u < kBatch; ++u) sum += first[u];
-  if (active) {
-    for (int cb = c0 + kBatch; cb < c1; cb += kBatch) {
-      int v[kBatch];
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u) v[u] = (cb + u < c1) ? chunk_counts[(size_t)(cb + u) * E + e] : 0;
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u) sum += v[u];
-    }
-  }
-  partial[part][lane] = sum;
-  __syncthreads();
-  if (!active) return;
-  int run = 0;
-  for (int q = 0; q < part; ++q) run += partial[q][lane];
-  if (part == 31) counts[e] = run + sum;
-#pragma unroll
-  for (int u = 0; u < kBatch; ++u) {
-    if (c0 + u < c1) chunk_counts[(size_t)(c0 + u) * E + e] = run;
-    run += first[u];
-  }
-  for (int cb = c0 + kBatch; cb < c1; cb += kBatch) {
-    int v[kBatch];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) v[u] = (cb + u < c1) ? chunk_counts[(size_t)(cb + u) * E + e] : 0;
+// Counts the slots [f0, f1) into hist[0..E) with all threads of the CTA (integer adds commute: the count does not
+// depend on their order).
+__device__ __forceinline__ void count_slots(const int32_t* __restrict__ topk_idx, int64_t f0, int64_t f1, int E, int* hist,
+                                            int* status) {
+  for (int64_t base = f0; base < f1; base += (int64_t)kThreads * kBatch) {
+    int ev[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
-      if (cb + u < c1) chunk_counts[(size_t)(cb + u) * E + e] = run;
-      run += v[u];
+      const int64_t f = base + u * kThreads + threadIdx.x;
+      ev[u] = (f < f1) ? __ldg(topk_idx + f) : -2;
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      if (base + u * kThreads + threadIdx.x >= f1) continue;
+      if (ev[u] >= 0 && ev[u] < E) atomicAdd(&hist[ev[u]], 1);
+      else flag_status(status, kStBadIndex);
     }
   }
 }
 
-// (3) every CTA scans the counts over experts itself (CTA 0 also stores the result -> offsets) and places its
-//     chunks at offsets[e] + (prefix of earlier chunks)[e]
-//     shared memory: run[warps][E] | counts_sh[E] | offsets_sh[E+1] | warp_sums[33]
-__global__ void __launch_bounds__(kChunkWarpsPerBlock * 32)
-layout_place_kernel(const int32_t* __restrict__ topk_idx, int64_t n_slots, int E, int n_chunks,
-                    const int32_t* __restrict__ chunk_prefix, const int32_t* __restrict__ counts,
-                    int32_t* __restrict__ offsets, int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm) {
+// chunk_counts[chunk][e] of the CTA's chunk.
+__global__ void __launch_bounds__(kThreads)
+layout_count_kernel(const int32_t* __restrict__ topk_idx, int64_t n_slots, int E, int chunk,
+                    int32_t* __restrict__ chunk_counts, int* status) {
+  extern __shared__ int sh[];
+  for (int e = threadIdx.x; e < E; e += kThreads) sh[e] = 0;
   pdl_wait();
   pdl_launch_dependents();
-  extern __shared__ int sh[];
-  int* counts_sh = sh + kChunkWarpsPerBlock * E;
-  int* offsets_sh = counts_sh + E;
-  int* warp_sums = offsets_sh + (E + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int e = threadIdx.x; e < E; e += blockDim.x) counts_sh[e] = counts[e];
   __syncthreads();
-  block_exclusive_scan(counts_sh, E, blockIdx.x == 0 ? offsets : nullptr, offsets_sh, warp_sums);
-  const int chunk = blockIdx.x * kChunkWarpsPerBlock + warp;
-  if (chunk >= n_chunks) return;
-  int* run = sh + warp * E;
-  for (int e = lane; e < E; e += 32) run[e] = offsets_sh[e] + chunk_prefix[(size_t)chunk * E + e];
-  __syncwarp();
-  const int64_t f0 = (int64_t)chunk * kLayoutChunk;
-  const int64_t f1 = min(f0 + kLayoutChunk, n_slots);
-  place_chunk(topk_idx, f0, f1, E, run, perm, inv_perm);
+  const int64_t f0 = (int64_t)blockIdx.x * chunk;
+  count_slots(topk_idx, f0, min(f0 + chunk, n_slots), E, sh, status);
+  __syncthreads();
+  for (int e = threadIdx.x; e < E; e += kThreads) chunk_counts[(size_t)blockIdx.x * E + e] = sh[e];
+}
+
+// base[e] += counts of the chunks before this CTA's, total[e] += those of the chunks behind it.  A thread takes V
+// consecutive experts and every parts-th chunk, kBatch chunks' loads in flight.
+template <int V>
+__device__ __forceinline__ void sum_chunks(const int32_t* __restrict__ chunk_counts, int E, int* base, int* total) {
+  const int EV = E / V, parts = max(1, kThreads / EV), n_chunks = (int)gridDim.x, me = (int)blockIdx.x;
+  for (int i = threadIdx.x; i < parts * EV; i += kThreads) {
+    const int part = i / EV, e = (i - part * EV) * V;
+    int before[V] = {}, after[V] = {};
+    for (int q = part; q < n_chunks; q += parts * kBatch) {
+      int v[kBatch][V];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int c = q + u * parts;
+        const int32_t* src = chunk_counts + (size_t)c * E + e;
+        if constexpr (V == 4) {
+          const int4 w = c < n_chunks ? *reinterpret_cast<const int4*>(src) : make_int4(0, 0, 0, 0);
+          v[u][0] = w.x; v[u][1] = w.y; v[u][2] = w.z; v[u][3] = w.w;
+        } else {
+          v[u][0] = c < n_chunks ? *src : 0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int c = q + u * parts;
+#pragma unroll
+        for (int x = 0; x < V; ++x) {
+          if (c < me) before[x] += v[u][x];
+          else if (c > me) after[x] += v[u][x];
+        }
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < V; ++x) {
+      if (before[x]) atomicAdd(&base[e + x], before[x]);
+      if (after[x]) atomicAdd(&total[e + x], after[x]);
+    }
+  }
+}
+
+// Places the CTA's chunk; CTA 0 also stores counts and offsets.  chunk_counts: every chunk's counts, or nullptr: the
+// CTA counts the other chunks itself.
+// shared memory: hist[kWarps][E] | base[E] | total[E] | offsets_sh[E+1] | warp_sums[33]
+__global__ void __launch_bounds__(kThreads)
+layout_place_kernel(const int32_t* __restrict__ topk_idx, int64_t n_slots, int E, int chunk,
+                    const int32_t* __restrict__ chunk_counts, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
+                    int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm, int* status) {
+  extern __shared__ int sh[];
+  int* hist = sh;                 // per warp: counts of its run, then their prefix over the warps before it
+  int* base = hist + kWarps * E;  // slots of earlier chunks, then the destination of the chunk's first slot
+  int* total = base + E;
+  int* offsets_sh = total + E;
+  int* warp_sums = offsets_sh + (E + 1);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt_mask = (1u << lane) - 1u;
+  for (int i = threadIdx.x; i < (kWarps + 2) * E; i += kThreads) sh[i] = 0;
+  pdl_wait();
+  pdl_launch_dependents();
+  const int64_t c0 = (int64_t)blockIdx.x * chunk, c1 = min(c0 + chunk, n_slots);
+  const int run = chunk / kWarps;  // a multiple of 32
+  const int64_t f0 = min(c0 + (int64_t)warp * run, c1), f1 = min(f0 + run, c1);
+  int* mine = hist + warp * E;
+  const bool one_step = run == 32;
+  // one step: the warp's index and its rank among the step's equals stay in registers
+  int e1 = -1, rank1 = 0;
+  if (one_step) {
+    if (f0 + lane < f1) e1 = __ldg(topk_idx + f0 + lane);
+    const bool valid = e1 >= 0 && e1 < E;
+    if (f0 + lane < f1 && !valid) flag_status(status, kStBadIndex);
+    if (!valid) e1 = -1;
+    const unsigned peers = __match_any_sync(0xffffffffu, valid ? e1 : E);  // (the slower, the more values there are)
+    rank1 = __popc(peers & lt_mask);
+    __syncthreads();  // the counters are zero
+    if (valid && rank1 == 0) mine[e1] = __popc(peers);
+  } else {
+    __syncthreads();
+    for (int64_t b = f0; b < f1; b += 32 * kBatch) {
+      int ev[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int64_t f = b + 32 * u + lane;
+        ev[u] = (f < f1) ? __ldg(topk_idx + f) : -2;
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        if (b + 32 * u + lane >= f1) continue;
+        if (ev[u] >= 0 && ev[u] < E) atomicAdd(&mine[ev[u]], 1);
+        else flag_status(status, kStBadIndex);
+      }
+    }
+  }
+  if (gridDim.x > 1) {
+    if (chunk_counts == nullptr) {
+      count_slots(topk_idx, 0, c0, E, base, nullptr);
+      count_slots(topk_idx, c1, n_slots, E, total, nullptr);
+    } else if (E % 4 == 0) {
+      sum_chunks<4>(chunk_counts, E, base, total);
+    } else {
+      sum_chunks<1>(chunk_counts, E, base, total);
+    }
+  }
+  __syncthreads();
+  // per expert: exclusive prefix over the warps' runs, and the total over all chunks
+  for (int e = threadIdx.x; e < E; e += kThreads) {
+    int sum = 0;
+#pragma unroll
+    for (int w0 = 0; w0 < kWarps; w0 += 16) {  // 16 reads in flight
+      int v[16];
+#pragma unroll
+      for (int w = 0; w < 16; ++w) v[w] = hist[(w0 + w) * E + e];
+#pragma unroll
+      for (int w = 0; w < 16; ++w) {
+        hist[(w0 + w) * E + e] = sum;
+        sum += v[w];
+      }
+    }
+    total[e] += base[e] + sum;  // later chunks, earlier ones, this one
+    if (blockIdx.x == 0) counts[e] = total[e];
+  }
+  __syncthreads();
+  block_exclusive_scan(total, E, blockIdx.x == 0 ? offsets : nullptr, offsets_sh, warp_sums);
+  for (int e = threadIdx.x; e < E; e += kThreads) base[e] += offsets_sh[e];
+  __syncthreads();
+  if (one_step) {
+    if (f0 + lane < f1) {
+      const int p = e1 >= 0 ? base[e1] + mine[e1] + rank1 : -1;
+      inv_perm[f0 + lane] = p;
+      if (p >= 0) perm[p] = (int32_t)(f0 + lane);
+    }
+    return;
+  }
+  for (int64_t b = f0; b < f1; b += 32 * kBatch) {
+    int ev[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int64_t f = b + 32 * u + lane;
+      ev[u] = (f < f1) ? __ldg(topk_idx + f) : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      if (b + 32 * u >= f1) break;  // uniform across the warp
+      const int64_t f = b + 32 * u + lane;
+      const int e = ev[u];
+      const bool valid = e >= 0 && e < E;
+      const unsigned peers = __match_any_sync(0xffffffffu, valid ? e : E);
+      int p = -1;
+      if (valid) p = base[e] + mine[e] + __popc(peers & lt_mask);
+      __syncwarp();
+      if (valid && (peers & lt_mask) == 0u) mine[e] += __popc(peers);  // the lowest lane of a group advances it
+      __syncwarp();
+      if (f < f1) {
+        inv_perm[f] = p;
+        if (valid) perm[p] = (int32_t)f;
+      }
+    }
+  }
 }
 
 __global__ void layout_empty_kernel(int E, int32_t* __restrict__ counts, int32_t* __restrict__ offsets) {
@@ -282,29 +286,25 @@ cudaError_t launch_layout(const int32_t* topk_idx, int64_t n_slots, int E, int32
     if (err == cudaSuccess && n_launches) *n_launches += 1;
     return err;
   }
-  const size_t fused_smem = ((size_t)kFusedWarps * E + (E + 1) + E + 33) * sizeof(int);
-  if (n_slots <= (int64_t)kFusedWarps * kFusedMaxSlotsPerWarp && fused_smem <= 200 * 1024) {
-    int spw = (int)((n_slots + kFusedWarps - 1) / kFusedWarps);
-    spw = (spw + 31) / 32 * 32;
-    if ((err = ensure_dynamic_smem(layout_fused_kernel, fused_smem)) != cudaSuccess) return err;
-    err = launch_pdl(true, layout_fused_kernel, dim3(1), dim3(kFusedWarps * 32), fused_smem, stream, topk_idx, (int)n_slots, E, spw, counts, offsets,
-                                                                     perm, inv_perm, status);
-    if (err == cudaSuccess && n_launches) *n_launches += 1;
-    return err;
+  // (every CTA reads n_chunks x E counts: fewer, larger chunks where E is large)
+  const int target = E > 512 ? kChunkTarget / 2 : kChunkTarget;
+  int64_t chunk = (n_slots + target - 1) / target;
+  chunk = chunk < kMinChunk ? kMinChunk : chunk > kMaxChunk ? kMaxChunk : (chunk + kMinChunk - 1) / kMinChunk * kMinChunk;
+  const int n_chunks = (int)((n_slots + chunk - 1) / chunk);
+  int n = 1;
+  const int32_t* chunk_counts = nullptr;
+  if (n_slots > kRecountMaxSlots) {
+    if ((err = launch_pdl(true, layout_count_kernel, dim3(n_chunks), dim3(kThreads), (size_t)E * sizeof(int), stream, topk_idx,
+                          n_slots, E, (int)chunk, scratch, status)) != cudaSuccess) return err;
+    chunk_counts = scratch;
+    ++n;
   }
-  const int n_chunks = (int)((n_slots + kLayoutChunk - 1) / kLayoutChunk);
-  const int blocks = (n_chunks + kChunkWarpsPerBlock - 1) / kChunkWarpsPerBlock;
-  const size_t chunk_smem = (size_t)kChunkWarpsPerBlock * E * sizeof(int);
-  if ((err = launch_pdl(true, layout_count_kernel, dim3(blocks), dim3(kChunkWarpsPerBlock * 32), chunk_smem, stream, topk_idx, n_slots, E, n_chunks,
-                                                                                scratch, status)) != cudaSuccess) return err;
-  if ((err = launch_pdl(true, layout_scan_kernel, dim3((E + 31) / 32), dim3(1024), 0, stream, scratch, n_chunks, E, counts)) != cudaSuccess) return err;
-  const size_t place_smem = chunk_smem + ((size_t)E + (E + 1) + 33) * sizeof(int);
-  launch_pdl(true, layout_place_kernel, dim3(blocks), dim3(kChunkWarpsPerBlock * 32), place_smem, stream, topk_idx, n_slots, E, n_chunks,
-                                                                                scratch, counts, offsets, perm,
-                                                                                inv_perm);
-  if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  if (n_launches) *n_launches += 3;
-  return cudaSuccess;
+  const size_t smem = ((size_t)(kWarps + 3) * E + 1 + 33) * sizeof(int);
+  if ((err = ensure_dynamic_smem(layout_place_kernel, smem)) != cudaSuccess) return err;
+  err = launch_pdl(true, layout_place_kernel, dim3(n_chunks), dim3(kThreads), smem, stream, topk_idx, n_slots, E, (int)chunk,
+                   chunk_counts, counts, offsets, perm, inv_perm, status);
+  if (err == cudaSuccess && n_launches) *n_launches += n;
+  return err;
 }
 
 }  // namespace moe
