@@ -308,24 +308,40 @@ int gemm_ctas(const moe_ctx* ctx) {
 }
 
 // The choice between the two tensor-core variants for a PREFILL context, per pass, from the rows per expert
-// R = rows / experts and the pass's K.  Measured on a B200 with the variants interleaved in long blocks
-// (DeepSeek-V3- and Qwen3-30B-shaped layers, uniform and Zipf routing, whole steps and per-pass stage times):
-//  * with tiles of up to 256 tokens the small-M kernel moves fewer bytes through shared memory per flop than the
-//    large-M kernel (one CTA's MMA operands come from shared memory, whose bandwidth both end up waiting for), but
-//    its tiles of more than 128 tokens fill tensor memory, so their epilogue is exposed: the longer K is, the less
-//    that weighs;
-//  * gated pass: K = 7168 -- small-M ahead by 4-13 % at every R up to 1024; K = 2048 -- level or ahead from R = 448
-//    to 1024, behind by 3-10 % below that;
-//  * down pass: K = 2048 -- small-M ahead up to R ~ 320 and 10-17 % behind above; K = 768 (12 k-blocks per tile: an
-//    exposed epilogue is a quarter of a tile) -- behind by 9-25 % at every R;
-//  * problems of up to 8192 rows, whose launches overlap with their neighbours, are 1.5-6 % faster on the small-M
-//    kernel at any shape: it builds its tile list and fetches weights before the previous kernel has finished;
-//  * FP8 (half the operand bytes per flop, so the issue cost of two MMAs per 16 K-elements shows): small-M up to
-//    R = 256 (gated, K >= 4096) and 128 (down, K >= 1536); with shorter K (half as many k-blocks per tile as bf16)
-//    large-M is 8-10 % ahead above the launch-overlap regime.
-constexpr int64_t kSmallMRowsGated = 1024, kSmallMRowsGatedShortKFrom = 448, kSmallMRowsDown = 320;
-constexpr int64_t kSmallMRowsFp8Gated = 256, kSmallMRowsFp8Down = 128;
-constexpr int kLongK = 4096, kShortDownK = 1536;
+// R = rows / experts and the pass's K.  The small-M kernel reads an expert's weights once for up to 256 rows, multiplies
+// exactly the rows there are and moves fewer bytes through shared memory per flop; the large-M kernel multiplies rows in
+// steps of 128 but always overlaps its epilogue with the next tile, which counts when K is short.  Both draw the GPU's
+// power limit at these sizes, so the lines below are whole steps in the sustained state (each variant run for 0.12 s
+// before it was timed for 0.12 s, in turns), gated / down pass, s = small-M, l = large-M, us:
+//   bf16  K = 2048 / 768 (hidden 2048, 128 experts):  R = 95 ss 289 sl 285 ll 280;  131 335 337 351;  156 358 366 397;
+//         187 397 397 414;  325 578 563 572;  512 808 785 820;  750 1121 1082 1106;  1500 2113 2036 2096
+//         K = 2560 / 1024 (512 experts):  31 ss 1315 sl 1380 ll 1490;  64 1482 1511 1579;  187 2197 2266 2541;
+//         312 3358 3381 3573;  375 3757 3748 3911;  468 4447 4445 4697
+//         K = 7168 / 2048 (256 experts + shared):  46 ss 3784 sl 4041 ll 4615;  281 8907 9599 10410;  500 14111 15087
+//         16142;  750 20017 19998 19769;  937 24815 25055 25740;  Zipf routing, 1024: 24911 25075 26394
+//   FP8   K = 2048 / 768:  93 ss 204 sl 202 ll 196;  156 271 273 271;  187 304 299 284;  375 506 479 448;  1500 1708 1566
+//         1466
+//         K = 2560 / 1024:  31 ss 744 sl 773 ll 879;  64 886 894 923;  156 1365 1390 1538;  218 1697 1610 1719;
+//         312 2337 2258 2252;  468 3306 3095 3040
+//         K = 7168 / 2048:  46 ss 2073 sl 2185 ll 2520;  128 3011 3154 3475;  281 5038 5137 5653;  437 7048 7042 7467;
+//         500 7904 7674 8118;  625 9928 9732 11110;  1000 14867 14629 16121
+constexpr int kLongK = 4096, kMidK = 2560, kMidDownK = 1024, kLongDownK = 2048;
+constexpr int64_t kOneTileRows = 120;     // an expert's rows fit one 128-row tile, spread included
+constexpr int64_t kShortKDownRows = 200;  // bf16 down pass, K < 1024: small-M between these two
+constexpr int64_t kMidKDownRows = 350;    // ... 1024 <= K < 2048: small-M up to here; from K = 2048 on at every R
+constexpr int64_t kFp8MidKRows = 300, kFp8MidKDownRows = 180, kFp8LongKDownRows = 400;
+
+bool small_m_is_faster(bool fp8, bool gated, int K, int64_t rows, int64_t E) {
+  const auto up_to = [&](int64_t r) { return rows <= r * E; };
+  if (gated) {
+    if (fp8) return K >= kLongK || (K >= kMidK && up_to(kFp8MidKRows));
+    return K >= kMidK || !up_to(kOneTileRows);
+  }
+  if (fp8) return K >= kLongDownK ? up_to(kFp8LongKDownRows) : K >= kMidDownK && up_to(kFp8MidKDownRows);
+  if (K >= kLongDownK) return true;
+  if (K >= kMidDownK) return up_to(kMidKDownRows);
+  return !up_to(kOneTileRows) && up_to(kShortKDownRows);
+}
 
 // moe_layer_host: the down pass in one piece for every 1.5 MB of output, up to four; two chunks of tokens from 200 rows
 // per expert and 4 MB a chunk on.  Measured on the Qwen3-30B-shaped layer with pinned buffers (whole call; before: copy,
@@ -346,17 +362,9 @@ int gemm_variant_of(const moe_ctx* ctx, const moe::GemmProblem& p) {
   if (ctx->cfg.phase == MOE_PHASE_DECODE) return MOE_GEMM_SMALL_M;
   if (ctx->cfg.row_gather == 1) return MOE_GEMM_LARGE_M;  // only the large-M kernel gathers its rows itself
   if (ctx->preemptible) return MOE_GEMM_SMALL_M;          // only the small-M kernel can stop between tiles
-  const int64_t E = p.E;  // 1 for a dense problem
-  bool small;
-  if (p.rows_bound <= moe::kGemmOverlapMaxRows) {
-    small = true;
-  } else if (p.fp8) {
-    small = p.K >= (p.gated ? kLongK : kShortDownK) && p.rows_bound <= (p.gated ? kSmallMRowsFp8Gated : kSmallMRowsFp8Down) * E;
-  } else if (p.gated) {
-    small = p.rows_bound <= kSmallMRowsGated * E && (p.K >= kLongK || p.rows_bound >= kSmallMRowsGatedShortKFrom * E);
-  } else {
-    small = p.K >= kShortDownK && p.rows_bound <= kSmallMRowsDown * E;
-  }
+  // problems of up to 8192 rows, whose launches overlap with their neighbours, are 1.5-6 % faster on the small-M kernel
+  // at any shape: it builds its tile list and fetches weights before the previous kernel has finished
+  const bool small = p.rows_bound <= moe::kGemmOverlapMaxRows || small_m_is_faster(p.fp8, p.gated, p.K, p.rows_bound, p.E);
   return small ? MOE_GEMM_SMALL_M : MOE_GEMM_LARGE_M;
 }
 
