@@ -681,7 +681,11 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
           const int c = c_first + m * c_step;
-          if (c < t.rows) {
+          // Leave, do not skip chunk by chunk: the unrolled chunks are kilobytes of code that a launch of small tiles would
+          // fetch from a cold instruction cache just to jump over them (tiny layer, 64 tokens: 28.5 -> 26.2 us a step,
+          // one-token V3-shaped decode 143.1 -> 138.1 us).
+          if (c >= t.rows) break;
+          {
             float g[16], u[16];
             tmem_ld_wait();
 #pragma unroll
@@ -710,7 +714,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
           const int c = c_first + m * c_step;
-          if (c < t.rows) {
+          if (c >= t.rows) break;
+          {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               const uint32_t mine = pk[m][i];
