@@ -340,18 +340,25 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       uint32_t head = 0, free_slots = R, kb_idx = 0, oldest = 0;
       bool ok = true;
       // Early set-up: until this thread has waited for the previous kernel, token-row copies are put off (their
-      // ring space is allocated and their bytes announced) while the weight boxes of up to kNB k-blocks go out.
+      // ring space is allocated and their bytes announced) while the weight boxes of up to kNB k-blocks of the first
+      // tile go out.  The copies put off are the ring's first allocations, so they are found again by walking it from
+      // its start (a list of them would live in local memory, which is cold here).
       bool dep_waited = !p.early_setup;
-      int n_def = 0;
-      uint32_t def_dst[kNB], def_full[kNB];
-      int def_k0[kNB], def_row0[kNB];
-      const CUtensorMap* def_map[kNB];
+      uint32_t n_def = 0, def_nx = 0;
+      int def_row0 = 0;
+      const CUtensorMap* def_map = nullptr;
       auto dep_wait_and_flush = [&]() {
         pdl_wait();
         pdl_launch_dependents();
         dep_waited = true;
-        for (int i = 0; i < n_def; ++i) tma_load_2d(def_dst[i], def_map[i], def_full[i], def_k0[i], def_row0[i]);
-        n_def = 0;
+        uint32_t h = 0;
+        for (uint32_t i = 0; i < n_def; ++i) {
+          if (h + (uint32_t)kWSlots > R) h = 0;
+          h += (uint32_t)kWSlots;
+          if (h + def_nx > R) h = 0;
+          tma_load_2d(base_addr + h * (uint32_t)kSlotBytes, def_map, bar_full + 8u * i, (int)i * kbk, def_row0);
+          h += def_nx;
+        }
       };
       [[maybe_unused]] long long prof_wait_empty = 0, prof_tiles = 0;
       [[maybe_unused]] const long long prof_start = clock64();
@@ -409,6 +416,11 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         const int w_e = t.dense ? 0 : p.e_base + t.e;
         const int num_kb = t.dense ? num_kb2 : num_kb1;
         const int fetch_kb = num_kb > 4 ? num_kb - 4 : 0;
+        if (!dep_waited) {
+          def_nx = n >> 4;
+          def_map = mx;
+          def_row0 = t.row0;
+        }
         for (int kb = 0, k0 = 0; kb < num_kb && ok; ++kb, k0 += kbk) {
           if (kb == fetch_kb) {
             if (p.yield_req != nullptr) {
@@ -458,16 +470,13 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
           if (dep_waited) {
             tma_load_2d(base_addr + head_x * (uint32_t)kSlotBytes, mx, full, k0, t.row0);
           } else {
-            def_dst[n_def] = base_addr + head_x * (uint32_t)kSlotBytes;
-            def_full[n_def] = full;
-            def_map[n_def] = mx;
-            def_k0[n_def] = k0;
-            def_row0[n_def] = t.row0;
             ++n_def;
           }
           head = head_x + nx;
           ++kb_idx;
         }
+        // (before the next tile's number is looked at: its atomic is still on its way)
+        if (!dep_waited) dep_wait_and_flush();
         if (stop_after && ok) {
           *stopped_here = 1;  // no further tile is taken: the other roles finish the published ones and leave
           if (!publish(-1)) ok = false;
