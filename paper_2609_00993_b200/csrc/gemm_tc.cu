@@ -46,6 +46,7 @@ constexpr int kGatherThreads = 128;
 constexpr int kThreadsGather = kThreads + kGatherThreads;
 constexpr int kMaxStages = 8;
 constexpr int kEpiStagingBytes = kEpilogueWarps * 32 * 128;  // per-warp 32 x 128-byte staging tiles
+constexpr int kScaleBytes = 2 * 256 * 4;                     // FP8: a tile's weight-row scales, double-buffered
 
 struct TcParams {
   const int32_t* offsets;  // [E+1] (already advanced to the first expert of the launch) or nullptr
@@ -139,14 +140,15 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
   static_assert(!(GATHER && FP8), "the row gather exists for bf16 operands only");
   constexpr int kbk = FP8 ? 2 * kBlockK : kBlockK;  // K elements per stage
   extern __shared__ uint8_t smem_raw[];
-  // carve: [stages] | epilogue staging (large-M) | barriers | tmem slot | abort | prefix[E+1] | seg[E+1]
+  // carve: [stages] | epilogue staging (large-M) | FP8: scales | barriers | tmem slot | abort | prefix[E+1] | seg[E+1]
   //   stage: W box0 | W box1 | X tile
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base_addr = (raw_addr + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (base_addr - raw_addr);
   const int stage_bytes = 2 * kWBoxBytes + p.x_tile_bytes;
   uint8_t* epi_smem = base + (size_t)p.n_stages * stage_bytes;  // kEpilogueWarps x 4 KB, large-M only
-  uint8_t* after = epi_smem + kEpiStagingBytes;
+  float* scales = reinterpret_cast<float*>(epi_smem + kEpiStagingBytes);
+  uint8_t* after = epi_smem + kEpiStagingBytes + (FP8 ? kScaleBytes : 0);
   uint64_t* bars = reinterpret_cast<uint64_t*>(after);  // full[S], empty[S], tmem_full[2], tmem_empty[2]
   const uint32_t bar_full = smem_u32(bars);
   const uint32_t bar_empty = bar_full + 8u * p.n_stages;
@@ -351,15 +353,27 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty + 8u * as);
       };
+      __nv_bfloat16* const out = t.dense ? p.out2 : p.out;
+      const int n_feat = t.dense ? p.n_feat2 : p.n_feat;
+      // FP8: the tile's scales are fetched while it is still being multiplied -- the row's in a register, the weight rows'
+      // (gated: 128 gate rows, then the 128 up rows) in shared memory.  They are different ones for every tile, so read
+      // where they are used every 32 columns waited for L2 (Qwen3-shaped layer, T = 6007: down pass 137 -> 118 us, T = 2000: 67 -> 55).
+      float rs = 0.f;
+      float* const sc = scales + as * 256u;
+      if (FP8) {
+        const float* const wsp =
+            t.dense ? p.w_scale2 : p.w_scale + (size_t)(p.e_base + t.e) * (GATED ? 2 : 1) * n_feat;
+        const int r = warp * 32 + lane;  // 0..127
+        if (r < t.rows) rs = __ldg((t.dense ? p.row_scale2 : p.row_scale) + t.row0 + r);
+        const int f = t.ft * kFeatPerTile + r;
+        const int f2 = GATED ? n_feat + f : f + 128;
+        sc[r] = f < n_feat ? __ldg(wsp + f) : 0.f;
+        sc[128 + r] = (GATED ? f : f2) < n_feat ? __ldg(wsp + f2) : 0.f;
+        asm volatile("barrier.cta.sync 1, 128;" ::: "memory");
+      }
       if (!mbar_wait(bar_tfull + 8u * as, aph, abort_flag, p.wait_limit_ns)) { ok = false; break; }
       tc_fence_after();
       const uint32_t d0 = tmem_base + as * acc_cols + lane_base;
-      __nv_bfloat16* const out = t.dense ? p.out2 : p.out;
-      const int n_feat = t.dense ? p.n_feat2 : p.n_feat;
-      // FP8: scales of this tile's rows and of its expert's weight rows (gate rows first, then up rows)
-      const float* const rsp = FP8 ? (t.dense ? p.row_scale2 : p.row_scale) + t.row0 : nullptr;
-      const float* const wsp =
-          FP8 ? (t.dense ? p.w_scale2 : p.w_scale + (size_t)(p.e_base + t.e) * (GATED ? 2 : 1) * n_feat) : nullptr;
       bool released = false;  // has this warp already handed the accumulator stage back?
       {
         // lane = token row, column = output feature.  Two 32-column chunks (128 bytes of a row) at a time go
@@ -370,7 +384,6 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         constexpr int kPairs = kFeatPerTile / 64;
         uint8_t* stage_tile = epi_smem + warp * 4096;  // 32 rows x 128 bytes
         const int rows_here = t.rows - warp * 32;       // rows of this warp's 32 that are valid (may be <= 0)
-        const float rs = (FP8 && lane < rows_here) ? rsp[warp * 32 + lane] : 0.f;  // FP8: this lane's row scale
         for (int pc = 0; pc < kPairs; ++pc) {
           const int f0 = t.ft * kFeatPerTile + pc * 64;
           if (f0 >= n_feat) break;  // uniform across the CTA
@@ -378,9 +391,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
           for (int h = 0; h < 2; ++h) {
             uint32_t ra[32], packed[16];
             tmem_ld32(d0 + (uint32_t)(pc * 64 + h * 32), ra);
-            // FP8: the 32 columns' weight-row scales (the same for every lane: broadcast loads); a chunk that
-            // reaches past n_feat reads no scales and is not stored either
-            const bool scaled = FP8 && f0 + h * 32 + 32 <= n_feat;
+            const float4* const sc4 = reinterpret_cast<const float4*>(sc + pc * 64 + h * 32);  // broadcast reads
             if (GATED) {
               uint32_t rb[32];
               tmem_ld32(d0 + (uint32_t)(128 + pc * 64 + h * 32), rb);
@@ -388,10 +399,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
               if (FP8) {
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                  const float4 sg = scaled ? __ldg(reinterpret_cast<const float4*>(wsp + f0 + h * 32) + q)
-                                           : make_float4(0.f, 0.f, 0.f, 0.f);
-                  const float4 su = scaled ? __ldg(reinterpret_cast<const float4*>(wsp + n_feat + f0 + h * 32) + q)
-                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+                  const float4 sg = sc4[q], su = sc4[32 + q];
                   ra[4 * q + 0] = __float_as_uint(__uint_as_float(ra[4 * q + 0]) * (rs * sg.x));
                   ra[4 * q + 1] = __float_as_uint(__uint_as_float(ra[4 * q + 1]) * (rs * sg.y));
                   ra[4 * q + 2] = __float_as_uint(__uint_as_float(ra[4 * q + 2]) * (rs * sg.z));
@@ -411,8 +419,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
               if (FP8) {
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                  const float4 sw = scaled ? __ldg(reinterpret_cast<const float4*>(wsp + f0 + h * 32) + q)
-                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+                  const float4 sw = sc4[q];
                   ra[4 * q + 0] = __float_as_uint(__uint_as_float(ra[4 * q + 0]) * (rs * sw.x));
                   ra[4 * q + 1] = __float_as_uint(__uint_as_float(ra[4 * q + 1]) * (rs * sw.y));
                   ra[4 * q + 2] = __float_as_uint(__uint_as_float(ra[4 * q + 2]) * (rs * sw.z));
@@ -644,7 +651,7 @@ cudaError_t launch_gemm_tc(const GemmProblem& p, const GemmDenseGroup* dense, in
   prm.inject_producer_stall = p.debug_stall ? 1 : 0;
   prm.wait_limit_ns = p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs;
   const int stage_bytes = 2 * kWBoxBytes + prm.x_tile_bytes;
-  const size_t tail = kEpiStagingBytes + (2 * kMaxStages + 4) * sizeof(uint64_t) +
+  const size_t tail = kEpiStagingBytes + (fp8 ? kScaleBytes : 0) + (2 * kMaxStages + 4) * sizeof(uint64_t) +
                       2 * sizeof(uint32_t) + 2 * (size_t)(prm.E + 1) * sizeof(int);
   int stages = (int)((kSmemBudget - 1024 - (int)tail) / stage_bytes);
   if (stages > kMaxStages) stages = kMaxStages;
