@@ -707,19 +707,15 @@ moe_status enqueue_row_movement(moe_ctx* ctx, const char* who, const void* x) {
   int n = 0;
   cudaError_t e = cudaSuccess;
   if (T > 0 && fp8) {
-    {
-      StageTimer tm(ctx, 8);
-      e = moe::launch_quantize_rows(x, T, ctx->cfg.hidden, b.xq_tok, b.sx_tok, ctx->stream, &n);
-    }
-    if (e == cudaSuccess) {
-      StageTimer tm(ctx, 2);
-      e = moe::launch_permute(b.xq_tok, ctx->inv_perm, b.xq, T, ctx->cfg.top_k, ctx->cfg.hidden / 2, ctx->status,
-                              ctx->stream, &n, b.sx_tok, b.sx, ctx->wait_limit_ns);
-    }
+    // (in token order only for the shared expert's pass)
+    const bool shared = ctx->cfg.n_shared != 0;
+    StageTimer tm(ctx, 8);
+    e = moe::launch_quantize_move(x, T, ctx->cfg.hidden, shared ? b.xq_tok : nullptr, shared ? b.sx_tok : nullptr,
+                                  ctx->inv_perm, ctx->cfg.top_k, b.xq, b.sx, ctx->stream, &n);
   } else if (T > 0 && !gathers_rows(ctx)) {
     StageTimer tm(ctx, 2);
     e = moe::launch_permute(x, ctx->inv_perm, b.x_perm, T, ctx->cfg.top_k, ctx->cfg.hidden, ctx->status, ctx->stream,
-                            &n, nullptr, nullptr, ctx->wait_limit_ns);
+                            &n, ctx->wait_limit_ns);
   }
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->launches += n;

@@ -73,12 +73,9 @@ cudaError_t launch_layout(const int32_t* topk_idx, int64_t n_slots, int E, int32
                           int* n_launches);
 
 // ---- a5 permute, a9 combine ----------------------------------------------------------------
-// H counts 2-byte columns (a row of H E4M3 codes is H/2 of them).  row_val / row_val_perm (optional): one fp32
-// value per source row is copied to each of its destination rows.
 // wait_limit_ns: time limit of the kernels' bounded waits (0 = the default of 2 s).
 cudaError_t launch_permute(const void* x, const int32_t* inv_perm, void* x_perm, int T, int k, int H, int* status,
-                           cudaStream_t stream, int* n_launches, const float* row_val = nullptr,
-                           float* row_val_perm = nullptr, unsigned long long wait_limit_ns = 0);
+                           cudaStream_t stream, int* n_launches, unsigned long long wait_limit_ns = 0);
 // Columns [c_begin, c_end) of the rows (c_end < 0: all; multiples of 8).
 cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32_t* inv_perm, const float* topk_w,
                            void* out, int T, int k, int H, int* status, cudaStream_t stream, int* n_launches,
@@ -164,9 +161,13 @@ struct GemmDenseGroup {
 };
 
 // FP8 variant: per-row dynamic quantisation of bf16 rows [rows, n] -> E4M3 codes [rows, n] + scale [rows]
-// (n a multiple of 8, at most 8192).
+// (n a multiple of 16, at most 8192).
 cudaError_t launch_quantize_rows(const void* x, int64_t rows, int n, void* q, float* scale, cudaStream_t stream,
                                  int* n_launches);
+// The same for T token rows, whose codes and scales also go to their k places in the dispatch: row inv_perm[t * k + j] of
+// q_perm / scale_perm (negative: dropped).  q and scale (token order) may be nullptr.
+cudaError_t launch_quantize_move(const void* x, int T, int n, void* q, float* scale, const int32_t* inv_perm, int k,
+                                 void* q_perm, float* scale_perm, cudaStream_t stream, int* n_launches);
 
 cudaError_t launch_gemm_validation(const GemmProblem& p, cudaStream_t stream, int* n_launches);
 
