@@ -19,7 +19,7 @@
 //              neighbouring lanes exchange values so that every store writes a feature pair.  The gated epilogue
 //              hands the accumulator back before its exchanges and stores.
 //   schedule   the tile list is ordered by expert size, largest first.  Its first waves are dealt statically (CTAs
-//              in step share weights and rows through L2), the last two waves' worth of tiles -- the smallest -- are
+//              in step share weights and rows through L2), the last waves' worth of tiles -- the smallest -- are
 //              handed out by an atomic counter to whichever CTA is free; the producer publishes the tiles it takes
 //              in a four-entry queue that the MMA issuer and the epilogue warps follow.
 //   set-up     with the launch overlap, the tile list is built and weight boxes are requested before the kernel
@@ -70,10 +70,13 @@ constexpr int kNB = 8;                                  // k-blocks in flight at
 constexpr int kXMaps = 16;                              // token-row boxes of 16 (b + 1) rows
 constexpr uint32_t kTmemCols = 512;
 constexpr int kQ = 4;                                   // entries of the CTA's tile queue
-#ifndef MOE_STREAM_DYN_WAVES
-#define MOE_STREAM_DYN_WAVES 2
-#endif
-constexpr int kDynWaves = MOE_STREAM_DYN_WAVES;         // waves' worth of tiles, at the list's end, handed out dynamically
+// Waves' worth of tiles, at the list's end, that are handed out dynamically: a fifth of them, between two and six.  Over
+// tens of waves the CTAs drift apart by more than two tiles (V3-shaped decode, 28 and 49 waves: six against two waves
+// 2111 -> 2089 us with 64 tokens, with FP8 weights and 128 tokens 1332 -> 1313 us on one GPU; on another that runs the same
+// steps in 2146 and 1355 us no difference); a launch of five waves, or one whose tiles
+// share weights through L2 while the CTAs are in step, wants two (37 tokens, 5 waves: 177.0 against 177.3 us; all but the
+// first wave dynamic: 8192-token Qwen3-shaped prefill 732 -> 742 us).
+constexpr int kMinDynWaves = 2, kMaxDynWaves = 6, kDynWavesOneIn = 5;
 
 struct StreamParams {
   const int32_t* offsets;  // [E+1] (already advanced to the first expert of the launch) or nullptr
@@ -385,12 +388,13 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       // A stop on request therefore takes effect after the tile that had already been taken.
       // The first waves are dealt statically (wave w: tile w * grid + the CTA's index, alternately forwards and
       // backwards): CTAs that run in step start the tiles that share an expert's weights or rows together, and the
-      // second reader finds them in L2.  The last kDynWaves waves' worth of tiles -- the smallest ones, the list being
+      // second reader finds them in L2.  The last few waves' worth of tiles -- the smallest ones, the list being
       // ordered by size -- go to whichever CTA is free, which evens out what the static part left uneven.  A pass that
       // can be stopped on request is dynamic throughout: its next launch only needs the counter to go on.
       const int grid = (int)gridDim.x;
       // (At least the first wave is static, which also spares every CTA a contended atomic at the start.)
-      const int w_static = p.all_dynamic ? 0 : max(1, total_tiles / grid - kDynWaves);
+      const int waves = total_tiles / grid;
+      const int w_static = p.all_dynamic ? 0 : max(1, waves - min(kMaxDynWaves, max(kMinDynWaves, waves / kDynWavesOneIn)));
       int sw = 0;
       auto next_tile = [&]() -> int {
         if (sw < w_static) {
