@@ -1015,8 +1015,12 @@ moe_status moe_grouped_ffn_fp8(moe_ctx* ctx, const void* wq_gate_up, const float
       if (pass == 0 && e == cudaSuccess) {
         {
           StageTimer tm(ctx, 9);
-          e = moe::launch_quantize_rows(b.act, N, c.inter, b.aq, b.sa, ctx->stream, &n);
-          if (e == cudaSuccess && shared)
+          // the shared expert's rows ride along if they are as long (a launch between the two passes is time in which no
+          // weights stream)
+          const bool ride = shared && c.shared_inter == c.inter;
+          e = moe::launch_quantize_rows(b.act, N, c.inter, b.aq, b.sa, ctx->stream, &n, ride ? b.act_shared : nullptr,
+                                        ride ? T : 0, b.aq_shared, b.sa_shared);
+          if (e == cudaSuccess && shared && !ride)
             e = moe::launch_quantize_rows(b.act_shared, T, c.shared_inter, b.aq_shared, b.sa_shared, ctx->stream, &n);
         }
         if (e == cudaSuccess) boundary();

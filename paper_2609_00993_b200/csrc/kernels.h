@@ -161,9 +161,10 @@ struct GemmDenseGroup {
 };
 
 // FP8 variant: per-row dynamic quantisation of bf16 rows [rows, n] -> E4M3 codes [rows, n] + scale [rows]
-// (n a multiple of 16, at most 8192).
+// (n a multiple of 16, at most 8192).  A second set of rows of the same length may ride in the launch.
 cudaError_t launch_quantize_rows(const void* x, int64_t rows, int n, void* q, float* scale, cudaStream_t stream,
-                                 int* n_launches);
+                                 int* n_launches, const void* x2 = nullptr, int64_t rows2 = 0, void* q2 = nullptr,
+                                 float* scale2 = nullptr);
 // The same for T token rows, whose codes and scales also go to their k places in the dispatch: row inv_perm[t * k + j] of
 // q_perm / scale_perm (negative: dropped).  q and scale (token order) may be nullptr.
 cudaError_t launch_quantize_move(const void* x, int T, int n, void* q, float* scale, const int32_t* inv_perm, int k,
