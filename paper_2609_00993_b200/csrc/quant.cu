@@ -50,8 +50,12 @@ quantize_rows_kernel(const uint4* __restrict__ x, long long rows, int n_pieces, 
                      float* __restrict__ scale_perm, const uint4* __restrict__ x2, long long rows2, uint4* __restrict__ q2,
                      float* __restrict__ scale2) {
   __shared__ uint32_t warp_max[kQuantThreads / 32];
+  // Without MOVE the next kernel is the down pass, which until it waits for this one reads only weights and the expert
+  // offsets: it may start while the kernel before this one is still finishing, and its weights are on their way when the
+  // codes are there (V3-shaped FP8 decode, one token 85.8 -> 84.3 us).  With MOVE the offsets themselves are that fresh.
+  if (!MOVE) pdl_launch_dependents();
   pdl_wait();
-  pdl_launch_dependents();
+  if (MOVE) pdl_launch_dependents();
   constexpr int kRowThreads = 32 * ROW_WARPS;
   const int tid = ROW_WARPS == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
   long long row = ROW_WARPS == 1 ? (long long)blockIdx.x * (kQuantThreads / 32) + (threadIdx.x >> 5)
