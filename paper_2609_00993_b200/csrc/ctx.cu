@@ -427,18 +427,22 @@ namespace moe {
 
 cudaError_t ensure_dynamic_smem_impl(const void* kern, size_t bytes) {
   static std::mutex mu;
-  static std::map<std::pair<const void*, int>, size_t> configured;  // (kernel, device) -> largest size set
+  static std::map<std::pair<const void*, int>, size_t> configured;  // (kernel, device) -> largest size set, plus one
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   std::lock_guard<std::mutex> lock(mu);
   size_t& have = configured[{kern, dev}];
-  if (bytes <= have) return cudaSuccess;
+  if (have != 0 && bytes < have) return cudaSuccess;
+  if (have == 0) {
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (err != cudaSuccess) return err;
+  }
   if (bytes > 48 * 1024) {
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (err != cudaSuccess) return err;
   }
-  have = bytes;
+  have = bytes + 1;
   return cudaSuccess;
 }
 

@@ -8,6 +8,9 @@ namespace moe {
 
 // Raises a kernel's dynamic shared-memory limit once per kernel, device and size, so that steady-state launches
 // make no driver calls besides the launch itself (which also keeps them legal while a stream is being captured).
+// The first time it also asks for the largest shared-memory carve-out, which the GEMM kernels need: an SM that one of the
+// small kernels left with more L1 has to drain before it can be divided anew (tiny layer, 64 tokens 23.9 -> 23.8 us a step;
+// one-token V3-shaped decode 134.2 -> 133.6 us).
 cudaError_t ensure_dynamic_smem_impl(const void* kern, size_t bytes);
 template <typename Kernel>
 inline cudaError_t ensure_dynamic_smem(Kernel kern, size_t bytes) {

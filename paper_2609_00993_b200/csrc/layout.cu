@@ -294,6 +294,7 @@ cudaError_t launch_layout(const int32_t* topk_idx, int64_t n_slots, int E, int32
   int n = 1;
   const int32_t* chunk_counts = nullptr;
   if (n_slots > kRecountMaxSlots) {
+    if ((err = ensure_dynamic_smem(layout_count_kernel, (size_t)E * sizeof(int))) != cudaSuccess) return err;
     if ((err = launch_pdl(true, layout_count_kernel, dim3(n_chunks), dim3(kThreads), (size_t)E * sizeof(int), stream, topk_idx,
                           n_slots, E, (int)chunk, scratch, status)) != cudaSuccess) return err;
     chunk_counts = scratch;

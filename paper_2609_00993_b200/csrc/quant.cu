@@ -139,7 +139,9 @@ cudaError_t launch(const void* x, int64_t rows, int n, void* q, float* scale, co
   const int np = warp_row ? (pieces + 31) / 32 : (pieces + kQuantThreads - 1) / kQuantThreads;
   const int64_t all = rows + rows2;
   const unsigned blocks = (unsigned)(warp_row ? (all + kQuantThreads / 32 - 1) / (kQuantThreads / 32) : all);
-  auto go = [&](auto kern) {
+  auto go = [&](auto kern) -> cudaError_t {
+    cudaError_t e = ensure_dynamic_smem(kern, 0);
+    if (e != cudaSuccess) return e;
     return launch_pdl(true, kern, dim3(blocks), dim3(kQuantThreads), 0, stream, static_cast<const uint4*>(x), (long long)rows,
                       pieces, static_cast<uint4*>(q), scale, inv_perm, k, static_cast<uint4*>(q_perm), scale_perm,
                       static_cast<const uint4*>(x2), (long long)rows2, static_cast<uint4*>(q2), scale2);

@@ -150,12 +150,15 @@ template <int VPT>
 cudaError_t launch_vpt(bool vec, const float* logits, const float* bias, int T, int E, int k, float scale,
                        int32_t* idx, float* w, cudaStream_t stream) {
   const int blocks = (T + kWarpsPerBlock - 1) / kWarpsPerBlock;
+  cudaError_t err = cudaSuccess;
   if constexpr (VPT >= 4) {
     if (vec) {
+      if ((err = ensure_dynamic_smem(route_kernel<VPT, true>, 0)) != cudaSuccess) return err;
       return launch_pdl(true, route_kernel<VPT, true>, dim3(blocks), dim3(kWarpsPerBlock * 32), 0, stream, logits, bias, T, E, k,
                         scale, idx, w);
     }
   }
+  if ((err = ensure_dynamic_smem(route_kernel<VPT, false>, 0)) != cudaSuccess) return err;
   return launch_pdl(true, route_kernel<VPT, false>, dim3(blocks), dim3(kWarpsPerBlock * 32), 0, stream, logits, bias, T, E, k, scale,
                     idx, w);
 }
