@@ -209,6 +209,7 @@ struct moe_ctx {
   std::mutex* yield_mu;
   int* stopped_host;  // pinned host word: CTAs that stopped in the last launch
   int64_t yields;     // launches that ended on a yield request
+  bool offsets_fresh; // the kernel right before the gated pass wrote the step's offsets (moe_layer, a few tokens)
   bool unmarked;      // launches have been enqueued since `done` was last recorded
   moe::StreamPlan* plans[2][4];  // tensor maps of the small-M GEMM: [buffer set][2 * (dense problem by itself) + down pass]
   unsigned long long wait_limit_ns;  // time limit of every bounded device-side wait (0 = the kernels' default)
@@ -381,8 +382,9 @@ cudaError_t run_gemm(moe_ctx* ctx, moe::GemmProblem p, const moe::GemmDenseGroup
   p.wait_limit_ns = ctx->wait_limit_ns;
   p.debug_stall = ctx->debug_stall;
   // Every GEMM launch comes after the step's row movement (or after another GEMM launch or a quantisation of the
-  // same step), which in turn waited for the layout kernels: the offsets are older than the previous kernel.
-  p.offsets_settled = true;
+  // same step), which in turn waited for the layout kernels: the offsets are older than the previous kernel.  Only a
+  // step that dispatched its tokens in one launch has them from the kernel before its gated pass.
+  p.offsets_settled = !(ctx->offsets_fresh && p.gated);
   p.tile_counters = reinterpret_cast<int*>(ctx->ws + kTileCounterOffset) + 2 * (ctx->gemm_seq++ % kTileCounterPairs);
   p.max_group_rows = T;
   p.plan = ctx->plans[ctx->cur][(p.offsets == nullptr ? 2 : 0) + (p.gated ? 0 : 1)];
@@ -502,6 +504,7 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
   for (int s = 0; s < l.n_sets; ++s) carve_set(*cfg, ctx->ws + kStatusBlock + (size_t)s * l.set_bytes, &ctx->sets[s]);
   ctx->host_pipeline = false;
   ctx->unmarked = false;
+  ctx->offsets_fresh = false;
   bool have_plans = true;
   for (int i = 0; i < 8; ++i) {
     moe::StreamPlan*& plan = ctx->plans[i / 4][i % 4];
@@ -677,6 +680,15 @@ moe_status moe_route(moe_ctx* ctx, const float* logits, const float* select_bias
 
 namespace {
 
+// The step's layout arrays: the caller's, or the context's own where there is none.
+void set_layout_arrays(moe_ctx* ctx, int32_t* counts, int32_t* offsets, int32_t* perm, int32_t* inv_perm) {
+  const BufferSet& b = ctx->sets[ctx->cur];
+  ctx->counts = counts ? counts : b.counts;
+  ctx->offsets = offsets ? offsets : b.offsets;
+  ctx->perm = perm ? perm : b.perm;
+  ctx->inv_perm = inv_perm ? inv_perm : b.inv_perm;
+}
+
 // First half of a dispatch: counts, exclusive scan, stable permutation (no rows move).
 moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx, int32_t T, int32_t* counts,
                           int32_t* offsets, int32_t* perm, int32_t* inv_perm) {
@@ -686,10 +698,7 @@ moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx
   if (misaligned(topk_idx) || misaligned(counts) || misaligned(offsets) || misaligned(perm) || misaligned(inv_perm))
     return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
   BufferSet& b = ctx->sets[ctx->cur];
-  ctx->counts = counts ? counts : b.counts;
-  ctx->offsets = offsets ? offsets : b.offsets;
-  ctx->perm = perm ? perm : b.perm;
-  ctx->inv_perm = inv_perm ? inv_perm : b.inv_perm;
+  set_layout_arrays(ctx, counts, offsets, perm, inv_perm);
   int n = 0;
   cudaError_t e;
   {
@@ -699,8 +708,21 @@ moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx
   }
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->T = T;
+  ctx->offsets_fresh = false;
   ctx->launches += n;
   return MOE_OK;
+}
+
+// Whether a step of a BF16 context starts with one launch instead of three: a few tokens, every argument fit for
+// moe_route and moe_dispatch_layout both -- or the calls themselves report what is wrong -- and no stage times wanted.
+bool dispatches_at_once(const moe_ctx* ctx, const float* logits, const float* select_bias, const void* x, int32_t T,
+                        const int32_t* topk_idx, const float* topk_w, const int32_t* counts, const int32_t* offsets,
+                        const int32_t* perm, const int32_t* inv_perm) {
+  const moe_config& c = ctx->cfg;
+  return (ctx->state == ST_IDLE || ctx->state == ST_ROUTED) && !ctx->profiling && c.weight_format == MOE_WEIGHTS_BF16 &&
+         T <= c.max_tokens && moe::small_dispatch_fits(T, c.n_experts, c.top_k) && logits && x && topk_idx && topk_w &&
+         !misaligned(logits) && !misaligned(select_bias) && !misaligned(x) && !misaligned(topk_idx) &&
+         !misaligned(topk_w) && !misaligned(counts) && !misaligned(offsets) && !misaligned(perm) && !misaligned(inv_perm);
 }
 
 // Second half: the routed data movement (an FP8 context quantises each token row once and moves the codes).
@@ -1075,8 +1097,27 @@ moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias
                      int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
                      int32_t* inv_perm, const void* w_gate_up, const void* w_down, const void* ws_gate_up,
                      const void* ws_down, void* out) {
-  moe_status st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
-  if (st == MOE_OK) st = moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm);
+  if (!ctx) return MOE_ERR_INVALID_ARG;
+  moe_status st;
+  if (dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm)) {
+    DeviceGuard guard(ctx->device);
+    set_layout_arrays(ctx, counts, offsets, perm, inv_perm);
+    const moe_config& c = ctx->cfg;
+    int n = 0;
+    const cudaError_t e = moe::launch_small_dispatch(
+        logits, select_bias, T, c.n_experts, c.top_k, c.routed_scale, topk_idx, topk_w, ctx->counts, ctx->offsets, ctx->perm,
+        ctx->inv_perm, x, gathers_rows(ctx) ? nullptr : ctx->sets[ctx->cur].x_perm, c.hidden, ctx->stream, &n);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "moe_layer");
+    ctx->T = T;
+    ctx->offsets_fresh = true;
+    ctx->state = ST_LAID_OUT;
+    ctx->split_step = false;
+    mark(ctx, n);
+    st = MOE_OK;
+  } else {
+    st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
+    if (st == MOE_OK) st = moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm);
+  }
   if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T);
   if (st == MOE_OK) st = moe_combine(ctx, topk_w, inv_perm, T, out);
   return st;

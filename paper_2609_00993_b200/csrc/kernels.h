@@ -29,19 +29,32 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(bool allow_overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t stream, Args&&... args) {
+inline cudaError_t launch_pdl_clusters(bool allow_overlap, int cluster_y, void (*kern)(KArgs...), dim3 grid, dim3 block,
+                                       size_t smem, cudaStream_t stream, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (allow_overlap) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster_y > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = attr[n].val.clusterDim.z = 1;
+    attr[n++].val.clusterDim.y = (unsigned)cluster_y;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = allow_overlap ? 1 : 0;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(bool allow_overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t stream, Args&&... args) {
+  return launch_pdl_clusters(allow_overlap, 1, kern, grid, block, smem, stream, static_cast<KArgs>(args)...);
 }
 // The GEMM kernels take the overlap only for problems of up to this many rows: measured on a B200, a step of a
 // few hundred microseconds gains 7 % from it (six launch latencies and prologues hidden), while steps of several
@@ -74,6 +87,14 @@ inline size_t layout_scratch_ints(int64_t n_slots, int E) {
 cudaError_t launch_layout(const int32_t* topk_idx, int64_t n_slots, int E, int32_t* counts, int32_t* offsets,
                           int32_t* perm, int32_t* inv_perm, int32_t* scratch, int* status, cudaStream_t stream,
                           int* n_launches);
+
+// ---- a1-a5 of a few tokens in one launch (the results of the three stages) -------------------
+// x_perm nullptr: no rows move.  Only where small_dispatch_fits (512 experts: 16 keys per lane).
+constexpr int kSmallDispatchMaxTokens = 64, kSmallDispatchMaxSlots = 1024;
+bool small_dispatch_fits(int T, int E, int k);
+cudaError_t launch_small_dispatch(const float* logits, const float* bias, int T, int E, int k, float scale, int32_t* idx,
+                                  float* w, int32_t* counts, int32_t* offsets, int32_t* perm, int32_t* inv_perm,
+                                  const void* x, void* x_perm, int H, cudaStream_t stream, int* n_launches);
 
 // ---- a5 permute, a9 combine ----------------------------------------------------------------
 // wait_limit_ns: time limit of the kernels' bounded waits (0 = the default of 2 s).

@@ -14,6 +14,7 @@
 #include <mutex>
 
 #include "kernels.h"
+#include "routing.cuh"
 
 namespace moe {
 namespace {
@@ -25,54 +26,6 @@ constexpr int kMaxChunk = 4096;           // ... and at most
 constexpr int kChunkTarget = 64;          // CTAs wanted between those two
 constexpr int64_t kRecountMaxSlots = 16384;  // see above
 constexpr int kBatch = 8;                 // loads issued together (latency hiding)
-
-__device__ __forceinline__ void flag_status(int* status, int code) {
-  if (status != nullptr) atomicCAS(status, kStOk, code);
-}
-
-// Block-wide exclusive scan of counts[0..E) -> offsets[0..E]; E <= 1024, blockDim.x a multiple of 32 and >= E...
-// handled in rounds of blockDim.x so that any E works.  `warp_sums` is 33 ints of shared scratch.
-__device__ void block_exclusive_scan(const int* counts_sh, int E, int32_t* __restrict__ offsets_out, int* offsets_sh,
-                                     int* warp_sums) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  int carry = 0;
-  for (int base = 0; base < E; base += blockDim.x) {
-    const int e = base + threadIdx.x;
-    const int v = (e < E) ? counts_sh[e] : 0;
-    int incl = v;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int n = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += n;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      int ws = (lane < nwarps) ? warp_sums[lane] : 0;
-      int wincl = ws;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, wincl, off);
-        if (lane >= off) wincl += n;
-      }
-      if (lane < nwarps) warp_sums[lane] = wincl - ws;  // exclusive prefix of the warp totals
-      if (lane == 31) warp_sums[32] = wincl;            // total of this round
-    }
-    __syncthreads();
-    const int excl = carry + warp_sums[warp] + incl - v;
-    if (e < E) {
-      offsets_sh[e] = excl;
-      if (offsets_out != nullptr) offsets_out[e] = excl;
-    }
-    carry += warp_sums[32];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    offsets_sh[E] = carry;
-    if (offsets_out != nullptr) offsets_out[E] = carry;
-  }
-  __syncthreads();
-}
 
 // Counts the slots [f0, f1) into hist[0..E) with all threads of the CTA (integer adds commute: the count does not
 // depend on their order).
@@ -212,18 +165,7 @@ layout_place_kernel(const int32_t* __restrict__ topk_idx, int64_t n_slots, int E
   __syncthreads();
   // per expert: exclusive prefix over the warps' runs, and the total over all chunks
   for (int e = threadIdx.x; e < E; e += kThreads) {
-    int sum = 0;
-#pragma unroll
-    for (int w0 = 0; w0 < kWarps; w0 += 16) {  // 16 reads in flight
-      int v[16];
-#pragma unroll
-      for (int w = 0; w < 16; ++w) v[w] = hist[(w0 + w) * E + e];
-#pragma unroll
-      for (int w = 0; w < 16; ++w) {
-        hist[(w0 + w) * E + e] = sum;
-        sum += v[w];
-      }
-    }
+    const int sum = prefix_over_warps(hist, E, e);
     total[e] += base[e] + sum;  // later chunks, earlier ones, this one
     if (blockIdx.x == 0) counts[e] = total[e];
   }
