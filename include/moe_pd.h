@@ -357,6 +357,13 @@ moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias
                      int32_t* inv_perm, const void* w_gate_up, const void* w_down, const void* ws_gate_up,
                      const void* ws_down, void* out);
 
+/* The same step of a context created for FP8 weights, with the arguments of moe_grouped_ffn_fp8. */
+moe_status moe_layer_fp8(moe_ctx* ctx, const float* logits, const float* select_bias, const void* x, int32_t T,
+                         int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
+                         int32_t* inv_perm, const void* wq_gate_up, const float* sw_gate_up, const void* wq_down,
+                         const float* sw_down, const void* wsq_gate_up, const float* sws_gate_up, const void* wsq_down,
+                         const float* sws_down, void* out);
+
 /* One whole step with HOST activations: copies logits_host [T,E] fp32 and x_host [T,H] bf16
  * to the device (cudaMemcpyAsync into context-owned staging), runs a1..a9, copies out
  * [T,H] bf16 back to out_host and waits for all of it before returning.  With pinned host

@@ -29,7 +29,7 @@ STATUS_NAMES = {0: "MOE_OK", 1: "MOE_ERR_INVALID_ARG", 2: "MOE_ERR_CAPACITY", 3:
 # every symbol include/moe_pd.h declares
 EXPORTS = ("moe_version", "moe_ctx_workspace_bytes", "moe_ctx_create", "moe_ctx_destroy", "moe_ctx_status",
            "moe_last_error", "moe_route", "moe_dispatch_layout", "moe_grouped_ffn", "moe_grouped_ffn_fp8", "moe_combine",
-           "moe_layer", "moe_layer_host", "moe_layer_host_submit", "moe_layer_host_wait",
+           "moe_layer", "moe_layer_fp8", "moe_layer_host", "moe_layer_host_submit", "moe_layer_host_wait",
            "moe_ctx_debug_ptrs", "moe_ctx_debug_ptrs_fp8", "moe_ctx_launch_count", "moe_ctx_set_profiling", "moe_ctx_read_profile",
            "moe_dispatch_layout_static", "moe_ctx_set_segments", "moe_ctx_abandon_step", "moe_turnstile_create", "moe_turnstile_destroy",
            "moe_turnstile_set_span", "moe_turnstile_begin_epoch", "moe_turnstile_publish", "moe_turnstile_task_done",
@@ -101,6 +101,8 @@ def load_library() -> ctypes.CDLL:
     lib.moe_combine.argtypes = [vp, vp, vp, i32, vp]
     lib.moe_layer.restype = i32
     lib.moe_layer.argtypes = [vp] * 4 + [i32] + [vp] * 11
+    lib.moe_layer_fp8.restype = i32
+    lib.moe_layer_fp8.argtypes = [vp] * 4 + [i32] + [vp] * 15
     lib.moe_layer_host.restype = i32
     lib.moe_layer_host.argtypes = [vp, vp, vp, vp, i32, vp, vp, vp, vp, vp]
     lib.moe_layer_host_submit.restype = i32
@@ -433,14 +435,20 @@ class MoeContext:
         """One step with FP8 weights; `w8` holds wq_gate_up, sw_gate_up, wq_down, sw_down and, with a shared
         expert, wsq_gate_up, sws_gate_up, wsq_down, sws_down (see workloads.make_weights_fp8)."""
         T, k, E = x.shape[0], self.cfg.top_k, self.cfg.n_experts
-        bufs, out = self._step_tensors(T, k, E, x.device, bufs, out)
-        self.moe_route(logits, select_bias, bufs["topk_idx"], bufs["topk_w"], T=T)
-        self.moe_dispatch_layout(bufs["topk_idx"], x, bufs["counts"], bufs["offsets"], bufs["perm"], bufs["inv_perm"],
-                                 T=T)
-        self.moe_grouped_ffn_fp8(w8["wq_gate_up"], w8["sw_gate_up"], w8["wq_down"], w8["sw_down"],
-                                 w8.get("wsq_gate_up"), w8.get("sws_gate_up"), w8.get("wsq_down"), w8.get("sws_down"),
-                                 T=T)
-        self.moe_combine(bufs["topk_w"], bufs["inv_perm"], out, T=T)
+        if bufs is None or out is None:
+            bufs, out = self._step_tensors(T, k, E, x.device, bufs, out)
+        i32, f32, u8, bf16 = torch.int32, torch.float32, torch.uint8, torch.bfloat16
+        st = self.lib.moe_layer_fp8(self.handle, _arg(logits, f32, "logits"), _arg(select_bias, f32, "select_bias"),
+                                    _arg(x, bf16, "x"), T, _arg(bufs["topk_idx"], i32, "topk_idx"),
+                                    _arg(bufs["topk_w"], f32, "topk_w"), _arg(bufs["counts"], i32, "counts"),
+                                    _arg(bufs["offsets"], i32, "offsets"), _arg(bufs["perm"], i32, "perm"),
+                                    _arg(bufs["inv_perm"], i32, "inv_perm"), _arg(w8["wq_gate_up"], u8, "wq_gate_up"),
+                                    _arg(w8["sw_gate_up"], f32, "sw_gate_up"), _arg(w8["wq_down"], u8, "wq_down"),
+                                    _arg(w8["sw_down"], f32, "sw_down"), _arg(w8.get("wsq_gate_up"), u8, "wsq_gate_up"),
+                                    _arg(w8.get("sws_gate_up"), f32, "sws_gate_up"), _arg(w8.get("wsq_down"), u8, "wsq_down"),
+                                    _arg(w8.get("sws_down"), f32, "sws_down"), _arg(out, bf16, "out"))
+        if st != MOE_OK:
+            self._check(st)
         return out, bufs
 
 

@@ -713,14 +713,14 @@ moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx
   return MOE_OK;
 }
 
-// Whether a step of a BF16 context starts with one launch instead of three: a few tokens, every argument fit for
-// moe_route and moe_dispatch_layout both -- or the calls themselves report what is wrong -- and no stage times wanted.
+// Whether a step routes and lays out in one launch: a few tokens, every argument fit for moe_route and
+// moe_dispatch_layout both -- or the calls themselves report what is wrong -- and no stage times wanted.
 bool dispatches_at_once(const moe_ctx* ctx, const float* logits, const float* select_bias, const void* x, int32_t T,
                         const int32_t* topk_idx, const float* topk_w, const int32_t* counts, const int32_t* offsets,
                         const int32_t* perm, const int32_t* inv_perm) {
   const moe_config& c = ctx->cfg;
-  return (ctx->state == ST_IDLE || ctx->state == ST_ROUTED) && !ctx->profiling && c.weight_format == MOE_WEIGHTS_BF16 &&
-         T <= c.max_tokens && moe::small_dispatch_fits(T, c.n_experts, c.top_k) && logits && x && topk_idx && topk_w &&
+  return (ctx->state == ST_IDLE || ctx->state == ST_ROUTED) && !ctx->profiling && T <= c.max_tokens &&
+         moe::small_dispatch_fits(T, c.n_experts, c.top_k) && logits && x && topk_idx && topk_w &&
          !misaligned(logits) && !misaligned(select_bias) && !misaligned(x) && !misaligned(topk_idx) &&
          !misaligned(topk_w) && !misaligned(counts) && !misaligned(offsets) && !misaligned(perm) && !misaligned(inv_perm);
 }
@@ -1093,32 +1093,64 @@ moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_per
   return MOE_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// moe_route and moe_dispatch_layout of a whole step, as one launch where that is possible (an FP8 context quantises and
+// moves its rows in a second one).
+moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits, const float* select_bias, const void* x,
+                              int32_t T, int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
+                              int32_t* inv_perm) {
+  if (!ctx) return MOE_ERR_INVALID_ARG;
+  if (!dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm)) {
+    const moe_status st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
+    return st == MOE_OK ? moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm) : st;
+  }
+  DeviceGuard guard(ctx->device);
+  set_layout_arrays(ctx, counts, offsets, perm, inv_perm);
+  const moe_config& c = ctx->cfg;
+  const bool fp8 = c.weight_format == MOE_WEIGHTS_FP8_E4M3;
+  int n = 0;
+  const cudaError_t e = moe::launch_small_dispatch(
+      logits, select_bias, T, c.n_experts, c.top_k, c.routed_scale, topk_idx, topk_w, ctx->counts, ctx->offsets, ctx->perm,
+      ctx->inv_perm, x, fp8 || gathers_rows(ctx) ? nullptr : ctx->sets[ctx->cur].x_perm, c.hidden, ctx->stream, &n);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, who);
+  ctx->T = T;
+  ctx->offsets_fresh = !fp8;
+  mark(ctx, n);
+  if (fp8) {
+    const moe_status st = enqueue_row_movement(ctx, who, x);
+    if (st != MOE_OK) return st;
+  }
+  ctx->state = ST_LAID_OUT;
+  ctx->split_step = false;
+  return MOE_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias, const void* x, int32_t T,
                      int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
                      int32_t* inv_perm, const void* w_gate_up, const void* w_down, const void* ws_gate_up,
                      const void* ws_down, void* out) {
-  if (!ctx) return MOE_ERR_INVALID_ARG;
-  moe_status st;
-  if (dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm)) {
-    DeviceGuard guard(ctx->device);
-    set_layout_arrays(ctx, counts, offsets, perm, inv_perm);
-    const moe_config& c = ctx->cfg;
-    int n = 0;
-    const cudaError_t e = moe::launch_small_dispatch(
-        logits, select_bias, T, c.n_experts, c.top_k, c.routed_scale, topk_idx, topk_w, ctx->counts, ctx->offsets, ctx->perm,
-        ctx->inv_perm, x, gathers_rows(ctx) ? nullptr : ctx->sets[ctx->cur].x_perm, c.hidden, ctx->stream, &n);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "moe_layer");
-    ctx->T = T;
-    ctx->offsets_fresh = true;
-    ctx->state = ST_LAID_OUT;
-    ctx->split_step = false;
-    mark(ctx, n);
-    st = MOE_OK;
-  } else {
-    st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
-    if (st == MOE_OK) st = moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm);
-  }
+  moe_status st = route_and_dispatch(ctx, "moe_layer", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
   if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T);
+  if (st == MOE_OK) st = moe_combine(ctx, topk_w, inv_perm, T, out);
+  return st;
+}
+
+moe_status moe_layer_fp8(moe_ctx* ctx, const float* logits, const float* select_bias, const void* x, int32_t T,
+                         int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
+                         int32_t* inv_perm, const void* wq_gate_up, const float* sw_gate_up, const void* wq_down,
+                         const float* sw_down, const void* wsq_gate_up, const float* sws_gate_up, const void* wsq_down,
+                         const float* sws_down, void* out) {
+  moe_status st =
+      route_and_dispatch(ctx, "moe_layer_fp8", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
+  if (st == MOE_OK)
+    st = moe_grouped_ffn_fp8(ctx, wq_gate_up, sw_gate_up, wq_down, sw_down, wsq_gate_up, sws_gate_up, wsq_down, sws_down, T);
   if (st == MOE_OK) st = moe_combine(ctx, topk_w, inv_perm, T, out);
   return st;
 }
