@@ -190,7 +190,7 @@ struct moe_ctx {
   struct Span { cudaEvent_t beg, end; int stage; };
   std::vector<Span> spans;
   size_t spans_used;
-  // pipelined host path: staging slots and two copy streams (created by the first moe_layer_host_submit)
+  // host path: staging slots, and a copy stream (two from the first moe_layer_host_submit on)
   struct HostSlot {
     float* logits;
     char* x;
@@ -199,8 +199,10 @@ struct moe_ctx {
     bool in_flight;
   } slots[MOE_HOST_SLOTS];
   cudaStream_t h2d_stream, d2h_stream;
-  cudaEvent_t copied_in, computed;  // stream positions inside moe_layer_host (a wait takes the last record before it)
-  bool host_pipeline;
+  // stream positions inside moe_layer_host (a wait takes the last record before it): copied in, of each chunk; computed
+  cudaEvent_t copied_in[2], computed;
+  bool host_stream;    // h2d_stream and those three exist
+  bool host_pipeline;  // d2h_stream and the slots' events exist
   // preemption of prefill GEMM passes at tile granularity (off by default)
   bool preemptible;
   int* yield_src;     // pinned host words {0, 1}: the sources of the copies that lower / raise the request
@@ -502,7 +504,7 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
   ctx->err[0] = 0;
   ctx->status = reinterpret_cast<int*>(ctx->ws);
   for (int s = 0; s < l.n_sets; ++s) carve_set(*cfg, ctx->ws + kStatusBlock + (size_t)s * l.set_bytes, &ctx->sets[s]);
-  ctx->host_pipeline = false;
+  ctx->host_stream = ctx->host_pipeline = false;
   ctx->unmarked = false;
   ctx->offsets_fresh = false;
   bool have_plans = true;
@@ -594,10 +596,11 @@ moe_status moe_ctx_destroy(moe_ctx* ctx) {
       cudaEventDestroy(ctx->slots[s].comp);
       cudaEventDestroy(ctx->slots[s].done);
     }
-    cudaEventDestroy(ctx->copied_in);
-    cudaEventDestroy(ctx->computed);
-    cudaStreamDestroy(ctx->h2d_stream);
     cudaStreamDestroy(ctx->d2h_stream);
+  }
+  if (ctx->host_stream) {
+    for (cudaEvent_t ev : {ctx->copied_in[0], ctx->copied_in[1], ctx->computed}) cudaEventDestroy(ev);
+    cudaStreamDestroy(ctx->h2d_stream);
   }
   {
     std::lock_guard<std::mutex> lock(g_registry_mutex);
@@ -854,31 +857,43 @@ moe_status grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, 
   return MOE_OK;
 }
 
-// The copy streams and events of the host path, created by its first call.
-moe_status ensure_host_streams(moe_ctx* ctx, const char* who) {
-  if (ctx->host_pipeline) return MOE_OK;
-  constexpr int kEvents = 3 * MOE_HOST_SLOTS + 2;
-  cudaEvent_t ev[kEvents] = {};
-  cudaStream_t st[2] = {};
-  cudaError_t e = cudaSuccess;
-  for (int i = 0; i < kEvents && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&st[i], cudaStreamNonBlocking);
-  if (e != cudaSuccess) {
-    for (int i = 0; i < kEvents; ++i)
-      if (ev[i]) cudaEventDestroy(ev[i]);
-    for (int i = 0; i < 2; ++i)
-      if (st[i]) cudaStreamDestroy(st[i]);
-    return cuda_fail(ctx, e, who);
+// A copy stream and n events (all given back if one of them cannot be had).
+cudaError_t create_stream_and_events(cudaStream_t* stream, cudaEvent_t* const* events, int n) {
+  cudaError_t e = cudaStreamCreateWithFlags(stream, cudaStreamNonBlocking);
+  for (int i = 0; i < n && e == cudaSuccess; ++i) {
+    e = cudaEventCreateWithFlags(events[i], cudaEventDisableTiming);
+    if (e == cudaSuccess) continue;
+    while (i-- > 0) cudaEventDestroy(*events[i]);
+    cudaStreamDestroy(*stream);
+    break;
   }
+  return e;
+}
+
+// The copy stream of moe_layer_host, created by its first call.  One serves both directions, because creating a stream
+// takes 0.06 to 0.5 ms, which the first pass of a context pays (Qwen3-shaped layer, 1531 tokens: 778 us with two streams and
+// every event of the pipelined form, 716 with one; later passes 489 with either).
+moe_status ensure_host_stream(moe_ctx* ctx, const char* who) {
+  if (ctx->host_stream) return MOE_OK;
+  cudaEvent_t* const events[] = {&ctx->copied_in[0], &ctx->copied_in[1], &ctx->computed};
+  const cudaError_t e = create_stream_and_events(&ctx->h2d_stream, events, 3);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, who);
+  ctx->host_stream = true;
+  return MOE_OK;
+}
+
+// The pipelined form copies out on a second stream, beside the copies in of the next slots.
+moe_status ensure_host_pipeline(moe_ctx* ctx, const char* who) {
+  const moe_status st = ensure_host_stream(ctx, who);
+  if (st != MOE_OK || ctx->host_pipeline) return st;
+  cudaEvent_t* events[3 * MOE_HOST_SLOTS];
   for (int s = 0; s < MOE_HOST_SLOTS; ++s) {
-    ctx->slots[s].h2d = ev[3 * s];
-    ctx->slots[s].comp = ev[3 * s + 1];
-    ctx->slots[s].done = ev[3 * s + 2];
+    events[3 * s] = &ctx->slots[s].h2d;
+    events[3 * s + 1] = &ctx->slots[s].comp;
+    events[3 * s + 2] = &ctx->slots[s].done;
   }
-  ctx->copied_in = ev[kEvents - 2];
-  ctx->computed = ev[kEvents - 1];
-  ctx->h2d_stream = st[0];
-  ctx->d2h_stream = st[1];
+  const cudaError_t e = create_stream_and_events(&ctx->d2h_stream, events, 3 * MOE_HOST_SLOTS);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->host_pipeline = true;
   return MOE_OK;
 }
@@ -1166,7 +1181,7 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
   if (T > ctx->cfg.max_tokens) return fail(ctx, MOE_ERR_CAPACITY, "T = %d exceeds max_tokens = %d", T, ctx->cfg.max_tokens);
   if (T > 0 && (!logits_host || !x_host || !out_host)) return fail(ctx, MOE_ERR_INVALID_ARG, "NULL host pointer");
   DeviceGuard guard(ctx->device);
-  moe_status st = ensure_host_streams(ctx, "moe_layer_host set-up");
+  moe_status st = ensure_host_stream(ctx, "moe_layer_host set-up");
   if (st != MOE_OK) return st;
   BufferSet& b = ctx->sets[ctx->cur];
   const moe_config& c = ctx->cfg;
@@ -1189,6 +1204,20 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
   if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->h2d_stream, ctx->computed, 0);
   for (const moe_ctx::HostSlot& s : ctx->slots)  // (a slot of the pipelined path may still be copying out of them)
     if (e == cudaSuccess && s.in_flight) e = cudaStreamWaitEvent(ctx->stream, s.done, 0);
+  // The copy stream takes everything that comes in, in the order of use, before anything that goes out.
+  for (int i = 0; i * chunk < T && e == cudaSuccess; ++i) {
+    const size_t t0 = (size_t)i * chunk, n_tok = std::min<size_t>(chunk, T - t0);
+    e = cudaMemcpyAsync(b.logits + t0 * c.n_experts, logits_host + t0 * c.n_experts, n_tok * c.n_experts * 4,
+                        cudaMemcpyHostToDevice, ctx->h2d_stream);
+    if (i == 0) {  // the first chunk's router does not wait for the rows
+      if (e == cudaSuccess) e = cudaEventRecord(ctx->copied_in[0], ctx->h2d_stream);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->copied_in[0], 0);
+    }
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(b.x_stage + t0 * row_bytes, static_cast<const char*>(x_host) + t0 * row_bytes, n_tok * row_bytes,
+                          cudaMemcpyHostToDevice, ctx->h2d_stream);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->copied_in[i], ctx->h2d_stream);
+  }
   for (int t0 = 0; (t0 < T || T == 0) && e == cudaSuccess && st == MOE_OK; t0 += chunk) {
     const int n_tok = std::min(chunk, T - t0);
     float* const logits = b.logits + (size_t)t0 * c.n_experts;
@@ -1197,21 +1226,12 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
     char* const out_to = static_cast<char*>(out_host) + (size_t)t0 * row_bytes;
     int32_t* const idx = b.topk_idx + (size_t)t0 * c.top_k;
     float* const w = b.topk_w + (size_t)t0 * c.top_k;
-    if (T > 0) {
-      e = cudaMemcpyAsync(logits, logits_host + (size_t)t0 * c.n_experts, (size_t)n_tok * c.n_experts * 4,
-                          cudaMemcpyHostToDevice, ctx->h2d_stream);
-      if (e == cudaSuccess) e = cudaEventRecord(ctx->copied_in, ctx->h2d_stream);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->copied_in, 0);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(x, static_cast<const char*>(x_host) + (size_t)t0 * row_bytes, (size_t)n_tok * row_bytes,
-                            cudaMemcpyHostToDevice, ctx->h2d_stream);
-      if (e == cudaSuccess) e = cudaEventRecord(ctx->copied_in, ctx->h2d_stream);
-      if (e != cudaSuccess) break;
-    }
+    const cudaEvent_t copied_in = ctx->copied_in[t0 > 0 ? 1 : 0];
+    if (t0 > 0 && (e = cudaStreamWaitEvent(ctx->stream, copied_in, 0)) != cudaSuccess) break;
     st = moe_route(ctx, logits, select_bias, n_tok, idx, w);
     if (st == MOE_OK) st = enqueue_layout(ctx, "moe_layer_host", idx, n_tok, nullptr, nullptr, nullptr, nullptr);
     if (st != MOE_OK) break;
-    if ((e = cudaStreamWaitEvent(ctx->stream, ctx->copied_in, 0)) != cudaSuccess) break;
+    if (T > 0 && (e = cudaStreamWaitEvent(ctx->stream, copied_in, 0)) != cudaSuccess) break;
     st = enqueue_row_movement(ctx, "moe_layer_host", x);
     if (st != MOE_OK) break;
     ctx->state = ST_LAID_OUT;
@@ -1231,10 +1251,10 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
       }
       ctx->launches += n;
       if (err == cudaSuccess) err = cudaEventRecord(ctx->computed, ctx->stream);
-      if (err == cudaSuccess) err = cudaStreamWaitEvent(ctx->d2h_stream, ctx->computed, 0);
+      if (err == cudaSuccess) err = cudaStreamWaitEvent(ctx->h2d_stream, ctx->computed, 0);
       if (err == cudaSuccess && n_tok > 0)
         err = cudaMemcpy2DAsync(out_to + (size_t)c0 * 2, row_bytes, out + (size_t)c0 * 2, row_bytes, (size_t)(c1 - c0) * 2,
-                                n_tok, cudaMemcpyDeviceToHost, ctx->d2h_stream);
+                                n_tok, cudaMemcpyDeviceToHost, ctx->h2d_stream);
       return err;
     };
     st = grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, n_tok, pieces > 1 ? piece_cols : 0, finish);
@@ -1247,7 +1267,7 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
   mark(ctx, 0);
   mark_position(ctx);
   // nothing of the caller's memory is in use when this returns, whatever happened
-  for (cudaStream_t s : {ctx->h2d_stream, ctx->stream, ctx->d2h_stream}) {
+  for (cudaStream_t s : {ctx->stream, ctx->h2d_stream}) {
     const cudaError_t sync = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = sync;
   }
@@ -1270,7 +1290,7 @@ moe_status moe_layer_host_submit(moe_ctx* ctx, int32_t slot, const float* logits
   if (T > 0 && (!logits_host || !x_host || !out_host)) return fail(ctx, MOE_ERR_INVALID_ARG, "NULL host pointer");
   DeviceGuard guard(ctx->device);
   cudaError_t e = cudaSuccess;
-  moe_status st = ensure_host_streams(ctx, "moe_layer_host_submit set-up");
+  moe_status st = ensure_host_pipeline(ctx, "moe_layer_host_submit set-up");
   if (st != MOE_OK) return st;
   moe_ctx::HostSlot& hs = ctx->slots[slot];
   BufferSet& b = ctx->sets[ctx->cur];
