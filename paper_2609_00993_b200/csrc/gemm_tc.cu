@@ -46,7 +46,7 @@ constexpr int kGatherThreads = 128;
 constexpr int kThreadsGather = kThreads + kGatherThreads;
 constexpr int kMaxStages = 8;
 constexpr int kEpiStagingBytes = kEpilogueWarps * 32 * 128;  // per-warp 32 x 128-byte staging tiles
-constexpr int kScaleBytes = 2 * 256 * 4;                     // FP8: a tile's weight-row scales, double-buffered
+constexpr int kScaleBytes = kEpilogueWarps * 256 * 4;        // FP8: a tile's weight-row scales, a copy per warp
 
 struct TcParams {
   const int32_t* offsets;  // [E+1] (already advanced to the first expert of the launch) or nullptr
@@ -356,20 +356,26 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
       __nv_bfloat16* const out = t.dense ? p.out2 : p.out;
       const int n_feat = t.dense ? p.n_feat2 : p.n_feat;
       // FP8: the tile's scales are fetched while it is still being multiplied -- the row's in a register, the weight rows'
-      // (gated: 128 gate rows, then the 128 up rows) in shared memory.  They are different ones for every tile, so read
-      // where they are used every 32 columns waited for L2 (Qwen3-shaped layer, T = 6007: down pass 137 -> 118 us, T = 2000: 67 -> 55).
+      // (gated: 128 gate rows, then the 128 up rows) in shared memory, because reads of L2 where they are used, every 32
+      // columns, are what the epilogue then waits for (Qwen3-shaped layer, T = 6007: down pass 137 against 118 us).  Each warp
+      // keeps a copy of its own: one for all four needs a barrier between them, which a warp whose accumulator wait has run
+      // out would never reach again (T = 6007, whole steps: 412.6 us with the barrier, 409.4 without).
       float rs = 0.f;
-      float* const sc = scales + as * 256u;
+      float* const sc = scales + warp * 256;
       if (FP8) {
         const float* const wsp =
             t.dense ? p.w_scale2 : p.w_scale + (size_t)(p.e_base + t.e) * (GATED ? 2 : 1) * n_feat;
         const int r = warp * 32 + lane;  // 0..127
         if (r < t.rows) rs = __ldg((t.dense ? p.row_scale2 : p.row_scale) + t.row0 + r);
-        const int f = t.ft * kFeatPerTile + r;
-        const int f2 = GATED ? n_feat + f : f + 128;
-        sc[r] = f < n_feat ? __ldg(wsp + f) : 0.f;
-        sc[128 + r] = (GATED ? f : f2) < n_feat ? __ldg(wsp + f2) : 0.f;
-        asm volatile("barrier.cta.sync 1, 128;" ::: "memory");
+        // n_feat is a multiple of 64: four scales are inside the weight rows or outside them as a whole
+        const int f = t.ft * kFeatPerTile + 4 * lane, f2 = GATED ? n_feat + f : f + 128;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 lo = f < n_feat ? __ldg(reinterpret_cast<const float4*>(wsp + f)) : zero;
+        const float4 hi = (GATED ? f : f2) < n_feat ? __ldg(reinterpret_cast<const float4*>(wsp + f2)) : zero;
+        __syncwarp();  // every lane has read the previous tile's
+        reinterpret_cast<float4*>(sc)[lane] = lo;
+        reinterpret_cast<float4*>(sc)[32 + lane] = hi;
+        __syncwarp();
       }
       if (!mbar_wait(bar_tfull + 8u * as, aph, abort_flag, p.wait_limit_ns)) { ok = false; break; }
       tc_fence_after();
