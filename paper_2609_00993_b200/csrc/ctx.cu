@@ -173,7 +173,7 @@ struct moe_ctx {
   int32_t* offsets;
   int32_t* perm;
   int32_t* inv_perm;
-  cudaEvent_t done;  // recorded after the last enqueue of every call
+  cudaEvent_t done;  // recorded after the last enqueue of every call (see PositionMark)
   int64_t launches;
   // pending-dispatch record of a split dispatch: what the second half needs (the arrays above, T) and the
   // stream position of the first half; at most one per context
@@ -213,6 +213,7 @@ struct moe_ctx {
   int64_t yields;     // launches that ended on a yield request
   bool offsets_fresh; // the kernel right before the gated pass wrote the step's offsets (moe_layer, a few tokens)
   bool unmarked;      // launches have been enqueued since `done` was last recorded
+  int calls_open;     // entry points being executed (the calls of a whole step are made by another)
   moe::StreamPlan* plans[2][4];  // tensor maps of the small-M GEMM: [buffer set][2 * (dense problem by itself) + down pass]
   unsigned long long wait_limit_ns;  // time limit of every bounded device-side wait (0 = the kernels' default)
   bool debug_stall;                  // failure-detection hook: the GEMM producers issue no copies
@@ -260,21 +261,31 @@ bool capturing(const moe_ctx* ctx) {
   return st != cudaStreamCaptureStatusNone;
 }
 
-// After the last enqueue of a call: count the launches.
+// Counts launches that have been enqueued.
 void mark(moe_ctx* ctx, int n) {
   ctx->launches += n;
   ctx->unmarked = true;
 }
 
-// Marks the stream position that moe_ctx_destroy asks about: at the end of a step (an event record between two kernels
-// of a step would cost host time on every call), or when a step is given up.  While the stream is being captured into a
-// CUDA graph nothing executes, so there is no position to mark (and an event recorded during capture could not be
-// queried later).
-void mark_position(moe_ctx* ctx) {
-  if (!ctx->unmarked) return;
-  ctx->unmarked = false;
-  if (!capturing(ctx)) cudaEventRecord(ctx->done, ctx->stream);
-}
+// Every entry point that enqueues holds one: when the outermost of them returns, however it returns, `done` is recorded
+// behind its last launch, for moe_ctx_destroy to ask about -- there and not in destroy, because what the caller puts on the
+// stream afterwards is not the context's.  The calls that make a whole step record once (a record costs host time, and a
+// step of the tiny layer is bound by that).  While the stream is being captured into a CUDA graph nothing executes, so
+// there is no position to mark (and an event recorded during capture could not be queried later).
+struct PositionMark {
+  moe_ctx* ctx;
+  explicit PositionMark(moe_ctx* c) : ctx(c) { ++ctx->calls_open; }
+  ~PositionMark() {
+    record();
+    --ctx->calls_open;
+  }
+  void record() {
+    if (ctx->calls_open > 1 || !ctx->unmarked) return;
+    ctx->unmarked = false;
+    DeviceGuard guard(ctx->device);
+    if (!capturing(ctx)) cudaEventRecord(ctx->done, ctx->stream);
+  }
+};
 
 // Brackets the launches of one stage with events when profiling is on.
 struct StageTimer {
@@ -506,6 +517,7 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
   for (int s = 0; s < l.n_sets; ++s) carve_set(*cfg, ctx->ws + kStatusBlock + (size_t)s * l.set_bytes, &ctx->sets[s]);
   ctx->host_stream = ctx->host_pipeline = false;
   ctx->unmarked = false;
+  ctx->calls_open = 0;
   ctx->offsets_fresh = false;
   bool have_plans = true;
   for (int i = 0; i < 8; ++i) {
@@ -582,7 +594,6 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
 moe_status moe_ctx_destroy(moe_ctx* ctx) {
   if (!ctx) return MOE_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
-  mark_position(ctx);  // (a step that stopped half way)
   cudaError_t q = cudaEventQuery(ctx->done);
   if (q == cudaErrorNotReady) return fail(ctx, MOE_ERR_STATE, "work is still in flight on the context's stream");
   if (q != cudaSuccess) (void)cudaGetLastError();
@@ -627,10 +638,6 @@ moe_status moe_ctx_destroy(moe_ctx* ctx) {
 moe_status moe_ctx_abandon_step(moe_ctx* ctx) {
   if (!ctx) return MOE_ERR_INVALID_ARG;
   if (ctx->state == ST_IDLE) return MOE_OK;
-  {
-    DeviceGuard guard(ctx->device);
-    mark_position(ctx);
-  }
   ctx->state = ST_IDLE;
   ctx->T = 0;
   ctx->pending_dispatch = false;  // a pending dispatch is retired with the step
@@ -666,6 +673,7 @@ moe_status moe_route(moe_ctx* ctx, const float* logits, const float* select_bias
   if (misaligned(logits) || misaligned(select_bias) || misaligned(topk_idx) || misaligned(topk_w))
     return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
   DeviceGuard guard(ctx->device);
+  PositionMark position(ctx);
   int n = 0;
   cudaError_t e;
   {
@@ -673,9 +681,9 @@ moe_status moe_route(moe_ctx* ctx, const float* logits, const float* select_bias
     e = moe::launch_route(logits, select_bias, T, ctx->cfg.n_experts, ctx->cfg.top_k, ctx->cfg.routed_scale, topk_idx,
                           topk_w, ctx->stream, &n);
   }
+  mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "moe_route");
   ctx->state = ST_ROUTED;
-  mark(ctx, n);
   return MOE_OK;
 }
 
@@ -709,10 +717,10 @@ moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx
     e = moe::launch_layout(topk_idx, (int64_t)T * ctx->cfg.top_k, ctx->cfg.n_experts, ctx->counts, ctx->offsets,
                            ctx->perm, ctx->inv_perm, b.scan, ctx->status, ctx->stream, &n);
   }
+  mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->T = T;
   ctx->offsets_fresh = false;
-  ctx->launches += n;
   return MOE_OK;
 }
 
@@ -746,8 +754,8 @@ moe_status enqueue_row_movement(moe_ctx* ctx, const char* who, const void* x) {
     e = moe::launch_permute(x, ctx->inv_perm, b.x_perm, T, ctx->cfg.top_k, ctx->cfg.hidden, ctx->status, ctx->stream,
                             &n, ctx->wait_limit_ns);
   }
+  mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
-  ctx->launches += n;
   return MOE_OK;
 }
 
@@ -785,6 +793,7 @@ moe_status grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, 
   if (misaligned(w_gate_up) || misaligned(w_down) || misaligned(x) || misaligned(ws_gate_up) || misaligned(ws_down))
     return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
   DeviceGuard guard(ctx->device);
+  PositionMark position(ctx);
   BufferSet& b = ctx->sets[ctx->cur];
   const moe_config& c = ctx->cfg;
   const int64_t N = (int64_t)T * c.top_k, Ncap = (int64_t)c.max_tokens * c.top_k;
@@ -851,9 +860,9 @@ moe_status grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, 
       }
     }
   }
+  mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "moe_grouped_ffn");
   ctx->state = ST_FFN_DONE;
-  mark(ctx, n);
   return MOE_OK;
 }
 
@@ -911,12 +920,12 @@ moe_status moe_dispatch_layout(moe_ctx* ctx, const int32_t* topk_idx, int32_t T,
     return fail(ctx, MOE_ERR_STATE, "moe_dispatch_layout called in the middle of a step");
   if (misaligned(x)) return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
   DeviceGuard guard(ctx->device);
+  PositionMark position(ctx);
   moe_status st = enqueue_layout(ctx, "moe_dispatch_layout", topk_idx, T, counts, offsets, perm, inv_perm);
   if (st == MOE_OK && x != nullptr) st = enqueue_row_movement(ctx, "moe_dispatch_layout", x);
   if (st != MOE_OK) return st;
   ctx->state = (x != nullptr || T == 0) ? ST_LAID_OUT : ST_LAYOUT_ONLY;  // an empty batch has no rows to move
   ctx->split_step = false;
-  mark(ctx, 0);
   return MOE_OK;
 }
 
@@ -928,12 +937,14 @@ moe_status moe_dispatch_notify(moe_ctx* ctx, const int32_t* topk_idx, int32_t T,
   if (ctx->state != ST_IDLE && ctx->state != ST_ROUTED)
     return fail(ctx, MOE_ERR_STATE, "moe_dispatch_notify called in the middle of a step");
   DeviceGuard guard(ctx->device);
-  moe_status st = enqueue_layout(ctx, "moe_dispatch_notify", topk_idx, T, counts, offsets, perm, inv_perm);
-  if (st != MOE_OK) return st;
+  {
+    PositionMark position(ctx);
+    const moe_status st = enqueue_layout(ctx, "moe_dispatch_notify", topk_idx, T, counts, offsets, perm, inv_perm);
+    if (st != MOE_OK) return st;
+  }
   ctx->state = ST_NOTIFIED;
   ctx->pending_dispatch = true;
   ctx->split_step = true;
-  mark(ctx, 0);
   if (!capturing(ctx)) cudaEventRecord(ctx->notified, ctx->stream);  // the record's stream position
   // boundary 0 of a segmented step: after notification, before any row moves
   if (ctx->seg_experts > 0 && ctx->boundary_fn) ctx->boundary_fn(ctx->boundary_user, 0, 1 + ffn_boundaries(ctx));
@@ -947,11 +958,11 @@ moe_status moe_dispatch_move(moe_ctx* ctx, const void* x) {
   if (ctx->T > 0 && !x) return fail(ctx, MOE_ERR_INVALID_ARG, "x is NULL");
   if (misaligned(x)) return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
   DeviceGuard guard(ctx->device);
+  PositionMark position(ctx);
   moe_status st = enqueue_row_movement(ctx, "moe_dispatch_move", x);
   if (st != MOE_OK) return st;  // the dispatch stays pending: retry, or abandon the step
   ctx->state = ST_LAID_OUT;
   ctx->pending_dispatch = false;
-  mark(ctx, 0);
   return MOE_OK;
 }
 
@@ -994,6 +1005,7 @@ moe_status moe_grouped_ffn_fp8(moe_ctx* ctx, const void* wq_gate_up, const float
       misaligned(wsq_gate_up) || misaligned(sws_gate_up) || misaligned(wsq_down) || misaligned(sws_down))
     return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
   DeviceGuard guard(ctx->device);
+  PositionMark position(ctx);
   BufferSet& b = ctx->sets[ctx->cur];
   const moe_config& c = ctx->cfg;
   const int64_t N = (int64_t)T * c.top_k, Ncap = (int64_t)c.max_tokens * c.top_k;
@@ -1076,9 +1088,9 @@ moe_status moe_grouped_ffn_fp8(moe_ctx* ctx, const void* wq_gate_up, const float
       if (e == cudaSuccess) boundary();
     }
   }
+  mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "moe_grouped_ffn_fp8");
   ctx->state = ST_FFN_DONE;
-  mark(ctx, n);
   return MOE_OK;
 }
 
@@ -1090,6 +1102,7 @@ moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_per
   if (misaligned(topk_w) || misaligned(inv_perm) || misaligned(out))
     return fail(ctx, MOE_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
   DeviceGuard guard(ctx->device);
+  PositionMark position(ctx);
   BufferSet& b = ctx->sets[ctx->cur];
   int n = 0;
   cudaError_t e;
@@ -1104,7 +1117,6 @@ moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_per
   ctx->split_step = false;
   if (ctx->n_sets == 2) ctx->cur ^= 1;  // D: the next step works in the other buffer set
   mark(ctx, n);
-  mark_position(ctx);
   return MOE_OK;
 }
 
@@ -1117,7 +1129,6 @@ namespace {
 moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits, const float* select_bias, const void* x,
                               int32_t T, int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
                               int32_t* inv_perm) {
-  if (!ctx) return MOE_ERR_INVALID_ARG;
   if (!dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm)) {
     const moe_status st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
     return st == MOE_OK ? moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm) : st;
@@ -1130,10 +1141,10 @@ moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits
   const cudaError_t e = moe::launch_small_dispatch(
       logits, select_bias, T, c.n_experts, c.top_k, c.routed_scale, topk_idx, topk_w, ctx->counts, ctx->offsets, ctx->perm,
       ctx->inv_perm, x, fp8 || gathers_rows(ctx) ? nullptr : ctx->sets[ctx->cur].x_perm, c.hidden, ctx->stream, &n);
+  mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->T = T;
   ctx->offsets_fresh = !fp8;
-  mark(ctx, n);
   if (fp8) {
     const moe_status st = enqueue_row_movement(ctx, who, x);
     if (st != MOE_OK) return st;
@@ -1151,6 +1162,8 @@ moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias
                      int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
                      int32_t* inv_perm, const void* w_gate_up, const void* w_down, const void* ws_gate_up,
                      const void* ws_down, void* out) {
+  if (!ctx) return MOE_ERR_INVALID_ARG;
+  PositionMark position(ctx);
   moe_status st = route_and_dispatch(ctx, "moe_layer", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
   if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T);
   if (st == MOE_OK) st = moe_combine(ctx, topk_w, inv_perm, T, out);
@@ -1162,6 +1175,8 @@ moe_status moe_layer_fp8(moe_ctx* ctx, const float* logits, const float* select_
                          int32_t* inv_perm, const void* wq_gate_up, const float* sw_gate_up, const void* wq_down,
                          const float* sw_down, const void* wsq_gate_up, const float* sws_gate_up, const void* wsq_down,
                          const float* sws_down, void* out) {
+  if (!ctx) return MOE_ERR_INVALID_ARG;
+  PositionMark position(ctx);
   moe_status st =
       route_and_dispatch(ctx, "moe_layer_fp8", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
   if (st == MOE_OK)
@@ -1181,6 +1196,7 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
   if (T > ctx->cfg.max_tokens) return fail(ctx, MOE_ERR_CAPACITY, "T = %d exceeds max_tokens = %d", T, ctx->cfg.max_tokens);
   if (T > 0 && (!logits_host || !x_host || !out_host)) return fail(ctx, MOE_ERR_INVALID_ARG, "NULL host pointer");
   DeviceGuard guard(ctx->device);
+  PositionMark position(ctx);
   moe_status st = ensure_host_stream(ctx, "moe_layer_host set-up");
   if (st != MOE_OK) return st;
   BufferSet& b = ctx->sets[ctx->cur];
@@ -1249,7 +1265,7 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
         err = moe::launch_combine(ctx->sets[ctx->cur].y_perm, y_shared, ctx->inv_perm, w, out, n_tok, c.top_k, c.hidden,
                                   ctx->status, ctx->stream, &n, ctx->wait_limit_ns, c0, c1);
       }
-      ctx->launches += n;
+      mark(ctx, n);
       if (err == cudaSuccess) err = cudaEventRecord(ctx->computed, ctx->stream);
       if (err == cudaSuccess) err = cudaStreamWaitEvent(ctx->h2d_stream, ctx->computed, 0);
       if (err == cudaSuccess && n_tok > 0)
@@ -1264,8 +1280,7 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
     if (ctx->n_sets == 2) ctx->cur ^= 1;
     if (T == 0) break;
   }
-  mark(ctx, 0);
-  mark_position(ctx);
+  position.record();  // before the wait, so that it has been passed when this returns
   // nothing of the caller's memory is in use when this returns, whatever happened
   for (cudaStream_t s : {ctx->stream, ctx->h2d_stream}) {
     const cudaError_t sync = cudaStreamSynchronize(s);
@@ -1289,6 +1304,7 @@ moe_status moe_layer_host_submit(moe_ctx* ctx, int32_t slot, const float* logits
   if (T > ctx->cfg.max_tokens) return fail(ctx, MOE_ERR_CAPACITY, "T = %d exceeds max_tokens = %d", T, ctx->cfg.max_tokens);
   if (T > 0 && (!logits_host || !x_host || !out_host)) return fail(ctx, MOE_ERR_INVALID_ARG, "NULL host pointer");
   DeviceGuard guard(ctx->device);
+  PositionMark position(ctx);
   cudaError_t e = cudaSuccess;
   moe_status st = ensure_host_pipeline(ctx, "moe_layer_host_submit set-up");
   if (st != MOE_OK) return st;
