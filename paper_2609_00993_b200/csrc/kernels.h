@@ -77,8 +77,8 @@ cudaError_t launch_route(const float* logits, const float* bias, int T, int E, i
                          float* w, cudaStream_t stream, int* n_launches);
 
 // ---- a2-a4 layout --------------------------------------------------------------------------
-// Scratch of the multi-CTA path: one row of E counts per chunk, and a chunk has 256 slots at least (the kernels use 1024
-// and more; the bound is also the documented limit of moe_dispatch_layout_static).
+// Scratch of the two-launch path: one row of E counts per chunk.  Sized for chunks of 256 slots, which is also the
+// documented limit of moe_dispatch_layout_static (the kernels use 1024 and more: rules.h).
 constexpr int kLayoutChunk = 256;
 inline size_t layout_scratch_ints(int64_t n_slots, int E) {
   int64_t chunks = (n_slots + kLayoutChunk - 1) / kLayoutChunk;

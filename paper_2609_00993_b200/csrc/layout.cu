@@ -8,22 +8,20 @@
 //   up to kRecountMaxSlots slots   one launch: every CTA counts the other chunks too (a few slots per thread);
 //   more                           a launch that counts each chunk, then the same kernel reading those counts.
 // The arithmetic is nothing; what it costs is launches, dependent round trips and the slots one SM can walk.  Back to
-// back in a CUDA graph, against one CTA up to 16384 slots and count -> scan -> place in three launches above: 512 slots of
-// 256 experts 4.1 -> 3.2 us, 5600 10.3 -> 5.9, 12248 of 128 17.7 -> 6.8, 32768 of 512 10.7 -> 8.5, 65536 of 128 8.4 -> 7.9,
-// 262144 of 256 14.3 -> 12.2.  (Recounting up to 32768 slots instead of 16384: 0.3 us less at 20000, 0.5 more at 32000.)
+// back in a CUDA graph: 512 slots of 256 experts 3.2 us, 5600 5.9, 12248 of 128 6.8, 32768 of 512 8.5, 65536 of 128 7.9,
+// 262144 of 256 12.2.  (Recounting up to 32768 slots instead of 16384: 0.3 us less at 20000, 0.5 more at 32000.)
+// How the slots are cut into chunks: rules.h.
 #include <mutex>
 
 #include "kernels.h"
 #include "routing.cuh"
+#include "rules.h"
 
 namespace moe {
 namespace {
 
 constexpr int kWarps = 32;                // warps (= runs) per CTA
 constexpr int kThreads = 32 * kWarps;
-constexpr int kMinChunk = 1024;           // slots per CTA at least: one step of 32 per warp
-constexpr int kMaxChunk = 4096;           // ... and at most
-constexpr int kChunkTarget = 64;          // CTAs wanted between those two
 constexpr int64_t kRecountMaxSlots = 16384;  // see above
 constexpr int kBatch = 8;                 // loads issued together (latency hiding)
 
@@ -228,10 +226,7 @@ cudaError_t launch_layout(const int32_t* topk_idx, int64_t n_slots, int E, int32
     if (err == cudaSuccess && n_launches) *n_launches += 1;
     return err;
   }
-  // (every CTA reads n_chunks x E counts: fewer, larger chunks where E is large)
-  const int target = E > 512 ? kChunkTarget / 2 : kChunkTarget;
-  int64_t chunk = (n_slots + target - 1) / target;
-  chunk = chunk < kMinChunk ? kMinChunk : chunk > kMaxChunk ? kMaxChunk : (chunk + kMinChunk - 1) / kMinChunk * kMinChunk;
+  const int64_t chunk = layout_chunk_slots(n_slots, E);
   const int n_chunks = (int)((n_slots + chunk - 1) / chunk);
   int n = 1;
   const int32_t* chunk_counts = nullptr;
@@ -299,8 +294,8 @@ extern "C" moe_status moe_dispatch_layout_static(const int32_t* topk_idx, int32_
     }
     scratch = g_static_scratch_addr[dev];
   }
-  // Nothing in the scratch has to start at zero: the count kernel writes every histogram cell that the
-  // scan and place kernels read afterwards, so what the previous call left behind is never seen.
+  // Nothing in the scratch has to start at zero: the count kernel writes every cell that the place kernel reads
+  // afterwards, so what the previous call left behind is never seen.
   cudaError_t e = moe::launch_layout(topk_idx, n_slots, n_experts, counts, offsets, perm, inv_perm, scratch,
                                      /*status=*/nullptr, static_cast<cudaStream_t>(cuda_stream), nullptr);
   if (e != cudaSuccess) {
