@@ -367,9 +367,10 @@ moe_status moe_layer_fp8(moe_ctx* ctx, const float* logits, const float* select_
 /* One whole step with HOST activations: copies logits_host [T,E] fp32 and x_host [T,H] bf16
  * to the device (cudaMemcpyAsync into context-owned staging), runs a1..a9, copies out
  * [T,H] bf16 back to out_host and waits for all of it before returning.  With pinned host
- * memory (recommended) the copies run on copy streams of the context and overlap the kernels:
- * the output leaves in pieces of columns while the down pass computes the next, and a large
- * prefill batch is cut into two chunks of tokens.  Results are those of the device calls, bit for bit.  select_bias and all weights are DEVICE pointers as above. */
+ * memory (recommended) and from half a megabyte of rows on the copies run on a copy stream of the context (created by
+ * its first call with 1.5 MB) and overlap the kernels: the output leaves in pieces of columns while the down pass computes
+ * the next, and a large prefill batch is cut into two chunks of tokens.  Results are those of the device calls, bit for
+ * bit.  select_bias and all weights are DEVICE pointers as above. */
 moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* select_bias, const void* x_host,
                           int32_t T, const void* w_gate_up, const void* w_down, const void* ws_gate_up,
                           const void* ws_down, void* out_host);
@@ -383,8 +384,8 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
  * slot's result has arrived in out_host (a no-op for a slot with nothing in flight).  A slot must be waited for
  * before it is submitted again (MOE_ERR_STATE otherwise); the host buffers of a submitted slot must stay valid
  * and untouched until its wait returns, and must be pinned for the copies to overlap anything.  Steps execute in
- * submission order.  The two copy streams and the events are created by the first submit on a context (host
- * resources, no device memory) and belong to that context alone; moe_ctx_destroy refuses while a slot is in
+ * submission order.  The two copy streams (one is that of moe_layer_host) and the events are created by the first submit on
+ * a context (host resources, no device memory) and belong to that context alone; moe_ctx_destroy refuses while a slot is in
  * flight.  Device-side arguments as for moe_layer_host.  Not for contexts created for FP8 weights. */
 #define MOE_HOST_SLOTS 4
 moe_status moe_layer_host_submit(moe_ctx* ctx, int32_t slot, const float* logits_host, const float* select_bias,

@@ -357,14 +357,16 @@ bool small_m_is_faster(bool fp8, bool gated, int K, int64_t rows, int64_t E) {
   return !up_to(kOneTileRows) && up_to(kShortKDownRows);
 }
 
-// moe_layer_host: the down pass in one piece for every 1.5 MB of output, up to four; two chunks of tokens from 200 rows
-// per expert and 4 MB a chunk on.  Measured on the Qwen3-30B-shaped layer with pinned buffers (whole call; before: copy,
-// compute, copy):
-//   T = 1531   534 us -> 513 (rows behind the router's work), 486 with two or four pieces, 520 with eight
-//   T = 701    369 us -> 343 with two pieces, 352 with four;  hidden 2560, 512 experts, T = 5001: 2517 -> 2261 us with four
-//   two chunks against one: T = 2600 (162 rows per expert) 737 : 690 us, 3500 (219) 824 : 845, 5200 (325) 1066 : 1235,
-//   8192 (512) 1400 : 1957 before;  three or four chunks at 8192: 1466, 1590 us.
-constexpr size_t kHostPieceBytes = 1536 * 1024, kHostChunkBytes = 4 << 20;
+// moe_layer_host.  Measured on the Qwen3-30B-shaped layer with pinned buffers, whole calls, us:
+//   copies beside the kernels | in order on the context's stream:  T = 16 (64 KB of rows) 178 | 165, 64 (256 KB) 239 | 235,
+//     128 (512 KB) 248 | 252, 384 (1.5 MB) 293 | 304, 1531 (6 MB) 488 | 529, 8192 1380 | 1950; tiny layer, T = 512 (256 KB)
+//     75 | 66, 2048 (1 MB) 107 | 108.  A context's first call, which creates the stream: T = 128 291 | 277, 256 (1 MB)
+//     321 | 314, 384 335 | 348, 1531 650 | 695, 8192 1680 | 2235 -- so only a call of 1.5 MB creates it.
+//   the down pass in one piece for every 1.5 MB of output, up to four: T = 1531 513 with one piece, 486 with two or four,
+//     520 with eight; T = 701 343 with two, 352 with four.
+//   two chunks of tokens | one: T = 2600 (162 rows per expert) 737 | 690, 3500 (219) 824 | 845, 5200 (325) 1066 | 1235;  three
+//     or four chunks at 8192: 1466, 1590.
+constexpr size_t kHostOverlapBytes = 512 * 1024, kHostPieceBytes = 1536 * 1024, kHostChunkBytes = 4 << 20;
 constexpr int kHostMaxPieces = 4, kHostChunkFromRows = 200;
 
 // AUTO: a DECODE context always streams; a PREFILL context chooses per launch from the problem's rows (T * top_k
@@ -879,29 +881,28 @@ cudaError_t create_stream_and_events(cudaStream_t* stream, cudaEvent_t* const* e
   return e;
 }
 
-// The copy stream of moe_layer_host, created by its first call.  One serves both directions, because creating a stream
-// takes 0.06 to 0.5 ms, which the first pass of a context pays (Qwen3-shaped layer, 1531 tokens: 778 us with two streams and
-// every event of the pipelined form, 716 with one; later passes 489 with either).
-moe_status ensure_host_stream(moe_ctx* ctx, const char* who) {
-  if (ctx->host_stream) return MOE_OK;
+// The copy stream of the host path.  moe_layer_host makes do with one for both directions: a second one is a second
+// creation, which a context pays for.
+cudaError_t ensure_host_stream(moe_ctx* ctx) {
+  if (ctx->host_stream) return cudaSuccess;
   cudaEvent_t* const events[] = {&ctx->copied_in[0], &ctx->copied_in[1], &ctx->computed};
   const cudaError_t e = create_stream_and_events(&ctx->h2d_stream, events, 3);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, who);
-  ctx->host_stream = true;
-  return MOE_OK;
+  ctx->host_stream = e == cudaSuccess;
+  return e;
 }
 
 // The pipelined form copies out on a second stream, beside the copies in of the next slots.
 moe_status ensure_host_pipeline(moe_ctx* ctx, const char* who) {
-  const moe_status st = ensure_host_stream(ctx, who);
-  if (st != MOE_OK || ctx->host_pipeline) return st;
+  cudaError_t e = ensure_host_stream(ctx);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, who);
+  if (ctx->host_pipeline) return MOE_OK;
   cudaEvent_t* events[3 * MOE_HOST_SLOTS];
   for (int s = 0; s < MOE_HOST_SLOTS; ++s) {
     events[3 * s] = &ctx->slots[s].h2d;
     events[3 * s + 1] = &ctx->slots[s].comp;
     events[3 * s + 2] = &ctx->slots[s].done;
   }
-  const cudaError_t e = create_stream_and_events(&ctx->d2h_stream, events, 3 * MOE_HOST_SLOTS);
+  e = create_stream_and_events(&ctx->d2h_stream, events, 3 * MOE_HOST_SLOTS);
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->host_pipeline = true;
   return MOE_OK;
@@ -1197,8 +1198,6 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
   if (T > 0 && (!logits_host || !x_host || !out_host)) return fail(ctx, MOE_ERR_INVALID_ARG, "NULL host pointer");
   DeviceGuard guard(ctx->device);
   PositionMark position(ctx);
-  moe_status st = ensure_host_stream(ctx, "moe_layer_host set-up");
-  if (st != MOE_OK) return st;
   BufferSet& b = ctx->sets[ctx->cur];
   const moe_config& c = ctx->cfg;
   const size_t row_bytes = (size_t)c.hidden * 2;
@@ -1207,85 +1206,111 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
   // the next is computed -- a piece costs two launches more, so there is one for every kHostPieceBytes, up to four.
   // A prefill batch of at least kHostChunkFromRows rows per expert is also cut into two chunks of tokens, so that the
   // second comes in while the first is computed; with fewer rows the pass is bound by streaming the weights, which each
-  // chunk would do again.  Segments and preemption keep their one sequence of boundaries.
-  // So does pageable memory, whose copies the runtime makes while the call waits.
+  // chunk would do again.  Segments and preemption keep their one sequence of boundaries; pageable memory is copied by the
+  // runtime while the call waits; and a few rows are there and back before a second stream is worth its events.
   cudaPointerAttributes attr;
   const bool pinned = T > 0 && cudaPointerGetAttributes(&attr, out_host) == cudaSuccess && attr.type == cudaMemoryTypeHost;
-  const bool whole = ctx->seg_experts > 0 || ctx->preemptible || c.gemm_variant == MOE_GEMM_VALIDATION || !pinned;
-  const bool halves = !whole && c.phase == MOE_PHASE_PREFILL &&
+  const bool overlap = pinned && T * row_bytes >= (ctx->host_stream ? kHostOverlapBytes : kHostPieceBytes) && ctx->seg_experts == 0 && !ctx->preemptible &&
+                       c.gemm_variant != MOE_GEMM_VALIDATION;
+  cudaError_t e = cudaSuccess;
+  moe_status st = MOE_OK;
+  for (const moe_ctx::HostSlot& s : ctx->slots)  // (a slot of the pipelined path may still be copying out of the staging)
+    if (e == cudaSuccess && s.in_flight) e = cudaStreamWaitEvent(ctx->stream, s.done, 0);
+  const bool halves = overlap && c.phase == MOE_PHASE_PREFILL &&
                       (int64_t)T * c.top_k >= (int64_t)kHostChunkFromRows * c.n_experts && T * row_bytes >= 2 * kHostChunkBytes;
   const int n_chunks = halves ? 2 : 1;
   const int chunk = ((T + n_chunks - 1) / n_chunks + 15) / 16 * 16;  // keeps every chunk's arrays 16-byte aligned
-  cudaError_t e = cudaEventRecord(ctx->computed, ctx->stream);  // the staging buffers are the stream's until here
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->h2d_stream, ctx->computed, 0);
-  for (const moe_ctx::HostSlot& s : ctx->slots)  // (a slot of the pipelined path may still be copying out of them)
-    if (e == cudaSuccess && s.in_flight) e = cudaStreamWaitEvent(ctx->stream, s.done, 0);
-  // The copy stream takes everything that comes in, in the order of use, before anything that goes out.
-  for (int i = 0; i * chunk < T && e == cudaSuccess; ++i) {
-    const size_t t0 = (size_t)i * chunk, n_tok = std::min<size_t>(chunk, T - t0);
-    e = cudaMemcpyAsync(b.logits + t0 * c.n_experts, logits_host + t0 * c.n_experts, n_tok * c.n_experts * 4,
-                        cudaMemcpyHostToDevice, ctx->h2d_stream);
+  auto tokens_of = [&](int i) { return std::min(chunk, T - i * chunk); };
+  auto copy_logits = [&](int i, cudaStream_t s) {
+    const size_t at = (size_t)i * chunk * c.n_experts;
+    return cudaMemcpyAsync(b.logits + at, logits_host + at, (size_t)tokens_of(i) * c.n_experts * 4, cudaMemcpyHostToDevice, s);
+  };
+  auto copy_rows = [&](int i, cudaStream_t s) {
+    const size_t at = (size_t)i * chunk * row_bytes;
+    return cudaMemcpyAsync(b.x_stage + at, static_cast<const char*>(x_host) + at, tokens_of(i) * row_bytes,
+                           cudaMemcpyHostToDevice, s);
+  };
+  auto copy_in = [&](int i) -> cudaError_t {  // on the copy stream
+    cudaError_t err = copy_logits(i, ctx->h2d_stream);
     if (i == 0) {  // the first chunk's router does not wait for the rows
-      if (e == cudaSuccess) e = cudaEventRecord(ctx->copied_in[0], ctx->h2d_stream);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->copied_in[0], 0);
+      if (err == cudaSuccess) err = cudaEventRecord(ctx->copied_in[0], ctx->h2d_stream);
+      if (err == cudaSuccess) err = cudaStreamWaitEvent(ctx->stream, ctx->copied_in[0], 0);
     }
+    if (err == cudaSuccess) err = copy_rows(i, ctx->h2d_stream);
+    return err == cudaSuccess ? cudaEventRecord(ctx->copied_in[i], ctx->h2d_stream) : err;
+  };
+
+  if (!overlap) {
+    if (T > 0 && e == cudaSuccess) e = copy_logits(0, ctx->stream);
+    if (T > 0 && e == cudaSuccess) e = copy_rows(0, ctx->stream);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(b.x_stage + t0 * row_bytes, static_cast<const char*>(x_host) + t0 * row_bytes, n_tok * row_bytes,
-                          cudaMemcpyHostToDevice, ctx->h2d_stream);
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->copied_in[i], ctx->h2d_stream);
-  }
-  for (int t0 = 0; (t0 < T || T == 0) && e == cudaSuccess && st == MOE_OK; t0 += chunk) {
-    const int n_tok = std::min(chunk, T - t0);
-    float* const logits = b.logits + (size_t)t0 * c.n_experts;
-    char* const x = b.x_stage + (size_t)t0 * row_bytes;
-    char* const out = b.out_stage + (size_t)t0 * row_bytes;
-    char* const out_to = static_cast<char*>(out_host) + (size_t)t0 * row_bytes;
-    int32_t* const idx = b.topk_idx + (size_t)t0 * c.top_k;
-    float* const w = b.topk_w + (size_t)t0 * c.top_k;
-    const cudaEvent_t copied_in = ctx->copied_in[t0 > 0 ? 1 : 0];
-    if (t0 > 0 && (e = cudaStreamWaitEvent(ctx->stream, copied_in, 0)) != cudaSuccess) break;
-    st = moe_route(ctx, logits, select_bias, n_tok, idx, w);
-    if (st == MOE_OK) st = enqueue_layout(ctx, "moe_layer_host", idx, n_tok, nullptr, nullptr, nullptr, nullptr);
-    if (st != MOE_OK) break;
-    if (T > 0 && (e = cudaStreamWaitEvent(ctx->stream, copied_in, 0)) != cudaSuccess) break;
-    st = enqueue_row_movement(ctx, "moe_layer_host", x);
-    if (st != MOE_OK) break;
-    ctx->state = ST_LAID_OUT;
-    ctx->split_step = false;
-    int pieces = 1;
-    if (!whole && t0 + n_tok == T)
-      pieces = (int)std::min<size_t>(kHostMaxPieces, 1 + (size_t)n_tok * row_bytes / kHostPieceBytes);
-    const int piece_cols = (c.hidden / pieces + 255) / 256 * 256;
-    const char* const y_shared = c.n_shared ? ctx->sets[ctx->cur].y_shared : nullptr;
-    auto finish = [&](int c0, int c1) -> cudaError_t {  // combine the columns [c0, c1) and send them
-      int n = 0;
-      cudaError_t err;
-      {
-        StageTimer tm(ctx, 7);
-        err = moe::launch_combine(ctx->sets[ctx->cur].y_perm, y_shared, ctx->inv_perm, w, out, n_tok, c.top_k, c.hidden,
-                                  ctx->status, ctx->stream, &n, ctx->wait_limit_ns, c0, c1);
-      }
-      mark(ctx, n);
-      if (err == cudaSuccess) err = cudaEventRecord(ctx->computed, ctx->stream);
-      if (err == cudaSuccess) err = cudaStreamWaitEvent(ctx->h2d_stream, ctx->computed, 0);
-      if (err == cudaSuccess && n_tok > 0)
-        err = cudaMemcpy2DAsync(out_to + (size_t)c0 * 2, row_bytes, out + (size_t)c0 * 2, row_bytes, (size_t)(c1 - c0) * 2,
-                                n_tok, cudaMemcpyDeviceToHost, ctx->h2d_stream);
-      return err;
-    };
-    st = grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, n_tok, pieces > 1 ? piece_cols : 0, finish);
-    if (st != MOE_OK) break;
-    if (pieces == 1) e = finish(0, c.hidden);
-    ctx->state = ST_IDLE;
-    if (ctx->n_sets == 2) ctx->cur ^= 1;
-    if (T == 0) break;
+      st = moe_layer(ctx, b.logits, select_bias, b.x_stage, T, b.topk_idx, b.topk_w, nullptr, nullptr, nullptr, nullptr,
+                     w_gate_up, w_down, ws_gate_up, ws_down, b.out_stage);
+    if (T > 0 && e == cudaSuccess && st == MOE_OK)
+      e = cudaMemcpyAsync(out_host, b.out_stage, T * row_bytes, cudaMemcpyDeviceToHost, ctx->stream);
+  } else {
+    // Creating a stream takes 0.06 to 0.5 ms, so the context's first such call copies its first chunk in on its own stream
+    // and creates the copy stream while the GPU is at the gated pass.
+    const bool have_stream = ctx->host_stream;
+    if (have_stream) {
+      if (e == cudaSuccess) e = cudaEventRecord(ctx->computed, ctx->stream);  // the staging is the stream's until here
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->h2d_stream, ctx->computed, 0);
+      // the copy stream takes everything that comes in, in the order of use, before anything that goes out
+      for (int i = 0; i < n_chunks && e == cudaSuccess; ++i) e = copy_in(i);
+    } else if (e == cudaSuccess) {
+      e = copy_logits(0, ctx->stream);
+    }
+    for (int i = 0; i < n_chunks && e == cudaSuccess; ++i) {
+      const int t0 = i * chunk, n_tok = tokens_of(i);
+      char* const x = b.x_stage + (size_t)t0 * row_bytes;
+      char* const out = b.out_stage + (size_t)t0 * row_bytes;
+      char* const out_to = static_cast<char*>(out_host) + (size_t)t0 * row_bytes;
+      int32_t* const idx = b.topk_idx + (size_t)t0 * c.top_k;
+      float* const w = b.topk_w + (size_t)t0 * c.top_k;
+      if (i > 0 && (e = cudaStreamWaitEvent(ctx->stream, ctx->copied_in[i], 0)) != cudaSuccess) break;
+      st = moe_route(ctx, b.logits + (size_t)t0 * c.n_experts, select_bias, n_tok, idx, w);
+      if (st == MOE_OK) st = enqueue_layout(ctx, "moe_layer_host", idx, n_tok, nullptr, nullptr, nullptr, nullptr);
+      if (st != MOE_OK) break;
+      if (i == 0) e = have_stream ? cudaStreamWaitEvent(ctx->stream, ctx->copied_in[0], 0) : copy_rows(0, ctx->stream);
+      if (e != cudaSuccess) break;
+      st = enqueue_row_movement(ctx, "moe_layer_host", x);
+      if (st != MOE_OK) break;
+      ctx->state = ST_LAID_OUT;
+      ctx->split_step = false;
+      const int pieces = i + 1 < n_chunks ? 1 : (int)std::min<size_t>(kHostMaxPieces, 1 + n_tok * row_bytes / kHostPieceBytes);
+      const int piece_cols = (c.hidden / pieces + 255) / 256 * 256;
+      const char* const y_shared = c.n_shared ? ctx->sets[ctx->cur].y_shared : nullptr;
+      auto finish = [&](int c0, int c1) -> cudaError_t {  // combine the columns [c0, c1) and send them
+        int n = 0;
+        cudaError_t err;
+        {
+          StageTimer tm(ctx, 7);
+          err = moe::launch_combine(ctx->sets[ctx->cur].y_perm, y_shared, ctx->inv_perm, w, out, n_tok, c.top_k, c.hidden,
+                                    ctx->status, ctx->stream, &n, ctx->wait_limit_ns, c0, c1);
+        }
+        mark(ctx, n);
+        if (err == cudaSuccess && !ctx->host_stream) {
+          err = ensure_host_stream(ctx);
+          for (int j = 1; j < n_chunks && err == cudaSuccess; ++j) err = copy_in(j);
+        }
+        if (err == cudaSuccess) err = cudaEventRecord(ctx->computed, ctx->stream);
+        if (err == cudaSuccess) err = cudaStreamWaitEvent(ctx->h2d_stream, ctx->computed, 0);
+        if (err != cudaSuccess) return err;
+        return cudaMemcpy2DAsync(out_to + (size_t)c0 * 2, row_bytes, out + (size_t)c0 * 2, row_bytes, (size_t)(c1 - c0) * 2, n_tok,
+                                 cudaMemcpyDeviceToHost, ctx->h2d_stream);
+      };
+      st = grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, n_tok, pieces > 1 ? piece_cols : 0, finish);
+      if (st != MOE_OK) break;
+      if (pieces == 1) e = finish(0, c.hidden);
+      ctx->state = ST_IDLE;
+      if (ctx->n_sets == 2) ctx->cur ^= 1;
+    }
   }
   position.record();  // before the wait, so that it has been passed when this returns
   // nothing of the caller's memory is in use when this returns, whatever happened
-  for (cudaStream_t s : {ctx->stream, ctx->h2d_stream}) {
-    const cudaError_t sync = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = sync;
-  }
+  cudaError_t sync = cudaStreamSynchronize(ctx->stream);
+  if (e == cudaSuccess) e = sync;
+  if (overlap && ctx->host_stream && (sync = cudaStreamSynchronize(ctx->h2d_stream)) != cudaSuccess && e == cudaSuccess) e = sync;
   if (st != MOE_OK || e != cudaSuccess) ctx->state = ST_IDLE;
   if (st != MOE_OK) return st;
   return e == cudaSuccess ? MOE_OK : cuda_fail(ctx, e, "moe_layer_host");
