@@ -410,7 +410,8 @@ moe_status moe_ctx_debug_ptrs_fp8(moe_ctx* ctx, void** xq, float** sx, void** aq
  * Stage order: 0 route, 1 layout (counts+scan+permutation), 2 permute rows, 3 routed GEMM1+SwiGLU,
  * 4 routed GEMM2, 5 shared GEMM1+SwiGLU, 6 shared GEMM2, 7 combine.  Without prefill segmentation the shared
  * expert's passes ride in the routed launches, so their time is part of stages 3 and 4 and stages 5 and 6
- * stay empty.  FP8 variant only: 8 quantise the GEMM1 input rows, 9 quantise the activation rows. */
+ * stay empty.  moe_layer and moe_layer_fp8 route, lay out and (bf16) move up to 64 tokens in one launch, which is
+ * stage 0; stages 1 and 2 then stay empty.  FP8 variant only: 8 quantise the GEMM1 input rows, 9 quantise the activation rows. */
 #define MOE_N_STAGES 10
 typedef struct {
   double ms[MOE_N_STAGES];

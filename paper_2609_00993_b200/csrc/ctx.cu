@@ -726,13 +726,13 @@ moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx
   return MOE_OK;
 }
 
-// Whether a step routes and lays out in one launch: a few tokens, every argument fit for moe_route and
-// moe_dispatch_layout both -- or the calls themselves report what is wrong -- and no stage times wanted.
+// Whether a step routes and lays out in one launch: a few tokens, and every argument fit for moe_route and
+// moe_dispatch_layout both -- or the calls themselves report what is wrong.
 bool dispatches_at_once(const moe_ctx* ctx, const float* logits, const float* select_bias, const void* x, int32_t T,
                         const int32_t* topk_idx, const float* topk_w, const int32_t* counts, const int32_t* offsets,
                         const int32_t* perm, const int32_t* inv_perm) {
   const moe_config& c = ctx->cfg;
-  return (ctx->state == ST_IDLE || ctx->state == ST_ROUTED) && !ctx->profiling && T <= c.max_tokens &&
+  return (ctx->state == ST_IDLE || ctx->state == ST_ROUTED) && T <= c.max_tokens &&
          moe::small_dispatch_fits(T, c.n_experts, c.top_k) && logits && x && topk_idx && topk_w &&
          !misaligned(logits) && !misaligned(select_bias) && !misaligned(x) && !misaligned(topk_idx) &&
          !misaligned(topk_w) && !misaligned(counts) && !misaligned(offsets) && !misaligned(perm) && !misaligned(inv_perm);
@@ -1139,9 +1139,13 @@ moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits
   const moe_config& c = ctx->cfg;
   const bool fp8 = c.weight_format == MOE_WEIGHTS_FP8_E4M3;
   int n = 0;
-  const cudaError_t e = moe::launch_small_dispatch(
-      logits, select_bias, T, c.n_experts, c.top_k, c.routed_scale, topk_idx, topk_w, ctx->counts, ctx->offsets, ctx->perm,
-      ctx->inv_perm, x, fp8 || gathers_rows(ctx) ? nullptr : ctx->sets[ctx->cur].x_perm, c.hidden, ctx->stream, &n);
+  cudaError_t e;
+  {
+    StageTimer tm(ctx, 0);
+    e = moe::launch_small_dispatch(logits, select_bias, T, c.n_experts, c.top_k, c.routed_scale, topk_idx, topk_w, ctx->counts,
+                                   ctx->offsets, ctx->perm, ctx->inv_perm, x,
+                                   fp8 || gathers_rows(ctx) ? nullptr : ctx->sets[ctx->cur].x_perm, c.hidden, ctx->stream, &n);
+  }
   mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->T = T;
