@@ -396,9 +396,10 @@ cudaError_t run_gemm(moe_ctx* ctx, moe::GemmProblem p, const moe::GemmDenseGroup
   const int variant = gemm_variant_of(ctx, p);
   p.wait_limit_ns = ctx->wait_limit_ns;
   p.debug_stall = ctx->debug_stall;
-  // Every GEMM launch comes after the step's row movement (or after another GEMM launch or a quantisation of the
-  // same step), which in turn waited for the layout kernels: the offsets are older than the previous kernel.  Only a
-  // step that dispatched its tokens in one launch has them from the kernel before its gated pass.
+  // Every GEMM launch comes after the step's row movement (or after another GEMM launch of the same step), which in turn
+  // waited for the layout kernels: the offsets are older than the previous kernel.  The quantisation between the passes
+  // lets the down pass start beside the gated one; the offsets are older than that, too.  Only a step that dispatched its
+  // tokens in one launch has them from the kernel before its gated pass.
   p.offsets_settled = !(ctx->offsets_fresh && p.gated);
   p.tile_counters = reinterpret_cast<int*>(ctx->ws + kTileCounterOffset) + 2 * (ctx->gemm_seq++ % kTileCounterPairs);
   p.max_group_rows = T;
@@ -1072,10 +1073,10 @@ moe_status moe_grouped_ffn_fp8(moe_ctx* ctx, const void* wq_gate_up, const float
           // the shared expert's rows ride along if they are as long (a launch between the two passes is time in which no
           // weights stream)
           const bool ride = shared && c.shared_inter == c.inter;
-          e = moe::launch_quantize_rows(b.act, N, c.inter, b.aq, b.sa, ctx->stream, &n, ride ? b.act_shared : nullptr,
+          e = moe::launch_quantize_rows(b.act, N, c.inter, b.aq, b.sa, true, ctx->stream, &n, ride ? b.act_shared : nullptr,
                                         ride ? T : 0, b.aq_shared, b.sa_shared);
           if (e == cudaSuccess && shared && !ride)
-            e = moe::launch_quantize_rows(b.act_shared, T, c.shared_inter, b.aq_shared, b.sa_shared, ctx->stream, &n);
+            e = moe::launch_quantize_rows(b.act_shared, T, c.shared_inter, b.aq_shared, b.sa_shared, true, ctx->stream, &n);
         }
         if (e == cudaSuccess) boundary();
       }

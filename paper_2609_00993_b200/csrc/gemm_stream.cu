@@ -109,9 +109,9 @@ struct StreamParams {
   // preemption at tile granularity (both null: off)
   const int* yield_req;
   int* stopped;
-  // The expert offsets were final before the PREVIOUS kernel of the stream started (and the weights always are):
-  // the tile list is built and weight boxes are fetched before this kernel waits for that previous kernel, which
-  // only the token rows (and the FP8 row scales) depend on.
+  // The expert offsets are older than every kernel that may still be running (and the weights always are): the tile list
+  // is built and weight boxes are fetched before this kernel waits for the previous one, which only the token rows (and
+  // the FP8 row scales) depend on.
   int32_t early_setup;
   int32_t sort_tiles;  // 0: every group has at most one tile of the smallest size, so their order does not matter
 };

@@ -18,12 +18,17 @@ inline cudaError_t ensure_dynamic_smem(Kernel kern, size_t bytes) {
 }
 
 // Programmatic dependent launch: the kernels of the library are launched with "programmatic stream serialization
-// allowed" (the GEMMs for small problems only, see kGemmOverlapMaxRows), so their CTAs may become resident and run their prologue (barrier set-up, tensor-memory allocation,
-// tensor-map prefetch) while the previous kernel of the stream is still draining; pdl_wait() then blocks until that
-// kernel has completed and its writes are visible.  Rules: every thread calls pdl_wait() before its first access to
-// global memory (reads AND writes: the predecessor may still be reading what this kernel overwrites), and
-// pdl_launch_dependents() right after it, which lets the NEXT kernel start its own prologue as soon as SM resources
-// free up.  A step of six dependent kernels sheds the launch latency and prologue of each of them this way.
+// allowed" (the GEMMs for small problems only, see kGemmOverlapMaxRows), so their CTAs may become resident and run their
+// prologue (barrier set-up, tensor-memory allocation, tensor-map prefetch) while the previous kernel of the stream is
+// still draining; pdl_wait() then blocks until that kernel has completed and its writes are visible.
+// Rules.  A thread calls pdl_wait() before it first touches global memory that an unfinished kernel may write (or, for its
+// own writes, read), and pdl_launch_dependents() right after that wait, never before it.  A kernel therefore starts when
+// everything before its predecessor has completed, and may read that -- but nothing of its predecessor -- before it waits
+// (offsets_settled below, and the tile counters, of which launches in a row use different pairs).
+// The one exception is a quantisation launched with release_early: it releases before it waits.  The kernel behind it (or
+// behind several of them in a row) may start while the kernel BEFORE the quantisation is still running, so that before its
+// wait it may read only what is older than that one: everything before it has completed, because it releases by the rule.
+// A kernel that is launched behind such a quantisation must be held against that.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -162,8 +167,9 @@ struct GemmProblem {
   // Every launch of a pass that may be stopped and launched again sets this (also a launch without yield_req that
   // finishes such a pass): all its tiles come from the counter, none is dealt statically.
   bool resumable = false;
-  // Small-M kernel: `offsets` was final before the previous kernel of the stream started, so the kernel may read it
-  // (and fetch weights) before it waits for that kernel; only the rows of A (and the FP8 row scales) wait.
+  // Small-M kernel: `offsets` was final before the previous kernel of the stream started (behind a quantisation that
+  // releases early: before the kernel in front of that one started), so the kernel may read it (and fetch weights) before
+  // it waits; only the rows of A (and the FP8 row scales) wait.
   bool offsets_settled = false;
   // Upper bound on the rows of any one group (a token reaches an expert at most once, so T), or 0 if unknown.  With
   // at most 16, every non-empty group is one tile of the same cost and the small-M kernel skips ordering them.
@@ -186,9 +192,13 @@ struct GemmDenseGroup {
 
 // FP8 variant: per-row dynamic quantisation of bf16 rows [rows, n] -> E4M3 codes [rows, n] + scale [rows]
 // (n a multiple of 16, at most 8192).  A second set of rows of the same length may ride in the launch.
-cudaError_t launch_quantize_rows(const void* x, int64_t rows, int n, void* q, float* scale, cudaStream_t stream,
-                                 int* n_launches, const void* x2 = nullptr, int64_t rows2 = 0, void* q2 = nullptr,
-                                 float* scale2 = nullptr);
+// release_early: the next kernel of the stream may start although neither this launch nor the one before it has finished
+// (rules above).  For the quantisation between the two passes: the down pass reads only weights and the offsets, which are
+// older than the gated pass, before it waits, so its weights are on their way when the codes are there (V3-shaped FP8
+// decode, one token 85.8 us a step without, 84.3 with).
+cudaError_t launch_quantize_rows(const void* x, int64_t rows, int n, void* q, float* scale, bool release_early,
+                                 cudaStream_t stream, int* n_launches, const void* x2 = nullptr, int64_t rows2 = 0,
+                                 void* q2 = nullptr, float* scale2 = nullptr);
 // The same for T token rows, whose codes and scales also go to their k places in the dispatch: row inv_perm[t * k + j] of
 // q_perm / scale_perm (negative: dropped).  q and scale (token order) may be nullptr.
 cudaError_t launch_quantize_move(const void* x, int T, int n, void* q, float* scale, const int32_t* inv_perm, int k,

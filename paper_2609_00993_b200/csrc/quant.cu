@@ -48,14 +48,11 @@ __global__ void __launch_bounds__(kQuantThreads)
 quantize_rows_kernel(const uint4* __restrict__ x, long long rows, int n_pieces, uint4* __restrict__ q,
                      float* __restrict__ scale, const int32_t* __restrict__ inv_perm, int k, uint4* __restrict__ q_perm,
                      float* __restrict__ scale_perm, const uint4* __restrict__ x2, long long rows2, uint4* __restrict__ q2,
-                     float* __restrict__ scale2) {
+                     float* __restrict__ scale2, bool release_early) {
   __shared__ uint32_t warp_max[kQuantThreads / 32];
-  // Without MOVE the next kernel is the down pass, which until it waits for this one reads only weights and the expert
-  // offsets: it may start while the kernel before this one is still finishing, and its weights are on their way when the
-  // codes are there (V3-shaped FP8 decode, one token 85.8 -> 84.3 us).  With MOVE the offsets themselves are that fresh.
-  if (!MOVE) pdl_launch_dependents();
+  if (release_early) pdl_launch_dependents();  // (see launch_quantize_rows)
   pdl_wait();
-  if (MOVE) pdl_launch_dependents();
+  if (!release_early) pdl_launch_dependents();
   constexpr int kRowThreads = 32 * ROW_WARPS;
   const int tid = ROW_WARPS == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
   long long row = ROW_WARPS == 1 ? (long long)blockIdx.x * (kQuantThreads / 32) + (threadIdx.x >> 5)
@@ -129,8 +126,8 @@ namespace {
 
 template <bool MOVE>
 cudaError_t launch(const void* x, int64_t rows, int n, void* q, float* scale, const int32_t* inv_perm, int k, void* q_perm,
-                   float* scale_perm, const void* x2, int64_t rows2, void* q2, float* scale2, cudaStream_t stream,
-                   int* n_launches) {
+                   float* scale_perm, const void* x2, int64_t rows2, void* q2, float* scale2, bool release_early,
+                   cudaStream_t stream, int* n_launches) {
   if (rows <= 0) return cudaSuccess;
   if (n <= 0 || n % 16 != 0 || n > 16 * kQuantThreads * kQuantMaxPieces || rows + rows2 > 0x7fffffffLL || k > 32)
     return cudaErrorNotSupported;
@@ -144,7 +141,7 @@ cudaError_t launch(const void* x, int64_t rows, int n, void* q, float* scale, co
     if (e != cudaSuccess) return e;
     return launch_pdl(true, kern, dim3(blocks), dim3(kQuantThreads), 0, stream, static_cast<const uint4*>(x), (long long)rows,
                       pieces, static_cast<uint4*>(q), scale, inv_perm, k, static_cast<uint4*>(q_perm), scale_perm,
-                      static_cast<const uint4*>(x2), (long long)rows2, static_cast<uint4*>(q2), scale2);
+                      static_cast<const uint4*>(x2), (long long)rows2, static_cast<uint4*>(q2), scale2, release_early);
   };
   cudaError_t err;
   if (warp_row)
@@ -159,14 +156,17 @@ cudaError_t launch(const void* x, int64_t rows, int n, void* q, float* scale, co
 
 }  // namespace
 
-cudaError_t launch_quantize_rows(const void* x, int64_t rows, int n, void* q, float* scale, cudaStream_t stream,
-                                 int* n_launches, const void* x2, int64_t rows2, void* q2, float* scale2) {
-  return launch<false>(x, rows, n, q, scale, nullptr, 0, nullptr, nullptr, x2, rows2, q2, scale2, stream, n_launches);
+cudaError_t launch_quantize_rows(const void* x, int64_t rows, int n, void* q, float* scale, bool release_early,
+                                 cudaStream_t stream, int* n_launches, const void* x2, int64_t rows2, void* q2,
+                                 float* scale2) {
+  return launch<false>(x, rows, n, q, scale, nullptr, 0, nullptr, nullptr, x2, rows2, q2, scale2, release_early, stream,
+                       n_launches);
 }
 
 cudaError_t launch_quantize_move(const void* x, int T, int n, void* q, float* scale, const int32_t* inv_perm, int k,
                                  void* q_perm, float* scale_perm, cudaStream_t stream, int* n_launches) {
-  return launch<true>(x, T, n, q, scale, inv_perm, k, q_perm, scale_perm, nullptr, 0, nullptr, nullptr, stream, n_launches);
+  return launch<true>(x, T, n, q, scale, inv_perm, k, q_perm, scale_perm, nullptr, 0, nullptr, nullptr, false, stream,
+                      n_launches);
 }
 
 }  // namespace moe
