@@ -66,11 +66,11 @@ typedef enum {
 } moe_status;
 
 /* GEMM kernel variants.  AUTO: a DECODE context uses small-M; a PREFILL context chooses per step and pass from
- * the step's rows per expert R = T * top_k / n_experts and the pass's K (hidden for the gated pass, inter for the
- * down pass): small-M for every problem of up to 8192 rows and, above that, wherever it was measured ahead (with bf16 the
- * gated pass at nearly every size and the down pass unless K is short; with FP8 where K is long or R is small); large-M
- * otherwise -- a function of T alone, so a step captured in a CUDA graph replays
- * the kernels it was captured with. */
+ * the step's rows per expert R = T * top_k / n_experts, the pass's K (hidden for the gated pass, inter for the down pass)
+ * and its number of tiles: small-M for every problem of up to 8192 rows and, above that, wherever it was measured ahead
+ * (with bf16 the gated pass unless K or the tiles are few, and the down pass unless K is short; with FP8 where K is long or
+ * R is small); large-M otherwise -- a function of T and the context's configuration alone, so a step captured in a CUDA
+ * graph replays the kernels it was captured with. */
 typedef enum {
   MOE_GEMM_AUTO = 0,
   MOE_GEMM_LARGE_M = 1,  /* tokens fill the 128-row MMA dimension; for experts of many hundreds of rows,

@@ -14,6 +14,7 @@
 
 #include "../../include/moe_pd.h"
 #include "kernels.h"
+#include "rules.h"
 
 namespace {
 
@@ -321,42 +322,6 @@ int gemm_ctas(const moe_ctx* ctx) {
   return (ctx->cfg.sm_budget > 0 && ctx->cfg.sm_budget < ctx->n_sms) ? ctx->cfg.sm_budget : ctx->n_sms;
 }
 
-// The choice between the two tensor-core variants for a PREFILL context, per pass, from the rows per expert
-// R = rows / experts and the pass's K.  The small-M kernel reads an expert's weights once for up to 256 rows, multiplies
-// exactly the rows there are and moves fewer bytes through shared memory per flop; the large-M kernel multiplies rows in
-// steps of 128 but always overlaps its epilogue with the next tile, which counts when K is short.  Both draw the GPU's
-// power limit at these sizes, so the lines below are whole steps in the sustained state (each variant run for 0.12 s
-// before it was timed for 0.12 s, in turns), gated / down pass, s = small-M, l = large-M, us:
-//   bf16  K = 2048 / 768 (hidden 2048, 128 experts):  R = 95 ss 289 sl 285 ll 280;  131 335 337 351;  156 358 366 397;
-//         187 397 397 414;  325 578 563 572;  512 808 785 820;  750 1121 1082 1106;  1500 2113 2036 2096
-//         K = 2560 / 1024 (512 experts):  31 ss 1315 sl 1380 ll 1490;  64 1482 1511 1579;  187 2197 2266 2541;
-//         312 3358 3381 3573;  375 3757 3748 3911;  468 4447 4445 4697
-//         K = 7168 / 2048 (256 experts + shared):  46 ss 3784 sl 4041 ll 4615;  281 8907 9599 10410;  500 14111 15087
-//         16142;  750 20017 19998 19769;  937 24815 25055 25740;  Zipf routing, 1024: 24911 25075 26394
-//   FP8   K = 2048 / 768:  93 ss 204 sl 202 ll 196;  156 271 273 271;  187 304 299 284;  375 506 479 448;  1500 1708 1566
-//         1466
-//         K = 2560 / 1024:  31 ss 744 sl 773 ll 879;  64 886 894 923;  156 1365 1390 1538;  218 1697 1610 1719;
-//         312 2337 2258 2252;  468 3306 3095 3040
-//         K = 7168 / 2048:  46 ss 2073 sl 2185 ll 2520;  128 3011 3154 3475;  281 5038 5137 5653;  437 7048 7042 7467;
-//         500 7904 7674 8118;  625 9928 9732 11110;  1000 14867 14629 16121
-constexpr int kLongK = 4096, kMidK = 2560, kMidDownK = 1024, kLongDownK = 2048;
-constexpr int64_t kOneTileRows = 120;     // an expert's rows fit one 128-row tile, spread included
-constexpr int64_t kShortKDownRows = 200;  // bf16 down pass, K < 1024: small-M between these two
-constexpr int64_t kMidKDownRows = 350;    // ... 1024 <= K < 2048: small-M up to here; from K = 2048 on at every R
-constexpr int64_t kFp8MidKRows = 300, kFp8MidKDownRows = 180, kFp8LongKDownRows = 400;
-
-bool small_m_is_faster(bool fp8, bool gated, int K, int64_t rows, int64_t E) {
-  const auto up_to = [&](int64_t r) { return rows <= r * E; };
-  if (gated) {
-    if (fp8) return K >= kLongK || (K >= kMidK && up_to(kFp8MidKRows));
-    return K >= kMidK || !up_to(kOneTileRows);
-  }
-  if (fp8) return K >= kLongDownK ? up_to(kFp8LongKDownRows) : K >= kMidDownK && up_to(kFp8MidKDownRows);
-  if (K >= kLongDownK) return true;
-  if (K >= kMidDownK) return up_to(kMidKDownRows);
-  return !up_to(kOneTileRows) && up_to(kShortKDownRows);
-}
-
 // moe_layer_host.  Measured on the Qwen3-30B-shaped layer with pinned buffers, whole calls, us:
 //   copies beside the kernels | in order on the context's stream:  T = 16 (64 KB of rows) 178 | 165, 64 (256 KB) 239 | 235,
 //     128 (512 KB) 248 | 252, 384 (1.5 MB) 293 | 304, 1531 (6 MB) 488 | 529, 8192 1380 | 1950; tiny layer, T = 512 (256 KB)
@@ -380,7 +345,7 @@ int gemm_variant_of(const moe_ctx* ctx, const moe::GemmProblem& p) {
   if (ctx->preemptible) return MOE_GEMM_SMALL_M;          // only the small-M kernel can stop between tiles
   // problems of up to 8192 rows, whose launches overlap with their neighbours, are 1.5-6 % faster on the small-M kernel
   // at any shape: it builds its tile list and fetches weights before the previous kernel has finished
-  const bool small = p.rows_bound <= moe::kGemmOverlapMaxRows || small_m_is_faster(p.fp8, p.gated, p.K, p.rows_bound, p.E);
+  const bool small = p.rows_bound <= moe::kGemmOverlapMaxRows || moe::small_m_is_faster(p.fp8, p.gated, p.K, p.n_feat, p.rows_bound, p.E, gemm_ctas(ctx));
   return small ? MOE_GEMM_SMALL_M : MOE_GEMM_LARGE_M;
 }
 

@@ -24,4 +24,62 @@ inline int64_t layout_chunk_slots(int64_t n_slots, int E) {
   return least > kLayoutMidChunk ? least : kLayoutMidChunk;
 }
 
+// ---- which tensor-core kernel takes a pass of a PREFILL context (AUTO), for problems of more than 8192 rows
+// From the rows per expert R = rows / experts, the pass's K and output features, and how many CTAs the grid has.  The small-M
+// kernel reads an expert's weights once for up to 256 rows, multiplies exactly the rows there are and moves fewer bytes per
+// flop; the large-M kernel multiplies rows in steps of 128, but its tiles are half as large and its epilogue always overlaps
+// the next tile, which counts where K is short.  Both draw the GPU's power limit in steps of a millisecond and more.
+// Whole steps in the sustained state, us, gated pass / down pass on s = small-M, l = large-M; "K / K' x E" is a layer of
+// hidden K, inter K' and E experts (the gated pass has K and K' features, the down pass K' and K).
+//   bf16, gated pass (sl : ll)
+//     512 / 2048 x 8    R = 1100 100 : 84, 8000 508 : 472;  768 / 512 x 128  100 102 : 99, 160 130 : 131, 300 182 : 181
+//     1024 / 512 x 64   192 (256 tiles of 256 rows) 101 : 96, 400 (512) 157 : 153, 700 (768) 231 : 233;  x 512  24 313 : 338, 160
+//                       (2048) 528 : 589;  1024 / 256 x 256  40 116 : 121, 200 (512) 212 : 208, 300 (1024) 277 : 284
+//     1280 / 768 x 128  72 181 : 182, 96 195 : 193, 160 250 : 271, 600 594 : 604;  1536 / 512 x 128  72 156 : 158, 96 169 : 168,
+//                       160 216 : 229, 300 319 : 331
+//     2048 / 768 x 128  72 261 : 268, 96 281 : 282, 108 291 : 289, 120 308 : 309, 144 348 : 392, 220 415 : 436;
+//                x 512  24 809 : 922, 48 890 : 963, 96 1024 : 1051, 160 1363 : 1679
+//     few tiles: 2048 / 768 x 4  2100 (216 tiles of 256 rows on 148 CTAs) 131 : 120, 4000 (384) 221 : 216, 8000 411 : 409;
+//                7168 / 512 x 8  1100 (160) 297 : 278, 2000 (256) 467 : 493
+//   bf16, down pass (ss : sl)
+//     2048 / 256 x 128  160 182 : 178, 400 352 : 330;  1536 / 512 x 128  160 218 : 216, 200 251 : 239, 600 553 : 521
+//     2048 / 768 x 128  72 263 : 261, 120 308 : 308, 144 339 : 348, 180 378 : 381, 200 403 : 395;  x 512  24 794 : 809, 48 869 :
+//                890, 96 1041 : 1024, 144 1236 : 1317, 200 1479 : 1457
+//     1792 / 1024 x 128  72 293 : 296, 112 331 : 329, 160 387 : 402, 300 603 : 610, 600 1019 : 996
+//     7168 / 2048 x 256 + shared  256 8222 : 8616, 500 14097 : 14535, 750 20305 : 20791, 1024 26879 : 26662
+//   FP8, gated pass (sl : ll)
+//     1024 / 256 x 256  40 95 : 94, 64 107 : 102;  1536 / 512 x 128  72 112 : 105, 160 166 : 160;  1792 / 1024 x 128  72 182 : 181,
+//                       160 273 : 288, 300 416 : 413
+//     2048 / 768 x 128  72 168 : 169, 96 182 : 179, 120 209 : 197, 160 250 : 254, 220 292 : 279;  x 512  24 464 : 514, 48 519 :
+//                560, 72 573 : 596, 96 628 : 632, 300 1417 : 1437;  2048 / 256 x 128  80 106 : 99, 160 154 : 143
+//     2560 / 1024 x 256  96 481 : 480, 128 569 : 607, 180 714 : 770;  2560 / 1536 x 128  250 634 : 659, 350 842 : 793
+//     4096 / 1536 x 128  320 1101 : 1179, 1000 2821 : 2926;  7168 / 2048 x 256 + shared  256 4681 : 5073, 1024 14100 : 14878;
+//     few features: 2560 / 768 x 64  140 157 : 157, 250 209 : 199;  3072 / 768 x 128  160 343 : 368, 250 438 : 436, 400 634 : 665;
+//                       4096 / 512 x 128  160 339 : 357, 200 378 : 375;  x 32  260 144 : 140, 800 331 : 316
+//   FP8, down pass (ss : sl)
+//     2560 / 1024 x 512  64 860 : 871, 96 972 : 960, 140 1208 : 1261, 180 1414 : 1429, 220 1678 : 1558;  x 128  96 261 : 256, 160
+//                360 : 352;  2560 / 1536 x 128  72 327 : 330, 112 383 : 378, 160 481 : 490, 200 558 : 538
+//     7168 / 2048 x 256 + shared  256 4603 : 4681, 384 6227 : 6163, 750 11352 : 10958
+constexpr int kMinGatedK = 640, kShortGatedK = 1152;               // bf16 gated pass
+constexpr int kMinDownK = 640, kMidDownK = 960, kLongDownK = 2048;  // down pass
+constexpr int kFp8ShortGatedK = 1792, kFp8MidGatedK = 2432, kFp8LongGatedK = 3584, kFp8FewFeatures = 1024;
+
+inline bool small_m_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t rows, int64_t E, int ctas) {
+  const auto up_to = [&](int64_t r) { return rows <= r * E; };
+  // the small-M kernel's tiles, in half waves of the grid; of fewer than one and a half waves half the second is idle, which
+  // 128-row tiles fill
+  const int64_t chunks = (rows + 255) / 256 > E ? (rows + 255) / 256 : E, feat_per_tile = gated ? 128 : 256;
+  const int64_t half_waves = 2 * chunks * ((n_feat + feat_per_tile - 1) / feat_per_tile) / ctas;
+  if (half_waves < 3) return false;
+  if (gated && !fp8) return K >= kShortGatedK || (K >= kMinGatedK && (up_to(64) || half_waves >= 8));
+  if (gated) {
+    if (K < kFp8MidGatedK) return K >= kFp8ShortGatedK && up_to(64);
+    return n_feat < kFp8FewFeatures ? up_to(200) : K >= kFp8LongGatedK || up_to(300);
+  }
+  if (fp8) return K >= kLongDownK ? up_to(400) : K >= kMidDownK && up_to(180);
+  if (K >= kLongDownK) return true;
+  if (K >= kMidDownK) return up_to(350);
+  return K >= kMinDownK && (up_to(64) || (!up_to(120) && up_to(190)));
+}
+
 }  // namespace moe

@@ -34,3 +34,24 @@ def test_layout_reads_stay_linear_in_the_batch(rules):
         assert chunks * E <= max(1, -(-n // 256)) * E
         assert chunks <= 148 or chunk < 4096, (n, E, chunk)
         assert chunks ** 2 * E * 4 <= 148 ** 2 * 1024 * 4
+
+
+@pytest.mark.parametrize("fp8,gated,K,n_feat,E,R,small", [
+    # whole steps of which one side was measured at least 2 % faster, per pass (csrc/rules.h has the times)
+    (0, 1, 512, 2048, 8, 1100, 0), (0, 1, 768, 512, 128, 100, 0), (0, 1, 1024, 512, 64, 192, 0), (0, 1, 1024, 512, 64, 400, 0),
+    (0, 1, 1024, 512, 512, 24, 1), (0, 1, 1024, 512, 512, 160, 1), (0, 1, 1024, 256, 256, 40, 1), (0, 1, 1024, 256, 256, 300, 1),
+    (0, 1, 1280, 768, 128, 160, 1), (0, 1, 1536, 512, 128, 300, 1), (0, 1, 2048, 768, 128, 72, 1), (0, 1, 2048, 768, 128, 144, 1),
+    (0, 1, 2048, 768, 512, 24, 1), (0, 1, 2048, 768, 512, 48, 1), (0, 1, 2048, 768, 512, 96, 1), (0, 1, 2048, 768, 512, 160, 1),
+    (0, 1, 2048, 768, 4, 2100, 0), (0, 1, 7168, 512, 8, 1100, 0), (0, 1, 7168, 512, 8, 2000, 1),
+    (0, 1, 7168, 2048, 256, 750, 1), (0, 1, 7168, 2048, 256, 1500, 1),
+    (0, 0, 256, 2048, 128, 160, 0), (0, 0, 512, 1536, 128, 200, 0), (0, 0, 512, 1024, 64, 192, 0), (0, 0, 768, 2048, 128, 144, 1),
+    (0, 0, 768, 2048, 512, 48, 1), (0, 0, 768, 2048, 128, 200, 0), (0, 0, 1024, 1792, 128, 160, 1), (0, 0, 1024, 1792, 128, 600, 0),
+    (0, 0, 2048, 7168, 256, 256, 1), (0, 0, 2048, 512, 8, 1100, 0),
+    (1, 1, 1024, 256, 256, 64, 0), (1, 1, 1536, 512, 128, 72, 0), (1, 1, 2048, 768, 128, 120, 0), (1, 1, 2048, 768, 128, 220, 0),
+    (1, 1, 2048, 768, 512, 24, 1), (1, 1, 2048, 768, 512, 48, 1), (1, 1, 2048, 256, 128, 80, 0), (1, 1, 2560, 1536, 128, 250, 1),
+    (1, 1, 2560, 1536, 128, 350, 0), (1, 1, 4096, 1536, 128, 600, 1), (1, 1, 7168, 2048, 256, 1024, 1), (1, 1, 3072, 768, 128, 160, 1),
+    (1, 1, 2560, 768, 64, 250, 0), (1, 1, 4096, 512, 128, 160, 1), (1, 1, 4096, 512, 32, 800, 0), (1, 1, 7168, 512, 8, 1100, 0),
+    (1, 0, 1024, 2560, 512, 140, 1), (1, 0, 1024, 2560, 512, 220, 0), (1, 0, 1536, 2560, 128, 200, 0), (1, 0, 2048, 7168, 256, 750, 0),
+])
+def test_the_kernel_that_was_measured_faster_is_chosen(rules, fp8, gated, K, n_feat, E, R, small):
+    assert rules(f"moe::small_m_is_faster({fp8}, {gated}, {K}, {n_feat}, {R * E}LL, {E}, 148)") == [small]
