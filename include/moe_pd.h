@@ -394,7 +394,8 @@ moe_status moe_layer_host_submit(moe_ctx* ctx, int32_t slot, const float* logits
 moe_status moe_layer_host_wait(moe_ctx* ctx, int32_t slot);
 
 /* Test/inspection only: device pointers into the buffer set of the step in progress (between steps: of
- * the step that finished last).  Rows
+ * the step that finished last; moe_layer_host may cut a batch into two chunks of tokens, and what it leaves is then that of
+ * the second).  Rows
  * [0, T*k) of x_perm [.,H], act [.,I], y_perm [.,H] and rows [0,T) of y_shared [.,H] are
  * defined after the respective stage.  Any out-pointer may be NULL. */
 moe_status moe_ctx_debug_ptrs(moe_ctx* ctx, void** x_perm, void** act, void** y_perm, void** y_shared,
