@@ -71,11 +71,10 @@ constexpr int kXMaps = 16;                              // token-row boxes of 16
 constexpr uint32_t kTmemCols = 512;
 constexpr int kQ = 4;                                   // entries of the CTA's tile queue
 // Waves' worth of tiles, at the list's end, that are handed out dynamically: a fifth of them, between two and six.  Over
-// tens of waves the CTAs drift apart by more than two tiles (V3-shaped decode, 28 and 49 waves: six against two waves
-// 2111 -> 2089 us with 64 tokens, with FP8 weights and 128 tokens 1332 -> 1313 us on one GPU; on another that runs the same
-// steps in 2146 and 1355 us no difference); a launch of five waves, or one whose tiles
-// share weights through L2 while the CTAs are in step, wants two (37 tokens, 5 waves: 177.0 against 177.3 us; all but the
-// first wave dynamic: 8192-token Qwen3-shaped prefill 732 -> 742 us).
+// tens of waves the CTAs drift apart by more than two tiles (V3-shaped decode, 28 and 49 waves: 2089 us with six, 2111 with
+// two, 64 tokens; FP8 weights, 128 tokens 1313 and 1332; level on a GPU that runs these steps in 2146 and 1355 us); a launch
+// of five waves, or one whose tiles share weights through L2 while the CTAs are in step, wants two (8192-token Qwen3-shaped
+// prefill 732 us; 742 with all but the first wave dynamic).
 constexpr int kMinDynWaves = 2, kMaxDynWaves = 6, kDynWavesOneIn = 5;
 
 struct StreamParams {
@@ -257,8 +256,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   // The tile list: experts by size class, largest first, ascending index within a class.  A stable counting sort --
   // counts per class by shared-memory atomics, a scan over the classes, then one warp places 32 experts at a time and
   // ranks equals by __match_any_sync -- because every CTA of every launch builds the list before its first copy.
-  // (Ranking each expert against all others, one shared-memory read per pair: a decode step of 24 tokens over 512
-  // experts took 403 us, 384 us now; 37 tokens over 128 experts 186.2 -> 184.0 us; 64 over 256 2161 -> 2152 us.)
+  // (24 tokens over 512 experts 384 us a step; 403 when each expert was ranked against all others, a shared-memory read per
+  // pair; 37 over 128 184.0 and 186.2, 64 over 256 2152 and 2161.)
   if (p.sort_tiles)
     for (int c = threadIdx.x; c < kSizeClasses; c += kThreads) class_pos[c] = 0;
   __syncthreads();
@@ -698,8 +697,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         for (int m = 0; m < 8; ++m) {
           const int c = c_first + m * c_step;
           // Leave, do not skip chunk by chunk: the unrolled chunks are kilobytes of code that a launch of small tiles would
-          // fetch from a cold instruction cache just to jump over them (tiny layer, 64 tokens: 28.5 -> 26.2 us a step,
-          // one-token V3-shaped decode 143.1 -> 138.1 us).
+          // fetch from a cold instruction cache just to jump over them: 2 to 5 us a step (one-token V3-shaped decode 138.1
+          // us leaving, 143.1 skipping).
           if (c >= t.rows) break;
           {
             float g[16], u[16];
@@ -1004,7 +1003,7 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
     tiles += (int64_t)((dense->rows + kMaxTileRows - 1) / kMaxTileRows) * prm.n_ft2;
   int grid = (int)(tiles < (int64_t)max_ctas ? tiles : (int64_t)max_ctas);
   if (grid < 1) grid = 1;
-  // one tile per CTA at most: any order will do (with the short epilogue, the tiny layer's 64-token step 25.5 -> 24.2 us)
+  // one tile per CTA at most: any order will do (1.3 us of the tiny layer's 64-token step)
   if (tiles <= (int64_t)grid) prm.sort_tiles = 0;
   const bool overlap = p.rows_bound <= kGemmOverlapMaxRows;
   cudaError_t err;

@@ -9,8 +9,8 @@ namespace moe {
 // Raises a kernel's dynamic shared-memory limit once per kernel, device and size, so that steady-state launches
 // make no driver calls besides the launch itself (which also keeps them legal while a stream is being captured).
 // The first time it also asks for the largest shared-memory carve-out, which the GEMM kernels need: an SM that one of the
-// small kernels left with more L1 has to drain before it can be divided anew (tiny layer, 64 tokens 23.9 -> 23.8 us a step;
-// one-token V3-shaped decode 134.2 -> 133.6 us).
+// small kernels left with more L1 has to drain before it can be divided anew (one-token V3-shaped decode 133.6 us a step
+// with it, 134.2 without).
 cudaError_t ensure_dynamic_smem_impl(const void* kern, size_t bytes);
 template <typename Kernel>
 inline cudaError_t ensure_dynamic_smem(Kernel kern, size_t bytes) {
@@ -61,11 +61,9 @@ inline cudaError_t launch_pdl(bool allow_overlap, void (*kern)(KArgs...), dim3 g
                               cudaStream_t stream, Args&&... args) {
   return launch_pdl_clusters(allow_overlap, 1, kern, grid, block, smem, stream, static_cast<KArgs>(args)...);
 }
-// The GEMM kernels take the overlap only for problems of up to this many rows: measured on a B200, a step of a
-// few hundred microseconds gains 7 % from it (six launch latencies and prologues hidden), while steps of several
-// milliseconds LOSE 1.5-5 % when their GEMM launches carry the attribute (the small kernels keep it at every size;
-// re-measured in the sustained regime with the small-M kernel's early set-up: a limit of 32768 rows or none at all
-// changes nothing on the weight-streaming workloads and costs 3-6 % on the tensor-bound one).
+// The GEMM kernels take the overlap only for problems of up to this many rows: a step of a few hundred microseconds gains
+// 7 % from it (six launch latencies and prologues hidden), while a limit of 32768 rows or none at all changes nothing on the
+// weight-streaming workloads and costs 3-6 % on the tensor-bound one (the small kernels keep it at every size).
 #ifndef MOE_GEMM_OVERLAP_MAX_ROWS
 #define MOE_GEMM_OVERLAP_MAX_ROWS 8192
 #endif
@@ -112,8 +110,7 @@ cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32
 
 // Tensor maps of one small-M GEMM launch (host memory, opaque outside gemm_stream.cu).  A context keeps one plan per
 // buffer set and pass; a launch whose operands (addresses and shapes) are the plan's re-encodes nothing.  (Looking 34
-// maps up per launch in a locked table cost 3.4 us of host time; with that, an event record per call and four calls from
-// Python a 64-token step of the tiny layer took 36.4 us, all of it host time; 28.3 us now, bound by the GPU.)
+// maps up per launch in a locked table costs 3.4 us of host time, in steps that take the GPU 20.)
 struct StreamPlan;
 StreamPlan* stream_plan_create();
 void stream_plan_destroy(StreamPlan* plan);

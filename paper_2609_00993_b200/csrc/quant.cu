@@ -12,9 +12,9 @@
 // pieces for every row a quarter to three quarters of them handled pieces that are not there.
 // The quantised row may go to several places: MOVE writes it to its k destination rows of the dispatch (k n bytes) and,
 // when the shared expert needs it, in token order too -- from registers, so that no second kernel reads it back.
-// Against eight 8-element vectors a thread for every row and a row movement of its own, FP8 steps: Qwen3-shaped layer
-// T = 6007 quantising x and moving it 37.8 -> 25.1 us, quantising the activation 35.0 -> 22.9 us; T = 1500 184.3 -> 177.9 us
-// a step; hidden 2560, 512 experts, T = 20000 164 -> 93 and 125 -> 79 us, 2162 -> 2124 us a step.
+// Bound by HBM on long steps: hidden 2560, 512 experts, T = 20000 moves x in 93 us (164 with eight 8-element vectors a
+// thread for every row and a row movement of its own) and quantises the activation in 79 (125); Qwen3-shaped layer,
+// T = 6007 25.1 (37.8) and 22.9 (35.0).
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
@@ -42,7 +42,7 @@ __device__ __forceinline__ uint32_t quantize4(uint32_t w0, uint32_t w1, float in
 // n_pieces: 16-element pieces of a row.  MOVE: row's codes also go to rows inv_perm[row * k + j], j < k, of q_perm
 // (negative: dropped), its scale to the same places of scale_perm; q / scale may then be nullptr.
 // A second set of rows of the same length (x2, rows2 of them -> q2, scale2) may ride in the launch, behind the first: the
-// shared expert's activation in a launch of its own cost 4 us a step (V3-shaped FP8 decode, one token 90.0 -> 85.8 us).
+// shared expert's activation in a launch of its own costs 4 us a step (V3-shaped FP8 decode, one token 90.0 against 85.8 us).
 template <int ROW_WARPS, int NP, bool MOVE>
 __global__ void __launch_bounds__(kQuantThreads)
 quantize_rows_kernel(const uint4* __restrict__ x, long long rows, int n_pieces, uint4* __restrict__ q,

@@ -4,11 +4,13 @@
 // L2, or from 17 tokens on a cluster shares the work and hands the expert indices round through distributed shared memory.
 // It then finds the positions of its own token's slots by counting (no scan, no round trip), and copies its piece of that
 // token's row, which it has loaded meanwhile.
-// Measured as whole steps, against the three launches (us): 8 experts, 2 of them, 256 features: 1 token 24.1 -> 21.1,
-// 16 24.6 -> 21.6, 64 24.5 -> 22.6; 128 experts, 8 of them, 2048 features: 1 token 36.8 -> 34.9, 16 135.4 -> 133.2, 37
-// 182.2 -> 180.8, 64 200.9 -> 199.4; 512 experts, 8 of them: 1 token 33.4 -> 31.2, 32 85.1 -> 82.0.
-// (In one CTA, two tokens a warp at 64: 24.5 -> 23.9 and 200.9 -> 201.3.  128 tokens over a cluster: 25.2 -> 23.9 with 8
-// experts but 206.1 -> 207.6 with 128, so 64 is the limit.)
+// Whole steps, this launch | the three, us: 8 experts, 2 of them, 256 features: 1 token 21.1 | 24.1, 16 21.6 | 24.6, 64
+// 22.6 | 24.5; 128 experts, 8 of them, 2048 features: 1 token 34.9 | 36.8, 16 133.2 | 135.4, 37 180.8 | 182.2, 64 199.4 |
+// 200.9; 512 experts, 8 of them: 1 token 31.2 | 33.4, 32 82.0 | 85.1.
+// (In one CTA, two tokens a warp at 64: 23.9 | 24.5 and 201.3 | 200.9.  128 tokens over a cluster: 23.9 | 25.2 with 8
+// experts but 207.6 | 206.1 with 128, so 64 is the limit.)
+// Beside another phase without SM budgets the clusters of 8 start as soon as the three launches did: decode steps of 64
+// tokens beside back-to-back V3-shaped prefill of 4096 take 3.35 ms on average, 3.55 in a build that makes three launches.
 #include "kernels.h"
 #include "routing.cuh"
 
