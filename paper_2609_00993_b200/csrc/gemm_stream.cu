@@ -46,22 +46,16 @@ namespace {
 
 using namespace tc;
 
-#ifndef MOE_STREAM_ISSUERS
-#define MOE_STREAM_ISSUERS 1
-#endif
 #ifndef MOE_STREAM_EPI_WARPS
 #define MOE_STREAM_EPI_WARPS 8
 #endif
-// MMA-issuing threads: one for both weight boxes (1) or one per box (2).  Two were measured and are no faster:
-// what the issuer waits for is the tensor pipe, which in turn waits for shared-memory bandwidth.
-constexpr int kIssuers = MOE_STREAM_ISSUERS;
 // Epilogue warps: 4 (each owns 32 TMEM lanes = 32 weight rows) or 8 (two warps per lane group, one taking the
 // even and one the odd 16-token chunks), which halves the time a tile of more than 128 tokens keeps the MMA
 // issuer waiting for its single accumulator.
 constexpr int kEpilogueWarps = MOE_STREAM_EPI_WARPS;
 constexpr int kProducerWarp = kEpilogueWarps;
-constexpr int kMmaWarp = kEpilogueWarps + 1;  // issuer of box 0 and TMEM owner; the next warp issues box 1 when kIssuers == 2
-constexpr int kThreads = 32 * (kEpilogueWarps + 1 + kIssuers);
+constexpr int kMmaWarp = kEpilogueWarps + 1;
+constexpr int kThreads = 32 * (kEpilogueWarps + 2);
 constexpr int kSizeClasses = 256;     // classes of expert size the tile list is ordered by
 constexpr int kSlotBytes = 2048;                        // ring granularity: 16 token rows of one k-block
 constexpr int kWSlots = 2 * kWBoxBytes / kSlotBytes;    // 16 slots: the two weight boxes
@@ -132,10 +126,12 @@ struct StreamMaps {
   CUtensorMap x[kXMaps], x2[kXMaps];  // token rows, boxes of 16, 32, ..., 256 rows (x2: the dense group's)
 };
 
-struct STile {
-  int e, row0, rows, ft;
-  bool dense;
+// A tile as the producer hands it to the other roles: one entry of the CTA's queue.
+struct __align__(16) STile {
+  int e;  // expert; kDenseTile: a tile of the dense group; kNoTile: no more tiles
+  int row0, rows, ft;
 };
+constexpr int kDenseTile = -1, kNoTile = -2;
 
 // An expert's (or the dense group's) rows in ceil(cnt / 256) chunks of equal size, rounded up to 16.
 __device__ __forceinline__ void chunking(int cnt, int& tiles, int& chunk) {
@@ -151,37 +147,39 @@ __device__ __forceinline__ int size_class(int cnt) {
   return kSizeClasses - 1 - (16 + (msb - 4) * 8 + (int)((u >> (msb - 3)) & 7u));
 }
 
-// tile -> (expert, first row, valid rows, feature tile).  The dense group's tiles come first (chunk major),
+// tile -> (expert, first row, valid rows, feature tile), by a whole warp.  The dense group's tiles come first (chunk major),
 // then the experts' in the order `order` (largest first): prefix[i] = chunks of the experts at positions < i.
-__device__ __forceinline__ STile decode_tile(int tile, int dense_tiles, int n_ft2, int rows2, int n_ft, int ft0, int E,
-                                             const int* prefix, const int* order, const int* beg, const int* cnts) {
+__device__ __forceinline__ STile decode_tile(int tile, int dense_tiles, const StreamParams& p, const int* prefix,
+                                             const int* order, const int* beg, const int* cnts) {
   STile t;
   int tiles, chunk;
   if (tile < dense_tiles) {
-    const int rt = tile / n_ft2;
-    chunking(rows2, tiles, chunk);
-    t.e = 0;
-    t.ft = ft0 + tile - rt * n_ft2;
+    const int rt = tile / p.n_ft2;
+    chunking(p.rows2, tiles, chunk);
+    t.e = kDenseTile;
+    t.ft = p.ft0 + tile - rt * p.n_ft2;
     t.row0 = rt * chunk;
-    t.rows = min(chunk, rows2 - t.row0);
-    t.dense = true;
+    t.rows = min(chunk, p.rows2 - t.row0);
     return t;
   }
   tile -= dense_tiles;
-  const int rt = tile / n_ft;
-  int lo = 0, hi = E;  // largest position in [0,E) with prefix[position] <= rt
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (prefix[mid] <= rt) lo = mid; else hi = mid;
+  const int rt = tile / p.n_ft;
+  // largest position in [0,E) with prefix[position] <= rt: 32 places at a time
+  int lo = 0;
+  for (int span = p.E; span > 1;) {
+    const int step = (span + 31) >> 5, at = lo + (int)(threadIdx.x & 31) * step;
+    const unsigned below = __ballot_sync(0xffffffffu, at < lo + span && prefix[at] <= rt);
+    const int skip = (__popc(below) - 1) * step;
+    lo += skip;
+    span = min(step, span - skip);
   }
   const int e = order[lo], cnt = cnts[e];
   chunking(cnt, tiles, chunk);
   const int mt = rt - prefix[lo];
   t.e = e;
-  t.ft = ft0 + tile - rt * n_ft;
+  t.ft = p.ft0 + tile - rt * p.n_ft;
   t.row0 = beg[e] + mt * chunk;
   t.rows = min(chunk, cnt - mt * chunk);
-  t.dense = false;
   return t;
 }
 
@@ -191,8 +189,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
                            const __grid_constant__ StreamMaps xmaps, const __grid_constant__ StreamParams p) {
   constexpr int kbk = FP8 ? 2 * kBlockK : kBlockK;  // K elements per k-block
   extern __shared__ uint8_t smem_raw[];
-  // carve: ring (ring_slots x 2 KB) | full[kNB] empty[kNB] tfull[2] tempty[2] tqfull[kQ] tqempty[kQ] | tmem slot
-  //        | abort | stopped | sizes[kNB] | tq[kQ] | prefix[E+1] | order[E] | beg[E] | cnts[E] | classes | chunk sums
+  // carve: ring (ring_slots x 2 KB) | full[kNB] empty[kNB] tfull[2] tempty[2] tqfull[kQ] tqempty[kQ] | tq[kQ] | tmem slot
+  //        | abort | stopped | sizes[kNB] | prefix[E+1] | order[E] | beg[E] | cnts[E] | classes | chunk sums
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base_addr = (raw_addr + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (base_addr - raw_addr);
@@ -203,12 +201,13 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   const uint32_t bar_tempty = bar_tfull + 16u;
   const uint32_t bar_tqfull = bar_tempty + 16u;         // the tile queue: an entry has been published
   const uint32_t bar_tqempty = bar_tqfull + 8u * kQ;    // ... and read by the issuer and every epilogue warp
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kNB + 4 + 2 * kQ);
+  static_assert((2 * kNB + 4 + 2 * kQ) % 2 == 0, "the queue's entries are 16-byte aligned");
+  STile* tq = reinterpret_cast<STile*>(bars + 2 * kNB + 4 + 2 * kQ);  // tile queue
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tq + kQ);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* stopped_here = reinterpret_cast<volatile int*>(tmem_slot + 2);  // the producer stopped on request
   int* sizes = reinterpret_cast<int*>(tmem_slot + 3);  // slots held by the k-blocks in flight (producer only)
-  volatile int* tq = reinterpret_cast<volatile int*>(sizes + kNB);  // tile queue entries (-1: no more tiles)
-  int* prefix = sizes + kNB + kQ;
+  int* prefix = sizes + kNB;
   int* order = prefix + (p.E + 1);
   int* beg = order + p.E;
   int* cnts = beg + p.E;
@@ -219,9 +218,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   [[maybe_unused]] const int unit = (int)blockIdx.x;
   if (threadIdx.x == 0) PROF_STAMP(0);
   constexpr int kFeatPerTile = GATED ? 128 : 256;
-  const int n_ft = p.n_ft, n_ft2 = p.n_ft2;
   const int num_kb1 = (p.K + kbk - 1) / kbk, num_kb2 = (p.K2 + kbk - 1) / kbk;
-  const int dense_tiles = p.rows2 > 0 ? ((p.rows2 + kMaxTileRows - 1) / kMaxTileRows) * n_ft2 : 0;
+  const int dense_tiles = p.rows2 > 0 ? ((p.rows2 + kMaxTileRows - 1) / kMaxTileRows) * p.n_ft2 : 0;
   const unsigned long long limit = p.wait_limit_ns;
 
   // ---- set-up: barriers and TMEM (before the previous kernel of the stream is known to be complete), then the
@@ -229,15 +227,15 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   if (threadIdx.x == 32 * kProducerWarp) {
     for (int s = 0; s < kNB; ++s) {
       mbar_init(bar_full + 8u * s, 1);
-      mbar_init(bar_empty + 8u * s, kIssuers);
+      mbar_init(bar_empty + 8u * s, 1);
     }
     for (int a = 0; a < 2; ++a) {
-      mbar_init(bar_tfull + 8u * a, kIssuers);
+      mbar_init(bar_tfull + 8u * a, 1);
       mbar_init(bar_tempty + 8u * a, kEpilogueWarps);
     }
     for (int q = 0; q < kQ; ++q) {
       mbar_init(bar_tqfull + 8u * q, 1);
-      mbar_init(bar_tqempty + 8u * q, kIssuers + kEpilogueWarps);
+      mbar_init(bar_tqempty + 8u * q, 1 + kEpilogueWarps);
     }
     *abort_flag = 0;
     *stopped_here = 0;
@@ -333,12 +331,12 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   if (threadIdx.x == 0) PROF_STAMP(2);
-  const int total_tiles = dense_tiles + prefix[p.E] * n_ft;
+  const int total_tiles = dense_tiles + prefix[p.E] * p.n_ft;
   const uint32_t R = (uint32_t)p.ring_slots;
 
   if (warp == kProducerWarp) {
-    // ================================================================= TMA producer (one lane)
-    if (lane == 0 && !p.inject_producer_stall) {
+    // ================================================================= TMA producer
+    if (!p.inject_producer_stall) {
       uint32_t head = 0, free_slots = R, kb_idx = 0, oldest = 0;
       bool ok = true;
       // Early set-up: until this thread has waited for the previous kernel, token-row copies are put off (their
@@ -358,7 +356,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
           if (h + (uint32_t)kWSlots > R) h = 0;
           h += (uint32_t)kWSlots;
           if (h + def_nx > R) h = 0;
-          tma_load_2d(base_addr + h * (uint32_t)kSlotBytes, def_map, bar_full + 8u * i, (int)i * kbk, def_row0);
+          if (elect_one())
+            tma_load_2d(base_addr + h * (uint32_t)kSlotBytes, def_map, bar_full + 8u * i, (int)i * kbk, def_row0);
           h += def_nx;
         }
       };
@@ -369,19 +368,22 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(yield_seen) : "l"(p.yield_req) : "memory");
       // Tiles are handed out by a counter in device memory, in the list's order (largest experts first): a CTA
       // that finishes early takes the next tile, whichever CTA would have had it.  The producer publishes every tile
-      // it takes -- and finally -1 -- in a small queue that the issuer and the epilogue warps follow.
+      // it takes -- and finally that there are no more -- in a small queue that the issuer and the epilogue warps follow.
       uint32_t tcount = 0;
-      auto publish = [&](int tile) -> bool {
+      auto publish = [&](const STile& t) -> bool {
         const uint32_t q = tcount % kQ, par = ((tcount / kQ) & 1u) ^ 1u;
         // the epilogue warps free an entry only after the tile before it, which needs its token rows: the copies
-        // put off by the early set-up go out before this thread blocks
-        if (!dep_waited && !mbar_try_wait(bar_tqempty + 8u * q, par)) dep_wait_and_flush();
-        if (!mbar_wait(bar_tqempty + 8u * q, par, abort_flag, limit)) return false;
-        tq[q] = tile;
-        mbar_arrive(bar_tqfull + 8u * q);
+        // put off by the early set-up go out before this warp blocks
+        if (!dep_waited && !__all_sync(0xffffffffu, mbar_try_wait(bar_tqempty + 8u * q, par))) dep_wait_and_flush();
+        if (!mbar_wait_warp(bar_tqempty + 8u * q, par, abort_flag, limit)) return false;
+        if (elect_one()) {
+          tq[q] = t;
+          mbar_arrive(bar_tqfull + 8u * q);
+        }
         ++tcount;
         return true;
       };
+      const STile no_more{kNoTile, 0, 0, 0};
       // The counter is read a few k-blocks before the current tile's last copy, so that the atomic's round trip hides
       // behind those copies -- and no earlier, so that a CTA does not hold a second tile while another CTA has none.
       // A stop on request therefore takes effect after the tile that had already been taken.
@@ -400,24 +402,25 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
           const int w = sw++;
           return w * grid + ((w & 1) ? grid - 1 - (int)blockIdx.x : (int)blockIdx.x);
         }
-        return w_static * grid + atomicAdd(p.tile_ctr, 1);
+        return lane == 0 ? w_static * grid + atomicAdd(p.tile_ctr, 1) : 0;
       };
-      int taken = next_tile();
+      int taken = next_tile();  // lane 0's counts
       for (;;) {
-        const int tile = taken < total_tiles ? taken : -1;
-        if (!publish(tile)) {
+        const int tile = __shfl_sync(0xffffffffu, taken, 0);
+        const STile t = tile < total_tiles ? decode_tile(tile, dense_tiles, p, prefix, order, beg, cnts) : no_more;
+        if (!publish(t)) {
           ok = false;
           break;
         }
-        if (tile < 0) break;
+        if (t.e == kNoTile) break;
+        const bool dense = t.e == kDenseTile;
         bool stop_after = false;
-        const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, order, beg, cnts);
         const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
         const int w_row0 = t.ft * kFeatPerTile;
-        const CUtensorMap* mw = t.dense ? &map_w2 : &map_w;
-        const CUtensorMap* mx = (t.dense ? xmaps.x2 : xmaps.x) + ((n >> 4) - 1u);  // the box of exactly n rows
-        const int w_e = t.dense ? 0 : p.e_base + t.e;
-        const int num_kb = t.dense ? num_kb2 : num_kb1;
+        const CUtensorMap* mw = dense ? &map_w2 : &map_w;
+        const CUtensorMap* mx = (dense ? xmaps.x2 : xmaps.x) + ((n >> 4) - 1u);  // the box of exactly n rows
+        const int w_e = dense ? 0 : p.e_base + t.e;
+        const int num_kb = dense ? num_kb2 : num_kb1;
         const int fetch_kb = num_kb > 4 ? num_kb - 4 : 0;
         if (!dep_waited) {
           def_nx = n >> 4;
@@ -429,7 +432,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
             if (p.yield_req != nullptr) {
               // the request word was read a tile ago, so looking at it here does not stall the pipeline; the read for
               // the next tile goes out now
-              stop_after = yield_seen != 0;
+              stop_after = __shfl_sync(0xffffffffu, yield_seen, 0) != 0;
               asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(yield_seen) : "l"(p.yield_req) : "memory");
             }
             if (!stop_after) taken = next_tile();
@@ -450,7 +453,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
               dep_wait_and_flush();
             while (free_slots < need || (count_limit && kb_idx - oldest >= (uint32_t)kNB)) {
               PROF_T0();
-              const bool got = mbar_wait(bar_empty + 8u * (oldest % kNB), (oldest / kNB) & 1u, abort_flag, limit);
+              const bool got = mbar_wait_warp(bar_empty + 8u * (oldest % kNB), (oldest / kNB) & 1u, abort_flag, limit);
               PROF_ADD(prof_wait_empty);
               if (!got) return false;
               free_slots += (uint32_t)sizes[oldest % kNB];
@@ -461,17 +464,19 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
           if (!reclaim((uint32_t)kWSlots + pad_w, true)) { ok = false; break; }
           free_slots -= (uint32_t)kWSlots + pad_w;
           const uint32_t full = bar_full + 8u * (kb_idx % kNB);
-          mbar_expect_tx(full, 2u * kWBoxBytes + n * 128u);
           // one copy per operand: both weight boxes (gated: the map's third dimension steps from the gate rows
           // to the up rows; down pass: 256 consecutive rows), then the n token rows
           const uint32_t st_w = base_addr + head_w * (uint32_t)kSlotBytes;
-          if (GATED) tma_load_4d(st_w, mw, full, k0, w_row0, 0, w_e);
-          else tma_load_3d(st_w, mw, full, k0, w_row0, w_e);
+          if (elect_one()) {
+            mbar_expect_tx(full, 2u * kWBoxBytes + n * 128u);
+            if (GATED) tma_load_4d(st_w, mw, full, k0, w_row0, 0, w_e);
+            else tma_load_3d(st_w, mw, full, k0, w_row0, w_e);
+          }
           if (!reclaim(nx + pad_x, false)) { ok = false; break; }
           free_slots -= nx + pad_x;
           sizes[kb_idx % kNB] = (int)((uint32_t)kWSlots + pad_w + nx + pad_x);
           if (dep_waited) {
-            tma_load_2d(base_addr + head_x * (uint32_t)kSlotBytes, mx, full, k0, t.row0);
+            if (elect_one()) tma_load_2d(base_addr + head_x * (uint32_t)kSlotBytes, mx, full, k0, t.row0);
           } else {
             ++n_def;
           }
@@ -482,26 +487,25 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         if (!dep_waited) dep_wait_and_flush();
         if (stop_after && ok) {
           *stopped_here = 1;  // no further tile is taken: the other roles finish the published ones and leave
-          if (!publish(-1)) ok = false;
+          if (!publish(no_more)) ok = false;
           break;
         }
       }
       if (!dep_waited) dep_wait_and_flush();
-      if (!ok) {
+      if (!ok && lane == 0) {
         *abort_flag = 1;
         atomicCAS(p.status, kStOk, kStTimeout);
       }
 #ifdef MOE_STREAM_PROF
-      atomicAdd(&g_stream_prof[8 * unit + 0], (unsigned long long)(clock64() - prof_start));
-      atomicAdd(&g_stream_prof[8 * unit + 1], (unsigned long long)prof_wait_empty);
+      if (lane == 0) {
+        atomicAdd(&g_stream_prof[8 * unit + 0], (unsigned long long)(clock64() - prof_start));
+        atomicAdd(&g_stream_prof[8 * unit + 1], (unsigned long long)prof_wait_empty);
+      }
 #endif
     }
   } else if (warp >= kMmaWarp) {
-    // ================================================================= MMA issuer(s) (one lane each)
-    // With two issuers, warp 5 multiplies weight box 0 into accumulator a and warp 6 box 1 into accumulator b;
-    // both wait on the same barriers, and every barrier they signal counts one arrival from each.
-    const bool do_a = kIssuers == 1 || warp == kMmaWarp, do_b = kIssuers == 1 || warp != kMmaWarp;
-    if (lane == 0) {
+    // ================================================================= MMA issuer
+    {
       uint32_t head = 0, kb_idx = 0, use0 = 0, use1 = 0, next_half = 0;
       bool ok = true;
       [[maybe_unused]] long long prof_wait_full = 0, prof_wait_acc = 0, prof_tiles = 0;
@@ -512,28 +516,28 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       uint32_t tcount = 0;
       for (;;) {
         const uint32_t q = tcount % kQ;
-        if (!mbar_wait(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) {
+        if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) {
           ok = false;
           break;
         }
-        const int tile = tq[q];
-        mbar_arrive(bar_tqempty + 8u * q);
+        const STile t = tq[q];
+        __syncwarp();
+        if (elect_one()) mbar_arrive(bar_tqempty + 8u * q);
         ++tcount;
-        if (tile < 0) break;
-        const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, order, beg, cnts);
+        if (t.e == kNoTile) break;
         const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
         const bool big = n > 128u;
         uint32_t d_a, d_b;
         PROF_T0();
         if (big) {
-          if (!mbar_wait(bar_tempty, (use0 & 1u) ^ 1u, abort_flag, limit) ||
-              !mbar_wait(bar_tempty + 8u, (use1 & 1u) ^ 1u, abort_flag, limit)) { ok = false; break; }
+          if (!mbar_wait_warp(bar_tempty, (use0 & 1u) ^ 1u, abort_flag, limit) ||
+              !mbar_wait_warp(bar_tempty + 8u, (use1 & 1u) ^ 1u, abort_flag, limit)) { ok = false; break; }
           d_a = tmem_base;
           d_b = tmem_base + 256u;
         } else {
           const uint32_t h = next_half;
           next_half ^= 1u;
-          if (!mbar_wait(bar_tempty + 8u * h, ((h ? use1 : use0) & 1u) ^ 1u, abort_flag, limit)) { ok = false; break; }
+          if (!mbar_wait_warp(bar_tempty + 8u * h, ((h ? use1 : use0) & 1u) ^ 1u, abort_flag, limit)) { ok = false; break; }
           d_a = tmem_base + 256u * h;
           d_b = d_a + 128u;
           if (h) ++use1; else ++use0;
@@ -544,7 +548,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
 #endif
         tc_fence_after();
         const uint32_t idesc = FP8 ? umma_idesc_e4m3(128, n) : umma_idesc(128, n);
-        const int num_kb = t.dense ? num_kb2 : num_kb1;
+        const int num_kb = t.e == kDenseTile ? num_kb2 : num_kb1;
         for (int kb = 0; kb < num_kb; ++kb) {
           if (head + (uint32_t)kWSlots > R) head = 0;  // the producer's allocation, step for step
           const uint32_t pos_w = head;
@@ -554,51 +558,52 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
           head += n >> 4;
           {
             PROF_T0();
-            const bool got = mbar_wait(bar_full + 8u * (kb_idx % kNB), (kb_idx / kNB) & 1u, abort_flag, limit);
+            const bool got = mbar_wait_warp(bar_full + 8u * (kb_idx % kNB), (kb_idx / kNB) & 1u, abort_flag, limit);
             PROF_ADD(prof_wait_full);
             if (!got) { ok = false; break; }
           }
           if (kb_idx == 0) PROF_STAMP(3);
           tc_fence_after();
           const uint32_t lo_w0 = lo_base + pos_w * lo_slot, lo_w1 = lo_w0 + lo_box, lo_x = lo_base + pos_x * lo_slot;
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
-            const uint32_t adv = (uint32_t)((kk * kUmmaK * 2) >> 4);  // +32 bytes per MMA, in 16-byte units
-            const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
-            if (FP8) {
-              if (do_a) umma_e4m3_lo(d_a, lo_w0 + adv, lo_x + adv, desc_hi, idesc, acc);
-              if (do_b) umma_e4m3_lo(d_b, lo_w1 + adv, lo_x + adv, desc_hi, idesc, acc);
-            } else {
-              if (do_a) umma_bf16_lo(d_a, lo_w0 + adv, lo_x + adv, desc_hi, idesc, acc);
-              if (do_b) umma_bf16_lo(d_b, lo_w1 + adv, lo_x + adv, desc_hi, idesc, acc);
+            for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
+              const uint32_t adv = (uint32_t)((kk * kUmmaK * 2) >> 4);  // +32 bytes per MMA, in 16-byte units
+              const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
+              if (FP8) {
+                umma_e4m3_lo(d_a, lo_w0 + adv, lo_x + adv, desc_hi, idesc, acc);
+                umma_e4m3_lo(d_b, lo_w1 + adv, lo_x + adv, desc_hi, idesc, acc);
+              } else {
+                umma_bf16_lo(d_a, lo_w0 + adv, lo_x + adv, desc_hi, idesc, acc);
+                umma_bf16_lo(d_b, lo_w1 + adv, lo_x + adv, desc_hi, idesc, acc);
+              }
             }
+            umma_commit(bar_empty + 8u * (kb_idx % kNB));  // the k-block's slots are free once these MMAs have read them
           }
-          umma_commit(bar_empty + 8u * (kb_idx % kNB));  // the k-block's slots are free once these MMAs have read them
           ++kb_idx;
         }
         if (!ok) break;
+        if (elect_one()) {
+          umma_commit(bar_tfull + (big ? 0u : 8u * (next_half ^ 1u)));
+          if (big) umma_commit(bar_tfull + 8u);
+        }
         if (big) {
-          umma_commit(bar_tfull);
-          umma_commit(bar_tfull + 8u);
           ++use0;
           ++use1;
-        } else {
-          umma_commit(bar_tfull + 8u * (next_half ^ 1u));
         }
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         *abort_flag = 1;
         atomicCAS(p.status, kStOk, kStTimeout);
       }
       PROF_STAMP(4);
 #ifdef MOE_STREAM_PROF
-      if (warp == kMmaWarp)
-      atomicAdd(&g_stream_prof[8 * unit + 2], (unsigned long long)(clock64() - prof_start));
-      if (warp == kMmaWarp) {
-      atomicAdd(&g_stream_prof[8 * unit + 3], (unsigned long long)prof_wait_full);
-      atomicAdd(&g_stream_prof[8 * unit + 4], (unsigned long long)prof_wait_acc);
-      atomicAdd(&g_stream_prof[8 * unit + 5], (unsigned long long)prof_tiles);
-      atomicAdd(&g_stream_prof[8 * unit + 6], (unsigned long long)kb_idx);
+      if (lane == 0) {
+        atomicAdd(&g_stream_prof[8 * unit + 2], (unsigned long long)(clock64() - prof_start));
+        atomicAdd(&g_stream_prof[8 * unit + 3], (unsigned long long)prof_wait_full);
+        atomicAdd(&g_stream_prof[8 * unit + 4], (unsigned long long)prof_wait_acc);
+        atomicAdd(&g_stream_prof[8 * unit + 5], (unsigned long long)prof_tiles);
+        atomicAdd(&g_stream_prof[8 * unit + 6], (unsigned long long)kb_idx);
       }
 #endif
     }
@@ -623,12 +628,12 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         ok = false;
         break;
       }
-      const int tile = tq[q];
+      const STile t = tq[q];
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_tqempty + 8u * q);
       ++tcount;
-      if (tile < 0) break;
-      const STile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, order, beg, cnts);
+      if (t.e == kNoTile) break;
+      const bool dense = t.e == kDenseTile;
       const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
       const bool big = n > 128u;
       uint32_t h = 0, d_a, d_b;
@@ -650,16 +655,16 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       tc_fence_after();
       d_a += lane_base;
       d_b += lane_base;
-      __nv_bfloat16* const out = t.dense ? p.out2 : p.out;
-      const int n_feat = t.dense ? p.n_feat2 : p.n_feat;
+      __nv_bfloat16* const out = dense ? p.out2 : p.out;
+      const int n_feat = dense ? p.n_feat2 : p.n_feat;
       const int f_a = t.ft * kFeatPerTile + fl;  // box 0 feature
       const int f_b = f_a + kWBoxRows;           // box 1 feature (down pass only)
       float ws_a = 1.f, ws_b = 1.f;              // FP8: scales of this lane's two weight rows
       const float* rsp = nullptr;
       if (FP8) {
-        rsp = (t.dense ? p.row_scale2 : p.row_scale) + t.row0;
+        rsp = (dense ? p.row_scale2 : p.row_scale) + t.row0;
         const float* const wsp =
-            t.dense ? p.w_scale2 : p.w_scale + (size_t)(p.e_base + t.e) * (GATED ? 2 : 1) * n_feat;
+            dense ? p.w_scale2 : p.w_scale + (size_t)(p.e_base + t.e) * (GATED ? 2 : 1) * n_feat;
         if (f_a < n_feat) ws_a = wsp[f_a];
         if (GATED ? f_a < n_feat : f_b < n_feat) ws_b = wsp[GATED ? n_feat + f_a : f_b];
       }
@@ -974,7 +979,7 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   prm.yield_req = preemptible ? p.yield_req : nullptr;
   prm.stopped = preemptible ? p.stopped : nullptr;
 
-  const size_t tail = (2 * kNB + 4 + 2 * kQ) * sizeof(uint64_t) + 3 * sizeof(uint32_t) + (kNB + kQ) * sizeof(int) +
+  const size_t tail = (2 * kNB + 4 + 2 * kQ) * sizeof(uint64_t) + 3 * sizeof(uint32_t) + kNB * sizeof(int) + kQ * sizeof(STile) +
                       (4 * (size_t)(prm.E + 1) + kSizeClasses + 32) * sizeof(int);
   const int slots = (int)((kSmemBudget - 1024 - (int)tail) / kSlotBytes);
   if (slots < 2 * (kWSlots + kMaxTileRows / 16)) return cudaErrorNotSupported;

@@ -217,8 +217,8 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
   const int total_tiles = dense_tiles + prefix[p.E] * n_ft;
 
   if (warp == kProducerWarp) {
-    // ================================================================= TMA producer (one lane)
-    if (lane == 0 && !p.inject_producer_stall) {
+    // ================================================================= TMA producer
+    if (!p.inject_producer_stall) {
       RingCursor ring;
       bool ok = true;
       for (int tile = unit; tile < total_tiles && ok; tile += n_units) {
@@ -233,24 +233,26 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         const bool short_x = !GATHER && x_rows < 128u;
         const CUtensorMap* mxs = (t.dense ? omaps.xs2 : omaps.xs) + (short_x ? x_rows / 32u - 1u : 0u);
         for (int kb = 0, k0 = 0; kb < num_kb; ++kb, k0 += kbk) {
-          if (!mbar_wait(bar_empty + 8u * ring.stage, ring.phase ^ 1u, abort_flag, p.wait_limit_ns)) { ok = false; break; }
+          if (!mbar_wait_warp(bar_empty + 8u * ring.stage, ring.phase ^ 1u, abort_flag, p.wait_limit_ns)) { ok = false; break; }
           const uint32_t full = bar_full + 8u * ring.stage;
           const uint32_t st = base_addr + ring.stage * (uint32_t)stage_bytes;
-          mbar_expect_tx(full, GATHER ? 2u * kWBoxBytes : (short_x ? 2u * kWBoxBytes + x_rows * 128u : (uint32_t)stage_bytes));
-          tma_load_3d(st, mw, full, k0, w_row0, w_e);
-          tma_load_3d(st + kWBoxBytes, mw, full, k0, w_row1, w_e);
-          if (!GATHER) tma_load_2d(st + 2 * kWBoxBytes, short_x ? mxs : mx, full, k0, t.row0);
+          if (elect_one()) {
+            mbar_expect_tx(full, GATHER ? 2u * kWBoxBytes : (short_x ? 2u * kWBoxBytes + x_rows * 128u : (uint32_t)stage_bytes));
+            tma_load_3d(st, mw, full, k0, w_row0, w_e);
+            tma_load_3d(st + kWBoxBytes, mw, full, k0, w_row1, w_e);
+            if (!GATHER) tma_load_2d(st + 2 * kWBoxBytes, short_x ? mxs : mx, full, k0, t.row0);
+          }
           ring.advance((uint32_t)p.n_stages);
         }
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         *abort_flag = 1;
         atomicCAS(p.status, kStOk, kStTimeout);
       }
     }
   } else if (warp == kMmaWarp) {
-    // ================================================================= MMA issuer (one lane)
-    if (lane == 0) {
+    // ================================================================= MMA issuer
+    {
       uint32_t tile_iter = 0;
       RingCursor ring;
       bool ok = true;
@@ -261,33 +263,32 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
       for (int tile = unit; tile < total_tiles && ok; tile += n_units, ++tile_iter) {
         const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, seg, tile_rows);
         const uint32_t as = tile_iter & 1u, aph = (tile_iter >> 1) & 1u;
-        if (!mbar_wait(bar_tempty + 8u * as, aph ^ 1u, abort_flag, p.wait_limit_ns)) { ok = false; break; }
+        if (!mbar_wait_warp(bar_tempty + 8u * as, aph ^ 1u, abort_flag, p.wait_limit_ns)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d0 = tmem_base + as * acc_cols;
         const uint32_t idesc = FP8 ? umma_idesc_e4m3(128, 256) : umma_idesc(128, 256);
         const int num_kb = t.dense ? num_kb2 : num_kb1;
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(bar_full + 8u * ring.stage, ring.phase, abort_flag, p.wait_limit_ns)) { ok = false; break; }
+          if (!mbar_wait_warp(bar_full + 8u * ring.stage, ring.phase, abort_flag, p.wait_limit_ns)) { ok = false; break; }
           if (GATHER) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // X rows came by cp.async
           tc_fence_after();
           const uint32_t lo_w0 = lo_base + ring.stage * lo_stage;  // weight box 0; box 1 and the X tile follow
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
-            const uint32_t adv = (uint32_t)((kk * kUmmaK * 2) >> 4);  // +32 bytes per MMA (16 bf16 or 32 E4M3), in 16-byte units
-            const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
-            auto mma = [&](uint32_t d, uint32_t a_lo, uint32_t b_lo) {
-              if (FP8) umma_e4m3_lo(d, a_lo, b_lo, desc_hi, idesc, acc);
-              else umma_bf16_lo(d, a_lo, b_lo, desc_hi, idesc, acc);
-            };
-            // the two weight boxes are contiguous: one N = 256 operand
-            mma(d0, lo_w0 + 2 * lo_box + adv, lo_w0 + adv);
+            for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
+              const uint32_t adv = (uint32_t)((kk * kUmmaK * 2) >> 4);  // +32 bytes per MMA (16 bf16 or 32 E4M3), in 16-byte units
+              const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
+              // the two weight boxes are contiguous: one N = 256 operand
+              if (FP8) umma_e4m3_lo(d0, lo_w0 + 2 * lo_box + adv, lo_w0 + adv, desc_hi, idesc, acc);
+              else umma_bf16_lo(d0, lo_w0 + 2 * lo_box + adv, lo_w0 + adv, desc_hi, idesc, acc);
+            }
+            umma_commit(bar_empty + 8u * ring.stage);  // the stage is free once these MMAs have read it
           }
-          umma_commit(bar_empty + 8u * ring.stage);  // the stage is free once these MMAs have read it
           ring.advance((uint32_t)p.n_stages);
         }
-        if (ok) umma_commit(bar_tfull + 8u * as);  // accumulator complete
+        if (ok && elect_one()) umma_commit(bar_tfull + 8u * as);  // accumulator complete
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         *abort_flag = 1;
         atomicCAS(p.status, kStOk, kStTimeout);
       }
