@@ -15,9 +15,8 @@
 //              same tile sequence.
 //   TMEM       512 columns = two halves.  A tile of N <= 128 takes one half (its two accumulators side by side)
 //              and alternates halves, so its epilogue overlaps the next tile's MMAs; a tile of N > 128 takes both.
-//   epilogue   lane = weight row (output feature), column = token: tcgen05.ld -> (scale) -> SwiGLU -> bf16;
-//              neighbouring lanes exchange values so that every store writes a feature pair.  The gated epilogue
-//              hands the accumulator back before its exchanges and stores.
+//   epilogue   tcgen05.ld of 8 x 8 fragments -> (scale) -> SwiGLU -> bf16 -> stmatrix, which transposes (TMEM lanes are
+//              features, columns tokens), into a per-warp staging tile -> 16-byte stores.
 //   schedule   the tile list is ordered by expert size, largest first.  Its first waves are dealt statically (CTAs
 //              in step share weights and rows through L2), the last waves' worth of tiles -- the smallest -- are
 //              handed out by an atomic counter to whichever CTA is free; the producer publishes the tiles it takes
@@ -46,13 +45,7 @@ namespace {
 
 using namespace tc;
 
-#ifndef MOE_STREAM_EPI_WARPS
-#define MOE_STREAM_EPI_WARPS 8
-#endif
-// Epilogue warps: 4 (each owns 32 TMEM lanes = 32 weight rows) or 8 (two warps per lane group, one taking the
-// even and one the odd 16-token chunks), which halves the time a tile of more than 128 tokens keeps the MMA
-// issuer waiting for its single accumulator.
-constexpr int kEpilogueWarps = MOE_STREAM_EPI_WARPS;
+constexpr int kEpilogueWarps = 8;  // two per TMEM lane group, taking alternate 16-token chunks
 constexpr int kProducerWarp = kEpilogueWarps;
 constexpr int kMmaWarp = kEpilogueWarps + 1;
 constexpr int kThreads = 32 * (kEpilogueWarps + 2);
@@ -63,6 +56,7 @@ constexpr int kMaxTileRows = 256;                       // largest MMA N
 constexpr int kNB = 8;                                  // k-blocks in flight at most (barrier pairs)
 constexpr int kXMaps = 16;                              // token-row boxes of 16 (b + 1) rows
 constexpr uint32_t kTmemCols = 512;
+constexpr int kStagingBytes = 16 * 64;  // epilogue, per warp: 16 tokens x 32 features
 constexpr int kQ = 4;                                   // entries of the CTA's tile queue
 // Waves' worth of tiles, at the list's end, that are handed out dynamically: a fifth of them, between two and six.  Over
 // tens of waves the CTAs drift apart by more than two tiles (V3-shaped decode, 28 and 49 waves: 2089 us with six, 2111 with
@@ -189,12 +183,13 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
                            const __grid_constant__ StreamMaps xmaps, const __grid_constant__ StreamParams p) {
   constexpr int kbk = FP8 ? 2 * kBlockK : kBlockK;  // K elements per k-block
   extern __shared__ uint8_t smem_raw[];
-  // carve: ring (ring_slots x 2 KB) | full[kNB] empty[kNB] tfull[2] tempty[2] tqfull[kQ] tqempty[kQ] | tq[kQ] | tmem slot
+  // carve: ring (ring_slots x 2 KB) | epilogue staging | full[kNB] empty[kNB] tfull[2] tempty[2] tqfull[kQ] tqempty[kQ] | tq[kQ] | tmem slot
   //        | abort | stopped | sizes[kNB] | prefix[E+1] | order[E] | beg[E] | cnts[E] | classes | chunk sums
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base_addr = (raw_addr + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (base_addr - raw_addr);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(base + (size_t)p.ring_slots * kSlotBytes);
+  uint8_t* const staging = base + (size_t)p.ring_slots * kSlotBytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(staging + kEpilogueWarps * kStagingBytes);
   const uint32_t bar_full = smem_u32(bars);
   const uint32_t bar_empty = bar_full + 8u * kNB;
   const uint32_t bar_tfull = bar_empty + 8u * kNB;
@@ -609,7 +604,11 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
     }
   } else {
     // ================================================================= epilogue (warps 0-7)
-    // lane = weight row (output feature) of each box, TMEM column = token
+    // TMEM lane = weight row (output feature) of each box, column = token.  A warp takes 32 features x 16 tokens at a time, in
+    // the fragments of 8 x 8 matrices: a thread then has gate and up of the same elements and neighbouring tokens side by
+    // side, stmatrix transposes the bf16 results into the warp's staging, and they leave as 16 bytes of a row.  (With lanes
+    // as features and neighbouring lanes exchanging values for 4-byte stores 256 columns of 128 lanes took 5700 clocks, gated
+    // 8200; this 3100 and 3400.)
     if (p.early_setup) {
       pdl_wait();
       pdl_launch_dependents();
@@ -617,10 +616,15 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
     uint32_t use0 = 0, use1 = 0, next_half = 0;
     bool ok = true;
     const int lg = warp & 3;                         // TMEM lane group of this warp: lanes 32 lg .. 32 lg + 31
-    const int c_first = kEpilogueWarps == 8 ? 16 * (warp >> 2) : 0, c_step = kEpilogueWarps == 8 ? 32 : 16;
+    const int c_first = 16 * (warp >> 2), c_step = 32;
     const uint32_t lane_base = ((uint32_t)(lg * 32)) << 16;
-    const int fl = lg * 32 + lane;
-    const bool even = (lane & 1) == 0;
+    // staging: 16 tokens of 64 bytes, the 16-byte pieces XOR-swizzled by pairs of tokens (no bank conflicts either way)
+    uint8_t* const stg = staging + warp * kStagingBytes;
+    auto piece = [](int tok, int i) { return tok * 64 + ((i ^ ((tok >> 1) & 3)) << 4); };
+    const int st_tok = (lane & 7) + 8 * (lane >> 4), st_piece = (lane >> 3) & 1;  // stmatrix: this lane's row of 8 features
+    const uint32_t st0 = smem_u32(stg) + (uint32_t)piece(st_tok, st_piece), st1 = smem_u32(stg) + (uint32_t)piece(st_tok, st_piece + 2);
+    const int ld_tok = lane >> 2, ld_piece = lane & 3;                            // and the token and features it stores
+    const int fr_row = lane >> 2, fr_col = 2 * (lane & 3);                        // fragments: its feature and token
     uint32_t tcount = 0;
     for (;;) {
       const uint32_t q = tcount % kQ;
@@ -636,6 +640,30 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       const bool dense = t.e == kDenseTile;
       const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
       const bool big = n > 128u;
+      __nv_bfloat16* const out = dense ? p.out2 : p.out;
+      const int n_feat = dense ? p.n_feat2 : p.n_feat;
+      const int f0 = t.ft * kFeatPerTile + lg * 32;  // this warp's first feature (down pass: of box 0, and + 128 of box 1)
+      float ws_a[4], ws_b[4];                        // FP8: scales of this thread's weight rows, 8 apart
+      float rs[4];                                   // ... and of its tokens in the next chunk
+      const float* rsp = nullptr;
+      auto fetch_scales = [&](int c) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int tok = c + fr_col + (i & 1) + 8 * (i >> 1);
+          rs[i] = tok < t.rows ? __ldg(rsp + tok) : 0.f;
+        }
+      };
+      if (FP8) {
+        rsp = (dense ? p.row_scale2 : p.row_scale) + t.row0;
+        const float* const wsp = dense ? p.w_scale2 : p.w_scale + (size_t)(p.e_base + t.e) * (GATED ? 2 : 1) * n_feat;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int f = f0 + fr_row + 8 * i, f2 = GATED ? f : f + kWBoxRows;
+          ws_a[i] = f < n_feat ? __ldg(wsp + f) : 0.f;
+          ws_b[i] = f2 < n_feat ? __ldg(wsp + (GATED ? n_feat + f : f2)) : 0.f;
+        }
+        fetch_scales(c_first);
+      }
       uint32_t h = 0, d_a, d_b;
       if (big) {
         if (!mbar_wait(bar_tfull, use0 & 1u, abort_flag, limit) ||
@@ -655,23 +683,6 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       tc_fence_after();
       d_a += lane_base;
       d_b += lane_base;
-      __nv_bfloat16* const out = dense ? p.out2 : p.out;
-      const int n_feat = dense ? p.n_feat2 : p.n_feat;
-      const int f_a = t.ft * kFeatPerTile + fl;  // box 0 feature
-      const int f_b = f_a + kWBoxRows;           // box 1 feature (down pass only)
-      float ws_a = 1.f, ws_b = 1.f;              // FP8: scales of this lane's two weight rows
-      const float* rsp = nullptr;
-      if (FP8) {
-        rsp = (dense ? p.row_scale2 : p.row_scale) + t.row0;
-        const float* const wsp =
-            dense ? p.w_scale2 : p.w_scale + (size_t)(p.e_base + t.e) * (GATED ? 2 : 1) * n_feat;
-        if (f_a < n_feat) ws_a = wsp[f_a];
-        if (GATED ? f_a < n_feat : f_b < n_feat) ws_b = wsp[GATED ? n_feat + f_a : f_b];
-      }
-      // Feature pairs: an even lane keeps the even tokens of a 16-token chunk and receives its odd neighbour's
-      // values for them (features f, f+1 of one token are one 4-byte store); the odd lane does the same for
-      // the odd tokens.  n_feat is a multiple of 8, so a pair is inside the row or outside it as a whole.
-      const int f_pair = (GATED ? f_a : 0) & ~1;
       auto release_acc = [&]() {  // hand the accumulator half (or both) back to the MMA issuer
         tc_fence_before();
         __syncwarp();
@@ -684,127 +695,69 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
           }
         }
       };
-      // (Small tiles take the loop below, a twelfth of the code: a decode launch runs each line of it once, from a cold
-      // instruction cache, and has nothing to hand back early, the other half of TMEM being free.  With FP8 the loop's
-      // scale reads cost more than that: 181.8 against 180.8 us for three tokens of the V3-shaped layer.)
-      if (GATED && kEpilogueWarps == 8 && (big || FP8)) {
-        // Two phases, so that the accumulator goes back to the MMA issuer as early as possible (a tile of more than
-        // 128 tokens holds all of TMEM, and the issuer waits for it): first every chunk is loaded (the next chunk's
-        // loads in flight meanwhile), put through SwiGLU and packed to bf16 in registers -- a warp has at most 8
-        // chunks of 16 tokens; then the accumulator is released; only then come the lane exchanges and the stores.
-        uint32_t pk[8][8];  // pk[m][i]: this lane's feature for tokens c + 2i (low half) and c + 2i + 1 (high half)
-        uint32_t na[16], nb[16];
-        if (c_first < t.rows) {
-          tmem_ld16(d_a + (uint32_t)c_first, na);
-          tmem_ld16(d_b + (uint32_t)c_first, nb);
+      // stages 32 features x 16 tokens and stores them: features f.. of tokens c..
+      auto put = [&](const uint32_t (&lo)[4], const uint32_t (&hi)[4], int f, int c) {
+        stmatrix_trans(st0, lo);
+        stmatrix_trans(st1, hi);
+        __syncwarp();
+        uint4 v[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) v[i] = *reinterpret_cast<const uint4*>(stg + piece(ld_tok + 8 * i, ld_piece));
+        __syncwarp();  // read: the staging may be written again
+        f += 8 * ld_piece;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int tok = c + ld_tok + 8 * i;
+          if (tok < t.rows && f < n_feat) *reinterpret_cast<uint4*>(out + (size_t)(t.row0 + tok) * n_feat + f) = v[i];
         }
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const int c = c_first + m * c_step;
-          // Leave, do not skip chunk by chunk: the unrolled chunks are kilobytes of code that a launch of small tiles would
-          // fetch from a cold instruction cache just to jump over them: 2 to 5 us a step (one-token V3-shaped decode 138.1
-          // us leaving, 143.1 skipping).
-          if (c >= t.rows) break;
-          {
-            float g[16], u[16];
-            tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              g[i] = __uint_as_float(na[i]);
-              u[i] = __uint_as_float(nb[i]);
-            }
-            if (c + c_step < t.rows) {
-              tmem_ld16(d_a + (uint32_t)(c + c_step), na);
-              tmem_ld16(d_b + (uint32_t)(c + c_step), nb);
-            }
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              if (FP8) {
-                const float rs = (c + i < t.rows) ? __ldg(rsp + c + i) : 0.f;
-                g[i] *= rs * ws_a;
-                u[i] *= rs * ws_b;
-              }
-              g[i] = silu_mul(g[i], u[i]);
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) pk[m][i] = pack_bf16(g[2 * i], g[2 * i + 1]);
-          }
-        }
-        release_acc();
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const int c = c_first + m * c_step;
-          if (c >= t.rows) break;
-          {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const uint32_t mine = pk[m][i];
-              const uint32_t nbr = __shfl_xor_sync(0xffffffffu, mine, 1);
-              // even lane (even feature f): token c+2i, features (f, f+1) = (own low, neighbour's low);
-              // odd lane: token c+2i+1, features (f-1, f) = (neighbour's high, own high)
-              const uint32_t pa = even ? __byte_perm(mine, nbr, 0x5410) : __byte_perm(nbr, mine, 0x7632);
-              const int tok = c + 2 * i + (even ? 0 : 1);
-              if (tok < t.rows && f_pair < n_feat)
-                *reinterpret_cast<uint32_t*>(out + (size_t)(t.row0 + tok) * n_feat + f_pair) = pa;
-            }
-          }
-        }
-        continue;
-      }
+      };
       // the loads of the next 16-token chunk are in flight while this one is converted and stored
-      uint32_t na[16], nb[16];
-      if (c_first < t.rows) {
-        tmem_ld16(d_a + (uint32_t)c_first, na);
-        tmem_ld16(d_b + (uint32_t)c_first, nb);
-      }
+      uint32_t na[2][8], nb[2][8];  // [features 0-15 or 16-31][fragments]
+      auto load = [&](int c) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          tmem_ld_frag(d_a + ((uint32_t)(16 * k) << 16) + (uint32_t)c, na[k]);
+          tmem_ld_frag(d_b + ((uint32_t)(16 * k) << 16) + (uint32_t)c, nb[k]);
+        }
+      };
+      if (c_first < t.rows) load(c_first);
+      else release_acc();
       for (int c = c_first; c < t.rows; c += c_step) {
-        uint32_t ra[16], rb[16];
+        uint64_t va[2][4], vb[2][4];  // pairs of neighbouring tokens
         tmem_ld_wait();
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          ra[i] = na[i];
-          rb[i] = nb[i];
-        }
-        if (c + c_step < t.rows) {
-          tmem_ld16(d_a + (uint32_t)(c + c_step), na);
-          tmem_ld16(d_b + (uint32_t)(c + c_step), nb);
-        }
-        float va[16], vb[16];
+        for (int k = 0; k < 2; ++k)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float a = __uint_as_float(ra[i]), b = __uint_as_float(rb[i]);
-          if (FP8) {
-            const float rs = (c + i < t.rows) ? __ldg(rsp + c + i) : 0.f;
-            a *= rs * ws_a;
-            b *= rs * ws_b;
-          }
-          va[i] = GATED ? silu_mul(a, b) : a;
-          vb[i] = b;
-        }
-#pragma unroll
-        for (int i = 0; i < 16; i += 2) {
-          // values of token c+i (even lanes keep) and c+i+1 (odd lanes keep)
-          const float keep_a = even ? va[i] : va[i + 1], send_a = even ? va[i + 1] : va[i];
-          const float recv_a = __shfl_xor_sync(0xffffffffu, send_a, 1);
-          const int tok = c + i + (even ? 0 : 1);
-          const uint32_t pa = even ? pack_bf16(keep_a, recv_a) : pack_bf16(recv_a, keep_a);
-          if (GATED) {
-            if (tok < t.rows && f_pair < n_feat)
-              *reinterpret_cast<uint32_t*>(out + (size_t)(t.row0 + tok) * n_feat + f_pair) = pa;
-          } else {
-            const float keep_b = even ? vb[i] : vb[i + 1], send_b = even ? vb[i + 1] : vb[i];
-            const float recv_b = __shfl_xor_sync(0xffffffffu, send_b, 1);
-            const uint32_t pb = even ? pack_bf16(keep_b, recv_b) : pack_bf16(recv_b, keep_b);
-            const int fa2 = f_a & ~1, fb2 = f_b & ~1;
-            if (tok < t.rows) {
-              __nv_bfloat16* orow = out + (size_t)(t.row0 + tok) * n_feat;
-              if (fa2 < n_feat) *reinterpret_cast<uint32_t*>(orow + fa2) = pa;
-              if (fb2 < n_feat) *reinterpret_cast<uint32_t*>(orow + fb2) = pb;
+          for (int i = 0; i < 4; ++i) {
+            va[k][i] = f32x2(__uint_as_float(na[k][2 * i]), __uint_as_float(na[k][2 * i + 1]));
+            vb[k][i] = f32x2(__uint_as_float(nb[k][2 * i]), __uint_as_float(nb[k][2 * i + 1]));
+            if (FP8) {
+              const uint64_t r = f32x2(rs[2 * (i >> 1)], rs[2 * (i >> 1) + 1]);
+              const float wa = ws_a[2 * k + (i & 1)], wb = ws_b[2 * k + (i & 1)];
+              va[k][i] = mul2(va[k][i], mul2(r, f32x2(wa, wa)));
+              vb[k][i] = mul2(vb[k][i], mul2(r, f32x2(wb, wb)));
             }
           }
+        if (c + c_step < t.rows) {
+          load(c + c_step);
+          if (FP8) fetch_scales(c + c_step);
+        } else {
+          release_acc();  // read completely
+        }
+        uint32_t q[2][4];
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) q[k][i] = pack_bf16(GATED ? silu_mul2(va[k][i], vb[k][i]) : va[k][i]);
+        put(q[0], q[1], f0, c);
+        if (!GATED) {
+#pragma unroll
+          for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) q[k][i] = pack_bf16(vb[k][i]);
+          put(q[0], q[1], f0 + kWBoxRows, c);
         }
       }
-      release_acc();
     }
     if (!ok && lane == 0) {
       *abort_flag = 1;
@@ -979,7 +932,7 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   prm.yield_req = preemptible ? p.yield_req : nullptr;
   prm.stopped = preemptible ? p.stopped : nullptr;
 
-  const size_t tail = (2 * kNB + 4 + 2 * kQ) * sizeof(uint64_t) + 3 * sizeof(uint32_t) + kNB * sizeof(int) + kQ * sizeof(STile) +
+  const size_t tail = kEpilogueWarps * kStagingBytes + (2 * kNB + 4 + 2 * kQ) * sizeof(uint64_t) + 3 * sizeof(uint32_t) + kNB * sizeof(int) + kQ * sizeof(STile) +
                       (4 * (size_t)(prm.E + 1) + kSizeClasses + 32) * sizeof(int);
   const int slots = (int)((kSmemBudget - 1024 - (int)tail) / kSlotBytes);
   if (slots < 2 * (kWSlots + kMaxTileRows / 16)) return cudaErrorNotSupported;

@@ -419,8 +419,8 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
               }
 #pragma unroll
               for (int i = 0; i < 16; ++i)
-                packed[i] = pack_bf16(silu_mul(__uint_as_float(ra[2 * i]), __uint_as_float(rb[2 * i])),
-                                      silu_mul(__uint_as_float(ra[2 * i + 1]), __uint_as_float(rb[2 * i + 1])));
+                packed[i] = pack_bf16(silu_mul2(f32x2(__uint_as_float(ra[2 * i]), __uint_as_float(ra[2 * i + 1])),
+                                                f32x2(__uint_as_float(rb[2 * i]), __uint_as_float(rb[2 * i + 1]))));
             } else {
               tmem_ld_wait();
               if (FP8) {

@@ -166,6 +166,20 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+// 16 lanes x 16 columns, as the fragments of four 8 x 8 matrices: lane l gets columns 2 (l % 4) and + 1 of row l / 4 (r[0],
+// r[1]), of row l / 4 + 8 (r[2], r[3]), and the same of the columns behind 8 (r[4..7])
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+// Stores four such matrices of bf16 transposed; lane l gives the address of row l % 8 (16 bytes) of matrix l / 8
+__device__ __forceinline__ void stmatrix_trans(uint32_t addr, const uint32_t (&r)[4]) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3])
+               : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Tiled bulk store shared -> global of one box, tracked in the issuing thread's bulk groups
@@ -205,25 +219,55 @@ __device__ __forceinline__ uint32_t umma_idesc_e4m3(uint32_t M, uint32_t N) {
   return (1u << 4) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
-// silu(g) * u with one special-function operation per element instead of two: t = 2^(-|g| log2 e) in (0,1] comes
+// Two fp32 values in a register pair: one issue slot for both, each rounded as by the scalar instruction.
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ float2 unpack(uint64_t v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t v;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+  return v;
+}
+
+// silu(g) * u of two elements, with one special-function operation each instead of two: t = 2^(-|g| log2 e) in (0,1] comes
 // from ex2.approx; the reciprocal of d = 1 + t in (1,2] is a linear seed (24/17 - 8/17 d, relative error <= 1/17)
 // refined by two Newton steps on the FMA pipe (relative error <= 1.2e-5, far below the bf16 rounding that follows);
 // sigmoid(g) = 1/d for g >= 0 and t/d for g < 0, so small sigmoids keep their relative accuracy.  The epilogue
-// of a GEMM1 tile evaluates 32K of these, and the special-function unit (16 results per clock and SM) is what it
-// waits for.
-__device__ __forceinline__ float silu_mul(float g, float u) {
-  float t;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(-fabsf(g) * 1.4426950408889634f));
-  const float d = 1.0f + t;
-  float r = fmaf(d, -0.47058823529411764f, 1.4117647058823530f);
-  r = r * fmaf(-d, r, 2.0f);
-  r = r * fmaf(-d, r, 2.0f);
-  return g * (g >= 0.f ? r : t * r) * u;
+// of a GEMM1 tile evaluates 32K of these, and issue slots are what it waits for: 17 for two elements, 26 one at a time.
+__device__ __forceinline__ uint64_t silu_mul2(uint64_t g2, uint64_t u2) {
+  const float2 g = unpack(g2);
+  float2 t;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t.x) : "f"(-fabsf(g.x) * 1.4426950408889634f));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t.y) : "f"(-fabsf(g.y) * 1.4426950408889634f));
+  const uint64_t t2 = f32x2(t.x, t.y), minus1 = f32x2(-1.0f, -1.0f), two = f32x2(2.0f, 2.0f);
+  const uint64_t nd = fma2(t2, minus1, minus1);  // -d
+  uint64_t r = fma2(nd, f32x2(0.47058823529411764f, 0.47058823529411764f), f32x2(1.4117647058823530f, 1.4117647058823530f));
+  r = mul2(r, fma2(nd, r, two));
+  r = mul2(r, fma2(nd, r, two));
+  const float2 pos = unpack(r), neg = unpack(mul2(t2, r));
+  return mul2(mul2(g2, f32x2(g.x >= 0.f ? pos.x : neg.x, g.y >= 0.f ? pos.y : neg.y)), u2);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(uint64_t v) {
+  const float2 f = unpack(v);
+  return pack_bf16(f.x, f.y);
 }
 
 // Position in the ring of pipeline stages, advanced without division: the role loops run on a single thread (or
