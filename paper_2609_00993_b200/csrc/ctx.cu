@@ -334,6 +334,8 @@ int gemm_ctas(const moe_ctx* ctx) {
 constexpr size_t kHostOverlapBytes = 512 * 1024, kHostPieceBytes = 1536 * 1024, kHostChunkBytes = 4 << 20;
 constexpr int kHostMaxPieces = 4, kHostChunkFromRows = 200;
 
+constexpr int kGemmPair = 100;  // (beside the public variants: the two-CTA kernel, which AUTO alone takes)
+
 // AUTO: a DECODE context always streams; a PREFILL context chooses per launch from the problem's rows (T * top_k
 // rows over n_experts; T rows over one group for the shared expert by itself) and K: the choice is a function of T
 // alone, so it is the same on every replay of a graph.
@@ -345,8 +347,11 @@ int gemm_variant_of(const moe_ctx* ctx, const moe::GemmProblem& p) {
   if (ctx->preemptible) return MOE_GEMM_SMALL_M;          // only the small-M kernel can stop between tiles
   // problems of up to 8192 rows, whose launches overlap with their neighbours, are 1.5-6 % faster on the small-M kernel
   // at any shape: it builds its tile list and fetches weights before the previous kernel has finished
-  const bool small = p.rows_bound <= moe::kGemmOverlapMaxRows || moe::small_m_is_faster(p.fp8, p.gated, p.K, p.n_feat, p.rows_bound, p.E, gemm_ctas(ctx));
-  return small ? MOE_GEMM_SMALL_M : MOE_GEMM_LARGE_M;
+  if (p.rows_bound <= moe::kGemmOverlapMaxRows) return MOE_GEMM_SMALL_M;
+  // A context on part of the SMs shares the GPU with another, whose CTAs need not leave whole pairs of SMs free.
+  const int ctas = gemm_ctas(ctx);
+  if (ctas == ctx->n_sms && moe::pair_is_faster(p.fp8, p.gated, p.K, p.n_feat, p.rows_bound, p.E, ctas)) return kGemmPair;
+  return moe::small_m_is_faster(p.fp8, p.gated, p.K, p.n_feat, p.rows_bound, p.E, ctas) ? MOE_GEMM_SMALL_M : MOE_GEMM_LARGE_M;
 }
 
 // GEMM1 gathers its rows itself only on the large-M tensor-core variant.
@@ -400,6 +405,7 @@ cudaError_t run_gemm(moe_ctx* ctx, moe::GemmProblem p, const moe::GemmDenseGroup
     }
     return e;
   }
+  if (variant == kGemmPair) return moe::launch_gemm_pair(p, dense, gemm_ctas(ctx), ctx->status, ctx->stream, n);
   if (variant == MOE_GEMM_SMALL_M) return moe::launch_gemm_stream(p, dense, gemm_ctas(ctx), ctx->status, ctx->stream, n);
   return moe::launch_gemm_tc(p, dense, gemm_ctas(ctx), ctx->status, ctx->stream, n);
 }

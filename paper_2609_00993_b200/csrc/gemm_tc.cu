@@ -514,11 +514,11 @@ cudaError_t launch_variant(Kernel kern, int threads, const CUtensorMap& mx, cons
 namespace tc {
 bool encode_map(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
                 const uint32_t* box, bool bytes) {
-  if (rank < 2 || rank > 4) return false;
-  cuuint64_t gdim[4];
-  cuuint64_t gstr[3];
-  cuuint32_t bdim[4];
-  cuuint32_t estr[4] = {1, 1, 1, 1};
+  if (rank < 2 || rank > 5) return false;
+  cuuint64_t gdim[5];
+  cuuint64_t gstr[4];
+  cuuint32_t bdim[5];
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   for (int i = 0; i < rank; ++i) { gdim[i] = dims[i]; bdim[i] = box[i]; }
   for (int i = 0; i + 1 < rank; ++i) gstr[i] = strides_bytes[i];
   CUresult r = g_encode(map, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), gdim, gstr,

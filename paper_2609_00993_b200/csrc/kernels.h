@@ -213,6 +213,10 @@ cudaError_t launch_gemm_tc(const GemmProblem& p, const GemmDenseGroup* dense, in
 // bytes the SMs ingest.  Same contract as launch_gemm_tc; no row gather.
 cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense, int max_ctas, int* status,
                                cudaStream_t stream, int* n_launches);
+// Two-CTA variant (swap-AB, a tile multiplied by a pair of SMs): needs clusters of two CTAs, that is whole pairs of free
+// SMs.  Same contract as launch_gemm_tc; no row gather, no preemption.
+cudaError_t launch_gemm_pair(const GemmProblem& p, const GemmDenseGroup* dense, int max_ctas, int* status,
+                             cudaStream_t stream, int* n_launches);
 // One-time driver entry-point lookup for tensor-map encoding; returns false (with a reason) if unavailable.
 bool gemm_tc_init(const char** why);
 

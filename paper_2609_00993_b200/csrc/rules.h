@@ -82,4 +82,44 @@ inline bool small_m_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t r
   return K >= kMinDownK && (up_to(64) || (!up_to(120) && up_to(190)));
 }
 
+// ---- ... and whether the two-CTA kernel takes it before either of them, where it may use all SMs (gemm_pair.cu)
+// It multiplies exactly the rows there are, like the small-M kernel, and every epilogue overlaps the next tile, like the
+// large-M kernel's; but a tile's operands come in the same number of bytes as the small-M kernel's (per flop) through twice as
+// many k-blocks, so with long K the small-M kernel stays ahead.  Whole steps in the sustained state, each over the best of the
+// nine combinations, gated pass / down pass on s = small-M, l = large-M, p = pairs (two runs of one differ by up to 1.5 %):
+//   bf16  2048 / 768 x 128    R = 69 ss 1.007 sl 1.000 sp 1.006 pp 1.009; 96 1.011 1.000 1.015 1.013; 162 1.021 1.065 1.009 1.000;
+//                             281 1.000 1.021 1.007 1.051; 512 1.030 1.021 1.000 1.022; 1000 1.040 1.035 1.012 1.000; 1875 1.062
+//                             1.035 1.014 1.000
+//         2560 / 1024 x 512   64 1.004 1.019 1.014 1.040; 187 1.000 1.053 1.004 1.016; 312 1.001 1.030 1.018 1.016; 469 1.000 1.021
+//                             1.002 1.035
+//         4096 / 1536 x 128   125 1.000 1.026 1.010 1.029; 375 1.000 1.033 1.012 1.033; 1000 1.014 1.029 1.000 1.038
+//         7168 / 2048 x 256   64 1.015 1.058 1.019 1.045; 128 1.008 1.048 1.000 1.031; 250 1.010 1.050 1.000 1.042; 500 1.024 1.017
+//          + shared           1.000 1.097; 937 1.037 1.009 1.000 1.111
+//         1024 / 512 x 64     156 ss 1.051 sl 1.022 ll 1.060 pl 1.000 pp 1.003; 375 1.067 1.031 1.022 1.000 1.021; 1250 1.059 1.029
+//                             1.035 1.000 1.007;  1536 / 512 x 128  156 1.030 1.030 1.117 1.018 1.000; 625 1.048 1.009 1.048 1.000 1.010
+//         few tiles: 512 / 2048 x 8  R = 1125 ll 1.005 pl 1.038; 7500 1.018 1.015;  7168 / 512 x 8  1125 1.000 1.022; 2000 1.062 1.007
+//   FP8   2048 / 768 x 128    69 sl 1.005 ll 1.019 pl 1.003 pp 1.007; 96 1.006 1.001 1.000 1.008; 156 1.082 1.156 1.062 1.000; 250 1.023
+//                             1.043 1.017 1.000; 375 1.022 1.005 1.000 1.030; 1000 1.045 1.048 1.026 1.000; 1875 1.056 1.041 1.045 1.000
+//         2560 / 1024 x 512   64 ss 1.017 sl 1.009 ps 1.010 pp 1.027; 125 1.004 1.030 1.015 1.023; 187 1.028 1.044 1.002 1.000; 312 1.008
+//                             1.005 1.000 1.003; 469 1.026 1.025 1.000 1.001
+//         4096 / 1536 x 128   125 ss 1.000 sp 1.002 ps 1.010 pp 1.015; 375 1.028 1.000 1.003 1.003; 1000 1.035 1.005 1.009 1.000
+//         7168 / 2048 x 256   128 ss 1.000 sp 1.002 pp 1.021; 250 1.005 1.000 1.015; 500 1.000 1.002 1.030; 937 1.027 1.000 1.050; skewed
+//          + shared           experts, 500 1.025 1.000 1.031
+//         1024 / 512 x 64     156 ll 1.028 pl 1.010 pp 1.000; 375 1.000 1.014 1.028; 1250 1.012 1.012 1.012
+//         2048 / 256 x 128    156 ps 1.000 pl 1.094 pp 1.000; 625 1.013 1.014 1.000
+inline bool pair_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t rows, int64_t E, int ctas) {
+  const auto over = [&](int64_t r) { return rows > r * E; };
+  const int64_t chunks = (rows + 255) / 256 > E ? (rows + 255) / 256 : E, feat_per_tile = gated ? 128 : 256;
+  const int64_t half_waves = 2 * chunks * ((n_feat + feat_per_tile - 1) / feat_per_tile) / ctas;
+  if (half_waves < 3) return false;
+  if (gated && !fp8) {
+    if (K < 640) return half_waves >= 16;
+    return K < 1792 ? over(96) : K < 2304 && over(768);
+  }
+  if (gated) return K < 1280 ? false : K < 2304 ? over(64) : K < 3072 ? over(160) : K < 5632 && over(256);
+  if (fp8) return K < 896 ? over(128) : K < 1280 ? over(180) : over(256);
+  if (K < 896) return K >= 640 && over(128);
+  return K < 1280 ? over(350) : K < 1792 ? over(512) : over(96);
+}
+
 }  // namespace moe
