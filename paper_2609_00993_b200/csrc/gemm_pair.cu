@@ -260,7 +260,7 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         const bool dense = t.e == kDenseTile;
         const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
         const CUtensorMap* mw = dense ? &map_w2 : &map_w;
-        const CUtensorMap* mx = (dense ? xmaps.x2 : xmaps.x) + ((n >> 4) - 1u);  // the box of n / 2 rows
+        const CUtensorMap* mx = rows_map(xmaps, p, t, n);  // the box of n / 2 rows
         const int w_e = dense ? 0 : p.e_base + t.e;
         const int w_row0 = t.ft * kFeatPerTile + (int)rank * (kFeatPerTile / 2);
         const int x_row0 = t.row0 + (int)(rank * (n >> 1));

@@ -226,7 +226,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
         const int w_row0 = t.ft * kFeatPerTile;
         const CUtensorMap* mw = dense ? &map_w2 : &map_w;
-        const CUtensorMap* mx = (dense ? xmaps.x2 : xmaps.x) + ((n >> 4) - 1u);  // the box of exactly n rows
+        const CUtensorMap* mx = rows_map(xmaps, p, t, n);  // the box of exactly n rows
         const int w_e = dense ? 0 : p.e_base + t.e;
         const int num_kb = dense ? num_kb2 : num_kb1;
         const int fetch_kb = num_kb > 4 ? num_kb - 4 : 0;

@@ -59,8 +59,10 @@ struct StreamParams {
   int32_t sort_tiles;  // 0: every group has at most one tile of the smallest size, so their order does not matter
 };
 
+// Token rows in boxes of 16, 32, ..., 256 rows; the dense group's in the two sizes it has, its equal chunks and its last one.
+// (With sixteen of those, too, a launch's parameters are 4.6 KB instead of 2.8.)
 struct StreamMaps {
-  CUtensorMap x[kXMaps], x2[kXMaps];  // token rows, boxes of 16, 32, ..., 256 rows (x2: the dense group's)
+  CUtensorMap x[kXMaps], x2[2];
 };
 
 // A tile as the producer hands it to the other roles: one entry of the CTA's queue.
@@ -120,6 +122,12 @@ __device__ __forceinline__ STile decode_tile(int tile, int dense_tiles, const St
   return t;
 }
 
+// The map of a tile's token rows, n of them with the padding to 16.
+__device__ __forceinline__ const CUtensorMap* rows_map(const StreamMaps& maps, const StreamParams& p, const STile& t,
+                                                       uint32_t n) {
+  return t.e != kDenseTile ? maps.x + ((n >> 4) - 1u) : maps.x2 + (t.row0 + t.rows == p.rows2 ? 1 : 0);
+}
+
 // First tiles of a launch that are dealt statically, in waves of `takers` (CTAs, or pairs of them).
 __device__ __forceinline__ int static_waves(int total_tiles, int takers) {
   const int waves = total_tiles / takers;
@@ -136,20 +144,24 @@ __device__ __forceinline__ void build_tile_list(const StreamParams& p, int* pref
   // ranks equals by __match_any_sync -- because every CTA of every launch builds the list before its first copy.
   // (24 tokens over 512 experts 384 us a step; 403 when each expert was ranked against all others, a shared-memory read per
   // pair; 37 over 128 184.0 and 186.2, 64 over 256 2152 and 2161.)
-  if (p.sort_tiles)
-    for (int c = threadIdx.x; c < kSizeClasses; c += THREADS) class_pos[c] = 0;
-  __syncthreads();
-  for (int e = threadIdx.x; e < p.E; e += THREADS) {
-    const int b = p.offsets ? p.offsets[e] : 0;
-    int c = p.offsets ? p.offsets[e + 1] - b : p.fixed_rows;
+  // Where the order does not matter the prefix is taken as the counts come in: one barrier instead of three, none up to 32
+  // experts.
+  auto fetch = [&](int e, int& b, int& c) {
+    b = p.offsets ? p.offsets[e] : 0;
+    c = p.offsets ? p.offsets[e + 1] - b : p.fixed_rows;
     if (c < 0) c = 0;
     beg[e] = b;
     cnts[e] = c;
-    if (p.sort_tiles) atomicAdd(&class_pos[size_class(c)], 1);
-    else order[e] = e;
-  }
-  __syncthreads();
+  };
   if (p.sort_tiles) {
+    for (int c = threadIdx.x; c < kSizeClasses; c += THREADS) class_pos[c] = 0;
+    __syncthreads();
+    for (int e = threadIdx.x; e < p.E; e += THREADS) {
+      int b, c;
+      fetch(e, b, c);
+      atomicAdd(&class_pos[size_class(c)], 1);
+    }
+    __syncthreads();
     if (warp == 0) {
       constexpr int kPer = kSizeClasses / 32;  // consecutive classes per lane
       int v[kPer], sum = 0;
@@ -187,7 +199,13 @@ __device__ __forceinline__ void build_tile_list(const StreamParams& p, int* pref
   // prefix[i]: row chunks of the experts at positions < i; warp w scans the 32-expert groups w, w + warps, ...
   for (int g = warp; 32 * g < p.E; g += THREADS / 32) {
     const int i = 32 * g + lane;
-    const int cnt = i < p.E ? cnts[order[i]] : 0;
+    int begin, cnt = 0;
+    if (p.sort_tiles) {
+      if (i < p.E) cnt = cnts[order[i]];
+    } else if (i < p.E) {
+      fetch(i, begin, cnt);
+      order[i] = i;
+    }
     const int tiles = (cnt + kMaxTileRows - 1) / kMaxTileRows;
     int incl = tiles;
 #pragma unroll
@@ -196,8 +214,9 @@ __device__ __forceinline__ void build_tile_list(const StreamParams& p, int* pref
       if (lane >= off) incl += n;
     }
     if (i < p.E) prefix[i] = incl - tiles;
-    if (lane == 31) chunk_sum[g] = incl;
+    if (lane == 31) (p.E <= 32 ? prefix[p.E] : chunk_sum[g]) = incl;
   }
+  if (p.E <= 32) return;
   __syncthreads();
   for (int g = warp; 32 * g < p.E; g += THREADS / 32) {
     int before = lane < g ? chunk_sum[lane] : 0;  // at most 32 groups
@@ -300,8 +319,7 @@ inline cudaError_t update_plan(StreamPlan& plan, const GemmProblem& p, const Gem
       const int chunks = (dense->rows + kMaxTileRows - 1) / kMaxTileRows;
       const int chunk = ((dense->rows + chunks - 1) / chunks + 15) & ~15;
       const int last = (dense->rows - (chunks - 1) * chunk + 15) & ~15;
-      if (!encode_x(&plan.xm.x2[chunk / 16 - 1], k, chunk / 16 - 1)) return cudaErrorInvalidValue;
-      if (last != chunk && !encode_x(&plan.xm.x2[last / 16 - 1], k, last / 16 - 1)) return cudaErrorInvalidValue;
+      if (!encode_x(&plan.xm.x2[0], k, chunk / 16 - 1) || !encode_x(&plan.xm.x2[1], k, last / 16 - 1)) return cudaErrorInvalidValue;
     }
     plan.key2 = k;
   }
