@@ -293,6 +293,14 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
       }
       if (!ok && lane == 0) give_up();
     }
+    if (lane == 0 && leader) {
+      // this pair takes no more tiles; the last one that says so puts the counters back for the next launch that uses them
+      __threadfence();
+      if (atomicAdd(p.done_ctr, 1) == (int)gridDim.x / 2 - 1) {
+        *p.done_ctr = 0;
+        *p.tile_ctr = 0;
+      }
+    }
   } else if (warp == kMmaWarp) {
     // ================================================================= MMA issuer (leader)
     if (leader) {
@@ -479,14 +487,6 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
   }
   cluster_sync();  // nothing of the other CTA's is on its way to this one's barriers
-  if (threadIdx.x == 0 && leader) {
-    // the last pair to get here puts the counters back for the next launch that uses them
-    __threadfence();
-    if (atomicAdd(p.done_ctr, 1) == (int)gridDim.x / 2 - 1) {
-      *p.done_ctr = 0;
-      *p.tile_ctr = 0;
-    }
-  }
   if (warp == kMmaWarp) {
     __syncwarp();
     tc_fence_after();

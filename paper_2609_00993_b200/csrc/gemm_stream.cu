@@ -311,6 +311,18 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       }
 #endif
     }
+    if (lane == 0) {
+      // This CTA takes no more tiles.  The last one that says so puts the counters back for the next launch that uses them
+      // -- here, beside the last tile's MMAs and epilogue, because at the CTA's end the next kernel waits for it (0.7 us).
+      // After a stop on request the tile counter stays: the next launch of the pass goes on where this one stopped.
+      if (*stopped_here) atomicAdd(p.stopped, 1);
+      __threadfence();
+      if (atomicAdd(p.done_ctr, 1) == (int)gridDim.x - 1) {
+        const bool any_stopped = p.stopped != nullptr && *reinterpret_cast<volatile int*>(p.stopped) != 0;
+        *p.done_ctr = 0;
+        if (!any_stopped) *p.tile_ctr = 0;
+      }
+    }
   } else if (warp >= kMmaWarp) {
     // ================================================================= MMA issuer
     {
@@ -583,17 +595,6 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0) PROF_STAMP(6);
-  if (threadIdx.x == 0) {
-    // The last CTA to get here puts the counters back for the next launch that uses them.  After a stop on request
-    // the tile counter stays: the next launch of the pass goes on where this one stopped taking tiles.
-    if (*stopped_here) atomicAdd(p.stopped, 1);
-    __threadfence();
-    if (atomicAdd(p.done_ctr, 1) == (int)gridDim.x - 1) {
-      const bool any_stopped = p.stopped != nullptr && *reinterpret_cast<volatile int*>(p.stopped) != 0;
-      *p.done_ctr = 0;
-      if (!any_stopped) *p.tile_ctr = 0;
-    }
-  }
   if (*abort_flag) {
     // give copies still in flight time to land in this CTA's shared memory before it is released
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
