@@ -69,8 +69,9 @@ typedef enum {
  * the step's rows per expert R = T * top_k / n_experts, the pass's K (hidden for the gated pass, inter for the down pass)
  * and its number of tiles: small-M for every problem of up to 8192 rows and, above that, wherever it was measured ahead
  * (with bf16 the gated pass unless K or the tiles are few, and the down pass unless K is short; with FP8 where K is long or
- * R is small); large-M otherwise -- a function of T and the context's configuration alone, so a step captured in a CUDA
- * graph replays the kernels it was captured with. */
+ * R is small); large-M otherwise.  Above 8192 rows a context without an SM budget first asks for a third kernel, small-M with
+ * a tile shared by two SMs, which AUTO alone takes, where that was measured ahead of both.  All of it is a function of T and
+ * the context's configuration alone, so a step captured in a CUDA graph replays the kernels it was captured with. */
 typedef enum {
   MOE_GEMM_AUTO = 0,
   MOE_GEMM_LARGE_M = 1,  /* tokens fill the 128-row MMA dimension; for experts of many hundreds of rows,

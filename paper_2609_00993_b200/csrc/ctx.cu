@@ -61,7 +61,7 @@ struct Layout {
 // Status block at the start of the workspace: word 0 the device status, word 1 the count of CTAs that stopped on a
 // yield request in the last preemptible launch, word 2 the yield request itself (device memory: every CTA polls it
 // before each tile, which a word in host memory would not survive -- 148 SMs reading it over PCIe serialise), and
-// from byte 64 on four pairs {next tile, CTAs finished} that the small-M GEMM launches use in rotation.
+// from byte 64 on four pairs {next tile, CTAs that take no more} that the swap-AB GEMM launches use in rotation.
 constexpr size_t kStatusBlock = 8192;
 constexpr size_t kTileCounterOffset = 64;
 constexpr int kTileCounterPairs = 4;
@@ -215,7 +215,7 @@ struct moe_ctx {
   bool offsets_fresh; // the kernel right before the gated pass wrote the step's offsets (moe_layer, a few tokens)
   bool unmarked;      // launches have been enqueued since `done` was last recorded
   int calls_open;     // entry points being executed (the calls of a whole step are made by another)
-  moe::StreamPlan* plans[2][4];  // tensor maps of the small-M GEMM: [buffer set][2 * (dense problem by itself) + down pass]
+  moe::StreamPlan* plans[2][4];  // tensor maps of the swap-AB GEMMs: [buffer set][2 * (dense problem by itself) + down pass]
   unsigned long long wait_limit_ns;  // time limit of every bounded device-side wait (0 = the kernels' default)
   bool debug_stall;                  // failure-detection hook: the GEMM producers issue no copies
   char err[256];
@@ -1067,7 +1067,12 @@ moe_status moe_grouped_ffn_fp8(moe_ctx* ctx, const void* wq_gate_up, const float
   return MOE_OK;
 }
 
-moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_perm, int32_t T, void* out) {
+}  // extern "C"
+
+namespace {
+
+// settled: topk_w and inv_perm are older than the down pass (a whole step's, which nothing came between)
+moe_status combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_perm, int32_t T, void* out, bool settled) {
   if (!ctx) return MOE_ERR_INVALID_ARG;
   if (ctx->state != ST_FFN_DONE) return fail(ctx, MOE_ERR_STATE, "moe_combine needs moe_grouped_ffn in the same step");
   if (T != ctx->T) return fail(ctx, MOE_ERR_INVALID_ARG, "T = %d differs from the layout's T = %d", T, ctx->T);
@@ -1083,7 +1088,7 @@ moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_per
     StageTimer tm(ctx, 7);
     e = moe::launch_combine(b.y_perm, ctx->cfg.n_shared ? b.y_shared : nullptr, inv_perm ? inv_perm : ctx->inv_perm,
                             topk_w, out, T, ctx->cfg.top_k, ctx->cfg.hidden, ctx->status, ctx->stream, &n,
-                            ctx->wait_limit_ns);
+                            ctx->wait_limit_ns, 0, -1, settled);
   }
   if (e != cudaSuccess) return cuda_fail(ctx, e, "moe_combine");
   ctx->state = ST_IDLE;
@@ -1091,6 +1096,14 @@ moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_per
   if (ctx->n_sets == 2) ctx->cur ^= 1;  // D: the next step works in the other buffer set
   mark(ctx, n);
   return MOE_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_perm, int32_t T, void* out) {
+  return combine(ctx, topk_w, inv_perm, T, out, false);
 }
 
 }  // extern "C"
@@ -1143,7 +1156,7 @@ moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias
   PositionMark position(ctx);
   moe_status st = route_and_dispatch(ctx, "moe_layer", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
   if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T);
-  if (st == MOE_OK) st = moe_combine(ctx, topk_w, inv_perm, T, out);
+  if (st == MOE_OK) st = combine(ctx, topk_w, inv_perm, T, out, ctx->seg_experts == 0 && !ctx->preemptible);
   return st;
 }
 
@@ -1158,7 +1171,7 @@ moe_status moe_layer_fp8(moe_ctx* ctx, const float* logits, const float* select_
       route_and_dispatch(ctx, "moe_layer_fp8", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
   if (st == MOE_OK)
     st = moe_grouped_ffn_fp8(ctx, wq_gate_up, sw_gate_up, wq_down, sw_down, wsq_gate_up, sws_gate_up, wsq_down, sws_down, T);
-  if (st == MOE_OK) st = moe_combine(ctx, topk_w, inv_perm, T, out);
+  if (st == MOE_OK) st = combine(ctx, topk_w, inv_perm, T, out, ctx->seg_experts == 0 && !ctx->preemptible);
   return st;
 }
 

@@ -103,12 +103,13 @@ cudaError_t launch_small_dispatch(const float* logits, const float* bias, int T,
 // wait_limit_ns: time limit of the kernels' bounded waits (0 = the default of 2 s).
 cudaError_t launch_permute(const void* x, const int32_t* inv_perm, void* x_perm, int T, int k, int H, int* status,
                            cudaStream_t stream, int* n_launches, unsigned long long wait_limit_ns = 0);
-// Columns [c_begin, c_end) of the rows (c_end < 0: all; multiples of 8).
+// Columns [c_begin, c_end) of the rows (c_end < 0: all; multiples of 8).  settled: inv_perm and topk_w were final before the
+// previous kernel of the stream started, so the kernel may read its first ones before it waits.
 cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32_t* inv_perm, const float* topk_w,
                            void* out, int T, int k, int H, int* status, cudaStream_t stream, int* n_launches,
-                           unsigned long long wait_limit_ns = 0, int c_begin = 0, int c_end = -1);
+                           unsigned long long wait_limit_ns = 0, int c_begin = 0, int c_end = -1, bool settled = false);
 
-// Tensor maps of one small-M GEMM launch (host memory, opaque outside gemm_stream.cu).  A context keeps one plan per
+// Tensor maps of one launch of the swap-AB kernels (host memory, opaque outside swap_ab.cuh).  A context keeps one plan per
 // buffer set and pass; a launch whose operands (addresses and shapes) are the plan's re-encodes nothing.  (Looking 34
 // maps up per launch in a locked table costs 3.4 us of host time, in steps that take the GPU 20.)
 struct StreamPlan;
@@ -150,9 +151,9 @@ struct GemmProblem {
   // failure-detection hook (the TMA producer issues nothing, so every consumer wait runs into the limit).
   unsigned long long wait_limit_ns = 0;
   bool debug_stall = false;
-  // Small-M kernel: two words of device memory, {next tile, CTAs finished}, zero before the launch; the launch's CTAs
-  // take their tiles from the first (an atomic counter over the size-ordered tile list) and the last CTA to finish
-  // puts both back to zero.  Consecutive launches of a stream must use different pairs: with the launch overlap the
+  // Swap-AB kernels: two words of device memory, {next tile, CTAs (pairs) that take no more}, zero before the launch; the
+  // launch's CTAs take their tiles from the first (an atomic counter over the size-ordered tile list) and the last one that
+  // finds none left puts both back to zero.  Consecutive launches of a stream must use different pairs: with the launch overlap the
   // next kernel's CTAs take tiles while this one's are still finishing.
   int* tile_counters = nullptr;
   // Preemption at tile granularity (small-M kernel only; both null = off).  Before it takes a tile a CTA reads
@@ -171,7 +172,7 @@ struct GemmProblem {
   // Upper bound on the rows of any one group (a token reaches an expert at most once, so T), or 0 if unknown.  With
   // at most 16, every non-empty group is one tile of the same cost and the small-M kernel skips ordering them.
   int32_t max_group_rows = 0;
-  StreamPlan* plan = nullptr;  // small-M kernel: the launch's tensor maps
+  StreamPlan* plan = nullptr;  // swap-AB kernels: the launch's tensor maps
 };
 
 // A dense group (the shared expert) that rides in the same launch as a grouped problem: its tiles are added

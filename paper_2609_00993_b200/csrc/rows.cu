@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kCombineThreads)
 combine_kernel(const __nv_bfloat16* __restrict__ y_perm, const __nv_bfloat16* __restrict__ y_shared,
                const int32_t* __restrict__ inv_perm, const float* __restrict__ topk_w, __nv_bfloat16* __restrict__ out,
                int T, int k, int H, int c_begin, int c_end, int col_blocks, int chunk_bytes, int stage_bytes, int n_stages,
-               int* status, unsigned long long wait_limit_ns) {
+               int* status, unsigned long long wait_limit_ns, bool settled) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
   const uint32_t bar_full = base + (uint32_t)(n_stages * stage_bytes);
@@ -183,6 +183,14 @@ combine_kernel(const __nv_bfloat16* __restrict__ y_perm, const __nv_bfloat16* __
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
+  // the first item's rows and weights, where they are older than the kernel before this one (launch_combine)
+  int first_row = -1;
+  float first_w = 0.f;
+  if (settled && warp == kCombineConsumers / 32 && lane < k) {
+    const size_t slot = (size_t)(blockIdx.x / col_blocks) * k + lane;  // (the grid is no larger than the items)
+    first_row = inv_perm[slot];
+    first_w = topk_w[slot];
+  }
   pdl_wait();
   pdl_launch_dependents();
 
@@ -194,9 +202,9 @@ combine_kernel(const __nv_bfloat16* __restrict__ y_perm, const __nv_bfloat16* __
       const int t = (int)(it / col_blocks), c0 = c_begin + (int)(it % col_blocks) * kCombineChunkCols;
       const uint32_t bytes = (uint32_t)(min(kCombineChunkCols, c_end - c0) * 2);
       const uint32_t s = (uint32_t)(n % n_stages), ph = (uint32_t)((n / n_stages) & 1);
-      int row = -1;
-      float wv = 0.f;
-      if (lane < k) {
+      int row = first_row;
+      float wv = first_w;
+      if (lane < k && !(settled && n == 0)) {
         row = __ldg(inv_perm + (size_t)t * k + lane);
         wv = __ldg(topk_w + (size_t)t * k + lane);
       }
@@ -302,7 +310,7 @@ cudaError_t launch_permute(const void* x, const int32_t* inv_perm, void* x_perm,
 
 cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32_t* inv_perm, const float* topk_w,
                            void* out, int T, int k, int H, int* status, cudaStream_t stream, int* n_launches,
-                           unsigned long long wait_limit_ns, int c_begin, int c_end) {
+                           unsigned long long wait_limit_ns, int c_begin, int c_end, bool settled) {
   if (c_end < 0) c_end = H;
   if (T <= 0 || c_begin >= c_end) return cudaSuccess;
   if (k > 32 || c_begin < 0 || c_end > H || c_begin % 8 != 0 || c_end % 8 != 0) return cudaErrorNotSupported;  // one gathering lane per row
@@ -323,7 +331,7 @@ cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32
     return launch_pdl(true, kern, dim3(grid), dim3(kCombineThreads), smem, stream, static_cast<const __nv_bfloat16*>(y_perm),
                       static_cast<const __nv_bfloat16*>(y_shared), inv_perm, topk_w, static_cast<__nv_bfloat16*>(out), T, k,
                       H, c_begin, c_end, col_blocks, chunk_bytes, stage_bytes, stages, status,
-                      wait_limit_ns ? wait_limit_ns : kWaitLimitNs);
+                      wait_limit_ns ? wait_limit_ns : kWaitLimitNs, settled);
   };
   cudaError_t err = k == 8 ? launch(combine_kernel<8>) : k == 4 ? launch(combine_kernel<4>)
                   : k == 2 ? launch(combine_kernel<2>) : launch(combine_kernel<0>);

@@ -29,6 +29,8 @@ inline int64_t layout_chunk_slots(int64_t n_slots, int E) {
 // kernel reads an expert's weights once for up to 256 rows, multiplies exactly the rows there are and moves fewer bytes per
 // flop; the large-M kernel multiplies rows in steps of 128, but its tiles are half as large and its epilogue always overlaps
 // the next tile, which counts where K is short.  Both draw the GPU's power limit in steps of a millisecond and more.
+// (Measured with an epilogue of the small-M kernel that took twice as long as today's, before pair_is_faster, below, was asked
+// first: the sizes at which the small-M kernel lost by its epilogue are now mostly the pair kernel's.)
 // Whole steps in the sustained state, us, gated pass / down pass on s = small-M, l = large-M; "K / K' x E" is a layer of
 // hidden K, inter K' and E experts (the gated pass has K and K' features, the down pass K' and K).
 //   bf16, gated pass (sl : ll)

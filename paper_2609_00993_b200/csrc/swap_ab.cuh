@@ -44,8 +44,8 @@ struct StreamParams {
   const float* row_scale2;
   const float* w_scale;
   const float* w_scale2;
-  // The launch's tile counter and the count of CTAs that have finished (two words in device memory, zero before the
-  // first launch that uses them; the last CTA to finish puts them back to zero).
+  // The launch's tile counter and the count of CTAs (pairs) that take no more tiles (two words in device memory, zero
+  // before the first launch that uses them; the last one puts them back to zero).
   int* tile_ctr;
   int* done_ctr;
   int32_t all_dynamic;  // every tile comes from the counter (a pass that may be launched again to go on)
