@@ -369,7 +369,7 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     const int fr_row = lane >> 2, fr_col = 2 * (lane & 3);                                     // its feature and token
     for (;;) {
       const uint32_t q = tcount % kQ;
-      if (!mbar_wait(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) { ok = false; break; }
+      if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) { ok = false; break; }
       const STile t = tq[q];
       __syncwarp();
       if (lane == 0) arrive_remote(tqempty_at_leader + 8u * q);
@@ -399,7 +399,7 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         }
         fetch_scales(c_first);
       }
-      if (!mbar_wait(bar_tfull + 8u * acc, acc_phase, abort_flag, limit)) { ok = false; break; }
+      if (!mbar_wait_warp(bar_tfull + 8u * acc, acc_phase, abort_flag, limit)) { ok = false; break; }
       tc_fence_after();
       const uint32_t d = tmem_base + acc * kAccCols + ((uint32_t)(lg * 32) << 16);
       auto release_acc = [&]() {  // hand the accumulator back to the MMA issuer

@@ -453,7 +453,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
     uint32_t tcount = 0;
     for (;;) {
       const uint32_t q = tcount % kQ;
-      if (!mbar_wait(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) {
+      if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) {
         ok = false;
         break;
       }
@@ -491,8 +491,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       }
       uint32_t h = 0, d_a, d_b;
       if (big) {
-        if (!mbar_wait(bar_tfull, use0 & 1u, abort_flag, limit) ||
-            !mbar_wait(bar_tfull + 8u, use1 & 1u, abort_flag, limit)) { ok = false; break; }
+        if (!mbar_wait_warp(bar_tfull, use0 & 1u, abort_flag, limit) ||
+            !mbar_wait_warp(bar_tfull + 8u, use1 & 1u, abort_flag, limit)) { ok = false; break; }
         ++use0;
         ++use1;
         d_a = tmem_base;
@@ -500,7 +500,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
       } else {
         h = next_half;
         next_half ^= 1u;
-        if (!mbar_wait(bar_tfull + 8u * h, (h ? use1 : use0) & 1u, abort_flag, limit)) { ok = false; break; }
+        if (!mbar_wait_warp(bar_tfull + 8u * h, (h ? use1 : use0) & 1u, abort_flag, limit)) { ok = false; break; }
         if (h) ++use1; else ++use0;
         d_a = tmem_base + 256u * h;
         d_b = d_a + 128u;

@@ -378,7 +378,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         reinterpret_cast<float4*>(sc)[32 + lane] = hi;
         __syncwarp();
       }
-      if (!mbar_wait(bar_tfull + 8u * as, aph, abort_flag, p.wait_limit_ns)) { ok = false; break; }
+      if (!mbar_wait_warp(bar_tfull + 8u * as, aph, abort_flag, p.wait_limit_ns)) { ok = false; break; }
       tc_fence_after();
       const uint32_t d0 = tmem_base + as * acc_cols + lane_base;
       bool released = false;  // has this warp already handed the accumulator stage back?
