@@ -406,6 +406,13 @@ moe_status moe_ctx_debug_ptrs(moe_ctx* ctx, void** x_perm, void** act, void** y_
  * (codes [N,H] / [N,I] uint8, scales [N] fp32).  Any out-pointer may be NULL. */
 moe_status moe_ctx_debug_ptrs_fp8(moe_ctx* ctx, void** xq, float** sx, void** aq, float** sa);
 
+/* Test/inspection only, host state: the kernels that the last routed gated pass and the last routed down pass were launched
+ * with (MOE_GEMM_*, or MOE_KERNEL_PAIR for the kernel that AUTO alone takes; MOE_GEMM_AUTO before the first), and how many
+ * tensor maps of the small-M and the pair kernel the context has encoded (none in a step whose operands are those of an
+ * earlier step on the same kernel).  Any out-pointer may be NULL. */
+#define MOE_KERNEL_PAIR 100
+moe_status moe_ctx_debug_gemm(const moe_ctx* ctx, int32_t* gated, int32_t* down, int64_t* maps_encoded);
+
 /* Per-stage device timing (measurement aid; off by default).  While enabled, every stage's launches are
  * bracketed by CUDA events on the context's stream.  moe_ctx_read_profile synchronises the stream, returns
  * the summed device time and the number of bracketed launches per stage since the last read, and resets.

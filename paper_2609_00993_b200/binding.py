@@ -20,6 +20,7 @@ MOE_OK = 0
 MOE_ERR_INVALID_ARG, MOE_ERR_CAPACITY, MOE_ERR_STATE, MOE_ERR_UNSUPPORTED = 1, 2, 3, 4
 MOE_ERR_CUDA, MOE_ERR_TIMEOUT, MOE_ERR_BAD_INDEX = 5, 6, 7
 MOE_GEMM_AUTO, MOE_GEMM_LARGE_M, MOE_GEMM_SMALL_M, MOE_GEMM_VALIDATION = 0, 1, 2, 3
+MOE_KERNEL_PAIR = 100
 MOE_WEIGHTS_BF16, MOE_WEIGHTS_FP8_E4M3 = 0, 1
 MOE_BOUNDARY_YIELD = -1
 
@@ -30,7 +31,7 @@ STATUS_NAMES = {0: "MOE_OK", 1: "MOE_ERR_INVALID_ARG", 2: "MOE_ERR_CAPACITY", 3:
 EXPORTS = ("moe_version", "moe_ctx_workspace_bytes", "moe_ctx_create", "moe_ctx_destroy", "moe_ctx_status",
            "moe_last_error", "moe_route", "moe_dispatch_layout", "moe_grouped_ffn", "moe_grouped_ffn_fp8", "moe_combine",
            "moe_layer", "moe_layer_fp8", "moe_layer_host", "moe_layer_host_submit", "moe_layer_host_wait",
-           "moe_ctx_debug_ptrs", "moe_ctx_debug_ptrs_fp8", "moe_ctx_launch_count", "moe_ctx_set_profiling", "moe_ctx_read_profile",
+           "moe_ctx_debug_ptrs", "moe_ctx_debug_ptrs_fp8", "moe_ctx_debug_gemm", "moe_ctx_launch_count", "moe_ctx_set_profiling", "moe_ctx_read_profile",
            "moe_dispatch_layout_static", "moe_ctx_set_segments", "moe_ctx_abandon_step", "moe_turnstile_create", "moe_turnstile_destroy",
            "moe_turnstile_set_span", "moe_turnstile_begin_epoch", "moe_turnstile_publish", "moe_turnstile_task_done",
            "moe_turnstile_d_enter", "moe_turnstile_d_release", "moe_turnstile_state", "moe_ctx_set_wait_limit",
@@ -111,6 +112,8 @@ def load_library() -> ctypes.CDLL:
     lib.moe_layer_host_wait.argtypes = [vp, i32]
     lib.moe_ctx_debug_ptrs.restype = i32
     lib.moe_ctx_debug_ptrs.argtypes = [vp] + [ctypes.POINTER(vp)] * 6
+    lib.moe_ctx_debug_gemm.restype = i32
+    lib.moe_ctx_debug_gemm.argtypes = [vp, ctypes.POINTER(i32), ctypes.POINTER(i32), ctypes.POINTER(i64)]
     lib.moe_ctx_abandon_step.restype = i32
     lib.moe_ctx_abandon_step.argtypes = [vp]
     lib.moe_ctx_launch_count.restype = i64
@@ -393,6 +396,12 @@ class MoeContext:
         esz = torch.empty(0, dtype=dtype).element_size()
         off = p.value - self.workspace.data_ptr()
         return self.workspace[off:off + n * esz].view(dtype).view(*shape)
+
+    def moe_ctx_debug_gemm(self) -> dict:
+        """Kernels of the last routed passes and the number of tensor maps encoded so far (host state)."""
+        gated, down, maps = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int64()
+        self._check(self.lib.moe_ctx_debug_gemm(self.handle, ctypes.byref(gated), ctypes.byref(down), ctypes.byref(maps)))
+        return {"gated": gated.value, "down": down.value, "maps_encoded": maps.value}
 
     def _step_tensors(self, T, k, E, device, bufs, out):
         """Allocates the step's arrays and output when the caller passes none.  torch allocates on its current

@@ -215,7 +215,10 @@ struct moe_ctx {
   bool offsets_fresh; // the kernel right before the gated pass wrote the step's offsets (moe_layer, a few tokens)
   bool unmarked;      // launches have been enqueued since `done` was last recorded
   int calls_open;     // entry points being executed (the calls of a whole step are made by another)
-  moe::StreamPlan* plans[2][4];  // tensor maps of the swap-AB GEMMs: [buffer set][2 * (dense problem by itself) + down pass]
+  // tensor maps of the swap-AB GEMMs: [buffer set][4 * (two-CTA kernel) + 2 * (dense problem by itself) + down pass]; one plan
+  // per kernel, so that calls that take the one and the other in turn each find theirs
+  moe::StreamPlan* plans[2][8];
+  int gemm_taken[2];  // kernels of the last routed passes, gated and down (moe_ctx_debug_gemm)
   unsigned long long wait_limit_ns;  // time limit of every bounded device-side wait (0 = the kernels' default)
   bool debug_stall;                  // failure-detection hook: the GEMM producers issue no copies
   char err[256];
@@ -334,7 +337,7 @@ int gemm_ctas(const moe_ctx* ctx) {
 constexpr size_t kHostOverlapBytes = 512 * 1024, kHostPieceBytes = 1536 * 1024, kHostChunkBytes = 4 << 20;
 constexpr int kHostMaxPieces = 4, kHostChunkFromRows = 200;
 
-constexpr int kGemmPair = 100;  // (beside the public variants: the two-CTA kernel, which AUTO alone takes)
+constexpr int kGemmPair = MOE_KERNEL_PAIR;  // (beside the public variants: the two-CTA kernel, which AUTO alone takes)
 
 // AUTO: a DECODE context always streams; a PREFILL context chooses per launch from the problem's rows (T * top_k
 // rows over n_experts; T rows over one group for the shared expert by itself) and K: the choice is a function of T
@@ -373,7 +376,8 @@ cudaError_t run_gemm(moe_ctx* ctx, moe::GemmProblem p, const moe::GemmDenseGroup
   p.offsets_settled = !(ctx->offsets_fresh && p.gated);
   p.tile_counters = reinterpret_cast<int*>(ctx->ws + kTileCounterOffset) + 2 * (ctx->gemm_seq++ % kTileCounterPairs);
   p.max_group_rows = T;
-  p.plan = ctx->plans[ctx->cur][(p.offsets == nullptr ? 2 : 0) + (p.gated ? 0 : 1)];
+  p.plan = ctx->plans[ctx->cur][(variant == kGemmPair ? 4 : 0) + (p.offsets == nullptr ? 2 : 0) + (p.gated ? 0 : 1)];
+  if (p.offsets != nullptr) ctx->gemm_taken[p.gated ? 0 : 1] = variant;
   if (variant == MOE_GEMM_VALIDATION) {
     cudaError_t e = moe::launch_gemm_validation(p, ctx->stream, n);
     if (e == cudaSuccess && dense != nullptr) {
@@ -494,11 +498,12 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
   ctx->calls_open = 0;
   ctx->offsets_fresh = false;
   bool have_plans = true;
-  for (int i = 0; i < 8; ++i) {
-    moe::StreamPlan*& plan = ctx->plans[i / 4][i % 4];
-    plan = i / 4 < l.n_sets ? moe::stream_plan_create() : nullptr;
-    if (i / 4 < l.n_sets && plan == nullptr) have_plans = false;
+  for (int i = 0; i < 16; ++i) {
+    moe::StreamPlan*& plan = ctx->plans[i / 8][i % 8];
+    plan = i / 8 < l.n_sets ? moe::stream_plan_create() : nullptr;
+    if (i / 8 < l.n_sets && plan == nullptr) have_plans = false;
   }
+  ctx->gemm_taken[0] = ctx->gemm_taken[1] = MOE_GEMM_AUTO;
   if (!have_plans) {
     free_ctx(ctx);
     return fail(nullptr, MOE_ERR_CUDA, "host allocation failed");
@@ -1483,6 +1488,19 @@ moe_status moe_ctx_debug_ptrs_fp8(moe_ctx* ctx, void** xq, float** sx, void** aq
   if (sx) *sx = b.sx;
   if (aq) *aq = b.aq;
   if (sa) *sa = b.sa;
+  return MOE_OK;
+}
+
+moe_status moe_ctx_debug_gemm(const moe_ctx* ctx, int32_t* gated, int32_t* down, int64_t* maps_encoded) {
+  if (!ctx) return MOE_ERR_INVALID_ARG;
+  if (gated) *gated = ctx->gemm_taken[0];
+  if (down) *down = ctx->gemm_taken[1];
+  if (maps_encoded) {
+    *maps_encoded = 0;
+    for (const auto& set : ctx->plans)
+      for (const moe::StreamPlan* plan : set)
+        if (plan != nullptr) *maps_encoded += moe::stream_plan_encoded(plan);
+  }
   return MOE_OK;
 }
 

@@ -626,6 +626,7 @@ StreamPlan* stream_plan_create() {
   return p;
 }
 void stream_plan_destroy(StreamPlan* plan) { delete plan; }
+int64_t stream_plan_encoded(const StreamPlan* plan) { return plan->encoded; }
 
 cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense, int max_ctas, int* status,
                                cudaStream_t stream, int* n_launches) {

@@ -115,6 +115,7 @@ cudaError_t launch_combine(const void* y_perm, const void* y_shared, const int32
 struct StreamPlan;
 StreamPlan* stream_plan_create();
 void stream_plan_destroy(StreamPlan* plan);
+int64_t stream_plan_encoded(const StreamPlan* plan);  // maps encoded since the plan was created
 
 // ---- a6-a8 grouped GEMM --------------------------------------------------------------------
 // One grouped GEMM pass:  out[r, :] = epilogue( A[r, :] . W[e]^T )  for r in expert e's segment.

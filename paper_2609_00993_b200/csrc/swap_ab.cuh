@@ -234,20 +234,21 @@ struct OperandKey {
   const void* A = nullptr;
   int64_t rows = 0;
   int32_t groups = 0, n_feat = 0, K = 0;
-  bool gated = false, fp8 = false, pair = false;
+  bool gated = false, fp8 = false;
   bool same_weights(const OperandKey& o) const {
-    return W == o.W && groups == o.groups && n_feat == o.n_feat && K == o.K && gated == o.gated && fp8 == o.fp8 &&
-           pair == o.pair;
+    return W == o.W && groups == o.groups && n_feat == o.n_feat && K == o.K && gated == o.gated && fp8 == o.fp8;
   }
-  bool same_rows(const OperandKey& o) const { return A == o.A && rows == o.rows && K == o.K && fp8 == o.fp8 && pair == o.pair; }
+  bool same_rows(const OperandKey& o) const { return A == o.A && rows == o.rows && K == o.K && fp8 == o.fp8; }
 };
 
 }  // namespace tc
 
+// (of one kernel: the boxes of the two-CTA kernel are not those of the other)
 struct StreamPlan {
   tc::OperandKey key, key2;  // the routed problem's and the dense group's
   CUtensorMap mw, mw2;
   tc::StreamMaps xm;
+  int64_t encoded = 0;  // maps encoded so far
 };
 
 namespace tc {
@@ -278,6 +279,7 @@ inline cudaError_t update_plan(StreamPlan& plan, const GemmProblem& p, const Gem
   const uint64_t esz = fp8 ? 1 : 2;                                // bytes per operand element
   const uint32_t box_k = (uint32_t)(fp8 ? 2 * kBlockK : kBlockK);  // 128 bytes of K per k-block row
   auto encode_w = [&](CUtensorMap* m, const OperandKey& k) {
+    ++plan.encoded;
     const uint64_t K = (uint64_t)k.K, n_feat = (uint64_t)k.n_feat, n_groups = (uint64_t)k.groups;
     if (k.gated && pair) {
       const uint64_t dims[5] = {K, 16, 2, n_feat / 16, n_groups};
@@ -297,13 +299,14 @@ inline cudaError_t update_plan(StreamPlan& plan, const GemmProblem& p, const Gem
     return encode_map(m, k.W, 3, dims, str, box, fp8);
   };
   auto encode_x = [&](CUtensorMap* m, const OperandKey& k, int b) {  // the box of a tile of 16 (b + 1) rows
+    ++plan.encoded;
     const uint64_t dims[2] = {(uint64_t)k.K, (uint64_t)k.rows};
     const uint64_t str[1] = {(uint64_t)k.K * esz};
     const uint32_t box[2] = {box_k, (pair ? 8u : 16u) * (uint32_t)(b + 1)};
     return encode_map(m, k.A, 2, dims, str, box, fp8);
   };
   {
-    const OperandKey k{p.W, p.A, p.rows_cap, groups, p.n_feat, p.K, p.gated, fp8, pair}, had = plan.key;
+    const OperandKey k{p.W, p.A, p.rows_cap, groups, p.n_feat, p.K, p.gated, fp8}, had = plan.key;
     plan.key = OperandKey{};  // a failure half way leaves no valid key
     if (!had.same_weights(k) && !encode_w(&plan.mw, k)) return cudaErrorInvalidValue;
     if (!had.same_rows(k))
@@ -312,7 +315,7 @@ inline cudaError_t update_plan(StreamPlan& plan, const GemmProblem& p, const Gem
     plan.key = k;
   }
   if (dense != nullptr) {
-    const OperandKey k{dense->W, dense->A, dense->rows, 1, dense->n_feat, dense->K, p.gated, fp8, pair}, had = plan.key2;
+    const OperandKey k{dense->W, dense->A, dense->rows, 1, dense->n_feat, dense->K, p.gated, fp8}, had = plan.key2;
     plan.key2 = OperandKey{};
     if (!had.same_weights(k) && !encode_w(&plan.mw2, k)) return cudaErrorInvalidValue;
     if (!had.same_rows(k)) {
