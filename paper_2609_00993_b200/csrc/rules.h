@@ -29,8 +29,12 @@ inline int64_t layout_chunk_slots(int64_t n_slots, int E) {
 // kernel reads an expert's weights once for up to 256 rows, multiplies exactly the rows there are and moves fewer bytes per
 // flop; the large-M kernel multiplies rows in steps of 128, but its tiles are half as large and its epilogue always overlaps
 // the next tile, which counts where K is short.  Both draw the GPU's power limit in steps of a millisecond and more.
-// (Measured with an epilogue of the small-M kernel that took twice as long as today's, before pair_is_faster, below, was asked
-// first: the sizes at which the small-M kernel lost by its epilogue are now mostly the pair kernel's.)
+// Measured with an epilogue of the small-M kernel that took twice as long as today's.  A context that has all SMs asks
+// pair_is_faster, below, first; one with an SM budget goes by these lines alone.  Measured again with budgets of 48, 74 and 100
+// SMs, 96 layers and sizes, today's kernels: the choice is within 1.5 % of the best of the four combinations in 77 of them.  It is
+// behind with FP8 where the large-M kernel multiplies much padding (2048 / 768 x 128, 162 rows per expert, that is 256: ll
+// against ss 1.14 with every budget, 281 rows 1.03; 2560 / 1024 x 512, 187 rows sl 1.06 with 100 SMs), and with 48 SMs where experts
+// have half a large-M tile of rows (64: ss 1.08, with FP8 1.15; 72: sl 1.05).
 // Whole steps in the sustained state, us, gated pass / down pass on s = small-M, l = large-M; "K / K' x E" is a layer of
 // hidden K, inter K' and E experts (the gated pass has K and K' features, the down pass K' and K).
 //   bf16, gated pass (sl : ll)
@@ -88,27 +92,75 @@ inline bool small_m_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t r
 // It multiplies exactly the rows there are, like the small-M kernel, and every epilogue overlaps the next tile, like the
 // large-M kernel's; but a tile's operands come in the same number of bytes as the small-M kernel's (per flop) through twice as
 // many k-blocks, so with long K the small-M kernel stays ahead.  Whole steps in the sustained state, each over the best of the
-// nine combinations, gated pass / down pass on s = small-M, l = large-M, p = pairs (two runs of one differ by up to 1.5 %):
-//   bf16  2048 / 768 x 128    R = 69 ss 1.007 sl 1.000 sp 1.006 pp 1.009; 96 1.011 1.000 1.015 1.013; 162 1.021 1.065 1.009 1.000;
-//                             281 1.000 1.021 1.007 1.051; 512 1.030 1.021 1.000 1.022; 1000 1.040 1.035 1.012 1.000; 1875 1.062
-//                             1.035 1.014 1.000
-//         2560 / 1024 x 512   64 1.004 1.019 1.014 1.040; 187 1.000 1.053 1.004 1.016; 312 1.001 1.030 1.018 1.016; 469 1.000 1.021
-//                             1.002 1.035
-//         4096 / 1536 x 128   125 1.000 1.026 1.010 1.029; 375 1.000 1.033 1.012 1.033; 1000 1.014 1.029 1.000 1.038
-//         7168 / 2048 x 256   64 1.015 1.058 1.019 1.045; 128 1.008 1.048 1.000 1.031; 250 1.010 1.050 1.000 1.042; 500 1.024 1.017
-//          + shared           1.000 1.097; 937 1.037 1.009 1.000 1.111
-//         1024 / 512 x 64     156 ss 1.051 sl 1.022 ll 1.060 pl 1.000 pp 1.003; 375 1.067 1.031 1.022 1.000 1.021; 1250 1.059 1.029
-//                             1.035 1.000 1.007;  1536 / 512 x 128  156 1.030 1.030 1.117 1.018 1.000; 625 1.048 1.009 1.048 1.000 1.010
-//         few tiles: 512 / 2048 x 8  R = 1125 ll 1.005 pl 1.038; 7500 1.018 1.015;  7168 / 512 x 8  1125 1.000 1.022; 2000 1.062 1.007
-//   FP8   2048 / 768 x 128    69 sl 1.005 ll 1.019 pl 1.003 pp 1.007; 96 1.006 1.001 1.000 1.008; 156 1.082 1.156 1.062 1.000; 250 1.023
-//                             1.043 1.017 1.000; 375 1.022 1.005 1.000 1.030; 1000 1.045 1.048 1.026 1.000; 1875 1.056 1.041 1.045 1.000
-//         2560 / 1024 x 512   64 ss 1.017 sl 1.009 ps 1.010 pp 1.027; 125 1.004 1.030 1.015 1.023; 187 1.028 1.044 1.002 1.000; 312 1.008
-//                             1.005 1.000 1.003; 469 1.026 1.025 1.000 1.001
-//         4096 / 1536 x 128   125 ss 1.000 sp 1.002 ps 1.010 pp 1.015; 375 1.028 1.000 1.003 1.003; 1000 1.035 1.005 1.009 1.000
-//         7168 / 2048 x 256   128 ss 1.000 sp 1.002 pp 1.021; 250 1.005 1.000 1.015; 500 1.000 1.002 1.030; 937 1.027 1.000 1.050; skewed
-//          + shared           experts, 500 1.025 1.000 1.031
-//         1024 / 512 x 64     156 ll 1.028 pl 1.010 pp 1.000; 375 1.000 1.014 1.028; 1250 1.012 1.012 1.012
-//         2048 / 256 x 128    156 ps 1.000 pl 1.094 pp 1.000; 625 1.013 1.014 1.000
+// nine combinations, gated pass / down pass on s = small-M, l = large-M, p = pairs (ls is never near the best).  Medians of eight
+// interleaved blocks of 0.1 s; the medians of the odd and of the even blocks are up to 1.5 % apart in 40 of 53 measurements, up
+// to 2.5 % in 47, and 6.5 % at worst (steps of a millisecond and more, where a block may meet another power state).
+//                               R     ss    sl    sp    ll    lp    ps    pl    pp
+//   bf16  2048 / 768 x 128    162  1.023 1.064 1.013 1.178 1.124 1.015 1.051 1.000
+//                             281  1.000 1.017 1.013 1.095 1.084 1.038 1.047 1.046
+//                             375  1.019 1.011 1.000 1.050 1.041 1.020 1.017 1.007
+//                             512  1.019 1.017 1.000 1.087 1.048 1.019 1.023 1.004
+//         4096 / 1536 x 128   300  1.000 1.031 1.000 1.139 1.102 1.032 1.063 1.034
+//                             350  1.006 1.003 1.000 1.061 1.059 1.022 1.034 1.022
+//                             420  1.017 1.052 1.000 1.185 1.139 1.042 1.084 1.045
+//                             480  1.013 1.040 1.000 1.105 1.080 1.047 1.076 1.073
+//                             540  1.008 1.028 1.000 1.107 1.079 1.023 1.047 1.015
+//         2560 / 1536 x 128   300  1.000 1.036 1.014 1.139 1.147 1.041 1.064 1.049
+//                             375  1.003 1.010 1.000 1.078 1.067 1.007 1.028 1.006
+//                             450  1.007 1.031 1.000 1.127 1.091 1.014 1.041 1.014
+//                             540  1.005 1.026 1.002 1.079 1.058 1.003 1.025 1.000
+//         2048 / 1408 x 64    300  1.000 1.032 1.017 1.099 1.085 1.030 1.061 1.046
+//                             375  1.003 1.016 1.003 1.037 1.033 1.001 1.015 1.000
+//                             450  1.024 1.046 1.018 1.094 1.070 1.015 1.028 1.000
+//   FP8   2048 / 768 x 128    128  1.008 1.022 1.008 1.063 1.034 1.000 1.026 1.000
+//                             156  1.040 1.076 1.018 1.157 1.097 1.021 1.061 1.000
+//                             260  1.019 1.018 1.000 1.040 1.021 1.017 1.018 1.000
+//                             300  1.003 1.007 1.000 1.034 1.025 1.017 1.021 1.016
+//                             340  1.019 1.004 1.007 1.000 1.004 1.017 1.002 1.006
+//                             375  1.033 1.017 1.018 1.030 1.033 1.024 1.009 1.000
+//                             420  1.042 1.048 1.010 1.086 1.050 1.022 1.036 1.000
+//                             540  1.019 1.009 1.006 1.024 1.015 1.005 1.007 1.000
+//         2560 / 1024 x 512   125  1.000 1.030 1.013 1.099 1.075 1.023 1.048 1.030
+//                             187  1.018 1.037 1.002 1.147 1.105 1.000 1.040 1.003
+//                             312  1.003 1.000 1.000 1.049 1.041 1.008 1.021 1.007
+//         2560 / 1024 x 128   187  1.046 1.058 1.023 1.132 1.092 1.024 1.043 1.000
+//                             260  1.009 1.012 1.000 1.057 1.047 1.014 1.019 1.007
+//                             375  1.029 1.012 1.012 1.024 1.023 1.013 1.006 1.000
+//         1280 / 768 x 128    160  1.046 1.077 1.033 1.134 1.088 1.018 1.045 1.000
+//                             300  1.011 1.002 1.006 1.000 1.005 1.016 1.006 1.012
+//                             512  1.037 1.028 1.015 1.021 1.007 1.022 1.016 1.000
+//         1536 / 512 x 128    160  1.048 1.093 1.029 1.125 1.065 1.016 1.063 1.000
+//                             300  1.002 1.011 1.000 1.030 1.023 1.015 1.019 1.015
+//                             512  1.040 1.034 1.015 1.033 1.015 1.031 1.018 1.000
+//         1024 / 512 x 64     156  1.041 1.043 1.030 1.037 1.026 1.018 1.021 1.000
+//                             260  1.081 1.047 1.069 1.000 1.022 1.053 1.015 1.033
+//                             375  1.077 1.048 1.069 1.000 1.013 1.034 1.013 1.032
+//                             512  1.056 1.029 1.040 1.000 1.007 1.026 1.006 1.016
+//                             700  1.058 1.035 1.033 1.006 1.001 1.023 1.004 1.000
+//                            1250  1.053 1.031 1.032 1.000 1.001 1.017 1.003 1.005
+// An earlier sweep, the layers and sizes it has alone, two blocks each (up to 4 % apart):
+//   bf16  2048 / 768 x 128    R = 69 ss 1.007 sl 1.000 sp 1.006 pp 1.009; 96 ss 1.011 sl 1.000 sp 1.015 pp 1.013; 1000 ss 1.040 sl 1.035
+//                             sp 1.012 pp 1.000; 1875 ss 1.062 sl 1.035 sp 1.014 pp 1.000
+//         4096 / 1536 x 128   125 ss 1.000 sl 1.026 sp 1.010 pp 1.029; 1000 ss 1.014 sl 1.029 sp 1.000 pp 1.038
+//         2560 / 1024 x 512   64 ss 1.004 sl 1.019 sp 1.014 pp 1.040; 187 ss 1.000 sl 1.053 sp 1.004 pp 1.016; 312 ss 1.001 sl 1.030
+//                             sp 1.018 pp 1.016; 469 ss 1.000 sl 1.021 sp 1.002 pp 1.035
+//         7168 / 2048 x 256   64 ss 1.015 sl 1.058 sp 1.019 pp 1.045; 128 ss 1.008 sl 1.048 sp 1.000 pp 1.031; 250 ss 1.010 sl 1.050
+//          + shared           sp 1.000 pp 1.042; 500 ss 1.024 sl 1.017 sp 1.000 pp 1.097; 937 ss 1.037 sl 1.009 sp 1.000 pp 1.111
+//         1024 / 512 x 64     156 ss 1.051 sl 1.022 ll 1.060 pl 1.000 pp 1.003; 375 ss 1.067 sl 1.031 ll 1.022 pl 1.000 pp 1.021; 1250
+//                             ss 1.059 sl 1.029 ll 1.035 pl 1.000 pp 1.007
+//         1536 / 512 x 128    156 ss 1.030 sl 1.030 ll 1.117 pl 1.018 pp 1.000; 625 ss 1.048 sl 1.009 ll 1.048 pl 1.000 pp 1.010
+//         few tiles: 512 / 2048 x 8  R = 1125 ll 1.005 pl 1.038; 7500 ll 1.018 pl 1.015;  7168 / 512 x 8  1125 ll 1.000 pl 1.022; 2000
+//                             ll 1.062 pl 1.007
+//   FP8   2048 / 768 x 128    69 sl 1.005 ll 1.019 pl 1.003 pp 1.007; 96 sl 1.006 ll 1.001 pl 1.000 pp 1.008; 1000 sl 1.045 ll 1.048 pl
+//                             1.026 pp 1.000; 1875 sl 1.056 ll 1.041 pl 1.045 pp 1.000
+//         2560 / 1024 x 512   64 ss 1.017 sl 1.009 ps 1.010 pp 1.027; 469 ss 1.026 sl 1.025 ps 1.000 pp 1.001
+//         4096 / 1536 x 128   125 ss 1.000 sp 1.002 ps 1.010 pp 1.015; 375 ss 1.028 sp 1.000 ps 1.003 pp 1.003; 1000 ss 1.035 sp 1.005
+//                             ps 1.009 pp 1.000
+//         7168 / 2048 x 256   128 ss 1.000 sp 1.002 pp 1.021; 250 ss 1.005 sp 1.000 pp 1.015; 500 ss 1.000 sp 1.002 pp 1.030; 937
+//          + shared           ss 1.027 sp 1.000 pp 1.050; skewed experts, 500 ss 1.025 sp 1.000 pp 1.031
+//         2048 / 256 x 128    156 ps 1.000 pl 1.094 pp 1.000; 625 ps 1.013 pl 1.014 pp 1.000
+// FP8 down passes with the shortest K and few tiles (1024 / 512 x 64): pairs while an expert is one chunk (156 rows 70.1 us, large-M
+// 71.6), not with two (260 rows 88.2 and 86.4, 375 102.8 and 102.4, 512 129.3 and 128.3), level with three (700 165.2).
 inline bool pair_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t rows, int64_t E, int ctas) {
   const auto over = [&](int64_t r) { return rows > r * E; };
   const int64_t chunks = (rows + 255) / 256 > E ? (rows + 255) / 256 : E, feat_per_tile = gated ? 128 : 256;
@@ -119,9 +171,9 @@ inline bool pair_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t rows
     return K < 1792 ? over(96) : K < 2304 && over(768);
   }
   if (gated) return K < 1280 ? false : K < 2304 ? over(64) : K < 3072 ? over(160) : K < 5632 && over(256);
-  if (fp8) return K < 896 ? over(128) : K < 1280 ? over(180) : over(256);
+  if (fp8) return K < 640 ? over(128) && (!over(208) || half_waves >= 8) : K < 896 ? over(128) : K < 1280 ? over(180) : over(256);
   if (K < 896) return K >= 640 && over(128);
-  return K < 1280 ? over(350) : K < 1792 ? over(512) : over(96);
+  return K < 1792 ? over(350) : over(96);
 }
 
 }  // namespace moe

@@ -51,6 +51,10 @@ def _choice(H, I, E, k, T, fp8):
     (7168, 2048, 256, 8, 16000, 0, 0, 1), (4096, 1536, 128, 8, 16000, 0, 0, 1), (2560, 1024, 512, 8, 4096, 0, 0, 0),
     (2048, 768, 128, 8, 2500, 1, 1, 1), (2560, 1024, 512, 8, 12000, 1, 1, 1), (7168, 2048, 256, 8, 30000, 1, 0, 1),
     (7168, 512, 8, 2, 4500, 0, 0, 0), (512, 2048, 8, 2, 4500, 0, 0, 0),
+    (4096, 1536, 128, 8, 6720, 0, 0, 1), (4096, 1536, 128, 8, 7680, 0, 0, 1), (2560, 1536, 128, 8, 7200, 0, 0, 1),
+    (2048, 1408, 64, 6, 4800, 0, 0, 1), (2048, 1408, 64, 6, 3200, 0, 0, 0), (2560, 1536, 128, 8, 4800, 0, 0, 0),
+    (1024, 512, 64, 4, 2500, 1, 0, 1), (1024, 512, 64, 4, 4160, 1, 0, 0), (1024, 512, 64, 4, 11200, 1, 0, 1), (1536, 512, 128, 8, 2560, 1, 1, 1),
+    (2048, 768, 128, 8, 6720, 1, 1, 1), (2048, 768, 128, 8, 4160, 0, 0, 1),
 ] + [(*v[:5], int(v[7]), *v[8]) for v in LAYERS.values()])
 def test_the_rule(rules, H, I, E, k, T, fp8, gated, down):  # noqa: F811
     assert rules(*_choice(H, I, E, k, T, fp8)) == [gated, down]
@@ -158,3 +162,23 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(name):
     torch.cuda.synchronize()
     assert ctx.moe_ctx_status() == B.MOE_OK and torch.equal(again, good)
     ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,I,E,k,T,fp8,down", [
+    (2560, 1536, 24, 8, 1050, False, B.MOE_GEMM_SMALL_M), (2560, 1536, 24, 8, 1051, False, B.MOE_KERNEL_PAIR),  # 350 rows
+    (1024, 512, 147, 4, 7733, True, B.MOE_GEMM_LARGE_M), (1024, 512, 148, 4, 7733, True, B.MOE_KERNEL_PAIR),    # four waves
+])
+def test_down_passes_on_either_side_of_a_line(H, I, E, k, T, fp8, down):
+    shape = wl.LayerShape("t", T=T, H=H, E=E, k=k, I=I)
+    w, a = (wl.make_weights_fp8 if fp8 else wl.make_weights)(shape, 3, DEV), wl.make_activations(shape, 4, DEV)
+    outs = []
+    for variant in (B.MOE_GEMM_AUTO, B.MOE_GEMM_LARGE_M):
+        ctx = _ctx(shape, fp8, gemm_variant=variant)
+        torch.cuda.synchronize()
+        outs.append(_run(ctx, fp8, w, a))
+        torch.cuda.synchronize()
+        assert ctx.moe_ctx_status() == B.MOE_OK
+        assert ctx.moe_ctx_debug_gemm()["down"] == (down if variant == B.MOE_GEMM_AUTO else B.MOE_GEMM_LARGE_M)
+        ctx.close()
+    assert torch.isfinite(outs[0].float()).all() and torch.equal(*outs)
