@@ -192,13 +192,13 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
   if (warp == kMmaWarp) pair_tmem_alloc(smem_u32(tmem_slot), kTmemCols);
   pdl_wait();
   pdl_launch_dependents();
-  build_tile_list<kThreads>(p, prefix, order, beg, cnts, class_pos, chunk_sum);
+  if (leader) build_tile_list<kThreads>(p, prefix, order, beg, cnts, class_pos, chunk_sum);  // it hands the tiles to both
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // both CTAs' barriers exist
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int total_tiles = dense_tiles + prefix[p.E] * p.n_ft;
+  const int total_tiles = leader ? dense_tiles + prefix[p.E] * p.n_ft : 0;
   auto give_up = [&]() {
     *abort_flag = 1;
     store_remote(at_rank(smem_u32(const_cast<int*>(abort_flag)), rank ^ 1u), 1);
@@ -528,7 +528,7 @@ cudaError_t launch_gemm_pair(const GemmProblem& p, const GemmDenseGroup* dense, 
   auto launch = [&](auto kern) -> cudaError_t {
     cudaError_t e = ensure_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(p.rows_bound <= kGemmOverlapMaxRows, kern, dim3(2 * pairs), dim3(kThreads), smem, stream, plan.mw, plan.mw2,
+    return launch_pdl(false, kern, dim3(2 * pairs), dim3(kThreads), smem, stream, plan.mw, plan.mw2,
                       plan.xm, prm);
   };
   if (p.fp8) err = p.gated ? launch(grouped_gemm_pair_kernel<true, true>) : launch(grouped_gemm_pair_kernel<false, true>);

@@ -325,108 +325,106 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
     }
   } else if (warp >= kMmaWarp) {
     // ================================================================= MMA issuer
-    {
-      uint32_t head = 0, kb_idx = 0, use0 = 0, use1 = 0, next_half = 0;
-      bool ok = true;
-      [[maybe_unused]] long long prof_wait_full = 0, prof_wait_acc = 0, prof_tiles = 0;
-      [[maybe_unused]] const long long prof_start = clock64();
-      const uint32_t desc_hi = (uint32_t)(umma_smem_desc(0) >> 32);
-      const uint32_t lo_base = (uint32_t)umma_smem_desc(base_addr);  // slot 0
-      constexpr uint32_t lo_slot = (uint32_t)kSlotBytes >> 4, lo_box = (uint32_t)kWBoxBytes >> 4;
-      uint32_t tcount = 0;
-      for (;;) {
-        const uint32_t q = tcount % kQ;
-        if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) {
-          ok = false;
-          break;
-        }
-        const STile t = tq[q];
-        __syncwarp();
-        if (elect_one()) mbar_arrive(bar_tqempty + 8u * q);
-        ++tcount;
-        if (t.e == kNoTile) break;
-        const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
-        const bool big = n > 128u;
-        uint32_t d_a, d_b;
-        PROF_T0();
-        if (big) {
-          if (!mbar_wait_warp(bar_tempty, (use0 & 1u) ^ 1u, abort_flag, limit) ||
-              !mbar_wait_warp(bar_tempty + 8u, (use1 & 1u) ^ 1u, abort_flag, limit)) { ok = false; break; }
-          d_a = tmem_base;
-          d_b = tmem_base + 256u;
-        } else {
-          const uint32_t h = next_half;
-          next_half ^= 1u;
-          if (!mbar_wait_warp(bar_tempty + 8u * h, ((h ? use1 : use0) & 1u) ^ 1u, abort_flag, limit)) { ok = false; break; }
-          d_a = tmem_base + 256u * h;
-          d_b = d_a + 128u;
-          if (h) ++use1; else ++use0;
-        }
-        PROF_ADD(prof_wait_acc);
+    uint32_t head = 0, kb_idx = 0, use0 = 0, use1 = 0, next_half = 0;
+    bool ok = true;
+    [[maybe_unused]] long long prof_wait_full = 0, prof_wait_acc = 0, prof_tiles = 0;
+    [[maybe_unused]] const long long prof_start = clock64();
+    const uint32_t desc_hi = (uint32_t)(umma_smem_desc(0) >> 32);
+    const uint32_t lo_base = (uint32_t)umma_smem_desc(base_addr);  // slot 0
+    constexpr uint32_t lo_slot = (uint32_t)kSlotBytes >> 4, lo_box = (uint32_t)kWBoxBytes >> 4;
+    uint32_t tcount = 0;
+    for (;;) {
+      const uint32_t q = tcount % kQ;
+      if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) {
+        ok = false;
+        break;
+      }
+      const STile t = tq[q];
+      __syncwarp();
+      if (elect_one()) mbar_arrive(bar_tqempty + 8u * q);
+      ++tcount;
+      if (t.e == kNoTile) break;
+      const uint32_t n = (uint32_t)((t.rows + 15) & ~15);
+      const bool big = n > 128u;
+      uint32_t d_a, d_b;
+      PROF_T0();
+      if (big) {
+        if (!mbar_wait_warp(bar_tempty, (use0 & 1u) ^ 1u, abort_flag, limit) ||
+            !mbar_wait_warp(bar_tempty + 8u, (use1 & 1u) ^ 1u, abort_flag, limit)) { ok = false; break; }
+        d_a = tmem_base;
+        d_b = tmem_base + 256u;
+      } else {
+        const uint32_t h = next_half;
+        next_half ^= 1u;
+        if (!mbar_wait_warp(bar_tempty + 8u * h, ((h ? use1 : use0) & 1u) ^ 1u, abort_flag, limit)) { ok = false; break; }
+        d_a = tmem_base + 256u * h;
+        d_b = d_a + 128u;
+        if (h) ++use1; else ++use0;
+      }
+      PROF_ADD(prof_wait_acc);
 #ifdef MOE_STREAM_PROF
-        ++prof_tiles;
+      ++prof_tiles;
 #endif
+      tc_fence_after();
+      const uint32_t idesc = FP8 ? umma_idesc_e4m3(128, n) : umma_idesc(128, n);
+      const int num_kb = t.e == kDenseTile ? num_kb2 : num_kb1;
+      for (int kb = 0; kb < num_kb; ++kb) {
+        if (head + (uint32_t)kWSlots > R) head = 0;  // the producer's allocation, step for step
+        const uint32_t pos_w = head;
+        head += (uint32_t)kWSlots;
+        if (head + (n >> 4) > R) head = 0;
+        const uint32_t pos_x = head;
+        head += n >> 4;
+        {
+          PROF_T0();
+          const bool got = mbar_wait_warp(bar_full + 8u * (kb_idx % kNB), (kb_idx / kNB) & 1u, abort_flag, limit);
+          PROF_ADD(prof_wait_full);
+          if (!got) { ok = false; break; }
+        }
+        if (kb_idx == 0) PROF_STAMP(3);
         tc_fence_after();
-        const uint32_t idesc = FP8 ? umma_idesc_e4m3(128, n) : umma_idesc(128, n);
-        const int num_kb = t.e == kDenseTile ? num_kb2 : num_kb1;
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (head + (uint32_t)kWSlots > R) head = 0;  // the producer's allocation, step for step
-          const uint32_t pos_w = head;
-          head += (uint32_t)kWSlots;
-          if (head + (n >> 4) > R) head = 0;
-          const uint32_t pos_x = head;
-          head += n >> 4;
-          {
-            PROF_T0();
-            const bool got = mbar_wait_warp(bar_full + 8u * (kb_idx % kNB), (kb_idx / kNB) & 1u, abort_flag, limit);
-            PROF_ADD(prof_wait_full);
-            if (!got) { ok = false; break; }
-          }
-          if (kb_idx == 0) PROF_STAMP(3);
-          tc_fence_after();
-          const uint32_t lo_w0 = lo_base + pos_w * lo_slot, lo_w1 = lo_w0 + lo_box, lo_x = lo_base + pos_x * lo_slot;
-          if (elect_one()) {
-#pragma unroll
-            for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
-              const uint32_t adv = (uint32_t)((kk * kUmmaK * 2) >> 4);  // +32 bytes per MMA, in 16-byte units
-              const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
-              if (FP8) {
-                umma_e4m3_lo(d_a, lo_w0 + adv, lo_x + adv, desc_hi, idesc, acc);
-                umma_e4m3_lo(d_b, lo_w1 + adv, lo_x + adv, desc_hi, idesc, acc);
-              } else {
-                umma_bf16_lo(d_a, lo_w0 + adv, lo_x + adv, desc_hi, idesc, acc);
-                umma_bf16_lo(d_b, lo_w1 + adv, lo_x + adv, desc_hi, idesc, acc);
-              }
-            }
-            umma_commit(bar_empty + 8u * (kb_idx % kNB));  // the k-block's slots are free once these MMAs have read them
-          }
-          ++kb_idx;
-        }
-        if (!ok) break;
+        const uint32_t lo_w0 = lo_base + pos_w * lo_slot, lo_w1 = lo_w0 + lo_box, lo_x = lo_base + pos_x * lo_slot;
         if (elect_one()) {
-          umma_commit(bar_tfull + (big ? 0u : 8u * (next_half ^ 1u)));
-          if (big) umma_commit(bar_tfull + 8u);
+#pragma unroll
+          for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
+            const uint32_t adv = (uint32_t)((kk * kUmmaK * 2) >> 4);  // +32 bytes per MMA, in 16-byte units
+            const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
+            if (FP8) {
+              umma_e4m3_lo(d_a, lo_w0 + adv, lo_x + adv, desc_hi, idesc, acc);
+              umma_e4m3_lo(d_b, lo_w1 + adv, lo_x + adv, desc_hi, idesc, acc);
+            } else {
+              umma_bf16_lo(d_a, lo_w0 + adv, lo_x + adv, desc_hi, idesc, acc);
+              umma_bf16_lo(d_b, lo_w1 + adv, lo_x + adv, desc_hi, idesc, acc);
+            }
+          }
+          umma_commit(bar_empty + 8u * (kb_idx % kNB));  // the k-block's slots are free once these MMAs have read them
         }
-        if (big) {
-          ++use0;
-          ++use1;
-        }
+        ++kb_idx;
       }
-      if (!ok && lane == 0) {
-        *abort_flag = 1;
-        atomicCAS(p.status, kStOk, kStTimeout);
+      if (!ok) break;
+      if (elect_one()) {
+        umma_commit(bar_tfull + (big ? 0u : 8u * (next_half ^ 1u)));
+        if (big) umma_commit(bar_tfull + 8u);
       }
-      PROF_STAMP(4);
-#ifdef MOE_STREAM_PROF
-      if (lane == 0) {
-        atomicAdd(&g_stream_prof[8 * unit + 2], (unsigned long long)(clock64() - prof_start));
-        atomicAdd(&g_stream_prof[8 * unit + 3], (unsigned long long)prof_wait_full);
-        atomicAdd(&g_stream_prof[8 * unit + 4], (unsigned long long)prof_wait_acc);
-        atomicAdd(&g_stream_prof[8 * unit + 5], (unsigned long long)prof_tiles);
-        atomicAdd(&g_stream_prof[8 * unit + 6], (unsigned long long)kb_idx);
+      if (big) {
+        ++use0;
+        ++use1;
       }
-#endif
     }
+    if (!ok && lane == 0) {
+      *abort_flag = 1;
+      atomicCAS(p.status, kStOk, kStTimeout);
+    }
+    PROF_STAMP(4);
+#ifdef MOE_STREAM_PROF
+    if (lane == 0) {
+      atomicAdd(&g_stream_prof[8 * unit + 2], (unsigned long long)(clock64() - prof_start));
+      atomicAdd(&g_stream_prof[8 * unit + 3], (unsigned long long)prof_wait_full);
+      atomicAdd(&g_stream_prof[8 * unit + 4], (unsigned long long)prof_wait_acc);
+      atomicAdd(&g_stream_prof[8 * unit + 5], (unsigned long long)prof_tiles);
+      atomicAdd(&g_stream_prof[8 * unit + 6], (unsigned long long)kb_idx);
+    }
+#endif
   } else {
     // ================================================================= epilogue (warps 0-7)
     // TMEM lane = weight row (output feature) of each box, column = token.  A warp takes 32 features x 16 tokens at a time, in

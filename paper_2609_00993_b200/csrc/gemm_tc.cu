@@ -252,46 +252,44 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     }
   } else if (warp == kMmaWarp) {
     // ================================================================= MMA issuer
-    {
-      uint32_t tile_iter = 0;
-      RingCursor ring;
-      bool ok = true;
-      // descriptor words: only the 14-bit start-address field of the low word changes between MMAs
-      const uint32_t desc_hi = (uint32_t)(umma_smem_desc(0) >> 32);
-      const uint32_t lo_base = (uint32_t)umma_smem_desc(base_addr);  // stage 0, weight box 0
-      const uint32_t lo_stage = (uint32_t)stage_bytes >> 4, lo_box = (uint32_t)kWBoxBytes >> 4;
-      for (int tile = unit; tile < total_tiles && ok; tile += n_units, ++tile_iter) {
-        const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, seg, tile_rows);
-        const uint32_t as = tile_iter & 1u, aph = (tile_iter >> 1) & 1u;
-        if (!mbar_wait_warp(bar_tempty + 8u * as, aph ^ 1u, abort_flag, p.wait_limit_ns)) { ok = false; break; }
+    uint32_t tile_iter = 0;
+    RingCursor ring;
+    bool ok = true;
+    // descriptor words: only the 14-bit start-address field of the low word changes between MMAs
+    const uint32_t desc_hi = (uint32_t)(umma_smem_desc(0) >> 32);
+    const uint32_t lo_base = (uint32_t)umma_smem_desc(base_addr);  // stage 0, weight box 0
+    const uint32_t lo_stage = (uint32_t)stage_bytes >> 4, lo_box = (uint32_t)kWBoxBytes >> 4;
+    for (int tile = unit; tile < total_tiles && ok; tile += n_units, ++tile_iter) {
+      const Tile t = decode_tile(tile, dense_tiles, n_ft2, p.rows2, n_ft, p.ft0, p.E, prefix, seg, tile_rows);
+      const uint32_t as = tile_iter & 1u, aph = (tile_iter >> 1) & 1u;
+      if (!mbar_wait_warp(bar_tempty + 8u * as, aph ^ 1u, abort_flag, p.wait_limit_ns)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d0 = tmem_base + as * acc_cols;
+      const uint32_t idesc = FP8 ? umma_idesc_e4m3(128, 256) : umma_idesc(128, 256);
+      const int num_kb = t.dense ? num_kb2 : num_kb1;
+      for (int kb = 0; kb < num_kb; ++kb) {
+        if (!mbar_wait_warp(bar_full + 8u * ring.stage, ring.phase, abort_flag, p.wait_limit_ns)) { ok = false; break; }
+        if (GATHER) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // X rows came by cp.async
         tc_fence_after();
-        const uint32_t d0 = tmem_base + as * acc_cols;
-        const uint32_t idesc = FP8 ? umma_idesc_e4m3(128, 256) : umma_idesc(128, 256);
-        const int num_kb = t.dense ? num_kb2 : num_kb1;
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait_warp(bar_full + 8u * ring.stage, ring.phase, abort_flag, p.wait_limit_ns)) { ok = false; break; }
-          if (GATHER) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // X rows came by cp.async
-          tc_fence_after();
-          const uint32_t lo_w0 = lo_base + ring.stage * lo_stage;  // weight box 0; box 1 and the X tile follow
-          if (elect_one()) {
+        const uint32_t lo_w0 = lo_base + ring.stage * lo_stage;  // weight box 0; box 1 and the X tile follow
+        if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
-              const uint32_t adv = (uint32_t)((kk * kUmmaK * 2) >> 4);  // +32 bytes per MMA (16 bf16 or 32 E4M3), in 16-byte units
-              const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
-              // the two weight boxes are contiguous: one N = 256 operand
-              if (FP8) umma_e4m3_lo(d0, lo_w0 + 2 * lo_box + adv, lo_w0 + adv, desc_hi, idesc, acc);
-              else umma_bf16_lo(d0, lo_w0 + 2 * lo_box + adv, lo_w0 + adv, desc_hi, idesc, acc);
-            }
-            umma_commit(bar_empty + 8u * ring.stage);  // the stage is free once these MMAs have read it
+          for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
+            const uint32_t adv = (uint32_t)((kk * kUmmaK * 2) >> 4);  // +32 bytes per MMA (16 bf16 or 32 E4M3), in 16-byte units
+            const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
+            // the two weight boxes are contiguous: one N = 256 operand
+            if (FP8) umma_e4m3_lo(d0, lo_w0 + 2 * lo_box + adv, lo_w0 + adv, desc_hi, idesc, acc);
+            else umma_bf16_lo(d0, lo_w0 + 2 * lo_box + adv, lo_w0 + adv, desc_hi, idesc, acc);
           }
-          ring.advance((uint32_t)p.n_stages);
+          umma_commit(bar_empty + 8u * ring.stage);  // the stage is free once these MMAs have read it
         }
-        if (ok && elect_one()) umma_commit(bar_tfull + 8u * as);  // accumulator complete
+        ring.advance((uint32_t)p.n_stages);
       }
-      if (!ok && lane == 0) {
-        *abort_flag = 1;
-        atomicCAS(p.status, kStOk, kStTimeout);
-      }
+      if (ok && elect_one()) umma_commit(bar_tfull + 8u * as);  // accumulator complete
+    }
+    if (!ok && lane == 0) {
+      *abort_flag = 1;
+      atomicCAS(p.status, kStOk, kStTimeout);
     }
   } else if (GATHER && warp >= kGatherWarp0) {
     // ================================================================= row gather (warps 6-9)

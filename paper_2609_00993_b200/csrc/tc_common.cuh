@@ -169,15 +169,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
 // 16 lanes x 16 columns, as the fragments of four 8 x 8 matrices: lane l gets columns 2 (l % 4) and + 1 of row l / 4 (r[0],
 // r[1]), of row l / 4 + 8 (r[2], r[3]), and the same of the columns behind 8 (r[4..7])
 __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[8]) {
@@ -282,9 +273,9 @@ __device__ __forceinline__ uint32_t pack_bf16(uint64_t v) {
   return pack_bf16(f.x, f.y);
 }
 
-// Position in the ring of pipeline stages, advanced without division: the role loops run on a single thread (or
-// a few), where every dependent scalar instruction's latency is exposed, so `it % stages` and `it / stages` per
-// k-block would cost more than the tensor core needs for the k-block's MMAs.
+// Position in the ring of pipeline stages, advanced without division: a role loop is one warp, where every dependent
+// instruction's latency is exposed, so `it % stages` and `it / stages` per k-block would cost more than the tensor core needs
+// for the k-block's MMAs.
 struct RingCursor {
   uint32_t stage = 0, phase = 0;
   __device__ __forceinline__ void advance(uint32_t n_stages) {
