@@ -227,6 +227,14 @@ def _stats(vals):
     return {"p50": percentile(vals, 50), "p99": percentile(vals, 99), "max": max(vals), "n": len(vals)}
 
 
+def gemm_kernels(B, ctx):
+    """The kernels the context's last routed passes were launched with."""
+    names = {B.MOE_GEMM_LARGE_M: "grouped_gemm_tc_kernel", B.MOE_GEMM_SMALL_M: "grouped_gemm_stream_kernel",
+             B.MOE_KERNEL_PAIR: "grouped_gemm_pair_kernel", B.MOE_GEMM_VALIDATION: "validation kernel"}
+    g = ctx.moe_ctx_debug_gemm()
+    return f"gated pass {names[g['gated']]}, down pass {names[g['down']]}"
+
+
 def decode_step_bytes(counts, shape, fp8=False):
     """Algorithmic HBM bytes of one decode step from the step's own per-expert counts: the weights of every
     non-empty expert and of the shared expert once, plus the rows in, the activation out and back in, the rows
@@ -382,6 +390,7 @@ def decode_under_prefill(torch, B, wl, dev, iters, warm, peaks, w):
             p_step(i)
     prof = ctx_p.moe_ctx_read_profile()
     ctx_p.moe_ctx_set_profiling(False)
+    p_kernels = gemm_kernels(B, ctx_p)
     st_us = {n: 1e3 * ms / c for n, (ms, c) in prof.items() if c}
     counts_p = bp["counts"].cpu().double()
     H, I = wl.C4_P.H, wl.C4_P.I
@@ -395,7 +404,7 @@ def decode_under_prefill(torch, B, wl, dev, iters, warm, peaks, w):
     res["prefill_v3"] = {
         "workload": "C4-P: T=4096 on the DeepSeek-V3-shaped layer (rows per expert 0..1300, mean 128), alone",
         "ms_per_step": p_alone_ms, "tokens_per_s": wl.C4_P.T / (p_alone_ms * 1e-3), "stages_us": {k_: round(v, 1) for k_, v in st_us.items()},
-        "roofline": {"kernel": "grouped_gemm_stream_kernel (both passes)", "bound": "hbm",
+        "roofline": {"kernel": p_kernels, "bound": "hbm",
                      "achieved": w_bytes / (gemm_us * 1e-6) / 1e9, "peak": hbm, "unit": "GB/s",
                      "frac": w_bytes / (gemm_us * 1e-6) / 1e9 / hbm, "bytes_per_step": w_bytes,
                      "note": "the weights of every non-empty expert and of the shared expert once over the two GEMM passes' time"},
@@ -744,6 +753,7 @@ def run_ours(args):
     l0 = ctx.moe_ctx_launch_count()
     ms_total = timed(args.steps, step)
     launches = ctx.moe_ctx_launch_count() - l0
+    step_kernels = gemm_kernels(B, ctx)
     ms_per_step = ms_total / args.steps
     value = whole_job_rate(T, world, ms_per_step * 1e-3)
 
@@ -939,7 +949,7 @@ def run_ours(args):
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
-            "config": {"workload": workload_name(shape), "phase": "prefill (small-M GEMM variant, chosen from 512 rows per expert)",
+            "config": {"workload": workload_name(shape), "phase": f"prefill ({step_kernels})",
                        "l2": "inputs larger than L2: 1.2 GB of weights streamed per step, 4 rotating input batches",
                        "parallelism": f"replicas x{world} (no data-path collective)"},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": T * E * 4 + T * H * 2,

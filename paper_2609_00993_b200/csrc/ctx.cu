@@ -216,7 +216,8 @@ struct moe_ctx {
   bool unmarked;      // launches have been enqueued since `done` was last recorded
   int calls_open;     // entry points being executed (the calls of a whole step are made by another)
   // tensor maps of the swap-AB GEMMs: [buffer set][4 * (two-CTA kernel) + 2 * (dense problem by itself) + down pass]; one plan
-  // per kernel, so that calls that take the one and the other in turn each find theirs
+  // per kernel, so that calls that take the one and the other in turn each find theirs (host time of a 64-token step after one of
+  // 2101, which takes the other kernel: 16.9 us; 19.2 with one plan for both)
   moe::StreamPlan* plans[2][8];
   int gemm_taken[2];  // kernels of the last routed passes, gated and down (moe_ctx_debug_gemm)
   unsigned long long wait_limit_ns;  // time limit of every bounded device-side wait (0 = the kernels' default)
@@ -339,9 +340,9 @@ constexpr int kHostMaxPieces = 4, kHostChunkFromRows = 200;
 
 constexpr int kGemmPair = MOE_KERNEL_PAIR;  // (beside the public variants: the two-CTA kernel, which AUTO alone takes)
 
-// AUTO: a DECODE context always streams; a PREFILL context chooses per launch from the problem's rows (T * top_k
-// rows over n_experts; T rows over one group for the shared expert by itself) and K: the choice is a function of T
-// alone, so it is the same on every replay of a graph.
+// AUTO: a DECODE context always streams (small-M); a PREFILL context chooses among the three kernels per launch, from the
+// problem's rows (T * top_k rows over n_experts; T rows over one group for the shared expert by itself), K, features and SMs: the
+// choice is a function of T alone, so it is the same on every replay of a graph.
 int gemm_variant_of(const moe_ctx* ctx, const moe::GemmProblem& p) {
   const int v = ctx->cfg.gemm_variant;
   if (v != MOE_GEMM_AUTO) return v;
@@ -351,7 +352,13 @@ int gemm_variant_of(const moe_ctx* ctx, const moe::GemmProblem& p) {
   // problems of up to 8192 rows, whose launches overlap with their neighbours, are 1.5-6 % faster on the small-M kernel
   // at any shape: it builds its tile list and fetches weights before the previous kernel has finished
   if (p.rows_bound <= moe::kGemmOverlapMaxRows) return MOE_GEMM_SMALL_M;
-  // A context on part of the SMs shares the GPU with another, whose CTAs need not leave whole pairs of SMs free.
+  // The pair kernel's lines were drawn on all SMs; a context on part of them keeps to the other two.  What else runs on the GPU
+  // is not asked: beside decode steps on a stream of higher priority, whose CTAs need not leave whole pairs of SMs free, batches
+  // with a pair down pass are level with those of the kernel that was next (M tokens/s, decode p50 / p99 in us; decode steps of 64
+  // tokens per batch): V3-shaped, 4096 tokens, one 0.556, 2227 / 5164 against small-M 0.561, 2225 / 5168, three 0.359, 3808 / 5495
+  // against 0.358, 3818 / 5495; 16384 tokens, one 1.009, 2637 / 10740 against 1.012, 2584 / 10410, three 0.820, 6415 / 11225
+  // against 0.817, 6820 / 10834; Qwen3-shaped, 8192 tokens, one 8.64, 232 / 595 against large-M 8.55, 231 / 578, three 6.22,
+  // 399 / 588 against 6.15, 408 / 593.
   const int ctas = gemm_ctas(ctx);
   if (ctas == ctx->n_sms && moe::pair_is_faster(p.fp8, p.gated, p.K, p.n_feat, p.rows_bound, p.E, ctas)) return kGemmPair;
   return moe::small_m_is_faster(p.fp8, p.gated, p.K, p.n_feat, p.rows_bound, p.E, ctas) ? MOE_GEMM_SMALL_M : MOE_GEMM_LARGE_M;
