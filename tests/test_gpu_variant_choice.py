@@ -1,5 +1,7 @@
-"""AUTO on either side of the lines where it changes over between the small-M and the large-M kernel: whichever it takes,
-the result is that of both, bit for bit (the order of the sums is the same)."""
+"""AUTO on either side of lines of the kernel choice: whichever kernel it takes, the result is that of the small-M and the large-M
+kernel, bit for bit (the order of the sums is the same).  These contexts have all SMs, so beyond some of the lines it is the pair
+kernel that takes over, and with the shortest K the lines named below are those of an older choice; test_gpu_variant_lines.py has
+both sides of today's lines and asks which kernel ran."""
 import pytest
 import torch
 

@@ -1,5 +1,6 @@
 """AUTO on either side of the lines that depend on the number of tiles and on short K: whichever kernel it takes, the result
-is that of both, bit for bit (the order of the sums is the same).  Which one it takes is tested in test_rules_cpu.py."""
+is that of both, bit for bit (the order of the sums is the same).  Which one it takes is asked on a context with part of the
+SMs, which never takes the pair kernel."""
 import pytest
 import torch
 
