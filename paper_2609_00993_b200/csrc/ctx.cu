@@ -65,6 +65,9 @@ struct Layout {
 constexpr size_t kStatusBlock = 8192;
 constexpr size_t kTileCounterOffset = 64;
 constexpr int kTileCounterPairs = 4;
+// ... and from byte 256 on the counters of a step whose passes and combine are one launch
+constexpr size_t kStepCounterOffset = 256;
+constexpr int kStepCounterWords = (int)((kStatusBlock - kStepCounterOffset) / sizeof(int));
 
 // Walks the carve of one buffer set; with base == nullptr it only measures.
 size_t carve_set(const moe_config& c, char* base, BufferSet* out) {
@@ -219,6 +222,7 @@ struct moe_ctx {
   // per kernel, so that calls that take the one and the other in turn each find theirs (host time of a 64-token step after one of
   // 2101, which takes the other kernel: 16.9 us; 19.2 with one plan for both)
   moe::StreamPlan* plans[2][8];
+  moe::StepPlan* step_plans[2];  // ... of the launch that makes both passes and the combine, per buffer set
   int gemm_taken[2];  // kernels of the last routed passes, gated and down (moe_ctx_debug_gemm)
   unsigned long long wait_limit_ns;  // time limit of every bounded device-side wait (0 = the kernels' default)
   bool debug_stall;                  // failure-detection hook: the GEMM producers issue no copies
@@ -319,6 +323,7 @@ struct StageTimer {
 void free_ctx(moe_ctx* ctx) {
   for (auto& set : ctx->plans)
     for (moe::StreamPlan* plan : set) moe::stream_plan_destroy(plan);
+  for (moe::StepPlan* plan : ctx->step_plans) moe::step_plan_destroy(plan);
   delete ctx;
 }
 
@@ -509,6 +514,10 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
     moe::StreamPlan*& plan = ctx->plans[i / 8][i % 8];
     plan = i / 8 < l.n_sets ? moe::stream_plan_create() : nullptr;
     if (i / 8 < l.n_sets && plan == nullptr) have_plans = false;
+  }
+  for (int i = 0; i < 2; ++i) {
+    ctx->step_plans[i] = i < l.n_sets ? moe::step_plan_create() : nullptr;
+    if (i < l.n_sets && ctx->step_plans[i] == nullptr) have_plans = false;
   }
   ctx->gemm_taken[0] = ctx->gemm_taken[1] = MOE_GEMM_AUTO;
   if (!have_plans) {
@@ -1126,7 +1135,7 @@ namespace {
 // moves its rows in a second one).
 moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits, const float* select_bias, const void* x,
                               int32_t T, int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
-                              int32_t* inv_perm) {
+                              int32_t* inv_perm, int zero_words) {
   if (!dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm)) {
     const moe_status st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
     return st == MOE_OK ? moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm) : st;
@@ -1141,7 +1150,8 @@ moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits
     StageTimer tm(ctx, 0);
     e = moe::launch_small_dispatch(logits, select_bias, T, c.n_experts, c.top_k, c.routed_scale, topk_idx, topk_w, ctx->counts,
                                    ctx->offsets, ctx->perm, ctx->inv_perm, x,
-                                   fp8 || gathers_rows(ctx) ? nullptr : ctx->sets[ctx->cur].x_perm, c.hidden, ctx->stream, &n);
+                                   fp8 || gathers_rows(ctx) ? nullptr : ctx->sets[ctx->cur].x_perm, c.hidden,
+                                   reinterpret_cast<int*>(ctx->ws + kStepCounterOffset), zero_words, ctx->stream, &n);
   }
   mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
@@ -1156,6 +1166,66 @@ moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits
   return MOE_OK;
 }
 
+// Whether a step that dispatches its tokens in one launch makes its passes and its combine in one, too: every argument fit for
+// them -- or the calls themselves report what is wrong.
+bool ffn_at_once(const moe_ctx* ctx, int32_t T, const void* w1, const void* w2, const void* w1_sh, const void* w2_sh,
+                 const void* out) {
+  const moe_config& c = ctx->cfg;
+  const bool shared = c.n_shared != 0;
+  if (c.weight_format != MOE_WEIGHTS_BF16 || c.gemm_variant != MOE_GEMM_AUTO || c.row_gather != 0 || ctx->seg_experts > 0 ||
+      ctx->preemptible ||
+      !moe::step_at_once_is_faster(T, c.top_k, c.n_experts, c.hidden, c.inter, shared ? c.shared_inter : 0, gemm_ctas(ctx)))
+    return false;
+  if (!w1 || !w2 || !out || (shared && (!w1_sh || !w2_sh))) return false;
+  return !misaligned(w1) && !misaligned(w2) && !misaligned(w1_sh) && !misaligned(w2_sh) && !misaligned(out) &&
+         moe::step_ffn_counters(c.n_experts, c.hidden) <= kStepCounterWords;
+}
+
+moe_status step_ffn(moe_ctx* ctx, const char* who, const void* w1, const void* w2, const void* w1_sh, const void* w2_sh,
+                    const void* x, const float* topk_w, void* out) {
+  DeviceGuard guard(ctx->device);
+  const moe_config& c = ctx->cfg;
+  const BufferSet& b = ctx->sets[ctx->cur];
+  moe::StepFfn f;
+  f.E = c.n_experts;
+  f.T = ctx->T;
+  f.k = c.top_k;
+  f.H = c.hidden;
+  f.I = c.inter;
+  f.Is = c.n_shared != 0 ? c.shared_inter : 0;
+  f.rows_cap = (int64_t)c.max_tokens * c.top_k;
+  f.w1 = w1;
+  f.w2 = w2;
+  f.w1_sh = w1_sh;
+  f.w2_sh = w2_sh;
+  f.x = b.x_perm;
+  f.x_sh = x;
+  f.act = b.act;
+  f.act_sh = b.act_shared;
+  f.y = b.y_perm;
+  f.y_sh = b.y_shared;
+  f.out = out;
+  f.offsets = ctx->offsets;
+  f.inv_perm = ctx->inv_perm;
+  f.topk_w = topk_w;
+  f.counters = reinterpret_cast<int*>(ctx->ws + kStepCounterOffset);
+  f.status = ctx->status;
+  f.wait_limit_ns = ctx->wait_limit_ns;
+  f.debug_stall = ctx->debug_stall;
+  int n = 0;
+  cudaError_t e;
+  {
+    StageTimer tm(ctx, 3);
+    e = moe::launch_step_ffn(f, ctx->step_plans[ctx->cur], gemm_ctas(ctx), ctx->stream, &n);
+  }
+  mark(ctx, n);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, who);
+  ctx->gemm_taken[0] = ctx->gemm_taken[1] = MOE_GEMM_SMALL_M;
+  ctx->state = ST_IDLE;
+  if (ctx->n_sets == 2) ctx->cur ^= 1;  // D: the next step works in the other buffer set
+  return MOE_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1166,7 +1236,11 @@ moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias
                      const void* ws_down, void* out) {
   if (!ctx) return MOE_ERR_INVALID_ARG;
   PositionMark position(ctx);
-  moe_status st = route_and_dispatch(ctx, "moe_layer", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
+  const bool at_once = ffn_at_once(ctx, T, w_gate_up, w_down, ws_gate_up, ws_down, out) &&
+                       dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
+  moe_status st = route_and_dispatch(ctx, "moe_layer", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm,
+                                     at_once ? moe::step_ffn_counters(ctx->cfg.n_experts, ctx->cfg.hidden) : 0);
+  if (at_once) return st == MOE_OK ? step_ffn(ctx, "moe_layer", w_gate_up, w_down, ws_gate_up, ws_down, x, topk_w, out) : st;
   if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T);
   if (st == MOE_OK) st = combine(ctx, topk_w, inv_perm, T, out, ctx->seg_experts == 0 && !ctx->preemptible);
   return st;
@@ -1180,7 +1254,7 @@ moe_status moe_layer_fp8(moe_ctx* ctx, const float* logits, const float* select_
   if (!ctx) return MOE_ERR_INVALID_ARG;
   PositionMark position(ctx);
   moe_status st =
-      route_and_dispatch(ctx, "moe_layer_fp8", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
+      route_and_dispatch(ctx, "moe_layer_fp8", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm, 0);
   if (st == MOE_OK)
     st = moe_grouped_ffn_fp8(ctx, wq_gate_up, sw_gate_up, wq_down, sw_down, wsq_gate_up, sws_gate_up, wsq_down, sws_down, T);
   if (st == MOE_OK) st = combine(ctx, topk_w, inv_perm, T, out, ctx->seg_experts == 0 && !ctx->preemptible);
@@ -1507,6 +1581,8 @@ moe_status moe_ctx_debug_gemm(const moe_ctx* ctx, int32_t* gated, int32_t* down,
     for (const auto& set : ctx->plans)
       for (const moe::StreamPlan* plan : set)
         if (plan != nullptr) *maps_encoded += moe::stream_plan_encoded(plan);
+    for (const moe::StepPlan* plan : ctx->step_plans)
+      if (plan != nullptr) *maps_encoded += moe::step_plan_encoded(plan);
   }
   return MOE_OK;
 }

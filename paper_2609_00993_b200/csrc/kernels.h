@@ -92,12 +92,14 @@ cudaError_t launch_layout(const int32_t* topk_idx, int64_t n_slots, int E, int32
                           int* n_launches);
 
 // ---- a1-a5 of a few tokens in one launch (the results of the three stages) -------------------
-// x_perm nullptr: no rows move.  Only where small_dispatch_fits (512 experts: 16 keys per lane).
+// x_perm nullptr: no rows move.  Only where small_dispatch_fits (512 experts: 16 keys per lane).  The n_zero words at `zero`
+// are set to zero (the counters of the step's next launch).
 constexpr int kSmallDispatchMaxTokens = 64, kSmallDispatchMaxSlots = 1024;
 bool small_dispatch_fits(int T, int E, int k);
 cudaError_t launch_small_dispatch(const float* logits, const float* bias, int T, int E, int k, float scale, int32_t* idx,
                                   float* w, int32_t* counts, int32_t* offsets, int32_t* perm, int32_t* inv_perm,
-                                  const void* x, void* x_perm, int H, cudaStream_t stream, int* n_launches);
+                                  const void* x, void* x_perm, int H, int* zero, int n_zero, cudaStream_t stream,
+                                  int* n_launches);
 
 // ---- a5 permute, a9 combine ----------------------------------------------------------------
 // wait_limit_ns: time limit of the kernels' bounded waits (0 = the default of 2 s).
@@ -188,6 +190,29 @@ struct GemmDenseGroup {
   const float* row_scale = nullptr;  // FP8 variant: [rows]
   const float* w_scale = nullptr;    // FP8 variant: [(gated?2:1)*n_feat]
 };
+
+// ---- a6-a9 of a few tokens in one launch (step_ffn.cu) ---------------------------------------
+// bf16; behind launch_small_dispatch, which zeroed the counters.
+constexpr int kStepMaxTokens = 64;
+struct StepFfn {
+  int E = 0, T = 0, k = 0, H = 0, I = 0, Is = 0;  // Is = 0: no shared expert
+  int64_t rows_cap = 0;                           // rows of x and act
+  const void *w1 = nullptr, *w2 = nullptr, *w1_sh = nullptr, *w2_sh = nullptr;  // gated and down weights, the shared expert's
+  const void *x = nullptr, *x_sh = nullptr;       // routed rows, token rows
+  void *act = nullptr, *act_sh = nullptr, *y = nullptr, *y_sh = nullptr, *out = nullptr;
+  const int32_t *offsets = nullptr, *inv_perm = nullptr;
+  const float* topk_w = nullptr;
+  int* counters = nullptr;  // step_ffn_counters words
+  int* status = nullptr;
+  unsigned long long wait_limit_ns = 0;
+  bool debug_stall = false;
+};
+struct StepPlan;  // the launch's tensor maps, kept per buffer set
+StepPlan* step_plan_create();
+void step_plan_destroy(StepPlan* plan);
+int64_t step_plan_encoded(const StepPlan* plan);
+int step_ffn_counters(int E, int H);
+cudaError_t launch_step_ffn(const StepFfn& f, StepPlan* plan, int max_ctas, cudaStream_t stream, int* n_launches);
 
 // FP8 variant: per-row dynamic quantisation of bf16 rows [rows, n] -> E4M3 codes [rows, n] + scale [rows]
 // (n a multiple of 16, at most 8192).  A second set of rows of the same length may ride in the launch.

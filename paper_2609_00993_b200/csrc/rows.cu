@@ -13,6 +13,7 @@
 #include <mutex>
 #include <tuple>
 
+#include "combine.cuh"
 #include "kernels.h"
 
 namespace moe {
@@ -146,16 +147,6 @@ constexpr int kCombineConsumers = 128;   // one 16-byte vector (8 columns) per c
 constexpr int kCombineThreads = kCombineConsumers + 32;
 constexpr int kCombineMaxStages = 4;
 
-// acc += w * v for eight bf16 values; a bf16 widens to fp32 by a 16-bit shift (low half) or a mask (high half)
-__device__ __forceinline__ void fma_bf16x8(float (&acc)[8], const uint4& v, float w) {
-  const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    acc[2 * q] = fmaf(w, __uint_as_float(u[q] << 16), acc[2 * q]);
-    acc[2 * q + 1] = fmaf(w, __uint_as_float(u[q] & 0xffff0000u), acc[2 * q + 1]);
-  }
-}
-
 // Columns [c_begin, c_end): out[t, c0:c1] = sum_j w[t,j] * y_perm[inv_perm[t*k+j], c0:c1] (+ y_shared[t, c0:c1]); ascending j, then shared.
 // dynamic shared memory, per stage: (k+1) row chunks of chunk_bytes | k weights | valid mask; then barriers.
 // Producer lane j gathers row j; lane 0 also fetches the shared row.  KT > 0 fixes k at compile time (the sum
@@ -253,11 +244,7 @@ combine_kernel(const __nv_bfloat16* __restrict__ y_perm, const __nv_bfloat16* __
               fma_bf16x8(acc, *reinterpret_cast<const uint4*>(mine + (size_t)j * chunk_bytes), wts[j]);
         }
         if (shared) fma_bf16x8(acc, *reinterpret_cast<const uint4*>(mine + (size_t)k * chunk_bytes), 1.0f);
-        uint4 o;
-        __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) oh[q] = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
-        *reinterpret_cast<uint4*>(out + (size_t)t * H + c0 + v * 8) = o;
+        *reinterpret_cast<uint4*>(out + (size_t)t * H + c0 + v * 8) = bf16x8(acc);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_empty + 8u * s);

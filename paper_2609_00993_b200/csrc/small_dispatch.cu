@@ -60,7 +60,8 @@ __global__ void __launch_bounds__(kMaxThreads)
 small_dispatch_kernel(const float* __restrict__ logits, const float* __restrict__ bias, int T, int E, int k, float scale,
                       int32_t* __restrict__ idx, float* __restrict__ w, int32_t* __restrict__ counts,
                       int32_t* __restrict__ offsets, int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm,
-                      const uint4* __restrict__ x, uint4* __restrict__ x_perm, int row_vecs, int n_ranks) {
+                      const uint4* __restrict__ x, uint4* __restrict__ x_perm, int row_vecs, int n_ranks, int* __restrict__ zero,
+                      int n_zero) {
   __shared__ unsigned long long s_cand[kMaxThreads / 32][32];
   __shared__ int s_sel[kMaxThreads / 32][32];
   __shared__ __align__(16) int s_idx[kSmallDispatchMaxSlots + 4];
@@ -74,6 +75,8 @@ small_dispatch_kernel(const float* __restrict__ logits, const float* __restrict_
   uint4 piece;
   const bool moves = x_perm != nullptr && t < T && col < row_vecs;
   if (moves) piece = x[(size_t)t * row_vecs + col];
+  if (blockIdx.x == 0)
+    for (int i = t * (int)blockDim.x + (int)threadIdx.x; i < n_zero; i += (int)(gridDim.y * blockDim.x)) zero[i] = 0;
   const int q = rank * n_warps + warp;
   int e = 0;
   if (q < T) {
@@ -139,7 +142,8 @@ bool small_dispatch_fits(int T, int E, int k) {
 
 cudaError_t launch_small_dispatch(const float* logits, const float* bias, int T, int E, int k, float scale, int32_t* idx,
                                   float* w, int32_t* counts, int32_t* offsets, int32_t* perm, int32_t* inv_perm,
-                                  const void* x, void* x_perm, int H, cudaStream_t stream, int* n_launches) {
+                                  const void* x, void* x_perm, int H, int* zero, int n_zero, cudaStream_t stream,
+                                  int* n_launches) {
   const bool vec = routes_in_vectors(logits, bias, E);
   const int per_lane = (E + 31) / 32, row_vecs = H / 8;
   // A warp per token.  More warps in a CTA than 16 are in one another's way (32 tokens in one CTA of 1024 threads instead of
@@ -153,7 +157,7 @@ cudaError_t launch_small_dispatch(const float* logits, const float* bias, int T,
     if (err != cudaSuccess) return err;
     return launch_pdl_clusters(true, n_ranks, kern, grid, dim3(threads), 0, stream, logits, bias, T, E, k, scale, idx, w, counts,
                                offsets, perm, inv_perm, static_cast<const uint4*>(x), static_cast<uint4*>(x_perm), row_vecs,
-                               n_ranks);
+                               n_ranks, zero, n_zero);
   };
   cudaError_t err;
   if (per_lane <= 1) err = go(small_dispatch_kernel<1, false>);

@@ -1,0 +1,63 @@
+"""Both passes and the combine of a few tokens in one launch, against the launches of the small-M kernel, bit for bit: groups of
+one to sixty-four rows, one expert and 512, rows that end within a feature tile, more tiles than CTAs and fewer, both buffer
+sets, steps on either side of the rule in turn; a step whose waits run out."""
+import pytest
+import torch
+
+from paper_2609_00993_b200 import binding as B
+from paper_2609_00993_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _step(ctx, a, logits, bias, w, T):
+    return ctx.layer(a["x"][:T], logits[:T], bias, w["w_gate_up"], w["w_down"], w["ws_gate_up"], w["ws_down"])
+
+
+def _context(shape, phase, variant, budget):
+    cfg = B.make_config(shape.H, shape.E, shape.k, shape.I, shape.shared_I, shape.T, phase, gemm_variant=variant, sm_budget=budget)
+    return B.MoeContext(cfg, workspace=torch.full((B.moe_ctx_workspace_bytes(cfg),), 0xFF, dtype=torch.uint8, device=DEV))
+
+
+@pytest.mark.parametrize("E,k,H,I,shared,budget", [
+    (1, 1, 64, 256, 0, 0), (8, 2, 256, 512, 0, 0), (5, 5, 192, 320, 256, 12), (33, 4, 1344, 704, 320, 1), (128, 8, 2048, 768, 0, 0),
+    (512, 8, 2560, 640, 512, 100), (64, 16, 704, 2112, 0, 148),
+])
+@pytest.mark.parametrize("phase", [B.MOE_PHASE_PREFILL, B.MOE_PHASE_DECODE])
+def test_one_launch_is_the_small_m_kernels(E, k, H, I, shared, budget, phase):
+    shape = wl.LayerShape("s", T=64, H=H, E=E, k=k, I=I, shared_I=shared)
+    w, a = wl.make_weights(shape, 31, DEV), wl.make_activations(shape, 32, DEV)
+    bias = torch.linspace(3.0, 0.0, E, device=DEV) if E > 8 else None  # experts of many rows and of none
+    one, many = (_context(shape, phase, v, budget) for v in (B.MOE_GEMM_AUTO, B.MOE_GEMM_SMALL_M))
+    torch.cuda.synchronize()
+    for T in (1, 16, 3, 17, 64, 33, 63):
+        got, want = (_step(c, a, a["logits"], bias, w, T) for c in (one, many))
+        torch.cuda.synchronize()
+        assert one.moe_ctx_status() == B.MOE_OK and many.moe_ctx_status() == B.MOE_OK
+        assert torch.equal(got[0], want[0]), T
+        for name in want[1]:
+            assert torch.equal(got[1][name], want[1][name]), (T, name)
+    n0 = one.moe_ctx_launch_count()
+    _step(one, a, a["logits"], bias, w, 2)
+    assert one.moe_ctx_launch_count() - n0 == 2
+    torch.cuda.synchronize()
+    one.close(), many.close()
+
+
+def test_a_wait_that_runs_out_is_reported_and_the_next_step_is_right():
+    shape = wl.LayerShape("s", T=20, H=256, E=16, k=4, I=512, shared_I=256)
+    w, a = wl.make_weights(shape, 41, DEV), wl.make_activations(shape, 42, DEV)
+    ctx = _context(shape, B.MOE_PHASE_DECODE, B.MOE_GEMM_AUTO, 0)
+    torch.cuda.synchronize()
+    want = _step(ctx, a, a["logits"], None, w, 20)[0].clone()
+    ctx.moe_ctx_set_wait_limit(20000)
+    ctx.moe_ctx_debug_inject_stall(True)
+    _step(ctx, a, a["logits"], None, w, 20)
+    torch.cuda.synchronize()
+    assert ctx.moe_ctx_status() == B.MOE_ERR_TIMEOUT
+    ctx.moe_ctx_debug_inject_stall(False)
+    got = _step(ctx, a, a["logits"], None, w, 20)[0]
+    torch.cuda.synchronize()
+    assert ctx.moe_ctx_status() == B.MOE_OK and torch.equal(got, want)
+    ctx.close()
