@@ -104,7 +104,8 @@ typedef struct {
   int32_t row_gather;   /* 0: moe_dispatch_layout writes x_perm (stage a5 is its own kernel).
                            1: with the large-M GEMM variant, GEMM1 gathers its rows from x
                               through perm while it runs; x_perm is not written, and x must
-                              be passed to moe_grouped_ffn.  Ignored by the other variants. */
+                              be passed to moe_grouped_ffn.  Ignored by the other variants.
+                           (The calls that make a whole step choose by themselves where 0.) */
   float routed_scale;   /* multiplies the routed weights; 1.0f unless the model says so */
   int32_t weight_format; /* moe_weight_format; FP8 adds the quantisation buffers to the workspace */
 } moe_config;
@@ -398,7 +399,8 @@ moe_status moe_layer_host_wait(moe_ctx* ctx, int32_t slot);
  * the step that finished last; moe_layer_host may cut a batch into two chunks of tokens, and what it leaves is then that of
  * the second).  Rows
  * [0, T*k) of x_perm [.,H], act [.,I], y_perm [.,H] and rows [0,T) of y_shared [.,H] are
- * defined after the respective stage.  Any out-pointer may be NULL. */
+ * defined after the respective stage (x_perm: not after a whole step whose gated pass gathered its rows, as
+ * moe_layer and moe_layer_host do from 8193 rows on).  Any out-pointer may be NULL. */
 moe_status moe_ctx_debug_ptrs(moe_ctx* ctx, void** x_perm, void** act, void** y_perm, void** y_shared,
                               int32_t** counts, int32_t** offsets);
 

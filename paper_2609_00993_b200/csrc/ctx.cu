@@ -215,6 +215,7 @@ struct moe_ctx {
   std::mutex* yield_mu;
   int* stopped_host;  // pinned host word: CTAs that stopped in the last launch
   int64_t yields;     // launches that ended on a yield request
+  bool gather_step;   // the step's gated pass gathers its rows from x: none have been moved
   bool offsets_fresh; // the kernel right before the gated pass wrote the step's offsets (moe_layer, a few tokens)
   bool unmarked;      // launches have been enqueued since `done` was last recorded
   int calls_open;     // entry points being executed (the calls of a whole step are made by another)
@@ -508,7 +509,7 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
   ctx->host_stream = ctx->host_pipeline = false;
   ctx->unmarked = false;
   ctx->calls_open = 0;
-  ctx->offsets_fresh = false;
+  ctx->offsets_fresh = ctx->gather_step = false;
   bool have_plans = true;
   for (int i = 0; i < 16; ++i) {
     moe::StreamPlan*& plan = ctx->plans[i / 8][i % 8];
@@ -715,8 +716,24 @@ moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx
   mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->T = T;
-  ctx->offsets_fresh = false;
+  ctx->offsets_fresh = ctx->gather_step = false;
   return MOE_OK;
+}
+
+// Whether the gated pass of a whole step of T tokens, whose rows it knows from the start, gathers them from x.
+bool step_gathers(const moe_ctx* ctx, int32_t T, const void* x) {
+  const moe_config& c = ctx->cfg;
+  if (c.gemm_variant != MOE_GEMM_AUTO || c.phase != MOE_PHASE_PREFILL || c.weight_format != MOE_WEIGHTS_BF16 || c.row_gather != 0 ||
+      ctx->seg_experts > 0 || ctx->preemptible || T < 1 || x == nullptr || misaligned(x) ||
+      gemm_ctas(ctx) != ctx->n_sms || !moe::gather_is_faster((int64_t)T * c.top_k, c.n_experts) || (int64_t)(T + 1) * c.hidden * 2 > 0xffffffffLL)
+    return false;
+  moe::GemmProblem g{};
+  g.rows_bound = (int64_t)T * c.top_k;
+  g.E = c.n_experts;
+  g.n_feat = c.inter;
+  g.K = c.hidden;
+  g.gated = true;
+  return gemm_variant_of(ctx, g) == MOE_GEMM_SMALL_M;
 }
 
 // Whether a step routes and lays out in one launch: a few tokens, and every argument fit for moe_route and
@@ -810,7 +827,7 @@ moe_status grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, 
     };
     moe::GemmProblem g1{b.x_perm, w_gate_up, b.act, ctx->offsets, 0, Ncap, N, c.n_experts, c.inter, c.hidden, true};
     moe::GemmProblem g2{b.act, w_down, b.y_perm, ctx->offsets, 0, Ncap, N, c.n_experts, c.hidden, c.inter, false};
-    if (gathers_rows(ctx)) {
+    if (gathers_rows(ctx) || ctx->gather_step) {
       g1.gather_src = x;
       g1.perm = ctx->perm;
       g1.top_k = c.top_k;
@@ -1137,8 +1154,16 @@ moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits
                               int32_t T, int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
                               int32_t* inv_perm, int zero_words) {
   if (!dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm)) {
-    const moe_status st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
-    return st == MOE_OK ? moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm) : st;
+    moe_status st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
+    if (st != MOE_OK) return st;
+    if (!step_gathers(ctx, T, x)) return moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm);
+    DeviceGuard guard(ctx->device);
+    st = enqueue_layout(ctx, who, topk_idx, T, counts, offsets, perm, inv_perm);
+    if (st != MOE_OK) return st;
+    ctx->gather_step = true;
+    ctx->state = ST_LAID_OUT;
+    ctx->split_step = false;
+    return MOE_OK;
   }
   DeviceGuard guard(ctx->device);
   set_layout_arrays(ctx, counts, offsets, perm, inv_perm);
@@ -1174,7 +1199,8 @@ bool ffn_at_once(const moe_ctx* ctx, int32_t T, const void* w1, const void* w2, 
   const bool shared = c.n_shared != 0;
   if (c.weight_format != MOE_WEIGHTS_BF16 || c.gemm_variant != MOE_GEMM_AUTO || c.row_gather != 0 || ctx->seg_experts > 0 ||
       ctx->preemptible ||
-      !moe::step_at_once_is_faster(T, c.top_k, c.n_experts, c.hidden, c.inter, shared ? c.shared_inter : 0, gemm_ctas(ctx)))
+      !moe::step_at_once_is_faster(T, c.top_k, c.n_experts, c.hidden, c.inter, shared ? c.shared_inter : 0, gemm_ctas(ctx),
+                                   gemm_ctas(ctx) == ctx->n_sms))
     return false;
   if (!w1 || !w2 || !out || (shared && (!w1_sh || !w2_sh))) return false;
   return !misaligned(w1) && !misaligned(w2) && !misaligned(w1_sh) && !misaligned(w2_sh) && !misaligned(out) &&
@@ -1348,7 +1374,8 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
       if (st != MOE_OK) break;
       if (i == 0) e = have_stream ? cudaStreamWaitEvent(ctx->stream, ctx->copied_in[0], 0) : copy_rows(0, ctx->stream);
       if (e != cudaSuccess) break;
-      st = enqueue_row_movement(ctx, "moe_layer_host", x);
+      ctx->gather_step = step_gathers(ctx, n_tok, x);
+      if (!ctx->gather_step) st = enqueue_row_movement(ctx, "moe_layer_host", x);
       if (st != MOE_OK) break;
       ctx->state = ST_LAID_OUT;
       ctx->split_step = false;

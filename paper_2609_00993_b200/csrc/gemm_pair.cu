@@ -501,7 +501,7 @@ cudaError_t launch_gemm_pair(const GemmProblem& p, const GemmDenseGroup* dense, 
   if (dense != nullptr && dense->rows <= 0) dense = nullptr;
   if (p.rows_bound <= 0 && dense == nullptr) return cudaSuccess;
   if (p.rows_bound <= 0) return cudaErrorInvalidValue;  // a dense group never comes without its routed pass
-  if (!swap_ab_supports(p, dense) || max_ctas < 2 || p.resumable || p.n_feat % 16 != 0 ||
+  if (!swap_ab_supports(p, dense) || max_ctas < 2 || p.resumable || p.gather_src != nullptr || p.n_feat % 16 != 0 ||
       (dense != nullptr && dense->n_feat % 16 != 0))
     return cudaErrorNotSupported;
   const int groups = p.offsets ? p.E : 1;

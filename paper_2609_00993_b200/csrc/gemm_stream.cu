@@ -26,6 +26,10 @@
 //
 // Warp roles (320 threads): warps 0-7 epilogue (two per TMEM lane group), warp 8 TMA producer, warp 9 MMA issuer
 // and TMEM owner.
+// The row-gather instantiation (gated pass, bf16; rules.h says when) adds warps 10 and 11, which fetch the token rows of a k-block out
+// of the unpermuted x by 16-byte cp.async copies, in TMA's swizzled layout, once the producer has made room for them; TMA then carries the
+// weights only.  (TMA's own gather takes 58 clocks for four rows of 128 bytes, three times what the k-block's MMAs take; two warps,
+// because with 14 in the CTA the epilogue's registers no longer fit.)
 // Every mbarrier wait is bounded: on expiry the kernel records a timeout in the status word, raises a CTA-wide
 // abort flag, lets copies in flight land, frees its TMEM and returns.
 // The same kernel serves E4M3 operands (kind::f8f6f4, 128 K-elements per k-block, accumulator scaled by the
@@ -47,6 +51,8 @@ constexpr int kEpilogueWarps = 8;  // two per TMEM lane group, taking alternate 
 constexpr int kProducerWarp = kEpilogueWarps;
 constexpr int kMmaWarp = kEpilogueWarps + 1;
 constexpr int kThreads = 32 * (kEpilogueWarps + 2);
+constexpr int kGatherWarp0 = kEpilogueWarps + 2, kGatherWarps = 2;
+constexpr int kThreadsGather = 32 * (kGatherWarp0 + kGatherWarps);
 constexpr int kSlotBytes = 2048;                        // ring granularity: 16 token rows of one k-block
 constexpr int kWSlots = 2 * kWBoxBytes / kSlotBytes;    // 16 slots: the two weight boxes
 constexpr int kNB = 8;                                  // k-blocks in flight at most (barrier pairs)
@@ -65,14 +71,16 @@ __device__ unsigned long long g_stream_ts[8 * 256];  // global-timer stamps of t
 #define PROF_STAMP(slot)
 #endif
 
-template <bool GATED, bool FP8>
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool GATED, bool FP8, bool GATHER>
+__global__ void __launch_bounds__(GATHER ? kThreadsGather : kThreads, 1)
 grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_w2,
                            const __grid_constant__ StreamMaps xmaps, const __grid_constant__ StreamParams p) {
+  static_assert(!GATHER || (GATED && !FP8), "rows are gathered for the gated pass of bf16 layers only");
   constexpr int kbk = FP8 ? 2 * kBlockK : kBlockK;  // K elements per k-block
+  constexpr int kCtaThreads = GATHER ? kThreadsGather : kThreads;
   extern __shared__ uint8_t smem_raw[];
-  // carve: ring (ring_slots x 2 KB) | epilogue staging | full[kNB] empty[kNB] tfull[2] tempty[2] tqfull[kQ] tqempty[kQ] | tq[kQ] | tmem slot
-  //        | abort | stopped | sizes[kNB] | prefix[E+1] | order[E] | beg[E] | cnts[E] | classes | chunk sums
+  // carve: ring (ring_slots x 2 KB) | epilogue staging | full[kNB] empty[kNB] tfull[2] tempty[2] tqfull[kQ] tqempty[kQ] (go[kNB])
+  //        | tq[kQ] | tmem slot | abort | stopped | sizes[kNB] | prefix[E+1] | order[E] | beg[E] | cnts[E] | classes | chunk sums
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base_addr = (raw_addr + 1023u) & ~1023u;
   uint8_t* base = smem_raw + (base_addr - raw_addr);
@@ -84,8 +92,10 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   const uint32_t bar_tempty = bar_tfull + 16u;
   const uint32_t bar_tqfull = bar_tempty + 16u;         // the tile queue: an entry has been published
   const uint32_t bar_tqempty = bar_tqfull + 8u * kQ;    // ... and read by the issuer and every epilogue warp
-  static_assert((2 * kNB + 4 + 2 * kQ) % 2 == 0, "the queue's entries are 16-byte aligned");
-  STile* tq = reinterpret_cast<STile*>(bars + 2 * kNB + 4 + 2 * kQ);  // tile queue
+  const uint32_t bar_go = bar_tqempty + 8u * kQ;        // row gather: there is room for the k-block's rows
+  constexpr int kBars = 2 * kNB + 4 + 2 * kQ + (GATHER ? kNB : 0);
+  static_assert(kBars % 2 == 0, "the queue's entries are 16-byte aligned");
+  STile* tq = reinterpret_cast<STile*>(bars + kBars);  // tile queue
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tq + kQ);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* stopped_here = reinterpret_cast<volatile int*>(tmem_slot + 2);  // the producer stopped on request
@@ -109,8 +119,9 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   // tile list (experts ordered by size, largest first)
   if (threadIdx.x == 32 * kProducerWarp) {
     for (int s = 0; s < kNB; ++s) {
-      mbar_init(bar_full + 8u * s, 1);
+      mbar_init(bar_full + 8u * s, GATHER ? 1 + 32 * kGatherWarps : 1);  // (a gathering thread's copies are an arrival of it)
       mbar_init(bar_empty + 8u * s, 1);
+      if (GATHER) mbar_init(bar_go + 8u * s, 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(bar_tfull + 8u * a, 1);
@@ -118,7 +129,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
     }
     for (int q = 0; q < kQ; ++q) {
       mbar_init(bar_tqfull + 8u * q, 1);
-      mbar_init(bar_tqempty + 8u * q, 1 + kEpilogueWarps);
+      mbar_init(bar_tqempty + 8u * q, 1 + kEpilogueWarps + (GATHER ? kGatherWarps : 0));
     }
     *abort_flag = 0;
     *stopped_here = 0;
@@ -134,7 +145,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
     pdl_launch_dependents();
   }
   if (threadIdx.x == 0) PROF_STAMP(1);
-  build_tile_list<kThreads>(p, prefix, order, beg, cnts, class_pos, chunk_sum);
+  build_tile_list<kCtaThreads>(p, prefix, order, beg, cnts, class_pos, chunk_sum);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -276,14 +287,16 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
           // to the up rows; down pass: 256 consecutive rows), then the n token rows
           const uint32_t st_w = base_addr + head_w * (uint32_t)kSlotBytes;
           if (elect_one()) {
-            mbar_expect_tx(full, 2u * kWBoxBytes + n * 128u);
+            mbar_expect_tx(full, 2u * kWBoxBytes + (GATHER ? 0u : n * 128u));
             if (GATED) tma_load_4d(st_w, mw, full, k0, w_row0, 0, w_e);
             else tma_load_3d(st_w, mw, full, k0, w_row0, w_e);
           }
           if (!reclaim(nx + pad_x, false)) { ok = false; break; }
           free_slots -= nx + pad_x;
           sizes[kb_idx % kNB] = (int)((uint32_t)kWSlots + pad_w + nx + pad_x);
-          if (dep_waited) {
+          if (GATHER) {
+            if (elect_one()) mbar_arrive(bar_go + 8u * (kb_idx % kNB));
+          } else if (dep_waited) {
             if (elect_one()) tma_load_2d(base_addr + head_x * (uint32_t)kSlotBytes, mx, full, k0, t.row0);
           } else {
             ++n_def;
@@ -322,6 +335,56 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         *p.done_ctr = 0;
         if (!any_stopped) *p.tile_ctr = 0;
       }
+    }
+  } else if (GATHER && warp >= kGatherWarp0) {
+    // ================================================================= row gather (warps 10 and 11)
+    // Row r of a tile is x[perm[row0 + r] / top_k] (the dense group's rows are their own).  Warp g takes rows 8 i + 4 g .. + 3 of a
+    // k-block, a lane 16 bytes of one of them, and puts them where TMA's 128-byte swizzle would.  A row past the tile's end is the
+    // tile's last one again.
+    uint32_t head = 0, kb_idx = 0, tcount = 0;
+    bool ok = true;
+    const int r0 = 4 * (warp - kGatherWarp0) + (lane >> 3), piece = lane & 7;
+    const uint32_t dst0 = base_addr + (uint32_t)(r0 * 128 + ((piece ^ r0) << 4));
+    for (;;) {
+      const uint32_t q = tcount % kQ;
+      if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) { ok = false; break; }
+      const STile t = tq[q];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_tqempty + 8u * q);
+      ++tcount;
+      if (t.e == kNoTile) break;
+      const bool dense = t.e == kDenseTile;
+      const uint32_t n = (uint32_t)((t.rows + 15) & ~15), nx = n >> 4;
+      const uint32_t row_bytes = (uint32_t)(dense ? p.K2 : p.K) * 2u;
+      const char* src = reinterpret_cast<const char*>(dense ? p.gather_src2 : p.gather_src);
+      uint32_t off[kMaxTileRows / 8];  // of this lane's piece in its rows
+#pragma unroll
+      for (int i = 0; i < kMaxTileRows / 8; ++i) {
+        if (8u * i >= n) break;
+        const int row = t.row0 + min(8 * i + r0, t.rows - 1);
+        off[i] = (uint32_t)(dense ? row : __ldg(p.perm + row) / p.top_k) * row_bytes + 16u * (uint32_t)piece;
+      }
+      const int num_kb = dense ? num_kb2 : num_kb1;
+      for (int kb = 0; kb < num_kb; ++kb, src += 2 * kBlockK) {
+        if (head + (uint32_t)kWSlots > R) head = 0;  // the producer's allocation, step for step
+        head += (uint32_t)kWSlots;
+        if (head + nx > R) head = 0;
+        const uint32_t dst = dst0 + head * (uint32_t)kSlotBytes;
+        head += nx;
+        if (!mbar_wait_warp(bar_go + 8u * (kb_idx % kNB), (kb_idx / kNB) & 1u, abort_flag, limit)) { ok = false; break; }
+#pragma unroll
+        for (int i = 0; i < kMaxTileRows / 8; ++i) {
+          if (8u * i >= n) break;
+          cp_async_16(dst + (uint32_t)(i * 1024), src + off[i]);
+        }
+        cp_async_arrive_on(bar_full + 8u * (kb_idx % kNB));
+        ++kb_idx;
+      }
+      if (!ok) break;
+    }
+    if (!ok && lane == 0) {
+      *abort_flag = 1;
+      atomicCAS(p.status, kStOk, kStTimeout);
     }
   } else if (warp >= kMmaWarp) {
     // ================================================================= MMA issuer
@@ -382,6 +445,7 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
           if (!got) { ok = false; break; }
         }
         if (kb_idx == 0) PROF_STAMP(3);
+        if (GATHER) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the rows came by cp.async
         tc_fence_after();
         const uint32_t lo_w0 = lo_base + pos_w * lo_slot, lo_w1 = lo_w0 + lo_box, lo_x = lo_base + pos_x * lo_slot;
         if (elect_one()) {
@@ -606,10 +670,10 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
 
 template <typename Kernel>
 cudaError_t launch_variant(Kernel kern, const CUtensorMap& mw, const CUtensorMap& mw2, const StreamMaps& xm,
-                           const StreamParams& prm, int grid, size_t smem, cudaStream_t stream, bool overlap) {
+                           const StreamParams& prm, int grid, int threads, size_t smem, cudaStream_t stream, bool overlap) {
   cudaError_t err = ensure_dynamic_smem(kern, smem);
   if (err != cudaSuccess) return err;
-  return launch_pdl(overlap, kern, dim3(grid), dim3(kThreads), smem, stream, mw, mw2, xm, prm);
+  return launch_pdl(overlap, kern, dim3(grid), dim3(threads), smem, stream, mw, mw2, xm, prm);
 }
 
 }  // namespace
@@ -632,6 +696,12 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   if (p.rows_bound <= 0 && dense == nullptr) return cudaSuccess;
   if (p.rows_bound <= 0) return cudaErrorInvalidValue;  // a dense group never comes without its routed pass
   if (!swap_ab_supports(p, dense)) return cudaErrorNotSupported;
+  const bool gather = p.gather_src != nullptr;
+  // (a row's offset in the source is 32 bits; what it reads comes from the kernel in front of it, so it does without the overlap)
+  if (gather && (!p.gated || p.fp8 || p.perm == nullptr || p.top_k < 1 || p.K % kBlockK != 0 ||
+                 (dense != nullptr && (dense->A == nullptr || dense->K % kBlockK != 0 || dense->rows * (int64_t)dense->K * 2 > 0xffffffffLL)) ||
+                 (p.rows_bound / p.top_k + 1) * (int64_t)p.K * 2 > 0xffffffffLL || p.rows_bound <= kGemmOverlapMaxRows))
+    return cudaErrorNotSupported;
   const int groups = p.offsets ? p.E : 1;
   const int e_begin = p.offsets ? p.e_begin : 0;
   const int e_end = (p.offsets && p.e_end >= 0) ? p.e_end : groups;
@@ -645,7 +715,7 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   int64_t tiles;
   if (!fill_params(prm, tiles, p, dense, e_begin, e_end, status)) return cudaErrorInvalidValue;
 
-  const size_t tail = kEpilogueWarps * kStagingBytes + (2 * kNB + 4 + 2 * kQ) * sizeof(uint64_t) + 3 * sizeof(uint32_t) + kNB * sizeof(int) + kQ * sizeof(STile) +
+  const size_t tail = kEpilogueWarps * kStagingBytes + (2 * kNB + 4 + 2 * kQ + (gather ? kNB : 0)) * sizeof(uint64_t) + 3 * sizeof(uint32_t) + kNB * sizeof(int) + kQ * sizeof(STile) +
                       (4 * (size_t)(prm.E + 1) + kSizeClasses + 32) * sizeof(int);
   const int slots = (int)((kSmemBudget - 1024 - (int)tail) / kSlotBytes);
   if (slots < 2 * (kWSlots + kMaxTileRows / 16)) return cudaErrorNotSupported;
@@ -663,12 +733,22 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   // one tile per CTA at most: any order will do (1.3 us of the tiny layer's 64-token step)
   if (tiles <= (int64_t)grid) prm.sort_tiles = 0;
   const bool overlap = p.rows_bound <= kGemmOverlapMaxRows;
+  if (gather) {
+    prm.early_setup = 0;
+    prm.gather_src = static_cast<const __nv_bfloat16*>(p.gather_src);
+    prm.gather_src2 = dense ? static_cast<const __nv_bfloat16*>(dense->A) : nullptr;
+    prm.perm = p.perm;
+    prm.top_k = p.top_k;
+  }
+  auto launch = [&](auto kern, int threads) {
+    return launch_variant(kern, plan.mw, plan.mw2, plan.xm, prm, grid, threads, smem, stream, overlap);
+  };
   if (p.fp8)
-    err = p.gated ? launch_variant(grouped_gemm_stream_kernel<true, true>, plan.mw, plan.mw2, plan.xm, prm, grid, smem, stream, overlap)
-                  : launch_variant(grouped_gemm_stream_kernel<false, true>, plan.mw, plan.mw2, plan.xm, prm, grid, smem, stream, overlap);
+    err = p.gated ? launch(grouped_gemm_stream_kernel<true, true, false>, kThreads) : launch(grouped_gemm_stream_kernel<false, true, false>, kThreads);
+  else if (gather)
+    err = launch(grouped_gemm_stream_kernel<true, false, true>, kThreadsGather);
   else
-    err = p.gated ? launch_variant(grouped_gemm_stream_kernel<true, false>, plan.mw, plan.mw2, plan.xm, prm, grid, smem, stream, overlap)
-                  : launch_variant(grouped_gemm_stream_kernel<false, false>, plan.mw, plan.mw2, plan.xm, prm, grid, smem, stream, overlap);
+    err = p.gated ? launch(grouped_gemm_stream_kernel<true, false, false>, kThreads) : launch(grouped_gemm_stream_kernel<false, false, false>, kThreads);
   if (err == cudaSuccess && n_launches) *n_launches += 1;
   return err;
 }

@@ -176,6 +176,17 @@ inline bool pair_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t rows
   return K < 1792 ? over(350) : over(96);
 }
 
+// ---- whether the gated pass of a whole bf16 step gathers its rows itself, where the small-M kernel takes it (gemm_stream.cu)
+// It saves the launch that moves the rows, and its write and re-read of them.  Up to 8192 rows that launch is hidden behind the set-up of
+// the gated pass, which would have to wait for the layout instead; with whole tiles of 256 rows the threads that gather cost what they
+// save.  Whole steps, us, rows moved | gathered (rows per expert; two runs of one side differ by 0.1 to 1 %):
+//   2048 / 768 x 128   69 253 | 245, 125 296 | 289, 250 425 | 421, 512 736 | 739, 750 1001 | 1002;  from host buffers 96 490 | 474, 256 (two
+//                      chunks) 1368 | 1378
+//   2560 / 1024 x 512  20 1246 | 1221, 64 1413 | 1388, 140 1776 | 1749, 187 2066 | 2072, 250 2607 | 2595, 312 3165 | 3211
+//   7168 / 2048 x 256 + shared  37 3498 | 3469, 69 3947 | 3915, 128 5087 | 5031, 219 7074 | 6959;  skewed experts 128 4133 | 4085
+// A context on part of the SMs moves its rows: V3-shaped, 1500 tokens on 48 SMs beside decode steps 13029 | 13224, skewed 2500 6129 | 6201.
+inline bool gather_is_faster(int64_t rows, int64_t E) { return rows > 8192 && rows < 256 * E; }
+
 // ---- whether a bf16 step of up to 64 tokens makes its passes and its combine in one launch (step_ffn.cu)
 // It gains a chain of launches and tiles half as large, which counts where there are few of them, and its weights stream over the seam
 // between the passes; its price is 1.2 to 1.5 us an SM for each tile, more than the HBM asks for where the down pass is short.  Whole steps,
@@ -190,11 +201,13 @@ inline bool pair_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t rows
 //                                            163.0 | 158.7, 64 181.3 | 182.6: a group of more than 16 rows takes twice the ring
 // Layers of inter below 256 would gain as well (256 / 128 x 8, 2, 64 tokens 16.9 | 15.0) but keep the launches of the stages: what
 // their stage times and their launches add up to is fixed for such steps.
-inline bool step_at_once_is_faster(int64_t T, int k, int E, int H, int I, int Is, int ctas) {
+// A context on part of the SMs takes it for few tiles only: its decode steps run beside a prefill batch on the others, from which a steadier
+// stream takes HBM that those SMs cannot make up for later (V3-shaped, skewed: 64 tokens beside 900, 4540 | 4642 for both).
+inline bool step_at_once_is_faster(int64_t T, int k, int E, int H, int I, int Is, int ctas, bool all_sms) {
   if (I < 256 || (Is > 0 && Is < 256)) return false;
   const int64_t slots = T * k, groups = slots < E ? slots : E, down = (H + 127) / 128;
   const int64_t tiles = groups * (I / 64 + down) + (Is > 0 ? Is / 64 + down : 0);
-  return tiles <= 4 * (int64_t)ctas || (I >= 640 && slots <= 3 * (int64_t)E);
+  return tiles <= 4 * (int64_t)ctas || (all_sms && I >= 640 && slots <= 3 * (int64_t)E);
 }
 
 }  // namespace moe

@@ -57,6 +57,11 @@ struct StreamParams {
   // the FP8 row scales) depend on.
   int32_t early_setup;
   int32_t sort_tiles;  // 0: every group has at most one tile of the smallest size, so their order does not matter
+  // row gather (the gated pass of bf16 layers, gemm_stream.cu): row r is gather_src[perm[r] / top_k], of the dense group gather_src2[r]
+  const __nv_bfloat16* gather_src;
+  const __nv_bfloat16* gather_src2;
+  const int32_t* perm;
+  int32_t top_k;
 };
 
 // Token rows in boxes of 16, 32, ..., 256 rows; the dense group's in the two sizes it has, its equal chunks and its last one.
@@ -258,7 +263,6 @@ inline bool swap_ab_supports(const GemmProblem& p, const GemmDenseGroup* dense) 
   if (dense != nullptr && (dense->K % 8 != 0 || dense->n_feat % 8 != 0)) return false;
   if (!encoder_ready()) return false;
   if (p.K % 8 != 0 || p.n_feat % 8 != 0 || p.E < 1 || p.E > 1024) return false;
-  if (p.gather_src != nullptr) return false;
   if (p.rows_bound > 0x7fffffffLL / 2) return false;
   return !(p.fp8 && (p.row_scale == nullptr || p.w_scale == nullptr || p.K % 16 != 0 || p.n_feat % 64 != 0 ||
                      (dense != nullptr && (dense->row_scale == nullptr || dense->w_scale == nullptr || dense->K % 16 != 0 ||

@@ -1,0 +1,58 @@
+"""Whole prefill steps whose gated pass gathers its rows, against the kernel that reads moved rows, bit for bit: experts of no row, of one,
+of a tile, of several and of all tokens; tiles that end within 8, 16 and 256 rows; the shared expert's rows; part of the SMs;
+the rows and bounds at which the rule begins and ends; host buffers."""
+import pytest
+import torch
+
+from paper_2609_00993_b200 import binding as B
+from paper_2609_00993_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("H,E,k,I,shared,T,budget,gathers", [
+    (1856, 48, 4, 704, 320, 2049, 0, True), (1856, 48, 4, 704, 320, 2048, 0, False),     # 8192 rows and more
+    (2368, 33, 8, 960, 0, 1055, 0, True), (2368, 33, 8, 960, 0, 1056, 0, False),         # 256 rows per expert and fewer
+    (2560, 512, 8, 320, 0, 1111, 0, True), (3072, 40, 9, 704, 576, 997, 0, True), (3072, 40, 9, 448, 576, 997, 37, False),
+])
+@pytest.mark.parametrize("skewed", [False, True])
+def test_gathered_rows_are_the_moved_ones(H, E, k, I, shared, T, budget, gathers, skewed):
+    shape = wl.LayerShape("g", T=T, H=H, E=E, k=k, I=I, shared_I=shared)
+    w, a = wl.make_weights(shape, 51, DEV), wl.make_activations(shape, 52, DEV)
+    # skewed: two experts get every token, the last third of the experts next to none
+    bias = torch.cat([torch.full((2,), 9.0), torch.zeros(E - 2 - E // 3), torch.full((E // 3,), -4.0)]).to(DEV) if skewed else None
+    res = []
+    for variant in (B.MOE_GEMM_AUTO, B.MOE_GEMM_SMALL_M):
+        cfg = B.make_config(H, E, k, I, shared, T, B.MOE_PHASE_PREFILL, gemm_variant=variant, sm_budget=budget)
+        ctx = B.MoeContext(cfg, workspace=torch.full((B.moe_ctx_workspace_bytes(cfg),), 0xFF, dtype=torch.uint8, device=DEV))
+        torch.cuda.synchronize()
+        for _ in range(2):
+            n0 = ctx.moe_ctx_launch_count()
+            out, bufs = ctx.layer(a["x"], a["logits"], bias, w["w_gate_up"], w["w_down"], w["ws_gate_up"], w["ws_down"])
+            n = ctx.moe_ctx_launch_count() - n0
+        torch.cuda.synchronize()
+        assert ctx.moe_ctx_status() == B.MOE_OK
+        if variant == B.MOE_GEMM_AUTO:
+            assert ctx.moe_ctx_debug_gemm()["gated"] == B.MOE_GEMM_SMALL_M
+        res.append((out, bufs, ctx.moe_ctx_debug_ptrs()["act"][:T * k].clone(), n))
+        ctx.close()
+    got, want = res
+    assert want[3] - got[3] == (1 if gathers else 0)
+    assert torch.equal(got[2], want[2]) and torch.equal(got[0], want[0])
+    assert all(torch.equal(got[1][n], want[1][n]) for n in want[1])
+
+
+def test_gathered_from_host_buffers():
+    shape = wl.LayerShape("g", T=1531, H=2048, E=128, k=8, I=256)
+    w, a = wl.make_weights(shape, 53, DEV), wl.make_activations(shape, 54, DEV)
+    ctx = B.MoeContext(B.make_config(2048, 128, 8, 256, 0, 1531, B.MOE_PHASE_PREFILL))
+    want = ctx.layer(a["x"], a["logits"], None, w["w_gate_up"], w["w_down"])[0]
+    x, logits = a["x"].cpu().pin_memory(), a["logits"].cpu().pin_memory()
+    out = torch.empty(1531, 2048, dtype=torch.bfloat16).pin_memory()
+    for _ in range(2):  # the call that creates the copy stream, and one that has it
+        out.zero_()
+        ctx.moe_layer_host(logits, None, x, w["w_gate_up"], w["w_down"], None, None, out)
+        assert torch.equal(out, want.cpu())
+    assert ctx.moe_ctx_status() == B.MOE_OK
+    ctx.close()
