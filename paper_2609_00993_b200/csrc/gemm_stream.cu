@@ -154,6 +154,54 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
   const int total_tiles = dense_tiles + prefix[p.E] * p.n_ft;
   const uint32_t R = (uint32_t)p.ring_slots;
 
+  // Row gather (warps 10 and 11).  Row r of a tile is x[perm[row0 + r] / top_k]; the dense group's rows are their own.  Warp g takes
+  // rows 8 i + 4 g .. + 3 of a k-block, a lane 16 bytes of one of them, and puts them where TMA's 128-byte swizzle would.  A row past
+  // the tile's end is the tile's last one again.
+  [[maybe_unused]] auto gather_rows = [&]() -> bool {
+    uint32_t head = 0, kb_idx = 0, tcount = 0;
+    bool ok = true;
+    const int r0 = 4 * (warp - kGatherWarp0) + (lane >> 3), piece = lane & 7;
+    const uint32_t dst0 = base_addr + (uint32_t)(r0 * 128 + ((piece ^ r0) << 4));
+    for (;;) {
+      const uint32_t q = tcount % kQ;
+      if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) { ok = false; break; }
+      const STile t = tq[q];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_tqempty + 8u * q);
+      ++tcount;
+      if (t.e == kNoTile) break;
+      const bool dense = t.e == kDenseTile;
+      const uint32_t n = (uint32_t)((t.rows + 15) & ~15), nx = n >> 4;
+      const uint32_t row_bytes = (uint32_t)(dense ? p.K2 : p.K) * 2u;
+      const char* src = reinterpret_cast<const char*>(dense ? p.gather_src2 : p.gather_src);
+      uint32_t off[kMaxTileRows / 8];  // of this lane's piece in its rows
+#pragma unroll
+      for (int i = 0; i < kMaxTileRows / 8; ++i) {
+        if (8u * i >= n) break;
+        const int row = t.row0 + min(8 * i + r0, t.rows - 1);
+        off[i] = (uint32_t)(dense ? row : __ldg(p.perm + row) / p.top_k) * row_bytes + 16u * (uint32_t)piece;
+      }
+      const int num_kb = dense ? num_kb2 : num_kb1;
+      for (int kb = 0; kb < num_kb; ++kb, src += 2 * kBlockK) {
+        if (head + (uint32_t)kWSlots > R) head = 0;  // the producer's allocation, step for step
+        head += (uint32_t)kWSlots;
+        if (head + nx > R) head = 0;
+        const uint32_t dst = dst0 + head * (uint32_t)kSlotBytes;
+        head += nx;
+        if (!mbar_wait_warp(bar_go + 8u * (kb_idx % kNB), (kb_idx / kNB) & 1u, abort_flag, limit)) { ok = false; break; }
+#pragma unroll
+        for (int i = 0; i < kMaxTileRows / 8; ++i) {
+          if (8u * i >= n) break;
+          cp_async_16(dst + (uint32_t)(i * 1024), src + off[i]);
+        }
+        cp_async_arrive_on(bar_full + 8u * (kb_idx % kNB));
+        ++kb_idx;
+      }
+      if (!ok) break;
+    }
+    return ok;
+  };
+
   if (warp == kProducerWarp) {
     // ================================================================= TMA producer
     if (!p.inject_producer_stall) {
@@ -336,58 +384,8 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
         if (!any_stopped) *p.tile_ctr = 0;
       }
     }
-  } else if (GATHER && warp >= kGatherWarp0) {
-    // ================================================================= row gather (warps 10 and 11)
-    // Row r of a tile is x[perm[row0 + r] / top_k] (the dense group's rows are their own).  Warp g takes rows 8 i + 4 g .. + 3 of a
-    // k-block, a lane 16 bytes of one of them, and puts them where TMA's 128-byte swizzle would.  A row past the tile's end is the
-    // tile's last one again.
-    uint32_t head = 0, kb_idx = 0, tcount = 0;
-    bool ok = true;
-    const int r0 = 4 * (warp - kGatherWarp0) + (lane >> 3), piece = lane & 7;
-    const uint32_t dst0 = base_addr + (uint32_t)(r0 * 128 + ((piece ^ r0) << 4));
-    for (;;) {
-      const uint32_t q = tcount % kQ;
-      if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) { ok = false; break; }
-      const STile t = tq[q];
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_tqempty + 8u * q);
-      ++tcount;
-      if (t.e == kNoTile) break;
-      const bool dense = t.e == kDenseTile;
-      const uint32_t n = (uint32_t)((t.rows + 15) & ~15), nx = n >> 4;
-      const uint32_t row_bytes = (uint32_t)(dense ? p.K2 : p.K) * 2u;
-      const char* src = reinterpret_cast<const char*>(dense ? p.gather_src2 : p.gather_src);
-      uint32_t off[kMaxTileRows / 8];  // of this lane's piece in its rows
-#pragma unroll
-      for (int i = 0; i < kMaxTileRows / 8; ++i) {
-        if (8u * i >= n) break;
-        const int row = t.row0 + min(8 * i + r0, t.rows - 1);
-        off[i] = (uint32_t)(dense ? row : __ldg(p.perm + row) / p.top_k) * row_bytes + 16u * (uint32_t)piece;
-      }
-      const int num_kb = dense ? num_kb2 : num_kb1;
-      for (int kb = 0; kb < num_kb; ++kb, src += 2 * kBlockK) {
-        if (head + (uint32_t)kWSlots > R) head = 0;  // the producer's allocation, step for step
-        head += (uint32_t)kWSlots;
-        if (head + nx > R) head = 0;
-        const uint32_t dst = dst0 + head * (uint32_t)kSlotBytes;
-        head += nx;
-        if (!mbar_wait_warp(bar_go + 8u * (kb_idx % kNB), (kb_idx / kNB) & 1u, abort_flag, limit)) { ok = false; break; }
-#pragma unroll
-        for (int i = 0; i < kMaxTileRows / 8; ++i) {
-          if (8u * i >= n) break;
-          cp_async_16(dst + (uint32_t)(i * 1024), src + off[i]);
-        }
-        cp_async_arrive_on(bar_full + 8u * (kb_idx % kNB));
-        ++kb_idx;
-      }
-      if (!ok) break;
-    }
-    if (!ok && lane == 0) {
-      *abort_flag = 1;
-      atomicCAS(p.status, kStOk, kStTimeout);
-    }
   } else if (warp >= kMmaWarp) {
-    // ================================================================= MMA issuer
+    // ================================================================= MMA issuer (row gather: and warps 10 and 11)
     uint32_t head = 0, kb_idx = 0, use0 = 0, use1 = 0, next_half = 0;
     bool ok = true;
     [[maybe_unused]] long long prof_wait_full = 0, prof_wait_acc = 0, prof_tiles = 0;
@@ -396,7 +394,9 @@ grouped_gemm_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __gr
     const uint32_t lo_base = (uint32_t)umma_smem_desc(base_addr);  // slot 0
     constexpr uint32_t lo_slot = (uint32_t)kSlotBytes >> 4, lo_box = (uint32_t)kWBoxBytes >> 4;
     uint32_t tcount = 0;
-    for (;;) {
+    const bool gathers = GATHER && warp >= kGatherWarp0;
+    if (gathers) ok = gather_rows();
+    while (!gathers) {
       const uint32_t q = tcount % kQ;
       if (!mbar_wait_warp(bar_tqfull + 8u * q, (tcount / kQ) & 1u, abort_flag, limit)) {
         ok = false;
