@@ -194,9 +194,10 @@ inline bool gather_is_faster(int64_t rows, int64_t E) { return rows > 8192 && ro
 //   few tiles      256 / 512 x 8, 2          1 token 18.6 | 15.8, 16 18.3 | 15.9, 64 19.2 | 17.0;  1024 / 2048 x 4, 2  1 31.8 | 23.8, 64 33.2 | 30.0
 //                  2048 / 768 x 128, 8       1 33.2 | 25.4, 3 53.0 | 49.8;  4096 / 4096 x 8, 2  1 65.9 | 50.0;  1024 / 256 x 64, 8  3 (288
 //                  tiles) 22.4 | 21.2, 8 (768) 26.5 | 28.4;  2048 / 256 x 128, 8  4 (640) 36.0 | 31.2, 32 (2560) 72.5 | 77.1
-//   a longer down  2048 / 768 x 128, 8       8 93.1 | 91.3, 20 142.9 | 142.4, 37 171.4 | 171.1, 64 189.0 | 189.6;  2560 / 1024 x 512, 8  16
-//   pass                                     264.4 | 256.4, 64 710.2 | 697.2;  7168 / 2048 x 256 + shared, 8  3 311.8 | 303.2, 8 725.1 | 694.3,
-//                                            64 2674 | 2642
+//   a longer down  2560 / 1024 x 512, 8      2 58.4 | 53.9, 4 90.7 | 86.2, 16 264.4 | 256.4, 64 710.2 | 697.2;  7168 / 2048 x 256 + shared, 8  3
+//   pass                                     311.8 | 303.2, 8 725.1 | 694.3, 20 1493 | 1463, 64 2674 | 2642;  2048 / 768 x 128, 8  4 61.9 | 57.3,
+//                                            5 67.2 | 64.8, 6 75.1 | 74.7, 7 (two full waves of the small-M kernel) 79.8 | 81.8, 9 97.6 | 94.7, 20
+//                                            140.1 | 141.2, 37 171.4 | 171.1
 //   many rows      7168 / 1024 x 64 + shared, 16  20 427.3 | 424.8, 64 (16 rows an expert) 449.9 | 460.6;  2048 / 1408 x 64 + shared, 6  20
 //                                            163.0 | 158.7, 64 181.3 | 182.6: a group of more than 16 rows takes twice the ring
 // Layers of inter below 256 would gain as well (256 / 128 x 8, 2, 64 tokens 16.9 | 15.0) but keep the launches of the stages: what
@@ -207,7 +208,8 @@ inline bool step_at_once_is_faster(int64_t T, int k, int E, int H, int I, int Is
   if (I < 256 || (Is > 0 && Is < 256)) return false;
   const int64_t slots = T * k, groups = slots < E ? slots : E, down = (H + 127) / 128;
   const int64_t tiles = groups * (I / 64 + down) + (Is > 0 ? Is / 64 + down : 0);
-  return tiles <= 4 * (int64_t)ctas || (all_sms && I >= 640 && slots <= 3 * (int64_t)E);
+  return tiles <= 4 * (int64_t)ctas ||
+         (all_sms && ((I >= 1024 && slots <= 3 * (int64_t)E) || (I >= 640 && 3 * slots <= (int64_t)E)));
 }
 
 }  // namespace moe
