@@ -699,7 +699,8 @@ cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense
   const bool gather = p.gather_src != nullptr;
   // (a row's offset in the source is 32 bits; what it reads comes from the kernel in front of it, so it does without the overlap)
   if (gather && (!p.gated || p.fp8 || p.perm == nullptr || p.top_k < 1 || p.K % kBlockK != 0 ||
-                 (dense != nullptr && (dense->A == nullptr || dense->K % kBlockK != 0 || dense->rows * (int64_t)dense->K * 2 > 0xffffffffLL)) ||
+                 (dense != nullptr && (dense->A == nullptr || dense->K % kBlockK != 0 ||
+                                       dense->rows * (int64_t)dense->K * 2 > 0xffffffffLL)) ||
                  (p.rows_bound / p.top_k + 1) * (int64_t)p.K * 2 > 0xffffffffLL || p.rows_bound <= kGemmOverlapMaxRows))
     return cudaErrorNotSupported;
   const int groups = p.offsets ? p.E : 1;

@@ -56,8 +56,9 @@ constexpr int kAccs = 4;
 constexpr uint32_t kAccCols = kStepMaxTokens, kTmemCols = kAccs * kAccCols;
 constexpr int kStagingBytes = 1024;  // epilogue, per warp: 16 tokens x 32 features
 constexpr int kQ = 4;
-constexpr int kTakeAhead = 4;  // k-blocks
-constexpr int kBatch = 4;  // k-blocks issued in one go
+// k-blocks before a tile's last at which the next tile's number is asked for (8 and 10 are level on long passes, 10 loses 1 % with 128
+// experts, 24 tokens), and k-blocks that are multiplied in one go
+constexpr int kTakeAhead = 4, kBatch = 4;
 constexpr int kGatedFeat = 64, kDownFeat = 128;  // output features of a tile
 constexpr int kCombineTokens = 4 * kFinishWarps;  // tokens of a combine tile: half a warp to two of them
 constexpr int kRowMaps = kStepMaxTokens / 16;
@@ -85,7 +86,7 @@ struct StepMaps {
 enum TileKind { kGated = 0, kDown = 1, kCombine = 2 };
 struct __align__(16) Tile {
   int group;  // (combine: the block of tokens); -1: no more
-  int kind, ft, pad;
+  int kind, ft, unused;
 };
 
 __device__ __forceinline__ int load_relaxed(const int* p) {
@@ -552,8 +553,8 @@ step_ffn_kernel(const __grid_constant__ StepMaps maps, const __grid_constant__ S
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_tempty + 8u * acc.stage);
       if (lane == 0) {
+        mbar_arrive(bar_tempty + 8u * acc.stage);
         mbar_arrive(bar_stored + 8u * q);
         mbar_arrive(bar_tqempty + 8u * q);
       }
@@ -647,7 +648,7 @@ static bool encode_step_maps(StepPlan& plan, const StepFfn& f) {
   auto gated = [&](CUtensorMap* m, const void* w, uint64_t K, uint64_t n_feat, uint64_t groups) {
     ++plan.encoded;
     const uint64_t dims[5] = {K, 16, 2, n_feat / 16, groups};
-    const uint64_t str[4] = {K * sizeof(__nv_bfloat16), n_feat * K * sizeof(__nv_bfloat16), 16 * K * sizeof(__nv_bfloat16), 2 * n_feat * K * sizeof(__nv_bfloat16)};
+    const uint64_t row = K * sizeof(__nv_bfloat16), str[4] = {row, n_feat * row, 16 * row, 2 * n_feat * row};
     const uint32_t box[5] = {(uint32_t)kBlockK, 16u, 2u, (uint32_t)kGatedFeat / 16u, 1u};
     return encode_map(m, w, 5, dims, str, box);
   };

@@ -61,3 +61,32 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_step_is_right():
     torch.cuda.synchronize()
     assert ctx.moe_ctx_status() == B.MOE_OK and torch.equal(got, want)
     ctx.close()
+
+
+def test_a_captured_step_starts_its_counters_anew():
+    shape = wl.LayerShape("s", T=40, H=512, E=12, k=3, I=320, shared_I=256)
+    w = wl.make_weights(shape, 71, DEV)
+    args = (None, w["w_gate_up"], w["w_down"], w["ws_gate_up"], w["ws_down"])
+    ctx = _context(shape, B.MOE_PHASE_PREFILL, B.MOE_GEMM_AUTO, 0)
+    a = wl.make_activations(shape, 72, DEV)
+    bufs, out = B.alloc_step_buffers(40, 3, 12, DEV), torch.empty(40, 512, dtype=torch.bfloat16, device=DEV)
+    ctx.layer(a["x"], a["logits"], *args, out=out, bufs=bufs)
+    torch.cuda.synchronize()
+    graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    cap = B.MoeContext(B.make_config(512, 12, 3, 320, 256, 40), stream=s)
+    with torch.cuda.stream(s):
+        cap.layer(a["x"], a["logits"], *args, out=out, bufs=bufs)
+    s.synchronize()
+    with torch.cuda.graph(graph, stream=s):
+        cap.layer(a["x"], a["logits"], *args, out=out, bufs=bufs)
+    for seed in (73, 74, 75):
+        b = wl.make_activations(shape, seed, DEV)
+        want = ctx.layer(b["x"], b["logits"], *args)[0]
+        a["x"].copy_(b["x"])
+        a["logits"].copy_(b["logits"])
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+    assert cap.moe_ctx_status() == B.MOE_OK
+    ctx.close(), cap.close()
