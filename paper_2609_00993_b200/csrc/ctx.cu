@@ -19,7 +19,8 @@
 namespace {
 
 // ST_NOTIFIED: the first half of a split dispatch has been enqueued (counts, scan, permutation) and the routed
-// data movement is pending; ST_LAYOUT_ONLY: a layout without rows (moe_dispatch_layout with x == NULL).
+// data movement is pending; ST_LAYOUT_ONLY: a layout without rows (moe_dispatch_layout with x == NULL, or a whole step whose
+// gated pass will gather them).
 enum StepState { ST_IDLE = 0, ST_ROUTED = 1, ST_LAID_OUT = 2, ST_LAYOUT_ONLY = 3, ST_FFN_DONE = 4, ST_NOTIFIED = 5 };
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -215,7 +216,6 @@ struct moe_ctx {
   std::mutex* yield_mu;
   int* stopped_host;  // pinned host word: CTAs that stopped in the last launch
   int64_t yields;     // launches that ended on a yield request
-  bool gather_step;   // the step's gated pass gathers its rows from x: none have been moved
   bool offsets_fresh; // the kernel right before the gated pass wrote the step's offsets (moe_layer, a few tokens)
   bool unmarked;      // launches have been enqueued since `done` was last recorded
   int calls_open;     // entry points being executed (the calls of a whole step are made by another)
@@ -509,7 +509,7 @@ moe_status moe_ctx_create(const moe_config* cfg, void* workspace, size_t workspa
   ctx->host_stream = ctx->host_pipeline = false;
   ctx->unmarked = false;
   ctx->calls_open = 0;
-  ctx->offsets_fresh = ctx->gather_step = false;
+  ctx->offsets_fresh = false;
   bool have_plans = true;
   for (int i = 0; i < 16; ++i) {
     moe::StreamPlan*& plan = ctx->plans[i / 8][i % 8];
@@ -716,7 +716,7 @@ moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx
   mark(ctx, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, who);
   ctx->T = T;
-  ctx->offsets_fresh = ctx->gather_step = false;
+  ctx->offsets_fresh = false;
   return MOE_OK;
 }
 
@@ -786,15 +786,16 @@ int ffn_boundaries(const moe_ctx* ctx) {
 
 namespace {
 
-// moe_grouped_ffn.  With piece_cols > 0 (an unsegmented step; a multiple of 256) the down pass runs in pieces of that many
-// output features, and after_piece(first, end) is called when each has been enqueued.
+// moe_grouped_ffn.  With `gather` (step_gathers) the layout moved no rows and the gated pass fetches them from x.  With
+// piece_cols > 0 (an unsegmented step; a multiple of 256) the down pass runs in pieces of that many output features, and
+// after_piece(first, end) is called when each has been enqueued.
 template <class AfterPiece>
 moe_status grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, const void* x, const void* ws_gate_up,
-                       const void* ws_down, int32_t T, int piece_cols, AfterPiece after_piece) {
+                       const void* ws_down, int32_t T, bool gather, int piece_cols, AfterPiece after_piece) {
   if (!ctx) return MOE_ERR_INVALID_ARG;
   if (ctx->cfg.weight_format != MOE_WEIGHTS_BF16)
     return fail(ctx, MOE_ERR_STATE, "the context was created for FP8 weights: call moe_grouped_ffn_fp8");
-  if (ctx->state != ST_LAID_OUT)
+  if (ctx->state != (gather ? ST_LAYOUT_ONLY : ST_LAID_OUT))
     return fail(ctx, MOE_ERR_STATE, "moe_grouped_ffn needs a moe_dispatch_layout with x in the same step");
   if (T != ctx->T) return fail(ctx, MOE_ERR_INVALID_ARG, "T = %d differs from the layout's T = %d", T, ctx->T);
   if (!w_gate_up || !w_down) return fail(ctx, MOE_ERR_INVALID_ARG, "routed weights are NULL");
@@ -827,7 +828,7 @@ moe_status grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, 
     };
     moe::GemmProblem g1{b.x_perm, w_gate_up, b.act, ctx->offsets, 0, Ncap, N, c.n_experts, c.inter, c.hidden, true};
     moe::GemmProblem g2{b.act, w_down, b.y_perm, ctx->offsets, 0, Ncap, N, c.n_experts, c.hidden, c.inter, false};
-    if (gathers_rows(ctx) || ctx->gather_step) {
+    if (gathers_rows(ctx) || gather) {
       g1.gather_src = x;
       g1.perm = ctx->perm;
       g1.top_k = c.top_k;
@@ -995,7 +996,7 @@ moe_status moe_ctx_pending_dispatch(moe_ctx* ctx, int32_t* pending, int32_t* tok
 
 moe_status moe_grouped_ffn(moe_ctx* ctx, const void* w_gate_up, const void* w_down, const void* x,
                            const void* ws_gate_up, const void* ws_down, int32_t T) {
-  return grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T, 0, [](int, int) { return cudaSuccess; });
+  return grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T, false, 0, [](int, int) { return cudaSuccess; });
 }
 
 moe_status moe_grouped_ffn_fp8(moe_ctx* ctx, const void* wq_gate_up, const float* sw_gate_up, const void* wq_down,
@@ -1149,19 +1150,18 @@ moe_status moe_combine(moe_ctx* ctx, const float* topk_w, const int32_t* inv_per
 namespace {
 
 // moe_route and moe_dispatch_layout of a whole step, as one launch where that is possible (an FP8 context quantises and
-// moves its rows in a second one).
+// moves its rows in a second one).  gather: no rows are moved (step_gathers, whose steps are never dispatched in one launch).
 moe_status route_and_dispatch(moe_ctx* ctx, const char* who, const float* logits, const float* select_bias, const void* x,
                               int32_t T, int32_t* topk_idx, float* topk_w, int32_t* counts, int32_t* offsets, int32_t* perm,
-                              int32_t* inv_perm, int zero_words) {
+                              int32_t* inv_perm, bool gather, int zero_words) {
   if (!dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm)) {
     moe_status st = moe_route(ctx, logits, select_bias, T, topk_idx, topk_w);
     if (st != MOE_OK) return st;
-    if (!step_gathers(ctx, T, x)) return moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm);
+    if (!gather) return moe_dispatch_layout(ctx, topk_idx, T, x, counts, offsets, perm, inv_perm);
     DeviceGuard guard(ctx->device);
     st = enqueue_layout(ctx, who, topk_idx, T, counts, offsets, perm, inv_perm);
     if (st != MOE_OK) return st;
-    ctx->gather_step = true;
-    ctx->state = ST_LAID_OUT;
+    ctx->state = ST_LAYOUT_ONLY;
     ctx->split_step = false;
     return MOE_OK;
   }
@@ -1264,10 +1264,12 @@ moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias
   PositionMark position(ctx);
   const bool at_once = ffn_at_once(ctx, T, w_gate_up, w_down, ws_gate_up, ws_down, out) &&
                        dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
+  const bool gather = step_gathers(ctx, T, x);
   moe_status st = route_and_dispatch(ctx, "moe_layer", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm,
-                                     at_once ? moe::step_ffn_counters(ctx->cfg.n_experts, ctx->cfg.hidden) : 0);
+                                     gather, at_once ? moe::step_ffn_counters(ctx->cfg.n_experts, ctx->cfg.hidden) : 0);
   if (at_once) return st == MOE_OK ? step_ffn(ctx, "moe_layer", w_gate_up, w_down, ws_gate_up, ws_down, x, topk_w, out) : st;
-  if (st == MOE_OK) st = moe_grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T);
+  if (st == MOE_OK)
+    st = grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, T, gather, 0, [](int, int) { return cudaSuccess; });
   if (st == MOE_OK) st = combine(ctx, topk_w, inv_perm, T, out, ctx->seg_experts == 0 && !ctx->preemptible);
   return st;
 }
@@ -1280,7 +1282,7 @@ moe_status moe_layer_fp8(moe_ctx* ctx, const float* logits, const float* select_
   if (!ctx) return MOE_ERR_INVALID_ARG;
   PositionMark position(ctx);
   moe_status st =
-      route_and_dispatch(ctx, "moe_layer_fp8", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm, 0);
+      route_and_dispatch(ctx, "moe_layer_fp8", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm, false, 0);
   if (st == MOE_OK)
     st = moe_grouped_ffn_fp8(ctx, wq_gate_up, sw_gate_up, wq_down, sw_down, wsq_gate_up, sws_gate_up, wsq_down, sws_down, T);
   if (st == MOE_OK) st = combine(ctx, topk_w, inv_perm, T, out, ctx->seg_experts == 0 && !ctx->preemptible);
@@ -1374,10 +1376,10 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
       if (st != MOE_OK) break;
       if (i == 0) e = have_stream ? cudaStreamWaitEvent(ctx->stream, ctx->copied_in[0], 0) : copy_rows(0, ctx->stream);
       if (e != cudaSuccess) break;
-      ctx->gather_step = step_gathers(ctx, n_tok, x);
-      if (!ctx->gather_step) st = enqueue_row_movement(ctx, "moe_layer_host", x);
+      const bool gather = step_gathers(ctx, n_tok, x);
+      if (!gather) st = enqueue_row_movement(ctx, "moe_layer_host", x);
       if (st != MOE_OK) break;
-      ctx->state = ST_LAID_OUT;
+      ctx->state = gather ? ST_LAYOUT_ONLY : ST_LAID_OUT;
       ctx->split_step = false;
       const int pieces = i + 1 < n_chunks ? 1 : (int)std::min<size_t>(kHostMaxPieces, 1 + n_tok * row_bytes / kHostPieceBytes);
       const int piece_cols = (c.hidden / pieces + 255) / 256 * 256;
@@ -1401,7 +1403,7 @@ moe_status moe_layer_host(moe_ctx* ctx, const float* logits_host, const float* s
         return cudaMemcpy2DAsync(out_to + (size_t)c0 * 2, row_bytes, out + (size_t)c0 * 2, row_bytes, (size_t)(c1 - c0) * 2, n_tok,
                                  cudaMemcpyDeviceToHost, ctx->h2d_stream);
       };
-      st = grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, n_tok, pieces > 1 ? piece_cols : 0, finish);
+      st = grouped_ffn(ctx, w_gate_up, w_down, x, ws_gate_up, ws_down, n_tok, gather, pieces > 1 ? piece_cols : 0, finish);
       if (st != MOE_OK) break;
       if (pieces == 1) e = finish(0, c.hidden);
       ctx->state = ST_IDLE;

@@ -56,3 +56,49 @@ def test_gathered_from_host_buffers():
         assert torch.equal(out, want.cpu())
     assert ctx.moe_ctx_status() == B.MOE_OK
     ctx.close()
+
+
+@pytest.mark.parametrize("H,E,k,I", [(2048, 128, 8, 768), (1024, 512, 8, 128)])
+@pytest.mark.parametrize("then", ["", "segments", "preemption"])
+@pytest.mark.parametrize("path", ["device", "host"])
+def test_a_gathered_batch_leaves_nothing_to_the_next_one(H, E, k, I, then, path):
+    """One context, batches that gather and batches that do not in turn, each against a context of its own."""
+    sizes = (4001, 37, 4001, 64, 1, 300, 1531, 7)
+    w = wl.make_weights(wl.LayerShape("g", T=1, H=H, E=E, k=k, I=I), 55, DEV)
+
+    def context(switched):
+        cfg = B.make_config(H, E, k, I, 0, max(sizes), B.MOE_PHASE_PREFILL)
+        ctx = B.MoeContext(cfg, workspace=torch.full((B.moe_ctx_workspace_bytes(cfg),), 0xFF, dtype=torch.uint8, device=DEV))
+        if switched:
+            switch(ctx)
+        return ctx
+
+    def switch(ctx):
+        if then == "segments":
+            ctx.moe_ctx_set_segments(E // 2, lambda i, n: None)
+        elif then == "preemption":
+            ctx.moe_ctx_set_preemption(True)
+
+    def step(ctx, a, T):
+        if path == "device":
+            out, bufs = ctx.layer(a["x"], a["logits"], None, w["w_gate_up"], w["w_down"])
+            torch.cuda.synchronize()
+            return {"out": out, **bufs}
+        out = torch.zeros(T, H, dtype=torch.bfloat16).pin_memory()
+        ctx.moe_layer_host(a["logits"].cpu().pin_memory(), None, a["x"].cpu().pin_memory(), w["w_gate_up"], w["w_down"], None, None, out)
+        return {"out": out}
+
+    kept = context(False)
+    for i, T in enumerate(sizes):
+        a = wl.make_activations(wl.LayerShape("g", T=T, H=H, E=E, k=k, I=I), 56 + i, DEV)
+        fresh = context(i > 0)
+        torch.cuda.synchronize()
+        want, got = step(fresh, a, T), step(kept, a, T)
+        assert fresh.moe_ctx_status() == B.MOE_OK and kept.moe_ctx_status() == B.MOE_OK
+        assert torch.isfinite(want["out"].float()).all()
+        for name in want:
+            assert torch.equal(got[name], want[name]), (T, name)
+        fresh.close()
+        if i == 0:
+            switch(kept)
+    kept.close()
