@@ -720,6 +720,13 @@ moe_status enqueue_layout(moe_ctx* ctx, const char* who, const int32_t* topk_idx
   return MOE_OK;
 }
 
+// Whether a whole step's passes will find nothing wrong with these pointers.  A step that they would refuse is routed and laid
+// out as the staged calls do it, rows and all, so that those can go on from there.
+bool passes_accept(const moe_ctx* ctx, const void* w1, const void* w2, const void* w1_sh, const void* w2_sh) {
+  return w1 && w2 && (ctx->cfg.n_shared == 0 || (w1_sh && w2_sh)) && !misaligned(w1) && !misaligned(w2) && !misaligned(w1_sh) &&
+         !misaligned(w2_sh);
+}
+
 // Whether the gated pass of a whole step of T tokens, whose rows it knows from the start, gathers them from x.
 bool step_gathers(const moe_ctx* ctx, int32_t T, const void* x) {
   const moe_config& c = ctx->cfg;
@@ -1202,8 +1209,7 @@ bool ffn_at_once(const moe_ctx* ctx, int32_t T, const void* w1, const void* w2, 
       !moe::step_at_once_is_faster(T, c.top_k, c.n_experts, c.hidden, c.inter, shared ? c.shared_inter : 0, gemm_ctas(ctx),
                                    gemm_ctas(ctx) == ctx->n_sms))
     return false;
-  if (!w1 || !w2 || !out || (shared && (!w1_sh || !w2_sh))) return false;
-  return !misaligned(w1) && !misaligned(w2) && !misaligned(w1_sh) && !misaligned(w2_sh) && !misaligned(out) &&
+  return passes_accept(ctx, w1, w2, w1_sh, w2_sh) && out && !misaligned(out) &&
          moe::step_ffn_counters(c.n_experts, c.hidden) <= kStepCounterWords;
 }
 
@@ -1264,7 +1270,7 @@ moe_status moe_layer(moe_ctx* ctx, const float* logits, const float* select_bias
   PositionMark position(ctx);
   const bool at_once = ffn_at_once(ctx, T, w_gate_up, w_down, ws_gate_up, ws_down, out) &&
                        dispatches_at_once(ctx, logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm);
-  const bool gather = step_gathers(ctx, T, x);
+  const bool gather = passes_accept(ctx, w_gate_up, w_down, ws_gate_up, ws_down) && step_gathers(ctx, T, x);
   moe_status st = route_and_dispatch(ctx, "moe_layer", logits, select_bias, x, T, topk_idx, topk_w, counts, offsets, perm, inv_perm,
                                      gather, at_once ? moe::step_ffn_counters(ctx->cfg.n_experts, ctx->cfg.hidden) : 0);
   if (at_once) return st == MOE_OK ? step_ffn(ctx, "moe_layer", w_gate_up, w_down, ws_gate_up, ws_down, x, topk_w, out) : st;

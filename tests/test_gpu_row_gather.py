@@ -102,3 +102,23 @@ def test_a_gathered_batch_leaves_nothing_to_the_next_one(H, E, k, I, then, path)
         if i == 0:
             switch(kept)
     kept.close()
+
+
+def test_a_step_whose_passes_are_refused_has_moved_its_rows():
+    """The staged calls go on from there, as behind a step that does not gather."""
+    T, H, E, k, I = 1100, 2048, 128, 8, 256
+    shape = wl.LayerShape("g", T=T, H=H, E=E, k=k, I=I)
+    w, a = wl.make_weights(shape, 57, DEV), wl.make_activations(shape, 58, DEV)
+    cfg = B.make_config(H, E, k, I, 0, T, B.MOE_PHASE_PREFILL)
+    ctx = B.MoeContext(cfg, workspace=torch.full((B.moe_ctx_workspace_bytes(cfg),), 0xFF, dtype=torch.uint8, device=DEV))
+    bufs, out = B.alloc_step_buffers(T, k, E, DEV), torch.empty(T, H, dtype=torch.bfloat16, device=DEV)
+    torch.cuda.synchronize()
+    with pytest.raises(B.MoeError, match="weights are NULL"):
+        ctx.layer(a["x"], a["logits"], None, w["w_gate_up"], None, out=out, bufs=bufs)
+    ctx.moe_grouped_ffn(w["w_gate_up"], w["w_down"], None, T=T)
+    ctx.moe_combine(bufs["topk_w"], bufs["inv_perm"], out)
+    want = ctx.layer(a["x"], a["logits"], None, w["w_gate_up"], w["w_down"])[0]
+    torch.cuda.synchronize()
+    assert ctx.moe_ctx_status() == B.MOE_OK
+    assert torch.isfinite(want.float()).all() and torch.equal(out, want)
+    ctx.close()
