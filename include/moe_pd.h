@@ -422,8 +422,10 @@ moe_status moe_ctx_debug_gemm(const moe_ctx* ctx, int32_t* gated, int32_t* down,
  * 4 routed GEMM2, 5 shared GEMM1+SwiGLU, 6 shared GEMM2, 7 combine.  Without prefill segmentation the shared
  * expert's passes ride in the routed launches, so their time is part of stages 3 and 4 and stages 5 and 6
  * stay empty.  moe_layer and moe_layer_fp8 route, lay out and (bf16) move up to 64 tokens in one launch, which is
- * stage 0; stages 1 and 2 then stay empty.  FP8 variant only: 8 quantise the GEMM1 input rows, 9 quantise the activation rows. */
-#define MOE_N_STAGES 10
+ * stage 0; stages 1 and 2 then stay empty.  Where moe_layer goes on to make both passes and the combine of such a step in one
+ * launch, too, that launch is stage 10 and stages 3, 4 and 7 stay empty.  Where the gated pass of a whole step gathers its rows,
+ * stage 2 stays empty.  FP8 variant only: 8 quantise the GEMM1 input rows, 9 quantise the activation rows. */
+#define MOE_N_STAGES 11
 typedef struct {
   double ms[MOE_N_STAGES];
   int64_t calls[MOE_N_STAGES];
@@ -434,7 +436,7 @@ moe_status moe_ctx_read_profile(moe_ctx* ctx, moe_stage_times* out);
 /* Kernels launched on this context since creation (for launch accounting in benchmarks). */
 int64_t moe_ctx_launch_count(const moe_ctx* ctx);
 
-/* Library version string, e.g. "moe_pd 0.1 (sm_100a)". */
+/* Library version string, e.g. "moe_pd 0.2 (sm_100a)". */
 const char* moe_version(void);
 
 #ifdef __cplusplus

@@ -41,7 +41,7 @@ EXPORTS = ("moe_version", "moe_ctx_workspace_bytes", "moe_ctx_create", "moe_ctx_
 BOUNDARY_FN = ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32)
 
 STAGE_NAMES = ("route", "layout", "permute", "gemm1_swiglu", "gemm2", "shared_gemm1_swiglu", "shared_gemm2", "combine",
-               "quantize_x", "quantize_act")
+               "quantize_x", "quantize_act", "ffn_combine")
 
 
 class moe_config(ctypes.Structure):
@@ -53,7 +53,7 @@ class moe_config(ctypes.Structure):
 
 
 class moe_stage_times(ctypes.Structure):
-    _fields_ = [("ms", ctypes.c_double * 10), ("calls", ctypes.c_int64 * 10)]
+    _fields_ = [("ms", ctypes.c_double * len(STAGE_NAMES)), ("calls", ctypes.c_int64 * len(STAGE_NAMES))]
 
 
 class MoeError(RuntimeError):

@@ -456,7 +456,7 @@ cudaError_t ensure_dynamic_smem_impl(const void* kern, size_t bytes) {
 
 extern "C" {
 
-const char* moe_version(void) { return "moe_pd 0.1 (sm_100a)"; }
+const char* moe_version(void) { return "moe_pd 0.2 (sm_100a)"; }
 
 size_t moe_ctx_workspace_bytes(const moe_config* cfg) {
   if (validate_config(cfg)) return 0;
@@ -1247,7 +1247,7 @@ moe_status step_ffn(moe_ctx* ctx, const char* who, const void* w1, const void* w
   int n = 0;
   cudaError_t e;
   {
-    StageTimer tm(ctx, 3);
+    StageTimer tm(ctx, 10);
     e = moe::launch_step_ffn(f, ctx->step_plans[ctx->cur], gemm_ctas(ctx), ctx->stream, &n);
   }
   mark(ctx, n);

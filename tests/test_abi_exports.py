@@ -25,6 +25,12 @@ def test_library_builds_and_exports_every_declared_symbol():
     assert "sm_100a" in B.moe_version()
 
 
+def test_the_stages_of_the_binding_are_the_headers():
+    text = open(os.path.join(ROOT, "include", "moe_pd.h")).read()
+    assert int(re.search(r"#define MOE_N_STAGES (\d+)", text).group(1)) == len(B.STAGE_NAMES)
+    assert ctypes.sizeof(B.moe_stage_times) == 16 * len(B.STAGE_NAMES)
+
+
 def test_host_only_entry_points_work_without_a_gpu():
     cfg = B.make_config(7168, 256, 8, 2048, 2048, 128, B.MOE_PHASE_DECODE)
     n = B.moe_ctx_workspace_bytes(cfg)

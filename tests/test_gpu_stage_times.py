@@ -17,9 +17,24 @@ DEV = "cuda"
     (65, True, {"route", "layout", "quantize_x", "gemm1_swiglu", "quantize_act", "gemm2", "combine"}),
 ])
 def test_stage_times_are_those_of_the_step(T, fp8, stages):
-    shape = wl.LayerShape("t", T=T, H=256, E=8, k=2, I=128)
+    _check(wl.LayerShape("t", T=T, H=256, E=8, k=2, I=128), fp8, stages)
+
+
+@pytest.mark.parametrize("T,H,E,k,I,stages", [
+    (64, 256, 8, 2, 512, {"route", "ffn_combine"}),       # both passes and the combine in one launch
+    (65, 256, 8, 2, 512, {"route", "layout", "permute", "gemm1_swiglu", "gemm2", "combine"}),
+    (64, 2048, 128, 8, 256, {"route", "gemm1_swiglu", "gemm2", "combine"}),  # too many tiles for that
+    (1055, 2368, 33, 8, 960, {"route", "layout", "gemm1_swiglu", "gemm2", "combine"}),             # the gated pass gathers
+    (1056, 2368, 33, 8, 960, {"route", "layout", "permute", "gemm1_swiglu", "gemm2", "combine"}),
+])
+def test_stages_that_are_one_launch_or_none(T, H, E, k, I, stages):
+    _check(wl.LayerShape("t", T=T, H=H, E=E, k=k, I=I), False, stages)
+
+
+def _check(shape, fp8, stages):
+    T = shape.T
     w, a = (wl.make_weights_fp8 if fp8 else wl.make_weights)(shape, 1, DEV), wl.make_activations(shape, 2, DEV)
-    ctx = B.MoeContext(B.make_config(256, 8, 2, 128, 0, T, weight_format=B.MOE_WEIGHTS_FP8_E4M3 if fp8 else B.MOE_WEIGHTS_BF16))
+    ctx = B.MoeContext(B.make_config(shape.H, shape.E, shape.k, shape.I, 0, T, weight_format=B.MOE_WEIGHTS_FP8_E4M3 if fp8 else B.MOE_WEIGHTS_BF16))
     torch.cuda.synchronize()
     outs, launches = [], []
     for profiling in (False, True):
