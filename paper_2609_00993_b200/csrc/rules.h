@@ -188,28 +188,46 @@ inline bool pair_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t rows
 inline bool gather_is_faster(int64_t rows, int64_t E) { return rows > 8192 && rows < 256 * E; }
 
 // ---- whether a bf16 step of up to 64 tokens makes its passes and its combine in one launch (step_ffn.cu)
-// It gains a chain of launches and tiles half as large, which counts where there are few of them, and its weights stream over the seam
-// between the passes; its price is 1.2 to 1.5 us an SM for each tile, more than the HBM asks for where the down pass is short.  Whole steps,
-// us, three launches | one, hidden / inter x experts, top-k:
-//   few tiles      256 / 512 x 8, 2          1 token 18.6 | 15.8, 16 18.3 | 15.9, 64 19.2 | 17.0;  1024 / 2048 x 4, 2  1 31.8 | 23.8, 64 33.2 | 30.0
-//                  2048 / 768 x 128, 8       1 33.2 | 25.4, 3 53.0 | 49.8;  4096 / 4096 x 8, 2  1 65.9 | 50.0;  1024 / 256 x 64, 8  3 (288
-//                  tiles) 22.4 | 21.2, 8 (768) 26.5 | 28.4;  2048 / 256 x 128, 8  4 (640) 36.0 | 31.2, 32 (2560) 72.5 | 77.1
-//   a longer down  2560 / 1024 x 512, 8      2 58.4 | 53.9, 4 90.7 | 86.2, 16 264.4 | 256.4, 64 710.2 | 697.2;  7168 / 2048 x 256 + shared, 8  3
-//   pass                                     311.8 | 303.2, 8 725.1 | 694.3, 20 1493 | 1463, 64 2674 | 2642;  2048 / 768 x 128, 8  4 61.9 | 57.3,
-//                                            5 67.2 | 64.8, 6 75.1 | 74.7, 7 (two full waves of the small-M kernel) 79.8 | 81.8, 9 97.6 | 94.7, 20
-//                                            140.1 | 141.2, 37 171.4 | 171.1
-//   many rows      7168 / 1024 x 64 + shared, 16  20 427.3 | 424.8, 64 (16 rows an expert) 449.9 | 460.6;  2048 / 1408 x 64 + shared, 6  20
-//                                            163.0 | 158.7, 64 181.3 | 182.6: a group of more than 16 rows takes twice the ring
-// Layers of inter below 256 would gain as well (256 / 128 x 8, 2, 64 tokens 16.9 | 15.0) but keep the launches of the stages: what
-// their stage times and their launches add up to is fixed for such steps.
+// It gains a chain of launches, and tiles half as large where the 256-row tiles of a pass are fewer than the CTAs or fill half of a
+// second wave; it loses 1.2 to 1.5 us of an SM for each tile, which shows where a tile's k-blocks are few, and seams between the tiles of a
+// CTA.  So few slots (T * k) gain at nearly any shape, many only where each CTA has about one tile, or where the weights take so long that
+// the stream over the seam between the passes counts.  The lines were drawn through 3600 layers and sizes at random (hidden and
+// inter 64 to 7168, 4 to 512 experts, top-1 to top-32, with and without a shared expert): steps called one by one, and steps replayed from a
+// graph over layers with weights of their own (in brackets), where a launch costs less.  Time with three launches over time with one,
+// geometric mean and worst:
+//   both passes' tiles on 7/8 of the CTAs, top-16 at most     1.14, 0.91 (1.12, 0.98);  with 132 to 148 tiles 1.07, 0.72 (0.97, 0.77)
+//   up to 12 slots                                            1.25, 1.02 (1.17, 0.97)
+//   hidden or inter from 1024 on, up to 28 slots              1.18, 1.01 (1.13, 0.95);  29 to 40 slots 1.11, 0.96 (1.03, 0.88);  where the
+//     256-row tiles of a pass fit the CTAs and its 128-row tiles do not: few tiles 1.12, 0.98 (1.06, 0.96), more 1.03, 0.96 (1.00, 0.94)
+//   both shorter, up to 16 slots and 4 tiles a CTA            1.12, 1.08 (0.99, 0.94);  17 to 28 slots 1.07, 0.93 (0.99, 0.90)
+//   4 tiles a CTA, up to 128 slots, top-8 at most             1.15, 0.97 (1.15, 1.04) with hidden or inter from 2048 on; 1.09, 0.94 (1.01, 0.93)
+//     where the 256-row tiles of a pass end within half a second wave
+//   what is left                                              1.01, 0.56 (0.96, 0.70):  256 / 256 x 32, top-16, 64 tokens 21.8 us | 29.9,
+//     960 / 640 x 16, 8, 31 tokens 24.6 | 30.5, 1024 / 512 x 16, 8, 64 25.0 | 28.4, 512 / 1472 x 8, 8, 61 28.4 | 32.5
+// A longer down pass, us from a graph, slots over experts in brackets: 7168 / 2048 x 256 + shared, 8  4 tokens 415 | 389, 32 (1) 1544 | 1515, 64
+//   (2) 2078 | 2048, skewed 64 617 | 625;  2560 / 1024 x 512, 8  8 160 | 153, 64 (1) 749 | 735;  4096 / 1536 x 128, 8  48 (3) 682 | 673;
+//   4096 / 2048 x 32, 4  24 (3) 246 | 237;  2048 / 768 x 128, 8  4 (0.25) 60.3 | 57.1, 5 66.6 | 65.4, 6 (0.38) 73.3 | 74.9;  7168 / 1024 x 64 +
+//   shared, 16  12 (3) 426 | 415, 64 (16) 463 | 479;  shorter hidden  1024 / 2048 x 64, 8  16 (2) 117 | 121.5;  1536 / 1536 x 64, 8  8 (1) 99.6 |
+//   101.8
 // A context on part of the SMs takes it for few tiles only: its decode steps run beside a prefill batch on the others, from which a steadier
 // stream takes HBM that those SMs cannot make up for later (V3-shaped, skewed: 64 tokens beside 900, 4540 | 4642 for both).
 inline bool step_at_once_is_faster(int64_t T, int k, int E, int H, int I, int Is, int ctas, bool all_sms) {
-  if (I < 256 || (Is > 0 && Is < 256)) return false;
-  const int64_t slots = T * k, groups = slots < E ? slots : E, down = (H + 127) / 128;
-  const int64_t tiles = groups * (I / 64 + down) + (Is > 0 ? Is / 64 + down : 0);
-  return tiles <= 4 * (int64_t)ctas ||
-         (all_sms && ((I >= 1024 && slots <= 3 * (int64_t)E) || (I >= 640 && 3 * slots <= (int64_t)E)));
+  const int64_t slots = T * k, groups = slots < E ? slots : E, dense = Is > 0 ? 1 : 0;
+  const auto over = [](int64_t n, int64_t d) { return (n + d - 1) / d; };
+  const int64_t gated = groups * (I / 64) + Is / 64, down = (groups + dense) * over(H, 128), tiles = gated + down;   // this kernel's
+  const int64_t gated256 = groups * over(I, 128) + over(Is, 128), down256 = (groups + dense) * over(H, 256);          // the small-M kernel's
+  const bool few = tiles <= 4 * (int64_t)ctas, is_long = H >= 1024 || I >= 1024;
+  if (!all_sms && !few) return false;
+  if (8 * tiles <= 7 * (int64_t)ctas) return k <= 16;
+  if (slots <= 12) return true;
+  // a wave of 256-row tiles against two of half as many rows
+  const bool level = (gated > ctas && gated256 <= ctas) || (down > ctas && down256 <= ctas);
+  if (level && few) return is_long && slots <= 28;
+  if (all_sms && H >= 2048 && (I >= 1024 ? slots <= 3 * (int64_t)E : I >= 640 && 3 * slots <= (int64_t)E)) return true;
+  if (level) return false;
+  if (is_long ? slots <= 28 : few && slots <= 16) return true;
+  const auto part = [&](int64_t t) { return t > ctas && 2 * t <= 3 * (int64_t)ctas; };
+  return few && k <= 8 && slots <= 128 && (H >= 2048 || I >= 2048 || part(gated256) || part(down256));
 }
 
 }  // namespace moe

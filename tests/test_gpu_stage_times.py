@@ -11,7 +11,7 @@ DEV = "cuda"
 
 
 @pytest.mark.parametrize("T,fp8,stages", [
-    (64, False, {"route", "gemm1_swiglu", "gemm2", "combine"}),
+    (64, False, {"route", "ffn_combine"}),  # both passes and the combine in one launch
     (65, False, {"route", "layout", "permute", "gemm1_swiglu", "gemm2", "combine"}),
     (64, True, {"route", "quantize_x", "gemm1_swiglu", "quantize_act", "gemm2", "combine"}),
     (65, True, {"route", "layout", "quantize_x", "gemm1_swiglu", "quantize_act", "gemm2", "combine"}),
@@ -21,9 +21,8 @@ def test_stage_times_are_those_of_the_step(T, fp8, stages):
 
 
 @pytest.mark.parametrize("T,H,E,k,I,stages", [
-    (64, 256, 8, 2, 512, {"route", "ffn_combine"}),       # both passes and the combine in one launch
-    (65, 256, 8, 2, 512, {"route", "layout", "permute", "gemm1_swiglu", "gemm2", "combine"}),
-    (64, 2048, 128, 8, 256, {"route", "gemm1_swiglu", "gemm2", "combine"}),  # too many tiles for that
+    (3, 2048, 128, 8, 768, {"route", "ffn_combine"}),
+    (64, 2048, 128, 8, 256, {"route", "gemm1_swiglu", "gemm2", "combine"}),  # too many slots for one launch
     (1055, 2368, 33, 8, 960, {"route", "layout", "gemm1_swiglu", "gemm2", "combine"}),             # the gated pass gathers
     (1056, 2368, 33, 8, 960, {"route", "layout", "permute", "gemm1_swiglu", "gemm2", "combine"}),
 ])

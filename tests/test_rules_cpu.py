@@ -55,3 +55,30 @@ def test_layout_reads_stay_linear_in_the_batch(rules):
 ])
 def test_the_kernel_that_was_measured_faster_is_chosen(rules, fp8, gated, K, n_feat, E, R, small):
     assert rules(f"moe::small_m_is_faster({fp8}, {gated}, {K}, {n_feat}, {R * E}LL, {E}, 148)") == [small]
+
+
+@pytest.mark.parametrize("H,I,E,k,Is,T,ctas,at_once", [
+    # whole steps measured in one launch and in three, at least 2 % apart unless at the edge of a line (csrc/rules.h)
+    (256, 512, 8, 2, 0, 64, 148, 1), (256, 128, 8, 2, 0, 64, 148, 1), (64, 64, 32, 16, 0, 64, 148, 1), (448, 320, 16, 10, 0, 47, 148, 0),  # 128 | 144 tiles
+    (320, 192, 4, 4, 64, 64, 148, 1), (64, 64, 32, 32, 0, 32, 148, 0), (128, 64, 64, 32, 1024, 12, 148, 0),                             # top-32
+    (6592, 128, 128, 12, 0, 1, 148, 1), (6592, 128, 128, 32, 0, 6, 148, 0), (704, 640, 64, 2, 0, 6, 148, 1),                              # 12 slots
+    (2048, 768, 128, 8, 0, 3, 148, 1), (1024, 256, 64, 8, 0, 3, 148, 1), (1024, 256, 64, 8, 0, 4, 148, 0), (1024, 960, 64, 2, 0, 14, 148, 0),
+    (768, 1792, 128, 4, 64, 7, 148, 0), (4160, 576, 32, 8, 0, 3, 148, 0), (704, 2112, 64, 16, 0, 1, 148, 1), (704, 2112, 64, 16, 0, 2, 148, 0),
+    (512, 512, 16, 4, 0, 4, 148, 1), (192, 512, 24, 4, 0, 8, 148, 0), (256, 256, 32, 8, 0, 64, 148, 0), (256, 256, 32, 16, 0, 64, 148, 0),
+    (4992, 2048, 4, 4, 2048, 11, 148, 0), (4928, 576, 8, 8, 576, 7, 148, 1), (1024, 2048, 4, 2, 0, 64, 148, 1), (1024, 2048, 8, 8, 0, 64, 148, 0),
+    (4096, 256, 16, 4, 0, 32, 148, 1), (4096, 256, 16, 4, 0, 33, 148, 0), (960, 640, 16, 8, 0, 31, 148, 0), (1024, 512, 16, 8, 0, 64, 148, 0),
+    (7168, 2048, 256, 8, 2048, 64, 148, 1), (2560, 1024, 512, 8, 0, 64, 148, 1), (4096, 1536, 128, 8, 0, 48, 148, 1),
+    (4096, 1536, 128, 8, 0, 49, 148, 0), (2048, 768, 128, 8, 0, 5, 148, 1), (2048, 768, 128, 8, 0, 6, 148, 0), (2048, 768, 128, 8, 0, 37, 148, 0),
+    (1536, 1536, 64, 8, 0, 8, 148, 0), (1024, 2048, 64, 8, 0, 16, 148, 0), (7168, 1024, 64, 16, 1024, 12, 148, 1), (7168, 1024, 64, 16, 1024, 13, 148, 0),
+    # on part of the SMs: few tiles only
+    (7168, 2048, 256, 8, 2048, 64, 100, 0), (7168, 2048, 256, 8, 2048, 1, 100, 0), (256, 512, 8, 2, 0, 64, 100, 1), (1024, 256, 64, 8, 0, 1, 48, 1),
+])
+def test_the_steps_made_in_one_launch(rules, H, I, E, k, Is, T, ctas, at_once):
+    assert rules(f"moe::step_at_once_is_faster({T}, {k}, {E}, {H}, {I}, {Is}, {ctas}, {int(ctas == 148)})") == [at_once]
+
+
+def test_the_rows_that_the_gated_pass_gathers(rules):
+    """Above 8192 rows (up to there moving them hides behind the pass's set-up) and below 256 rows an expert."""
+    cases = [(8192, 128, 0), (8193, 128, 1), (1025 * 8, 128, 1), (4001 * 8, 128, 1), (4096 * 8, 128, 0), (8447, 33, 1), (8448, 33, 0), (8193, 32, 0),
+             (4096 * 8, 512, 1), (7000 * 8, 256, 1), (8192 * 8, 256, 0)]
+    assert rules(*[f"moe::gather_is_faster({rows}LL, {E})" for rows, E, _ in cases]) == [g for _, _, g in cases]
