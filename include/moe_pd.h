@@ -400,7 +400,7 @@ moe_status moe_layer_host_wait(moe_ctx* ctx, int32_t slot);
  * the second).  Rows
  * [0, T*k) of x_perm [.,H], act [.,I], y_perm [.,H] and rows [0,T) of y_shared [.,H] are
  * defined after the respective stage (x_perm: not after a whole step whose gated pass gathered its rows, as
- * moe_layer and moe_layer_host do from 8193 rows on).  Any out-pointer may be NULL. */
+ * moe_layer and moe_layer_host may do from 8193 rows on).  Any out-pointer may be NULL. */
 moe_status moe_ctx_debug_ptrs(moe_ctx* ctx, void** x_perm, void** act, void** y_perm, void** y_shared,
                               int32_t** counts, int32_t** offsets);
 

@@ -732,7 +732,7 @@ bool step_gathers(const moe_ctx* ctx, int32_t T, const void* x) {
   const moe_config& c = ctx->cfg;
   if (c.gemm_variant != MOE_GEMM_AUTO || c.phase != MOE_PHASE_PREFILL || c.weight_format != MOE_WEIGHTS_BF16 || c.row_gather != 0 ||
       ctx->seg_experts > 0 || ctx->preemptible || T < 1 || x == nullptr || misaligned(x) ||
-      gemm_ctas(ctx) != ctx->n_sms || !moe::gather_is_faster((int64_t)T * c.top_k, c.n_experts) || (int64_t)(T + 1) * c.hidden * 2 > 0xffffffffLL)
+      gemm_ctas(ctx) != ctx->n_sms || !moe::gather_is_faster((int64_t)T * c.top_k, c.n_experts, c.hidden, c.inter) || (int64_t)(T + 1) * c.hidden * 2 > 0xffffffffLL)
     return false;
   moe::GemmProblem g{};
   g.rows_bound = (int64_t)T * c.top_k;

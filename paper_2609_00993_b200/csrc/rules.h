@@ -177,15 +177,23 @@ inline bool pair_is_faster(bool fp8, bool gated, int K, int n_feat, int64_t rows
 }
 
 // ---- whether the gated pass of a whole bf16 step gathers its rows itself, where the small-M kernel takes it (gemm_stream.cu)
-// It saves the launch that moves the rows, and its write and re-read of them.  Up to 8192 rows that launch is hidden behind the set-up of
-// the gated pass, which would have to wait for the layout instead; with whole tiles of 256 rows the threads that gather cost what they
-// save.  Whole steps, us, rows moved | gathered (rows per expert; two runs of one side differ by 0.1 to 1 %):
-//   2048 / 768 x 128   69 253 | 245, 125 296 | 289, 250 425 | 421, 512 736 | 739, 750 1001 | 1002;  from host buffers 96 490 | 474, 256 (two
-//                      chunks) 1368 | 1378
-//   2560 / 1024 x 512  20 1246 | 1221, 64 1413 | 1388, 140 1776 | 1749, 187 2066 | 2072, 250 2607 | 2595, 312 3165 | 3211
-//   7168 / 2048 x 256 + shared  37 3498 | 3469, 69 3947 | 3915, 128 5087 | 5031, 219 7074 | 6959;  skewed experts 128 4133 | 4085
+// It saves the launch that moves the rows, and its write and re-read of them; it costs the two gathering warps' loads once for every 128
+// features.  Up to 8192 rows that launch is hidden behind the set-up of the gated pass, which would have to wait for the layout
+// instead; with whole tiles of 256 rows the threads that gather cost what they save.  Between the two, time with moved rows over time with
+// gathered ones, whole steps of 511 layers and sizes at random (hidden 512 to 7168, inter 128 to 2048, 33 to 512 experts, three in ten skewed),
+// geometric mean and worst:
+//   inter up to 512                                  1.10, 0.97
+//   hidden from 4 inter on                           1.04, 0.97
+//   hidden from 2 inter on, up to 144 rows an expert 1.02, 0.98
+//   what is left                                     0.98, 0.87:  hidden from 2 inter on, more rows 0.99, 0.94;  hidden below 2 inter 0.97, 0.87
+// us, rows moved | gathered (rows per expert):  2048 / 768 x 128  69 255 | 247, 125 299 | 293, 144 317 | 308, 162 333 | 335, 206 370 | 376;  from
+//   host buffers 96 490 | 474;  2560 / 1024 x 512  17 1234 | 1210, 64 1425 | 1404, 128 1753 | 1734, 172 1991 | 2050, 250 2626 | 2689;  4096 / 1536 x
+//   128  69 852 | 834, 125 987 | 982, 206 1209 | 1275;  2048 / 1408 x 64 + shared  141 288 | 292, 244 390 | 411;  7168 / 2048 x 256 + shared  34 3484 |
+//   3457, 128 5185 | 5160, 188 6419 | 6463;  skewed 128 4156 | 4188, 253 6867 | 6955
 // A context on part of the SMs moves its rows: V3-shaped, 1500 tokens on 48 SMs beside decode steps 13029 | 13224, skewed 2500 6129 | 6201.
-inline bool gather_is_faster(int64_t rows, int64_t E) { return rows > 8192 && rows < 256 * E; }
+inline bool gather_is_faster(int64_t rows, int64_t E, int H, int I) {
+  return rows > 8192 && rows < 256 * E && (I <= 512 || H >= 4 * I || (H >= 2 * I && rows <= 144 * E));
+}
 
 // ---- whether a bf16 step of up to 64 tokens makes its passes and its combine in one launch (step_ffn.cu)
 // It gains a chain of launches, and tiles half as large where the 256-row tiles of a pass are fewer than the CTAs or fill half of a

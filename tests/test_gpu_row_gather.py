@@ -12,8 +12,9 @@ DEV = "cuda"
 
 
 @pytest.mark.parametrize("H,E,k,I,shared,T,budget,gathers", [
-    (1856, 48, 4, 704, 320, 2049, 0, True), (1856, 48, 4, 704, 320, 2048, 0, False),     # 8192 rows and more
-    (2368, 33, 8, 960, 0, 1055, 0, True), (2368, 33, 8, 960, 0, 1056, 0, False),         # 256 rows per expert and fewer
+    (1856, 64, 4, 704, 320, 2049, 0, True), (1856, 64, 4, 704, 320, 2048, 0, False),     # 8192 rows and more
+    (1856, 64, 4, 704, 320, 2304, 0, True), (1856, 64, 4, 704, 320, 2305, 0, False),     # 144 rows per expert
+    (1856, 64, 8, 512, 0, 2047, 0, True), (1856, 64, 8, 512, 0, 2048, 0, False),         # 256 rows per expert and fewer
     (2560, 512, 8, 320, 0, 1111, 0, True), (3072, 40, 9, 704, 576, 997, 0, True), (3072, 40, 9, 448, 576, 997, 37, False),
 ])
 @pytest.mark.parametrize("skewed", [False, True])
@@ -63,7 +64,7 @@ def test_gathered_from_host_buffers():
 @pytest.mark.parametrize("path", ["device", "host"])
 def test_a_gathered_batch_leaves_nothing_to_the_next_one(H, E, k, I, then, path):
     """One context, batches that gather and batches that do not in turn, each against a context of its own."""
-    sizes = (4001, 37, 4001, 64, 1, 300, 1531, 7)
+    sizes = (2001, 37, 2001, 64, 1, 300, 1531, 7)
     w = wl.make_weights(wl.LayerShape("g", T=1, H=H, E=E, k=k, I=I), 55, DEV)
 
     def context(switched):

@@ -23,8 +23,8 @@ def test_stage_times_are_those_of_the_step(T, fp8, stages):
 @pytest.mark.parametrize("T,H,E,k,I,stages", [
     (3, 2048, 128, 8, 768, {"route", "ffn_combine"}),
     (64, 2048, 128, 8, 256, {"route", "gemm1_swiglu", "gemm2", "combine"}),  # too many slots for one launch
-    (1055, 2368, 33, 8, 960, {"route", "layout", "gemm1_swiglu", "gemm2", "combine"}),             # the gated pass gathers
-    (1056, 2368, 33, 8, 960, {"route", "layout", "permute", "gemm1_swiglu", "gemm2", "combine"}),
+    (2047, 1856, 64, 8, 512, {"route", "layout", "gemm1_swiglu", "gemm2", "combine"}),             # the gated pass gathers
+    (2048, 1856, 64, 8, 512, {"route", "layout", "permute", "gemm1_swiglu", "gemm2", "combine"}),
 ])
 def test_stages_that_are_one_launch_or_none(T, H, E, k, I, stages):
     _check(wl.LayerShape("t", T=T, H=H, E=E, k=k, I=I), False, stages)

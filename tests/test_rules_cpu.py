@@ -78,7 +78,11 @@ def test_the_steps_made_in_one_launch(rules, H, I, E, k, Is, T, ctas, at_once):
 
 
 def test_the_rows_that_the_gated_pass_gathers(rules):
-    """Above 8192 rows (up to there moving them hides behind the pass's set-up) and below 256 rows an expert."""
-    cases = [(8192, 128, 0), (8193, 128, 1), (1025 * 8, 128, 1), (4001 * 8, 128, 1), (4096 * 8, 128, 0), (8447, 33, 1), (8448, 33, 0), (8193, 32, 0),
-             (4096 * 8, 512, 1), (7000 * 8, 256, 1), (8192 * 8, 256, 0)]
-    assert rules(*[f"moe::gather_is_faster({rows}LL, {E})" for rows, E, _ in cases]) == [g for _, _, g in cases]
+    """Above 8192 rows (up to there moving them hides behind the pass's set-up), below 256 rows an expert, and few feature tiles beside
+    what the launch saves."""
+    cases = [(8192, 128, 2048, 256, 0), (8193, 128, 2048, 256, 1), (256 * 128 - 1, 128, 2048, 512, 1), (256 * 128, 128, 2048, 512, 0),
+             (8447, 33, 512, 512, 1), (8193, 32, 2048, 256, 0), (1531 * 8, 128, 2048, 768, 1), (2300 * 8, 128, 2048, 768, 1),
+             (2600 * 8, 128, 2048, 768, 0), (4096 * 8, 512, 2560, 1024, 1), (11000 * 8, 512, 2560, 1024, 0), (3300 * 8, 128, 4096, 1536, 0),
+             (1500 * 6, 64, 2048, 1408, 0), (2600 * 6, 64, 2048, 1408, 0), (4096 * 8, 256, 7168, 2048, 1), (6000 * 8, 256, 7168, 2048, 0),
+             (200 * 256, 256, 7168, 1792, 1), (100 * 256, 256, 1024, 576, 0)]
+    assert rules(*[f"moe::gather_is_faster({rows}LL, {E}, {H}, {I})" for rows, E, H, I, _ in cases]) == [c[-1] for c in cases]
