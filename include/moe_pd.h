@@ -70,8 +70,9 @@ typedef enum {
  * and its number of tiles: small-M for every problem of up to 8192 rows and, above that, wherever it was measured ahead
  * (with bf16 the gated pass unless K or the tiles are few, and the down pass unless K is short; with FP8 where K is long or
  * R is small); large-M otherwise.  Above 8192 rows a context without an SM budget first asks for a third kernel, small-M with
- * a tile shared by two SMs, which AUTO alone takes, where that was measured ahead of both.  All of it is a function of T and
- * the context's configuration alone, so a step captured in a CUDA graph replays the kernels it was captured with. */
+ * a tile shared by two SMs, which AUTO alone takes, where that was measured ahead of both.  moe_layer with bf16 weights makes
+ * both passes and the combine of up to 64 tokens in one launch where that was measured ahead of three.  All of it is a function
+ * of T and the context's configuration alone, so a step captured in a CUDA graph replays the kernels it was captured with. */
 typedef enum {
   MOE_GEMM_AUTO = 0,
   MOE_GEMM_LARGE_M = 1,  /* tokens fill the 128-row MMA dimension; for experts of many hundreds of rows,
@@ -411,7 +412,8 @@ moe_status moe_ctx_debug_ptrs_fp8(moe_ctx* ctx, void** xq, float** sx, void** aq
 /* Test/inspection only, host state: the kernels that the last routed gated pass and the last routed down pass were launched
  * with (MOE_GEMM_*, or MOE_KERNEL_PAIR for the kernel that AUTO alone takes; MOE_GEMM_AUTO before the first), and how many
  * tensor maps of the small-M and the pair kernel the context has encoded (none in a step whose operands are those of an
- * earlier step on the same kernel).  Any out-pointer may be NULL. */
+ * earlier step on the same kernel).  A launch that makes both passes and the combine counts as small-M.  Any out-pointer may be
+ * NULL. */
 #define MOE_KERNEL_PAIR 100
 moe_status moe_ctx_debug_gemm(const moe_ctx* ctx, int32_t* gated, int32_t* down, int64_t* maps_encoded);
 

@@ -353,7 +353,7 @@ int gemm_variant_of(const moe_ctx* ctx, const moe::GemmProblem& p) {
   const int v = ctx->cfg.gemm_variant;
   if (v != MOE_GEMM_AUTO) return v;
   if (ctx->cfg.phase == MOE_PHASE_DECODE) return MOE_GEMM_SMALL_M;
-  if (ctx->cfg.row_gather == 1) return MOE_GEMM_LARGE_M;  // only the large-M kernel gathers its rows itself
+  if (ctx->cfg.row_gather == 1) return MOE_GEMM_LARGE_M;  // whose kernel gathers at any size
   if (ctx->preemptible) return MOE_GEMM_SMALL_M;          // only the small-M kernel can stop between tiles
   // problems of up to 8192 rows, whose launches overlap with their neighbours, are 1.5-6 % faster on the small-M kernel
   // at any shape: it builds its tile list and fetches weights before the previous kernel has finished
@@ -370,7 +370,8 @@ int gemm_variant_of(const moe_ctx* ctx, const moe::GemmProblem& p) {
   return moe::small_m_is_faster(p.fp8, p.gated, p.K, p.n_feat, p.rows_bound, p.E, ctas) ? MOE_GEMM_SMALL_M : MOE_GEMM_LARGE_M;
 }
 
-// GEMM1 gathers its rows itself only on the large-M tensor-core variant.
+// row_gather = 1: the staged calls move no rows and the large-M kernel fetches them.  (Whole steps of a context with 0 decide by
+// step_gathers, and the small-M kernel fetches them.)
 bool gathers_rows(const moe_ctx* ctx) {
   const int v = ctx->cfg.gemm_variant;
   return ctx->cfg.row_gather == 1 &&
@@ -382,11 +383,11 @@ cudaError_t run_gemm(moe_ctx* ctx, moe::GemmProblem p, const moe::GemmDenseGroup
   const int variant = gemm_variant_of(ctx, p);
   p.wait_limit_ns = ctx->wait_limit_ns;
   p.debug_stall = ctx->debug_stall;
-  // Every GEMM launch comes after the step's row movement (or after another GEMM launch of the same step), which in turn
+  // A GEMM launch comes after the step's row movement (or after another GEMM launch of the same step), which in turn
   // waited for the layout kernels: the offsets are older than the previous kernel.  The quantisation between the passes
-  // lets the down pass start beside the gated one; the offsets are older than that, too.  Only a step that dispatched its
-  // tokens in one launch has them from the kernel before its gated pass.
-  p.offsets_settled = !(ctx->offsets_fresh && p.gated);
+  // lets the down pass start beside the gated one; the offsets are older than that, too.  But a step that dispatched its tokens in
+  // one launch, and one that gathers its rows, have them from the kernel before their gated pass.
+  p.offsets_settled = !(p.gated && (ctx->offsets_fresh || p.gather_src != nullptr));
   p.tile_counters = reinterpret_cast<int*>(ctx->ws + kTileCounterOffset) + 2 * (ctx->gemm_seq++ % kTileCounterPairs);
   p.max_group_rows = T;
   p.plan = ctx->plans[ctx->cur][(variant == kGemmPair ? 4 : 0) + (p.offsets == nullptr ? 2 : 0) + (p.gated ? 0 : 1)];

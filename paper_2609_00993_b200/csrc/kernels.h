@@ -140,8 +140,9 @@ struct GemmProblem {
   int32_t e_end = -1;      // e_end < 0 means E
   int32_t f_begin = 0;     // ... and output features [f_begin, f_end) only (f_begin a multiple of 256; f_end < 0 means
   int32_t f_end = -1;      // n_feat); a dense group in the same launch then has the same n_feat and range
-  // Row gather (tensor-core large-M gated pass only): when gather_src is set, A is not read; row p of the
-  // operand is gather_src[perm[p] / top_k, :] instead (gather_src is bf16 [T, K], perm is [rows_bound]).
+  // Row gather (bf16 gated pass of the large-M kernel, and of the small-M kernel above kGemmOverlapMaxRows rows): when gather_src
+  // is set, A is not read; row p of the operand is gather_src[perm[p] / top_k, :] instead (gather_src is bf16 [T, K], perm is
+  // [rows_bound]).
   const void* gather_src = nullptr;
   const int32_t* perm = nullptr;
   int32_t top_k = 1;
@@ -237,7 +238,7 @@ cudaError_t launch_gemm_tc(const GemmProblem& p, const GemmDenseGroup* dense, in
                            cudaStream_t stream, int* n_launches);
 // Weight-streaming variant (swap-AB with the MMA N following each expert's row count, up to 256 tokens per tile,
 // operands in a byte ring): the variant for experts of up to a few hundred rows, where the step is bound by the
-// bytes the SMs ingest.  Same contract as launch_gemm_tc; no row gather.
+// bytes the SMs ingest.  Same contract as launch_gemm_tc; row gather in bf16 gated passes above kGemmOverlapMaxRows rows.
 cudaError_t launch_gemm_stream(const GemmProblem& p, const GemmDenseGroup* dense, int max_ctas, int* status,
                                cudaStream_t stream, int* n_launches);
 // Two-CTA variant (swap-AB, a tile multiplied by a pair of SMs): needs clusters of two CTAs, that is whole pairs of free
